@@ -968,10 +968,12 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   const int nsel2 = a->rac_nsel_2;
   uint8_t* mask2 = P(L.mask2);
   if (nsel2 > 0) {
-    // the scores are complete when the first projection ends (integer totals): ranking only
-    s = run_rank(g.keys2, I, nsel2, mask2, a->sel2, st);
-    if (s != QUADS_OK) return s;
-    QUADS_CUDA_OK(launch_kernel(mask_codes_kernel, dim3(di.sm_count * 8), dim3(256), (size_t)(0), st, P(L.r2q_pad), header + kHdrPaddedRows, I, mask2));
+    // the scores are complete when the first projection ends (integer totals)
+    const bool want_mask = a->sel2 || a->hq || a->hsf || a->r2q || a->r2sf;
+    QUADS_CUDA_OK(set_max_dynamic_smem<select_mask_kernel>(16384 * 8 + 16384 / 2));
+    QUADS_CUDA_OK(launch_kernel(select_mask_kernel, dim3(di.sm_count), dim3(kSelectThreads), (size_t)I * 8 + I / 2, st, P(L.r2q_pad), header,
+                                tile_rows, g.keys2, I, nsel2, want_mask ? mask2 : (uint8_t*)nullptr));
+    if (a->sel2) QUADS_CUDA_OK(launch_kernel(sel_list_kernel, dim3(1), dim3(1024), (size_t)0, st, mask2, I, a->sel2));
   } else if (a->r2q) {
     QUADS_CUDA_OK(cudaMemsetAsync(mask2, 0, I, st));
   }

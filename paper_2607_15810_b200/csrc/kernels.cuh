@@ -58,7 +58,9 @@ __global__ void rac_dispatch_kernel(int H, const uint8_t* mask, const int32_t* h
                                     const int32_t* tile_rows, const int32_t* row_token, const uint8_t* xq,
                                     const uint8_t* xsf, const uint8_t* rq, const uint8_t* rsf, uint8_t* xq_pad,
                                     uint8_t* xsf_tiled, uint8_t* rq_pad, uint8_t* rsf_tiled);
-__global__ void mask_codes_kernel(uint8_t* codes, const int* n_rows_ptr, int C, const uint8_t* mask);
+constexpr int kSelectThreads = 512;   // one CTA per SM: the CTAs of an SM would only repeat each other's search
+__global__ void select_mask_kernel(uint8_t* codes, const int32_t* header, const int32_t* tile_rows,
+                                   const unsigned long long* score_keys, int C, int n_sel, uint8_t* mask_out /* or NULL */);
 __global__ void combine_kernel(const uint16_t* y_pad, const int32_t* pos_pad, const float* wts, int T, int H,
                                int topk, uint16_t* out, float* out_f32);
 __global__ void export_site2_kernel(int A, const int32_t* n_rows_ptr, int I, const int32_t* perm, const int32_t* pos_pad,
