@@ -78,6 +78,11 @@ quads_status make_codes_map(CUtensorMap* map, const void* base, uint64_t rows, u
   return r == CUDA_SUCCESS ? QUADS_OK : QUADS_ERR_CUDA;
 }
 
+// The same bytes for row gathers: box one row of 128 bytes.
+quads_status make_gather_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t row_bytes) {
+  return make_codes_map(map, base, rows, row_bytes, 1);
+}
+
 // 2D map over tiled scale factors viewed as [atoms, 128 x u32] (512-byte atoms), box =
 // kGemmKSteps atoms, no swizzle; used by the CTA-pair GEMM only.
 quads_status make_sf_map(CUtensorMap* map, const void* base, uint64_t atoms) {
@@ -266,23 +271,21 @@ int gemm_cta_group_for(int64_t rows, int experts) {
   return rows >= (int64_t)1024 * (experts > 0 ? experts : 1) ? 2 : 1;
 }
 
-// Ranking of C order-preserving 64-bit score keys: mask of the n_sel largest (+ their ascending list).
-quads_status run_rank(const unsigned long long* keys, int C, int n_sel, uint8_t* mask, int32_t* sel_export,
-                      cudaStream_t st) {
+// Ranking of C order-preserving 64-bit score keys: mask of the n_sel largest.
+quads_status run_rank(const unsigned long long* keys, int C, int n_sel, uint8_t* mask, cudaStream_t st) {
   QUADS_CUDA_OK(set_max_dynamic_smem<rank_select_kernel>(128 * 1024));
   QUADS_CUDA_OK(launch_kernel(rank_select_kernel, dim3((C + 15) / 16), dim3(256), (size_t)((size_t)C * 8), st, keys, C, n_sel, mask));
-  if (sel_export) {
-    QUADS_CUDA_OK(launch_kernel(sel_list_kernel, dim3(1), dim3(1024), (size_t)(0), st, mask, C, sel_export));
-  }
-  QUADS_CUDA_OK(cudaGetLastError());
   return QUADS_OK;
 }
 
-quads_status run_select(const float* partials, const int* n_part_ptr, int n_part_mul, int n_part_fixed, int C,
-                        int n_sel, double* slice_sums, unsigned int* counters, unsigned long long* keys,
-                        uint8_t* mask, int32_t* sel_export, cudaStream_t st) {
-  QUADS_CUDA_OK(launch_kernel(score_reduce_kernel, dim3((C + 31) / 32, kScoreSlices), dim3(256), (size_t)(0), st, partials, n_part_ptr, n_part_mul, n_part_fixed, C, slice_sums, counters, keys));
-  return run_rank(keys, C, n_sel, mask, sel_export, st);
+// Selection and masking of a code matrix in one launch (see select_mask_kernel).
+template <bool kDoubleKeys>
+quads_status run_select_mask(uint8_t* codes, int n_rows_fixed, uint32_t flip, const int32_t* header, const int32_t* tile_rows,
+                             const unsigned long long* keys, int C, int n_sel, uint8_t* mask_out, int sm_count, cudaStream_t st) {
+  QUADS_CUDA_OK(set_max_dynamic_smem<select_mask_kernel<kDoubleKeys>>(16384 * 12 + 16384 / 2));
+  QUADS_CUDA_OK(launch_kernel(select_mask_kernel<kDoubleKeys>, dim3(sm_count), dim3(kSelectThreads), (size_t)C * 12 + C / 2, st, codes,
+                              n_rows_fixed, flip, header, tile_rows, keys, C, n_sel, mask_out));
+  return QUADS_OK;
 }
 
 }  // namespace
@@ -725,10 +728,16 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   const size_t pad_rows = (size_t)L.m_tiles_max * 128;
   const int cta_group = gemm_cta_group_for(dense ? (int64_t)T : (int64_t)A, dense ? 1 : E);
 
+  // few rows per expert (decode-sized batches): operands swapped, weights on the M side
+  static const bool no_swap = getenv("QUADS_NO_SWAP") != nullptr;
+  const bool swapped = !dense && !no_swap && cta_group == 1 && gemm_swapped_ok(A, E, L.m_tiles_max);
+  // Few tokens: the front of the call is two kernels of one cluster each (one for a dense projection), which
+  // clear what has to start at zero themselves.
+  const bool small = a->operand_mode == QUADS_W4A4 && cta_group == 1 && front_small_fits(T, H, swapped);
   g_trace.n = 0;
   trace_mark("start", st);
   // header (status word included) and the amax word start at zero
-  QUADS_CUDA_OK(cudaMemsetAsync(ws, 0, L.ids, st));
+  if (!small) QUADS_CUDA_OK(cudaMemsetAsync(ws, 0, L.ids, st));
   trace_mark("memset", st);
 
   if (dense && a->operand_mode != QUADS_W4A4) {
@@ -759,160 +768,207 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
     return QUADS_OK;
   }
 
+  const int nsel13 = a->rac_nsel_13;
+  uint8_t* mask13 = P(L.mask13);
+  if (small) {
+    if (!dense) {
+      SmallRouteArgs r{};
+      r.logits = a->router_logits;
+      r.T = T; r.E = E; r.topk = topk; r.renormalize = a->renormalize; r.e_lo = e_lo; r.e_hi = e_lo + e_cnt;
+      r.wts = wts; r.offsets = offsets; r.tile_prefix = tile_prefix; r.tile_expert = tile_expert; r.tile_rows = tile_rows;
+      r.header = header; r.perm = perm; r.pos_pad = pos_pad; r.row_token = row_token; r.row_weight = row_weight;
+      r.zero_u64 = reinterpret_cast<unsigned long long*>(P(L.keys2)); r.n_zero = I;
+      r.ids_out = a->topk_ids; r.wts_out = a->topk_w; r.offsets_out = a->expert_offsets; r.perm_out = a->perm;
+      if ((s = launch_route_small(r, st)) != QUADS_OK) return s;
+      trace_mark("route", st);
+    }
+    SmallFrontArgs f{};
+    f.x = x; f.T = T; f.H = H; f.topk = topk; f.n_sel = nsel13;
+    f.gs_in = a->a13_gs; f.pos_pad = dense ? nullptr : pos_pad;
+    f.after_routing = !dense; f.token_order = swapped;
+    f.xq_pad = P(swapped ? L.xq_tok : L.xq_pad); f.xsf = P(swapped ? L.xsf_tok : L.xsf);
+    f.rq_pad = P(swapped ? L.rq_tok : L.rq_pad); f.rsf = P(swapped ? L.rsf_tok : L.rsf);
+    f.amax_bits = amax_bits; f.header = header; f.gs_store = a->a13_gs_out;
+    f.mask_out = a->sel13 ? mask13 : nullptr;
+    f.xq_exp = a->xq; f.xsf_exp = a->xsf; f.rq_exp = a->rq; f.rsf_exp = a->rsf;
+    if ((s = launch_front_small(f, st)) != QUADS_OK) return s;
+    if (a->sel13 && nsel13 > 0)
+      QUADS_CUDA_OK(launch_kernel(sel_list_kernel, dim3(1), dim3(1024), (size_t)0, st, mask13, H, a->sel13));
+    trace_mark("front", st);
+  }
+
   // ---- routing and dispatch order: on a side stream, next to the activation chain below
   // (declared in this order: on an early return the guard joins first, then the lock is released)
   std::unique_lock<std::mutex> side_lock(g_side_mu, std::defer_lock);
   SideJoinGuard side_guard;
   SideStream* side = nullptr;
-  if (!dense && !g_trace.enabled) {
-    side_lock.lock();                       // event record / wait pairs of two host threads must not interleave
-    side = side_stream();
-    if (!side) side_lock.unlock();
-  }
-  cudaStream_t rs = st;
-  if (side) {
-    QUADS_CUDA_OK(cudaEventRecord(side->fork, st));
-    QUADS_CUDA_OK(cudaStreamWaitEvent(side->stream, side->fork, 0));
-    side_guard.arm(side, st);
-    rs = side->stream;
-  }
-  if (dense) {
-    QUADS_CUDA_OK(launch_kernel(dense_dispatch_kernel, dim3((T + 255) / 256), dim3(256), (size_t)(0), st, T, cta_group, pos_pad, row_token, row_weight, tile_expert, tile_rows, header));
-  } else {
-    int32_t* chunk_counts = reinterpret_cast<int32_t*>(P(L.chunk_counts));
-    int32_t* chunk_base = reinterpret_cast<int32_t*>(P(L.chunk_base));
-    int32_t* expert_total = reinterpret_cast<int32_t*>(P(L.expert_total));
-    {
-      auto route = E <= 32 ? route_kernel_t<1> : (E <= 64 ? route_kernel_t<2> : (E <= 128 ? route_kernel_t<4> : route_kernel_t<8>));
-      QUADS_CUDA_OK(launch_kernel(route, dim3(L.n_chunks), dim3(256), (size_t)(0), rs, a->router_logits, T, E, topk,
-                                  a->renormalize, ids, wts, chunk_counts, expert_total, a->topk_ids, a->topk_w, e_lo, e_lo + e_cnt));
+  if (!small) {
+    if (!dense && !g_trace.enabled) {
+      side_lock.lock();                       // event record / wait pairs of two host threads must not interleave
+      side = side_stream();
+      if (!side) side_lock.unlock();
     }
-    trace_mark("route", st);
-    QUADS_CUDA_OK(launch_kernel(scan_kernel, dim3(E), dim3(256), (size_t)(0), rs, E, L.n_chunks, cta_group, chunk_counts, expert_total, chunk_base, offsets, tile_prefix, tile_expert, tile_rows, header, a->expert_offsets));
-    trace_mark("scan", st);
-    QUADS_CUDA_OK(launch_kernel(permute_kernel, dim3(L.n_chunks), dim3(128), (size_t)(0), rs, T, E, topk, L.n_chunks, ids, wts, chunk_base, offsets, tile_prefix, perm, pos_pad, row_token, row_weight, a->perm, e_lo, e_lo + e_cnt));
-  }
-  trace_mark("permute", st);
-
-  // ---- per-tensor scale of x
-  // ---- per-tensor scale of x: folded into the quantization kernel (cooperative launch, grid
-  // barrier) when all of its CTAs fit on the GPU at once; else a kernel of its own
-  const int rq_block = H / 16 > 256 ? 256 : (H / 16 + 31) / 32 * 32;
-  static const bool no_fused_amax = getenv("QUADS_NO_FUSED_AMAX") != nullptr;
-  bool fused_amax = false;
-  if (!a->a13_gs && !no_fused_amax && !g_trace.enabled) {
-    // resident CTAs per SM for the two block sizes in use (128 and 256 threads); same on every sm_100 device
-    static std::atomic<int> per_sm_cache[2] = {{0}, {0}};
-    std::atomic<int>& slot = per_sm_cache[rq_block > 128 ? 1 : 0];
-    int per_sm = slot.load();
-    if (per_sm == 0) {
-      QUADS_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rac_quant_kernel, rq_block > 128 ? 256 : 128, 0));
-      slot.store(per_sm);
+    cudaStream_t rs = st;
+    if (side) {
+      QUADS_CUDA_OK(cudaEventRecord(side->fork, st));
+      QUADS_CUDA_OK(cudaStreamWaitEvent(side->stream, side->fork, 0));
+      side_guard.arm(side, st);
+      rs = side->stream;
     }
-    fused_amax = (int64_t)per_sm * di.sm_count >= L.stats_ctas;
-  }
-  if (!a->a13_gs && !fused_amax) {
-    const int64_t chunks = (int64_t)T * (H / 8);
-    int gx = (int)((chunks + 2047) / 2048);
-    if (gx > di.sm_count * 8) gx = di.sm_count * 8;
-    QUADS_CUDA_OK(launch_kernel(amax_kernel, dim3(gx, 1), dim3(256), (size_t)(0), st, x, T, H, H, 0, amax_bits));
-  }
-  trace_mark("amax", st);
-  // ---- site 13: quantize (+ residual + statistics), selection, dispatch scatter
-  const int nsel13 = a->rac_nsel_13;
-  const bool totals13 = (int64_t)L.stats_ctas * H <= ((int64_t)1 << 18);
-  uint8_t* mask13 = P(L.mask13);
-  {
-    const uint16_t* xp = x;
-    int Tt = T, Hh = H, rows_per_cta = L.rows_per_cta, with_res = nsel13 > 0 ? 1 : 0;
-    const float* gs13 = a->a13_gs;
-    unsigned int* arrivals = fused_amax ? reinterpret_cast<unsigned int*>(header + kHdrArrivals) : nullptr;
-    int32_t* status_word = header + kHdrStatus;
-    float* gs_store = a->a13_gs_out;
-    // Column scores of site 13: integer totals added by every CTA when there are few of them (the
-    // selection is then one ranking kernel; decode-sized batches), else one partial row per CTA and a
-    // reduction kernel (586 x 2048 integer reductions at the end of the kernel cost 20 us, the
-    // reduction kernel 9)
-    float* partials = totals13 ? nullptr : reinterpret_cast<float*>(P(L.partials13));
-    unsigned long long* totals = totals13 ? reinterpret_cast<unsigned long long*>(P(L.keys13)) : nullptr;
-    // a CTA's partial sum covers rows_per_cta rows (< rows * 2^18 in units of the squared scale); the
-    // stats_ctas partial sums of a column must fit 62 bits together
-    int cap_bits = 18, ctas_log2 = 0;
-    while ((1 << (cap_bits - 18)) < rows_per_cta) ++cap_bits;
-    while ((1 << ctas_log2) < L.stats_ctas) ++ctas_log2;
-    int score_bits = std::max(0, std::min(26, 62 - cap_bits - ctas_log2));
-    uint8_t *xq_tok = P(L.xq_tok), *xsf_tok = P(L.xsf_tok), *rq_tok = P(L.rq_tok), *rsf_tok = P(L.rsf_tok);
-    uint8_t *xq_exp = a->xq, *xsf_exp = a->xsf;
-    if (fused_amax) {
-      void* args[] = {&xp, &Tt, &Hh, &gs13, &amax_bits, &arrivals, &status_word, &gs_store, &rows_per_cta, &with_res,
-                      &partials, &xq_tok, &xsf_tok, &rq_tok, &rsf_tok, &xq_exp, &xsf_exp, &totals, &score_bits, &cap_bits};
-      QUADS_CUDA_OK(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(rac_quant_kernel), dim3(L.stats_ctas),
-                                                dim3(rq_block), args, 0, st));
-      note_launch();
+    if (dense) {
+      QUADS_CUDA_OK(launch_kernel(dense_dispatch_kernel, dim3((T + 255) / 256), dim3(256), (size_t)(0), st, T, cta_group, pos_pad, row_token, row_weight, tile_expert, tile_rows, header));
     } else {
-      QUADS_CUDA_OK(launch_kernel(rac_quant_kernel, dim3(L.stats_ctas), dim3(rq_block), (size_t)(0), st, xp, Tt, Hh, gs13,
-                                  amax_bits, arrivals, status_word, gs_store, rows_per_cta, with_res, partials, xq_tok,
-                                  xsf_tok, rq_tok, rsf_tok, xq_exp, xsf_exp, totals, score_bits, cap_bits));
+      int32_t* chunk_counts = reinterpret_cast<int32_t*>(P(L.chunk_counts));
+      int32_t* chunk_base = reinterpret_cast<int32_t*>(P(L.chunk_base));
+      int32_t* expert_total = reinterpret_cast<int32_t*>(P(L.expert_total));
+      {
+        auto route = E <= 32 ? route_kernel_t<1> : (E <= 64 ? route_kernel_t<2> : (E <= 128 ? route_kernel_t<4> : route_kernel_t<8>));
+        QUADS_CUDA_OK(launch_kernel(route, dim3(L.n_chunks), dim3(256), (size_t)(0), rs, a->router_logits, T, E, topk,
+                                    a->renormalize, ids, wts, chunk_counts, expert_total, a->topk_ids, a->topk_w, e_lo, e_lo + e_cnt));
+      }
+      trace_mark("route", st);
+      QUADS_CUDA_OK(launch_kernel(scan_kernel, dim3(E), dim3(256), (size_t)(0), rs, E, L.n_chunks, cta_group, chunk_counts, expert_total, chunk_base, offsets, tile_prefix, tile_expert, tile_rows, header, a->expert_offsets));
+      trace_mark("scan", st);
+      QUADS_CUDA_OK(launch_kernel(permute_kernel, dim3(L.n_chunks), dim3(128), (size_t)(0), rs, T, E, topk, L.n_chunks, ids, wts, chunk_base, offsets, tile_prefix, perm, pos_pad, row_token, row_weight, a->perm, e_lo, e_lo + e_cnt));
     }
-  }
-  trace_mark("rac_stats", st);
-  // The dispatched copies of Q(x) need only the dispatch order and the codes: with a side stream
-  // they are written there, next to the channel selection; the residual copies (which need the
-  // selection and the dispatch tables, not the other copies) follow on the main stream and may run
-  // beside them: the two streams meet again only in front of the first projection.
-  const bool split_scatter = side != nullptr && nsel13 > 0;
-  auto dispatch = [&](int parts, cudaStream_t s_) {
-    auto k = parts == 1 ? rac_dispatch_kernel<1> : (parts == 2 ? rac_dispatch_kernel<2> : rac_dispatch_kernel<3>);
-    return launch_kernel(k, dim3(L.m_tiles_max), dim3(256), (size_t)(0), s_, H, mask13, header,
-                         tile_rows, row_token, P(L.xq_tok), P(L.xsf_tok), P(L.rq_tok), P(L.rsf_tok), P(L.xq_pad),
-                         P(L.xsf), P(L.rq_pad), P(L.rsf));
-  };
-  if (side) {
-    if (split_scatter) {
-      QUADS_CUDA_OK(cudaEventRecord(side->tables, side->stream));      // routing tables complete
-      QUADS_CUDA_OK(cudaEventRecord(side->mid, st));
-      QUADS_CUDA_OK(cudaStreamWaitEvent(side->stream, side->mid, 0));
-      QUADS_CUDA_OK(dispatch(1, side->stream));
+    trace_mark("permute", st);
+
+    // ---- per-tensor scale of x
+    // ---- per-tensor scale of x: folded into the quantization kernel (cooperative launch, grid
+    // barrier) when all of its CTAs fit on the GPU at once; else a kernel of its own
+    const int rq_block = H / 16 > 256 ? 256 : (H / 16 + 31) / 32 * 32;
+    static const bool no_fused_amax = getenv("QUADS_NO_FUSED_AMAX") != nullptr;
+    bool fused_amax = false;
+    if (!a->a13_gs && !no_fused_amax && !g_trace.enabled) {
+      // resident CTAs per SM for the two block sizes in use (128 and 256 threads); same on every sm_100 device
+      static std::atomic<int> per_sm_cache[2] = {{0}, {0}};
+      std::atomic<int>& slot = per_sm_cache[rq_block > 128 ? 1 : 0];
+      int per_sm = slot.load();
+      if (per_sm == 0) {
+        QUADS_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rac_quant_kernel, rq_block > 128 ? 256 : 128, 0));
+        slot.store(per_sm);
+      }
+      fused_amax = (int64_t)per_sm * di.sm_count >= L.stats_ctas;
     }
-  }
-  if (nsel13 > 0) {
-    if (totals13)
-      s = run_rank(reinterpret_cast<unsigned long long*>(P(L.keys13)), H, nsel13, mask13, a->sel13, st);
-    else
-      s = run_select(reinterpret_cast<float*>(P(L.partials13)), nullptr, 1, L.stats_ctas, H, nsel13,
-                     reinterpret_cast<double*>(P(L.scores13)), reinterpret_cast<unsigned int*>(P(L.counters13)),
-                     reinterpret_cast<unsigned long long*>(P(L.keys13)), mask13, a->sel13, st);
-    if (s != QUADS_OK) return s;
-  }
-  trace_mark("select13", st);
-  if (split_scatter) {
-    QUADS_CUDA_OK(cudaStreamWaitEvent(st, side->tables, 0));
-  } else if (side) {
-    side_guard.join();
-    side_lock.unlock();
-  }
-  {
-    const int parts = split_scatter ? 2 : (nsel13 > 0 ? 3 : 1);
-    QUADS_CUDA_OK(dispatch(parts, st));
-    if (nsel13 > 0 && (a->rq || a->rsf)) {
-      // verification export of the masked residual in token order (no dispatched copies: top-k of 0)
-      const int64_t chunks = (int64_t)T * (H / 32);
-      QUADS_CUDA_OK(launch_kernel(rac_scatter_kernel, dim3((unsigned)((chunks + 255) / 256)), dim3(256), (size_t)(0), st, T, H, 2, mask13, 0, pos_pad, P(L.xq_tok), P(L.xsf_tok), P(L.rq_tok), P(L.rsf_tok), P(L.xq_pad), P(L.xsf), P(L.rq_pad), P(L.rsf), a->rq, a->rsf));
+    if (!a->a13_gs && !fused_amax) {
+      const int64_t chunks = (int64_t)T * (H / 8);
+      int gx = (int)((chunks + 2047) / 2048);
+      if (gx > di.sm_count * 8) gx = di.sm_count * 8;
+      QUADS_CUDA_OK(launch_kernel(amax_kernel, dim3(gx, 1), dim3(256), (size_t)(0), st, x, T, H, H, 0, amax_bits));
     }
+    trace_mark("amax", st);
+    // ---- site 13: quantize (+ residual + statistics), selection, dispatch scatter
+    const bool totals13 = (int64_t)L.stats_ctas * H <= ((int64_t)1 << 18);
+    {
+      const uint16_t* xp = x;
+      int Tt = T, Hh = H, rows_per_cta = L.rows_per_cta, with_res = nsel13 > 0 ? 1 : 0;
+      const float* gs13 = a->a13_gs;
+      unsigned int* arrivals = fused_amax ? reinterpret_cast<unsigned int*>(header + kHdrArrivals) : nullptr;
+      int32_t* status_word = header + kHdrStatus;
+      float* gs_store = a->a13_gs_out;
+      // Column scores of site 13: integer totals added by every CTA when there are few of them (the
+      // selection is then one ranking kernel; decode-sized batches), else one partial row per CTA and a
+      // reduction kernel (586 x 2048 integer reductions at the end of the kernel cost 20 us, the
+      // reduction kernel 9)
+      float* partials = totals13 ? nullptr : reinterpret_cast<float*>(P(L.partials13));
+      unsigned long long* totals = totals13 ? reinterpret_cast<unsigned long long*>(P(L.keys13)) : nullptr;
+      // a CTA's partial sum covers rows_per_cta rows (< rows * 2^18 in units of the squared scale); the
+      // stats_ctas partial sums of a column must fit 62 bits together
+      int cap_bits = 18, ctas_log2 = 0;
+      while ((1 << (cap_bits - 18)) < rows_per_cta) ++cap_bits;
+      while ((1 << ctas_log2) < L.stats_ctas) ++ctas_log2;
+      int score_bits = std::max(0, std::min(26, 62 - cap_bits - ctas_log2));
+      uint8_t *xq_tok = P(L.xq_tok), *xsf_tok = P(L.xsf_tok), *rq_tok = P(L.rq_tok), *rsf_tok = P(L.rsf_tok);
+      uint8_t *xq_exp = a->xq, *xsf_exp = a->xsf;
+      if (fused_amax) {
+        void* args[] = {&xp, &Tt, &Hh, &gs13, &amax_bits, &arrivals, &status_word, &gs_store, &rows_per_cta, &with_res,
+                        &partials, &xq_tok, &xsf_tok, &rq_tok, &rsf_tok, &xq_exp, &xsf_exp, &totals, &score_bits, &cap_bits};
+        QUADS_CUDA_OK(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(rac_quant_kernel), dim3(L.stats_ctas),
+                                                  dim3(rq_block), args, 0, st));
+        note_launch();
+      } else {
+        QUADS_CUDA_OK(launch_kernel(rac_quant_kernel, dim3(L.stats_ctas), dim3(rq_block), (size_t)(0), st, xp, Tt, Hh, gs13,
+                                    amax_bits, arrivals, status_word, gs_store, rows_per_cta, with_res, partials, xq_tok,
+                                    xsf_tok, rq_tok, rsf_tok, xq_exp, xsf_exp, totals, score_bits, cap_bits));
+      }
+    }
+    trace_mark("rac_stats", st);
+    unsigned long long* keys13 = reinterpret_cast<unsigned long long*>(P(L.keys13));
+    if (nsel13 > 0 && !totals13) {
+      QUADS_CUDA_OK(launch_kernel(score_reduce_kernel, dim3((H + 31) / 32, kScoreSlices), dim3(256), (size_t)0, st,
+                                  reinterpret_cast<float*>(P(L.partials13)), (const int*)nullptr, 1, L.stats_ctas, H,
+                                  reinterpret_cast<double*>(P(L.scores13)), reinterpret_cast<unsigned int*>(P(L.counters13)), keys13));
+    }
+    // verification exports of the selection and, from codes stored with `flip` applied, of the masked residual
+    auto export13 = [&](uint32_t flip) -> quads_status {
+      if (a->sel13) QUADS_CUDA_OK(launch_kernel(sel_list_kernel, dim3(1), dim3(1024), (size_t)0, st, mask13, H, a->sel13));
+      if (a->rq || a->rsf) {
+        const int64_t chunks = (int64_t)T * (H / 32);
+        QUADS_CUDA_OK(launch_kernel(export_residual_kernel, dim3((unsigned)((chunks + 255) / 256)), dim3(256), (size_t)0, st, T, H,
+                                    mask13, flip, P(L.rq_tok), P(L.rsf_tok), a->rq, a->rsf));
+      }
+      return QUADS_OK;
+    };
+    if (swapped) {
+      // the first projection gathers out of the token-order codes: the residual is masked and negated in place
+      if (nsel13 > 0) {
+        uint8_t* mask_out = (a->sel13 || a->rq) ? mask13 : nullptr;
+        s = totals13 ? run_select_mask<false>(P(L.rq_tok), T, 0x88888888u, header, tile_rows, keys13, H, nsel13, mask_out, di.sm_count, st)
+                     : run_select_mask<true>(P(L.rq_tok), T, 0x88888888u, header, tile_rows, keys13, H, nsel13, mask_out, di.sm_count, st);
+        if (s != QUADS_OK || (s = export13(0x88888888u)) != QUADS_OK) return s;
+      }
+      trace_mark("select13+mask", st);
+      if (side) {
+        side_guard.join();
+        side_lock.unlock();
+      }
+    } else {
+      // The dispatched copies of Q(x) need only the dispatch order and the codes: with a side stream
+      // they are written there, next to the channel selection; the residual copies (which need the
+      // selection and the dispatch tables, not the other copies) follow on the main stream and may run
+      // beside them: the two streams meet again only in front of the first projection.
+      const bool split_scatter = side != nullptr && nsel13 > 0;
+      auto dispatch = [&](int parts, cudaStream_t s_) {
+        auto k = parts == 1 ? rac_dispatch_kernel<1> : (parts == 2 ? rac_dispatch_kernel<2> : rac_dispatch_kernel<3>);
+        return launch_kernel(k, dim3(L.m_tiles_max), dim3(256), (size_t)(0), s_, H, mask13, header,
+                             tile_rows, row_token, P(L.xq_tok), P(L.xsf_tok), P(L.rq_tok), P(L.rsf_tok), P(L.xq_pad),
+                             P(L.xsf), P(L.rq_pad), P(L.rsf));
+      };
+      if (split_scatter) {
+        QUADS_CUDA_OK(cudaEventRecord(side->tables, side->stream));      // routing tables complete
+        QUADS_CUDA_OK(cudaEventRecord(side->mid, st));
+        QUADS_CUDA_OK(cudaStreamWaitEvent(side->stream, side->mid, 0));
+        QUADS_CUDA_OK(dispatch(1, side->stream));
+      }
+      if (nsel13 > 0) {
+        if ((s = run_rank(keys13, H, nsel13, mask13, st)) != QUADS_OK) return s;
+        if ((s = export13(0u)) != QUADS_OK) return s;
+      }
+      trace_mark("select13", st);
+      if (split_scatter) {
+        QUADS_CUDA_OK(cudaStreamWaitEvent(st, side->tables, 0));
+      } else if (side) {
+        side_guard.join();
+        side_lock.unlock();
+      }
+      QUADS_CUDA_OK(dispatch(split_scatter ? 2 : (nsel13 > 0 ? 3 : 1), st));
+      if (split_scatter) {
+        side_guard.join();
+        side_lock.unlock();
+      }
+    }
+    trace_mark("rac_dispatch", st);
   }
-  if (split_scatter) {
-    side_guard.join();
-    side_lock.unlock();
-  }
-  trace_mark("rac_dispatch", st);
   // ---- tensor maps
-  // few rows per expert (decode-sized batches): operands swapped, weights on the M side
-  static const bool no_swap = getenv("QUADS_NO_SWAP") != nullptr;
-  const bool swapped = !dense && !no_swap && cta_group == 1 && gemm_swapped_ok(A, E, L.m_tiles_max);
   const uint32_t act_box = swapped ? 16 : 128;
   GemmMaps m1;
-  if ((s = make_codes_map(&m1.a, P(L.xq_pad), pad_rows, H / 2, act_box)) != QUADS_OK) return s;
-  if ((s = make_codes_map(&m1.r, P(L.rq_pad), pad_rows, H / 2, act_box)) != QUADS_OK) return s;
+  if (swapped) {                                    // the first projection gathers its rows out of the token-order codes
+    if ((s = make_gather_map(&m1.a, P(L.xq_tok), T, H / 2)) != QUADS_OK) return s;
+    if ((s = make_gather_map(&m1.r, P(L.rq_tok), T, H / 2)) != QUADS_OK) return s;
+  } else {
+    if ((s = make_codes_map(&m1.a, P(L.xq_pad), pad_rows, H / 2, act_box)) != QUADS_OK) return s;
+    if ((s = make_codes_map(&m1.r, P(L.rq_pad), pad_rows, H / 2, act_box)) != QUADS_OK) return s;
+  }
   if ((s = make_codes_map(&m1.b, a->w13_q, (uint64_t)e_cnt * N1, H / 2)) != QUADS_OK) return s;
   if (cta_group == 2) {
     const uint64_t a_atoms = (uint64_t)(pad_rows / 128) * (H / 64);
@@ -928,14 +984,15 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   g.a_sf = P(L.xsf); g.r_sf = P(L.rsf);
   g.b_sf = a->w13_sf; g.b_sf_expert_stride = quads_sf_tiled_bytes(N1, H);
   g.b_gs = a->w13_gs; g.a_gs = a->a13_gs; g.a_amax_bits = amax_bits;
-  g.row_token = row_token; g.row_weight = row_weight;
   g.tile_prefix = tile_prefix; g.offsets = offsets;
+  g.row_token = row_token; g.xsf_tok = P(L.xsf_tok); g.rsf_tok = P(L.rsf_tok);
   g.status = header + kHdrStatus;
   g.b_rows_per_expert = N1;
   g.n_experts = e_cnt;
   g.expert_lo = e_lo;
   if (dense) {
     g.n_out = a->N;
+    g.dense_rows = T;
     g.n_tiles_n = (a->N + 255) / 256;
     g.half1_row_offset = 128;
     g.out_bf16 = static_cast<uint16_t*>(a->out);
@@ -970,9 +1027,9 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   if (nsel2 > 0) {
     // the scores are complete when the first projection ends (integer totals)
     const bool want_mask = a->sel2 || a->hq || a->hsf || a->r2q || a->r2sf;
-    QUADS_CUDA_OK(set_max_dynamic_smem<select_mask_kernel>(16384 * 8 + 16384 / 2));
-    QUADS_CUDA_OK(launch_kernel(select_mask_kernel, dim3(di.sm_count), dim3(kSelectThreads), (size_t)I * 8 + I / 2, st, P(L.r2q_pad), header,
-                                tile_rows, g.keys2, I, nsel2, want_mask ? mask2 : (uint8_t*)nullptr));
+    if ((s = run_select_mask<false>(P(L.r2q_pad), 0, 0u, header, tile_rows, g.keys2, I, nsel2, want_mask ? mask2 : nullptr,
+                                    di.sm_count, st)) != QUADS_OK)
+      return s;
     if (a->sel2) QUADS_CUDA_OK(launch_kernel(sel_list_kernel, dim3(1), dim3(1024), (size_t)0, st, mask2, I, a->sel2));
   } else if (a->r2q) {
     QUADS_CUDA_OK(cudaMemsetAsync(mask2, 0, I, st));

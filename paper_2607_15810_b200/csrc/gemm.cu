@@ -163,13 +163,13 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p, const CUtensorMap
   // Per-tile metadata (expert, valid rows) and the per-expert weight scales are read by every
   // role at every tile; dependent global loads there would sit on the critical path of short K
   // loops, so they are staged in shared memory once (single-CTA variant, when they fit).
-  const int m_tiles_all = p.header[kHdrMTiles];
+  const int m_tiles_all = EPI == kEpiStore ? (p.dense_rows + kBM * CG - 1) / (kBM * CG) * CG : p.header[kHdrMTiles];
   float* inv_lut = reinterpret_cast<float*>(smem_gen + C::kBarOffset + 256);   // 128 entries, SwiGLU epilogue
   if (EPI == kEpiSwiGLU && threadIdx.x < 128) inv_lut[threadIdx.x] = quant_inv_entry(threadIdx.x, p.h_gs[0]);
   uint8_t* tab_expert = smem_gen + C::kBarOffset + 256 + 512;
   uint8_t* tab_rows = tab_expert + kMaxTableTiles;
   float* tab_gs = reinterpret_cast<float*>(tab_rows + kMaxTableTiles);
-  const bool tables = (CG == 1) && m_tiles_all <= kMaxTableTiles && p.n_experts <= kMaxExperts;
+  const bool tables = (CG == 1) && EPI != kEpiStore && m_tiles_all <= kMaxTableTiles && p.n_experts <= kMaxExperts;
   if (tables) {
     for (int i = threadIdx.x; i < m_tiles_all; i += blockDim.x) {
       tab_expert[i] = (uint8_t)p.tile_expert[i];
@@ -182,8 +182,9 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p, const CUtensorMap
   // and the activation amax need that kernel.
   pdl_sync();
   __syncthreads();                          // tables and the reciprocal table are visible to every role
-  auto expert_of = [&](int mt) -> int { return tables ? (int)tab_expert[mt] : p.tile_expert[mt]; };
-  auto rows_of = [&](int mt) -> int { return tables ? (int)tab_rows[mt] : p.tile_rows[mt]; };
+  // (a dense projection has one weight and its rows in order: no tables)
+  auto expert_of = [&](int mt) -> int { return EPI == kEpiStore ? 0 : tables ? (int)tab_expert[mt] : p.tile_expert[mt]; };
+  auto rows_of = [&](int mt) -> int { return EPI == kEpiStore ? max(0, min(kBM, p.dense_rows - mt * kBM)) : tables ? (int)tab_rows[mt] : p.tile_rows[mt]; };
   auto gs_of = [&](int e) -> float { return tables ? tab_gs[e] : p.b_gs[e]; };
 
   const int m_groups = m_tiles_all / CG;            // M-tiles come in groups of CG (same expert)
@@ -454,7 +455,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p, const CUtensorMap
       } else {
         const int n0 = nt * 256 + cq * 64;
         if (valid && n0 < p.n_out) {
-          uint4* dst = reinterpret_cast<uint4*>(p.out_bf16 + (size_t)p.row_token[prow] * p.n_out + n0);
+          uint4* dst = reinterpret_cast<uint4*>(p.out_bf16 + (size_t)prow * p.n_out + n0);
 #pragma unroll
           for (int i = 0; i < 8; ++i)
             dst[i] = make_uint4(f32x2_to_bf16x2(acc[8 * i] * scale, acc[8 * i + 1] * scale),

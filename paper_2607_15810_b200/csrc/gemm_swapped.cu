@@ -8,13 +8,21 @@
 //
 //   Dt[f, t] = sum_k  W^[e, f, k] X^[t, k]  +  sum_k  W^[e, f, k] (-M R^)[t, k]
 //
-// with the same operands, scales and dispatch layout as the row-major kernel (gemm.cu): the
-// quantized activations / residuals sit in padded dispatch order (128-row slots per expert), a
-// chunk is one quarter (32 consecutive rows) of a slot.  Its block scales are column `chunk` of the
-// slot's 128-row scale atom, but the MMA accepts N-side scales only at even column offsets: an odd
-// chunk is therefore computed as the second half of a 64-row N tile whose first 32 rows are whatever
-// precedes the chunk's rows in shared memory (the operand descriptor starts 4 KB early; those
-// accumulator columns are never read), with the scales read from the even column before it.
+// on 128-row slots per expert as in the row-major kernel (gemm.cu); a chunk is one quarter (32
+// consecutive rows) of a slot.
+//
+// The first projection gathers: a chunk's rows come straight out of the token-order codes (TMA gather, four
+// rows per instruction) and its scales out of the token-order scales (16 bytes per row and stage, through
+// registers, into column 0 of an atom of its own), so that nothing has to copy every token to its top-k
+// places first (16 writing SMs took 10 us for that at 256 tokens).  For the few rows of a chunk that is
+// a handful of instructions per stage for a warp of its own; for 128-row tiles it was measured slower than the
+// copy (gemm.cu's operands are copied).
+// The second projection's operands are written in padded dispatch order by the first one's epilogue, with
+// tiled scales.  A chunk's scales are then column `chunk` of the slot's 128-row scale atom, but the MMA
+// accepts N-side scales only at even column offsets: an odd chunk is computed as the second half of a
+// 64-row N tile whose first 32 rows are whatever precedes the chunk's rows in shared memory (the operand
+// descriptor starts 4 KB early; those accumulator columns are never read), with the scales read from the
+// even column before it.
 // Small activation tiles leave room for four (six) stages of weights: what bounds this kernel is
 // the number of weight bytes in flight per SM, not the MMAs.
 //
@@ -24,8 +32,10 @@
 //                      as in the row-major kernel (codes, scales, residual, column scores);
 //   second projection: tile = 128 output features; epilogue = bf16 rows for the combine kernel.
 //
-// Roles: warp 0 producer (TMA + bulk copies, ring of stages), warp 1 MMA issuer, warps 2..9
-// epilogue (thread = feature, 16 token columns each).  Two accumulator buffers.  Every wait is
+// Roles: warp 0 loads weights and their scales into a ring of stages, warp 10 the activation side, warp 1
+// issues the MMAs, warps 2..9 are the epilogue (thread = feature, 16 token columns each).  Two accumulator
+// buffers.  Only the activation side and the epilogue wait for the preceding kernel: the weights and the
+// routing tables are older, so the ring fills while that kernel still runs.  Every wait is
 // bounded (status word, as in gemm.cu).
 #include "kernels.cuh"
 #include "tcgen05.cuh"
@@ -43,7 +53,8 @@ constexpr int kTileW = 128 * kStageKBytes;          // 128 weight rows of one st
 constexpr int kTileX = kChunk * kStageKBytes;       // one chunk of activation rows
 constexpr int kSfStage = kKSteps * 512;             // one 128-row scale atom per K step
 constexpr int kEpiWarps = 8;
-constexpr int kThreads = 64 + 32 * kEpiWarps;
+constexpr int kThreads = 64 + 32 * kEpiWarps + 32;
+constexpr int kActWarp = 2 + kEpiWarps;             // loads the activation / residual rows and their scales
 constexpr int kMaxChunkList = 2048;                 // (slot, chunk) entries, 2 bytes each
 constexpr int kMaxSlots = kMaxChunkList / 4;
 constexpr int kTmemCols = 512;
@@ -94,6 +105,20 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// Four rows of the tensor map (box: one row) into 4 x 128 bytes, swizzled like a tile.
+__device__ __forceinline__ void tma_gather4(uint32_t dst, const CUtensorMap* map, int x, int y0, int y1, int y2, int y3, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cta.global.tile::gather4.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
+      ::"r"(dst), "l"(map), "r"(x), "r"(y0), "r"(y1), "r"(y2), "r"(y3), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void st_shared_u32(uint32_t addr, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+// 16 scale bytes of one row and stage (8 in a stage of two K steps; rows start at multiples of 8 bytes).
+__device__ __forceinline__ uint4 load_row_scales(const uint8_t* p, int atoms) {
+  const uint2 a = __ldg(reinterpret_cast<const uint2*>(p));
+  const uint2 b = atoms > 2 ? __ldg(reinterpret_cast<const uint2*>(p) + 1) : make_uint2(0u, 0u);
+  return make_uint4(a.x, a.y, b.x, b.y);
+}
+
 __device__ __forceinline__ void epi_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory"); }
 // Barrier over the epilogue warps that also agrees on `ok` (true only if true in every thread), so
 // that the warps leave the item loop together when a wait was abandoned.
@@ -121,7 +146,7 @@ gemm_swapped_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_x
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) { mbar_init(bar_full + 8 * s, 1); mbar_init(bar_empty + 8 * s, 1); }
+    for (int s = 0; s < kStages; ++s) { mbar_init(bar_full + 8 * s, 2); mbar_init(bar_empty + 8 * s, 1); }   // full: both loading warps
     for (int b = 0; b < 2; ++b) { mbar_init(bar_tfull + 8 * b, 1); mbar_init(bar_tempty + 8 * b, kEpiWarps); }
     bars->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -167,10 +192,10 @@ gemm_swapped_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_x
     }
     if (lane == 0) bars->n_items_chunks = total;
   }
-  // Everything above reads only what kernels before the preceding one produced (routing tables,
-  // weight scales): it overlaps the preceding kernel's tail.  The operands need that kernel.
-  pdl_sync();
   __syncthreads();
+  // Up to here, and in the weight loader, only what kernels before the preceding one produced is read (routing
+  // tables, weights): it overlaps the preceding kernel.  The other roles wait for that kernel in their branch.
+  if (warp < 2) asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); else pdl_sync();
   const int n_chunks = bars->n_items_chunks;
   const int n_ft = p.n_tiles_n;                       // feature tiles of 128
   const int total_items = n_chunks * n_ft;
@@ -179,23 +204,18 @@ gemm_swapped_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_x
   const bool resid = p.has_resid != 0;
 
   if (warp == 0) {
-    // ------------------------------------------------------------ producer
+    // ------------------------------------------------------------ weight loader
     const bool issuer = elect_one();
     uint32_t stage = 0, phase = 0;
     bool ok = true;
     for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x) {
       const int ch = item / n_ft, ft = item - ch * n_ft;
-      const int mt = chunk_list[ch] >> 2, c = chunk_list[ch] & 3;
-      const int e = (int)tab_expert[mt] - p.expert_lo;                 // index into this call's weights
+      const int e = (int)tab_expert[chunk_list[ch] >> 2] - p.expert_lo;   // index into this call's weights
       const int wrow0 = e * p.b_rows_per_expert + ft * 128;            // gate rows (or the only rows)
       const int wrow1 = wrow0 + p.half1_row_offset;                   // up rows
-      const int xrow = mt * 128 + c * kChunk;
       const uint8_t* wsf = p.b_sf + (size_t)e * p.b_sf_expert_stride;
       const uint8_t* wsf0 = wsf + (size_t)ft * kt_count * 512u;
       const uint8_t* wsf1 = wsf + (size_t)((p.half1_row_offset >> 7) + ft) * kt_count * 512u;
-      const uint8_t* xsf = p.a_sf + (size_t)mt * kt_count * 512u;
-      const uint8_t* rsf = p.r_sf + (size_t)mt * kt_count * 512u;
-      const int n_box = (min(kChunk, (int)tab_rows[mt] - c * kChunk) + kBoxRows - 1) / kBoxRows;   // 1 or 2
       for (int ks = 0; ks < k_stages; ++ks) {
         ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, p.status);
         if (!ok) break;
@@ -206,26 +226,91 @@ gemm_swapped_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_x
           const uint32_t full = bar_full + 8 * stage;
           const int kc = ks * kStageKBytes;
           const size_t sf_off = (size_t)ks * (size_t)kSfStage;
-          mbar_expect_tx(full, (uint32_t)(C::kNumW * kTileW + n_box * (kBoxRows * kStageKBytes) * (resid ? 2 : 1)) +
-                                   sf_bytes * (uint32_t)(C::kNumW + (resid ? 2 : 1)));
+          mbar_expect_tx(full, (uint32_t)C::kNumW * (kTileW + sf_bytes));
           tma_load_2d(sb, &tm_w, kc, wrow0, full);
           if (kDual) tma_load_2d(sb + kTileW, &tm_w, kc, wrow1, full);
-          for (int b = 0; b < n_box; ++b) {
-            tma_load_2d(sb + C::kOffX + b * (kBoxRows * kStageKBytes), &tm_x, kc, xrow + b * kBoxRows, full);
-            if (resid) tma_load_2d(sb + C::kOffR + b * (kBoxRows * kStageKBytes), &tm_r, kc, xrow + b * kBoxRows, full);
-          }
           bulk_load(sb + C::kOffSfW, wsf0 + sf_off, sf_bytes, full);
           if (kDual) bulk_load(sb + C::kOffSfW + kSfStage, wsf1 + sf_off, sf_bytes, full);
-          bulk_load(sb + C::kOffSfX, xsf + sf_off, sf_bytes, full);
-          if (resid) bulk_load(sb + C::kOffSfR, rsf + sf_off, sf_bytes, full);
         }
         __syncwarp();
         if (++stage == kStages) { stage = 0; phase ^= 1u; }
       }
     }
-    for (int s = 0; s < kStages && ok; ++s) {          // drain
+    for (int s = 0; s < kStages && ok; ++s) {          // drain: every armed stage lands and is consumed before the CTA may exit
       ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, p.status);
       if (++stage == kStages) { stage = 0; phase ^= 1u; }
+    }
+  } else if (warp == kActWarp) {
+    // ------------------------------------------------------------ activation loader
+    uint32_t stage = 0, phase = 0;
+    bool ok = true;
+    for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x) {
+      const int ch = item / n_ft;
+      const int mt = chunk_list[ch] >> 2, c = chunk_list[ch] & 3;
+      const int n_rows = min(kChunk, (int)tab_rows[mt] - c * kChunk);
+      if (kDual) {
+        // lane = row of the chunk (rows beyond the valid ones repeat the last); lanes 0..7 gather four rows of
+        // codes each, lanes 8..15 four rows of the residual
+        const int tok = p.row_token[mt * 128 + c * kChunk + min(lane, n_rows - 1)];
+        const int g4 = (lane & 7) * 4;
+        const int y0 = __shfl_sync(0xFFFFFFFFu, tok, g4), y1 = __shfl_sync(0xFFFFFFFFu, tok, g4 + 1);
+        const int y2 = __shfl_sync(0xFFFFFFFFu, tok, g4 + 2), y3 = __shfl_sync(0xFFFFFFFFu, tok, g4 + 3);
+        const bool gathers = g4 < n_rows && (lane < 8 || (resid && lane < 16));
+        const CUtensorMap* map = lane < 8 ? &tm_x : &tm_r;
+        const uint32_t dst = (lane < 8 ? C::kOffX : C::kOffR) + (uint32_t)g4 * kStageKBytes;
+        const uint32_t bytes = (uint32_t)((n_rows + 3) / 4) * (4 * kStageKBytes) * (resid ? 2u : 1u);
+        const size_t so = (size_t)tok * (p.K >> 4);
+        uint4 vx = load_row_scales(p.xsf_tok + so, min(kKSteps, kt_count)), vr = make_uint4(0, 0, 0, 0);
+        if (resid) vr = load_row_scales(p.rsf_tok + so, min(kKSteps, kt_count));
+        for (int ks = 0; ks < k_stages; ++ks) {
+          ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, p.status);
+          if (!ok) break;
+          const int atoms = min(kKSteps, kt_count - ks * kKSteps);
+          const uint32_t sb = smem_base + stage * C::kStageBytes, full = bar_full + 8 * stage;
+          if (gathers) tma_gather4(sb + dst, map, ks * kStageKBytes, y0, y1, y2, y3, full);
+          const uint32_t ax = sb + C::kOffSfX + lane * 16, ar = sb + C::kOffSfR + lane * 16;
+          st_shared_u32(ax, vx.x); st_shared_u32(ax + 512, vx.y);
+          if (atoms > 2) { st_shared_u32(ax + 1024, vx.z); st_shared_u32(ax + 1536, vx.w); }
+          if (resid) {
+            st_shared_u32(ar, vr.x); st_shared_u32(ar + 512, vr.y);
+            if (atoms > 2) { st_shared_u32(ar + 1024, vr.z); st_shared_u32(ar + 1536, vr.w); }
+          }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // the copies to tensor memory read these words
+          __syncwarp();
+          if (lane == 0) mbar_expect_tx(full, bytes);
+          if (ks + 1 < k_stages) {                     // the next stage's scales, a stage ahead of their use
+            const int na = min(kKSteps, kt_count - (ks + 1) * kKSteps);
+            vx = load_row_scales(p.xsf_tok + so + (ks + 1) * 16, na);
+            if (resid) vr = load_row_scales(p.rsf_tok + so + (ks + 1) * 16, na);
+          }
+          if (++stage == kStages) { stage = 0; phase ^= 1u; }
+        }
+      } else {
+        const bool issuer = elect_one();
+        const int xrow = mt * 128 + c * kChunk;
+        const uint8_t* xsf = p.a_sf + (size_t)mt * kt_count * 512u;
+        const uint8_t* rsf = p.r_sf + (size_t)mt * kt_count * 512u;
+        const int n_box = (n_rows + kBoxRows - 1) / kBoxRows;          // 1 or 2
+        for (int ks = 0; ks < k_stages; ++ks) {
+          ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, p.status);
+          if (!ok) break;
+          if (issuer) {
+            const uint32_t sf_bytes = (uint32_t)min(kKSteps, kt_count - ks * kKSteps) * 512u;
+            const uint32_t sb = smem_base + stage * C::kStageBytes, full = bar_full + 8 * stage;
+            const int kc = ks * kStageKBytes;
+            const size_t sf_off = (size_t)ks * (size_t)kSfStage;
+            mbar_expect_tx(full, (uint32_t)(n_box * (kBoxRows * kStageKBytes) + sf_bytes) * (resid ? 2u : 1u));
+            for (int b = 0; b < n_box; ++b) {
+              tma_load_2d(sb + C::kOffX + b * (kBoxRows * kStageKBytes), &tm_x, kc, xrow + b * kBoxRows, full);
+              if (resid) tma_load_2d(sb + C::kOffR + b * (kBoxRows * kStageKBytes), &tm_r, kc, xrow + b * kBoxRows, full);
+            }
+            bulk_load(sb + C::kOffSfX, xsf + sf_off, sf_bytes, full);
+            if (resid) bulk_load(sb + C::kOffSfR, rsf + sf_off, sf_bytes, full);
+          }
+          __syncwarp();
+          if (++stage == kStages) { stage = 0; phase ^= 1u; }
+        }
+      }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
@@ -237,10 +322,11 @@ gemm_swapped_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_x
     constexpr uint32_t kSfHi = (uint32_t)(128 >> 4) | (1u << 14);
     for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x, ++it) {
       const int ch = item / n_ft;
-      const int mt = chunk_list[ch] >> 2, c = chunk_list[ch] & 3;
-      const int n_rows = min(kChunk, (int)tab_rows[mt] - c * kChunk);
+      const int mt = chunk_list[ch] >> 2, quarter = chunk_list[ch] & 3;
+      const int n_rows = min(kChunk, (int)tab_rows[mt] - quarter * kChunk);
       const int n_pad = (n_rows + 15) & ~15;                          // 16 or 32 token rows
-      const int n_lead = (c & 1) * kChunk;                            // odd chunk: 32 rows of filler come first
+      const int c = kDual ? 0 : quarter;                              // column of the atoms that holds the chunk's scales
+      const int n_lead = (c & 1) * kChunk;                            // odd column: 32 rows of filler come first
       const int n_mma = n_lead + n_pad;                               // N of the MMAs: 16 .. 64
       // E2M1 x E2M1, UE4M3 block scales, both operands K-major, M = 128, N = n_mma
       const uint32_t idesc = (1u << 7) | (1u << 10) | ((uint32_t)(n_mma >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
@@ -319,7 +405,7 @@ gemm_swapped_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_x
       const int e = tab_expert[mt];
       const int n_rows = min(kChunk, (int)tab_rows[mt] - c * kChunk);
       const int n_pad = (n_rows + 15) & ~15;
-      const int col0 = (c & 1) * kChunk;          // the chunk's first accumulator column
+      const int col0 = kDual ? 0 : (c & 1) * kChunk;   // the chunk's first accumulator column
       const int row0 = mt * 128 + c * kChunk;     // padded dispatch row of the chunk's first token
       const float scale = __fmul_rn(a_gs, tab_gs[e - p.expert_lo]);
       const int buf = it & 1;

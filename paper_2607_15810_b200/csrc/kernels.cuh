@@ -49,17 +49,16 @@ __global__ void score_reduce_kernel(const float* partials, const int* n_part_ptr
                                     unsigned long long* score_keys);
 __global__ void rank_select_kernel(const unsigned long long* score_keys, int C, int n_sel, uint8_t* mask);
 __global__ void sel_list_kernel(const uint8_t* mask, int C, int32_t* sel_export);
-__global__ void rac_scatter_kernel(int T, int H, int parts, const uint8_t* mask, int topk,
-                                   const int32_t* pos_pad, const uint8_t* xq, const uint8_t* xsf, const uint8_t* rq,
-                                   const uint8_t* rsf, uint8_t* xq_pad, uint8_t* xsf_tiled, uint8_t* rq_pad,
-                                   uint8_t* rsf_tiled, uint8_t* rq_exp, uint8_t* rsf_exp);
+__global__ void export_residual_kernel(int T, int H, const uint8_t* mask, uint32_t flip, const uint8_t* rq, const uint8_t* rsf,
+                                       uint8_t* rq_exp, uint8_t* rsf_exp);
 template <int kParts>   // bit 0: copies of Q(x), bit 1: masked, negated copies of the residual
 __global__ void rac_dispatch_kernel(int H, const uint8_t* mask, const int32_t* header,
                                     const int32_t* tile_rows, const int32_t* row_token, const uint8_t* xq,
                                     const uint8_t* xsf, const uint8_t* rq, const uint8_t* rsf, uint8_t* xq_pad,
                                     uint8_t* xsf_tiled, uint8_t* rq_pad, uint8_t* rsf_tiled);
 constexpr int kSelectThreads = 512;   // one CTA per SM: the CTAs of an SM would only repeat each other's search
-__global__ void select_mask_kernel(uint8_t* codes, const int32_t* header, const int32_t* tile_rows,
+template <bool kDoubleKeys>
+__global__ void select_mask_kernel(uint8_t* codes, int n_rows_fixed, uint32_t flip, const int32_t* header, const int32_t* tile_rows,
                                    const unsigned long long* score_keys, int C, int n_sel, uint8_t* mask_out /* or NULL */);
 __global__ void combine_kernel(const uint16_t* y_pad, const int32_t* pos_pad, const float* wts, int T, int H,
                                int topk, uint16_t* out, float* out_f32);
@@ -86,6 +85,39 @@ __global__ void permute_kernel(int T, int E, int topk, int n_chunks, const int32
 __global__ void dense_dispatch_kernel(int T, int tile_group, int32_t* pos_pad, int32_t* row_token, float* row_weight,
                                       int32_t* tile_expert, int32_t* tile_rows, int32_t* header);
 
+// ---- small_batch.cu: the front of a call with few tokens, two kernels of one cluster each
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallRouteMaxTokens = 512;
+constexpr int kSmallMaxUnits = 16;    // units of 128 channels a CTA of the front kernel takes (H <= 16384 on 8 CTAs)
+struct SmallRouteArgs {
+  const float* logits;
+  int T, E, topk, renormalize, e_lo, e_hi;
+  float* wts;
+  int32_t *offsets, *tile_prefix, *tile_expert, *tile_rows, *header, *perm, *pos_pad, *row_token;
+  float* row_weight;
+  unsigned long long* zero_u64;       // n_zero words cleared for the kernels that follow
+  int n_zero;
+  int32_t* ids_out;                   // exports, each may be NULL
+  float* wts_out;
+  int32_t *offsets_out, *perm_out;
+};
+struct SmallFrontArgs {
+  const uint16_t* x;
+  int T, H, topk, n_sel;
+  const float* gs_in;                 // per-tensor scale, or NULL: amax-derived (the bits go to amax_bits)
+  int after_routing;                  // launched behind route_small_kernel (else it is the call's first kernel)
+  int token_order;                    // outputs in token order, scales [T, H/16]; else dispatched copies, tiled scales
+  const int32_t* pos_pad;             // [T * topk] dispatched rows, or NULL: row t is token t (topk = 1)
+  uint8_t *xq_pad, *xsf, *rq_pad, *rsf;
+  uint32_t* amax_bits;
+  int32_t* header;                    // its status word is cleared when there is no routing kernel to do it
+  float* gs_store;                    // exports, each may be NULL
+  uint8_t *mask_out, *xq_exp, *xsf_exp, *rq_exp, *rsf_exp;
+};
+bool front_small_fits(int T, int H, bool token_order);
+quads_status launch_route_small(const SmallRouteArgs& a, cudaStream_t st);
+quads_status launch_front_small(const SmallFrontArgs& a, cudaStream_t st);
+
 // ---- gemm.cu
 #ifndef QUADS_GEMM_KSTEPS
 #define QUADS_GEMM_KSTEPS 4
@@ -101,6 +133,7 @@ struct GemmParams {
   int b_rows_per_expert; // weight rows per expert
   int half1_row_offset;  // weight-row distance from the tile's first half to its second half
   int has_resid;         // 1: also accumulate the (negated, masked) residual operand
+  int dense_rows;        // > 0: one weight and this many activation rows in token order, no routing tables
   int n_experts;         // entries of b_gs (the experts whose weights this call holds)
   int expert_lo;         // global id of the first of them: weights / scales are indexed by (expert - expert_lo)
   const int32_t* header;
@@ -114,9 +147,10 @@ struct GemmParams {
   const float* a_gs;     // per-tensor activation scale (pointer), or NULL ...
   const uint32_t* a_amax_bits;  // ... then derived from this amax word
   // epilogue: store / combine
-  const int32_t* row_token;
-  const float* row_weight;
-  uint16_t* out_bf16;    // kEpiStore: [T, n_out]
+  const int32_t* row_token;    // operand-swapped first projection: token of a padded dispatch row, and the scales of
+  const uint8_t* xsf_tok;      // its activation / residual operands in token order, [tokens, K/16]
+  const uint8_t* rsf_tok;
+  uint16_t* out_bf16;    // kEpiStore: [dense_rows, n_out]
   uint16_t* y_pad;       // kEpiCombine: bf16 [padded dispatch rows, n_out], one row per assignment
   // epilogue: SwiGLU + requantize (site 2)
   const float* h_gs;     // per-tensor scale of h
@@ -141,9 +175,10 @@ struct GemmMaps {
 };
 
 // Operand-swapped variant for few rows per expert (weights on the M side, tokens in chunks of 32
-// on the N side; epi = kEpiSwiGLU or kEpiCombine).  Maps: a / r = activation / residual codes with
-// boxes of 16 rows, b = weight codes with boxes of 128 rows; p.n_tiles_n counts tiles of 128
-// output features.  Usable when assignments <= 32 * experts and the slot tables fit.
+// on the N side; epi = kEpiSwiGLU or kEpiCombine).  Maps: a / r = activation / residual codes -- of
+// the tokens, with boxes of one row, for the first projection, which gathers its rows; of the padded
+// dispatch rows, with boxes of 16 rows, for the second -- b = weight codes with boxes of 128 rows;
+// p.n_tiles_n counts tiles of 128 output features.  Usable when assignments <= 32 * experts and the slot tables fit.
 bool gemm_swapped_ok(int64_t assignments, int n_experts, int m_tiles_max);
 quads_status launch_gemm_swapped(int epi, const GemmParams& p, const GemmMaps& m, int n_sms, cudaStream_t stream);
 

@@ -915,14 +915,6 @@ sel_list_kernel(const uint8_t* __restrict__ mask, int C, int32_t* __restrict__ s
     if (mask[i]) sel_export[pos++] = i;
 }
 
-// ---------------------------------------------------------------------------
-// Site-13 dispatch: copy every token row's codes and scales into each of its
-// dispatched copies (padded dispatch order, tiled scale layout).  The residual
-// is masked on the way (Eq. residual-recon: codes of unselected channels are
-// cleared) and stored NEGATED (sign bits flipped) so that the GEMM can
-// accumulate W Q(x) + W (-M Q(dx)) with two plain MMAs.  Pure data movement:
-// one thread per (token, 32 channels = 16 code bytes).
-// ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t nibble_mask8(const uint8_t* m) {
   // m[0..7] in {0,1} -> 0xF per selected nibble
   const uint2 v = *reinterpret_cast<const uint2*>(m);
@@ -935,54 +927,25 @@ __device__ __forceinline__ uint32_t nibble_mask8(const uint8_t* m) {
   return out;
 }
 
+// Verification export of the masked residual in token order (Eq. residual-recon: codes of unselected channels
+// cleared), from codes stored with `flip` XORed into every word.  One thread per (token, 32 channels).
 __global__ void __launch_bounds__(256)
-rac_scatter_kernel(int T, int H, int parts, const uint8_t* __restrict__ mask, int topk,
-                   const int32_t* __restrict__ pos_pad, const uint8_t* __restrict__ xq,
-                   const uint8_t* __restrict__ xsf, const uint8_t* __restrict__ rq, const uint8_t* __restrict__ rsf,
-                   uint8_t* __restrict__ xq_pad, uint8_t* __restrict__ xsf_tiled, uint8_t* __restrict__ rq_pad,
-                   uint8_t* __restrict__ rsf_tiled, uint8_t* __restrict__ rq_exp, uint8_t* __restrict__ rsf_exp) {
+export_residual_kernel(int T, int H, const uint8_t* __restrict__ mask, uint32_t flip, const uint8_t* __restrict__ rq,
+                       const uint8_t* __restrict__ rsf, uint8_t* __restrict__ rq_exp, uint8_t* __restrict__ rsf_exp) {
   pdl_sync();
-  const int per_row = H >> 5;                         // 16-byte chunks of codes per row
-  const int64_t n_chunks = (int64_t)T * per_row;
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n_chunks; g += (int64_t)gridDim.x * blockDim.x) {
+  const int per_row = H >> 5;
+  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= (int64_t)T * per_row) return;
   const int t = (int)(g / per_row), c = (int)(g - (int64_t)t * per_row);
   const size_t co = (size_t)t * (H >> 1) + c * 16;
-  const bool do_x = (parts & 1) != 0, with_residual = (parts & 2) != 0;
-  uint4 xv = make_uint4(0, 0, 0, 0), rv = make_uint4(0, 0, 0, 0);
-  const bool sf_owner = (c & 1) == 0;                 // even chunks also move 4 scale bytes (64 channels)
-  uint32_t xs = 0, rs = 0;
-  if (do_x) {
-    xv = __ldg(reinterpret_cast<const uint4*>(xq + co));
-    if (sf_owner) xs = __ldg(reinterpret_cast<const uint32_t*>(xsf + (size_t)t * (H >> 4) + c * 2));
-  }
-  if (with_residual) {
-    rv = __ldg(reinterpret_cast<const uint4*>(rq + co));
-    const uint8_t* m = mask + c * 32;
-    rv.x &= nibble_mask8(m); rv.y &= nibble_mask8(m + 8);
-    rv.z &= nibble_mask8(m + 16); rv.w &= nibble_mask8(m + 24);
-    if (sf_owner) rs = __ldg(reinterpret_cast<const uint32_t*>(rsf + (size_t)t * (H >> 4) + c * 2));
-    if (rq_exp) *reinterpret_cast<uint4*>(rq_exp + co) = rv;
-    if (rsf_exp && sf_owner) *reinterpret_cast<uint32_t*>(rsf_exp + (size_t)t * (H >> 4) + c * 2) = rs;
-    rv.x ^= 0x88888888u; rv.y ^= 0x88888888u; rv.z ^= 0x88888888u; rv.w ^= 0x88888888u;
-  }
-  const int kt_count = H >> 6;
-  for (int s0 = 0; s0 < topk; s0 += 8) {
-    int p[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) p[j] = (s0 + j < topk) ? __ldg(pos_pad + t * topk + s0 + j) : -1;   // all loads first
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if (p[j] < 0) continue;
-      const size_t po = (size_t)p[j] * (H >> 1) + c * 16;
-      if (do_x) __stcs(reinterpret_cast<uint4*>(xq_pad + po), xv);
-      if (with_residual) __stcs(reinterpret_cast<uint4*>(rq_pad + po), rv);
-      if (sf_owner) {
-        const size_t so = sf_tiled_offset(p[j], c * 2, kt_count);
-        if (do_x) *reinterpret_cast<uint32_t*>(xsf_tiled + so) = xs;
-        if (with_residual) *reinterpret_cast<uint32_t*>(rsf_tiled + so) = rs;
-      }
-    }
-  }
+  uint4 v = *reinterpret_cast<const uint4*>(rq + co);
+  const uint8_t* m = mask + c * 32;
+  v.x = (v.x ^ flip) & nibble_mask8(m); v.y = (v.y ^ flip) & nibble_mask8(m + 8);
+  v.z = (v.z ^ flip) & nibble_mask8(m + 16); v.w = (v.w ^ flip) & nibble_mask8(m + 24);
+  if (rq_exp) *reinterpret_cast<uint4*>(rq_exp + co) = v;
+  if (rsf_exp) {
+    const size_t so = (size_t)t * (H >> 4) + c * 2;
+    *reinterpret_cast<uint16_t*>(rsf_exp + so) = *reinterpret_cast<const uint16_t*>(rsf + so);
   }
 }
 
@@ -993,7 +956,9 @@ rac_scatter_kernel(int T, int H, int parts, const uint8_t* __restrict__ mask, in
 // as whole, contiguous regions.  Written from the source side instead (one thread per token
 // chunk), every 512-byte scale atom is touched by 128 different tokens at 128 different times,
 // 4 bytes each: partially written sectors get evicted and the memory system pays for them.
-// The residual is masked (Eq. residual-recon) and sign-flipped on the way, as above.
+// The residual is masked on the way (Eq. residual-recon: codes of unselected channels are cleared) and
+// stored NEGATED (sign bits flipped), so that the GEMM can accumulate W Q(x) + W (-M Q(dx)) with two
+// plain MMAs.
 // grid = upper bound of the tile count (tiles beyond header[kHdrMTiles] leave at once), 256 threads.
 // ---------------------------------------------------------------------------
 constexpr int kDispatchSlab = 32;                   // scale atoms (K = 64 each) staged per pass
@@ -1136,18 +1101,23 @@ template __global__ void rac_dispatch_kernel<3>(int, const uint8_t*, const int32
 // Against a ranking kernel (C / 16 CTAs, one rank per key) and a mask kernel behind it: decode layer of
 // 256 tokens 126.3 -> 120.4 us, of one token 55.8 -> 52.5 us, prefill of 8192 unchanged (522.7 us).  With
 // eight CTAs of 256 threads per SM, each repeating the search, the same layers took 133.6 and 65.7 us.
-// dynamic shared memory: C keys of 8 bytes, then C / 8 mask words.
+// With n_rows_fixed > 0 the matrix has that many rows, all valid (site 13 in token order); `flip` is XORed
+// into every word of the result (the residual operand is stored negated).
+// dynamic shared memory: C keys of 8 bytes, C words of scratch, C / 8 mask words.
+template <bool kDoubleKeys>
 __global__ void __launch_bounds__(kSelectThreads)
-select_mask_kernel(uint8_t* __restrict__ codes, const int32_t* __restrict__ header, const int32_t* __restrict__ tile_rows,
+select_mask_kernel(uint8_t* __restrict__ codes, int n_rows_fixed, uint32_t flip, const int32_t* __restrict__ header,
+                   const int32_t* __restrict__ tile_rows,
                    const unsigned long long* __restrict__ score_keys, int C, int n_sel, uint8_t* __restrict__ mask_out) {
   pdl_sync();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned long long* sc = reinterpret_cast<unsigned long long*>(smem_raw);
-  uint32_t* nib = reinterpret_cast<uint32_t*>(smem_raw + (size_t)C * 8);
+  uint32_t* images = reinterpret_cast<uint32_t*>(smem_raw + (size_t)C * 8);
+  uint32_t* nib = images + C;
   __shared__ SelectScratch scratch;
   for (int i = threadIdx.x; i < C; i += kSelectThreads) sc[i] = __ldcg(score_keys + i);
   const int per_row = C >> 5;
-  const int n_rows = header[kHdrMTiles] * 128;
+  const int n_rows = n_rows_fixed > 0 ? n_rows_fixed : header[kHdrMTiles] * 128;
   const int cols = min(per_row, kSelectThreads), rows_per_pass = kSelectThreads / cols;
   const int rl = threadIdx.x / cols;
   const int first = rl < rows_per_pass ? blockIdx.x * rows_per_pass + rl : n_rows;
@@ -1159,7 +1129,7 @@ select_mask_kernel(uint8_t* __restrict__ codes, const int32_t* __restrict__ head
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int r = r0 + u * step;
-      if (r < n_rows && (r & 127) < __ldg(tile_rows + (r >> 7))) on |= 1u << u;
+      if (r < n_rows && (n_rows_fixed > 0 || (r & 127) < __ldg(tile_rows + (r >> 7)))) on |= 1u << u;
     }
 #pragma unroll
     for (int u = 0; u < 8; ++u)
@@ -1168,7 +1138,7 @@ select_mask_kernel(uint8_t* __restrict__ codes, const int32_t* __restrict__ head
   const int c_first = threadIdx.x % cols;
   fetch(c_first, first);
   __syncthreads();
-  const Selection sel = select_largest<kSelectThreads>(sc, C, n_sel, &scratch);
+  const Selection sel = select_largest<kDoubleKeys>(sc, images, C, n_sel, &scratch);
   for (int w = threadIdx.x; w < (C >> 3); w += kSelectThreads) {
     uint32_t m = 0;
 #pragma unroll
@@ -1186,12 +1156,18 @@ select_mask_kernel(uint8_t* __restrict__ codes, const int32_t* __restrict__ head
 #pragma unroll
       for (int u = 0; u < 8; ++u)
         if (on >> u & 1) {
-          v[u].x &= m.x; v[u].y &= m.y; v[u].z &= m.z; v[u].w &= m.w;
+          v[u].x = (v[u].x & m.x) ^ flip; v[u].y = (v[u].y & m.y) ^ flip;
+          v[u].z = (v[u].z & m.z) ^ flip; v[u].w = (v[u].w & m.w) ^ flip;
           reinterpret_cast<uint4*>(codes + (size_t)(r0 + u * step) * (C >> 1))[c] = v[u];
         }
     }
   }
 }
+
+template __global__ void select_mask_kernel<false>(uint8_t*, int, uint32_t, const int32_t*, const int32_t*, const unsigned long long*,
+                                                   int, int, uint8_t*);
+template __global__ void select_mask_kernel<true>(uint8_t*, int, uint32_t, const int32_t*, const int32_t*, const unsigned long long*,
+                                                  int, int, uint8_t*);
 
 // Weighted top-k combine: out[t, :] = sum over the token's slots, in slot order,
 // of weight * y[row of (t, slot), :], accumulated in float32, rounded to bf16.

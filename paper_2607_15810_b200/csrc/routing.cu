@@ -41,7 +41,7 @@ route_kernel_t(const float* __restrict__ logits, int T, int E, int topk, int ren
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
       const int e = j * 32 + lane;
-      v[a][j] = (t < T && e < E) ? logits[(size_t)t * E + e] : -INFINITY;
+      v[a][j] = (t < T && e < E) ? logits[(size_t)t * E + e] + 0.f : -INFINITY;   // -0 counts as +0
     }
   }
 #pragma unroll
