@@ -5,7 +5,9 @@
 
 namespace quads {
 
-constexpr int kSelList = 512;                 // keys around the boundary that are listed and sorted out by one warp
+constexpr int kSelBins = 1024;
+constexpr int kSelFew = 128;                  // so few keys in the boundary's bin are ranked among each other
+constexpr int kSelList = 512;                 // (more of them only when their images are equal)
 
 // Key j is selected iff key > thr, or key == thr and j < tie_end (ties go to the lower index).
 struct Selection {
@@ -17,30 +19,20 @@ struct Selection {
 };
 
 struct SelectScratch {
-  uint32_t key[2][kSelList];
-  int idx[2][kSelList];
-  uint32_t cnt[3][32];
+  uint32_t hist[kSelBins];
+  uint32_t mn[32], mx[32], sum[32];
   int n_list;
+  struct __align__(16) Entry { unsigned long long key; int idx; int pad; } list[kSelList];
   Selection result;
 };
 
-// Bounds of the boundary in a monotone 32-bit image of the keys: c_lo >= n keys are >= lo, c_hi < n are >= hi.
-struct SelectBounds {
-  uint32_t lo, hi;
-  int c_lo, c_hi;
-};
-
-// One round of tightening by a warp: lane l has counted c keys >= its own threshold t (0: none).
-__device__ __forceinline__ void select_tighten(SelectBounds& b, uint32_t t, int c, int n) {
-  const bool above = c >= n;                                 // the boundary is at or above t
-  b.lo = max(b.lo, __reduce_max_sync(0xFFFFFFFFu, above ? t : 0u));
-  b.c_lo = min(b.c_lo, (int)__reduce_min_sync(0xFFFFFFFFu, (unsigned)(above ? c : 0x7FFFFFFF)));
-  b.hi = min(b.hi, __reduce_min_sync(0xFFFFFFFFu, above ? 0xFFFFFFFFu : t));
-  b.c_hi = max(b.c_hi, (int)__reduce_max_sync(0xFFFFFFFFu, (unsigned)(above ? 0 : c)));
-}
-
-__device__ __forceinline__ int select_count4(const uint4& k, uint32_t t) {
-  return (k.x >= t ? 1 : 0) + (k.y >= t ? 1 : 0) + (k.z >= t ? 1 : 0) + (k.w >= t ? 1 : 0);
+// Monotone 32-bit image of a key: the high word of a double (its exponent and 20 bits), or, for an integer, the
+// position of its leading one and the 26 bits behind it.
+template <bool kDoubleKeys>
+__device__ __forceinline__ uint32_t select_image(unsigned long long k) {
+  if (kDoubleKeys) return (uint32_t)(k >> 32);
+  const int lz = __clzll((long long)(k | 1ull));
+  return ((uint32_t)(64 - lz) << 26) - (1u << 26) + ((uint32_t)((k << lz) >> 37) & 0x3FFFFFFu);
 }
 
 // Exact search among more than kSelList keys whose images are equal (all of them at `image`): by value, then by
@@ -67,49 +59,77 @@ __device__ Selection select_ties(const unsigned long long* sc, const uint32_t* k
 
 // All threads of the block call it with the same arguments, after a barrier behind the stores to `sc`
 // (shared memory); it returns behind another one.  C is a multiple of 128, at most 16384; the block has at
-// least 128 threads, a multiple of 32; `k32` is scratch of C words, 16-byte aligned.  kDoubleKeys: the keys are the
-// bit patterns of non-negative doubles, else integers.
-//   1. Every lane of a warp takes one of 32 sampled keys as its threshold and counts the keys above it in the
-//      warp's share, on 32-bit images of the keys (float, rounded down): the boundary lies between two
-//      neighbouring samples, which leaves C / 16 keys or so.
-//   2. Those are listed, and one warp repeats the step on the list until at most 32 are left, which it ranks
-//      by exact key and index.
-// Three block barriers and no long serial chain, where a bisection pays one barrier and some hundred
-// dependent instructions per halving (measured in front_small_kernel at C = 2048: 8 000 to 21 000 cycles).
+// least 128 threads, a multiple of 32; `k32` is scratch of C words.  kDoubleKeys: the keys are the bit patterns
+// of non-negative doubles, else integers.
+//   1. A histogram of 1024 bins over the range of the keys' 32-bit images tells which bin the boundary lies in; while
+//      that bin holds many keys it is divided again (outliers stretch the range of the first one).
+//   2. Its keys are listed and ranked among each other by exact key and index.
+// Latency bounds it: a handful of barriers and little code, because code that runs once per launch is fetched
+// cold.  In front_small_kernel (1024 threads, C = 2048) it takes 6 300 cycles; a bisection with one barrier and some
+// hundred dependent instructions per halving took 8 000 to 21 000, 32 sampled thresholds instead of the bins 7 500.
 template <bool kDoubleKeys>
 __device__ Selection select_largest(const unsigned long long* sc, uint32_t* k32, int C, int n_sel, SelectScratch* s) {
   Selection r;
   if (n_sel >= C) { r.thr = 0; r.tie_end = 0x7FFFFFFF; return r; }
   if (n_sel <= 0) { r.thr = ~0ull; r.tie_end = 0; return r; }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nt = blockDim.x, nw = nt >> 5;
+  uint32_t mn = 0xFFFFFFFFu, mx = 0u;
   for (int i = threadIdx.x; i < C; i += nt) {
-    const unsigned long long k = sc[i];
-    k32[i] = __float_as_uint(kDoubleKeys ? __double2float_rz(__longlong_as_double((long long)k)) : __ull2float_rz(k));
+    const uint32_t k = select_image<kDoubleKeys>(sc[i]);
+    k32[i] = k;
+    mn = min(mn, k);
+    mx = max(mx, k);
   }
-  if (threadIdx.x < 96) (&s->cnt[0][0])[threadIdx.x] = 0;
+  for (int i = threadIdx.x; i < kSelBins; i += nt) s->hist[i] = 0;
+  mn = __reduce_min_sync(0xFFFFFFFFu, mn);
+  mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+  if (lane == 0) { s->mn[warp] = mn; s->mx[warp] = mx; }
   if (threadIdx.x == 0) s->n_list = 0;
   __syncthreads();
-  SelectBounds b{0u, 0xFFFFFFFFu, C, 0};
-  const uint4* k4 = reinterpret_cast<const uint4*>(k32);
-  int round = 0;
-  uint32_t t = k32[(int)(((unsigned)lane * (unsigned)C) >> 5) + (C >> 6)];     // sampled thresholds
+  uint32_t lo = __reduce_min_sync(0xFFFFFFFFu, lane < nw ? s->mn[lane] : 0xFFFFFFFFu);
+  uint32_t range = __reduce_max_sync(0xFFFFFFFFu, lane < nw ? s->mx[lane] : 0u) - lo;
+  int need = n_sel, m, shift;                  // `need` of the m keys with lo <= image <= lo + range are selected
   for (;;) {
-    int c = 0;
-    for (int i = warp; i < (C >> 2); i += nw) c += select_count4(k4[i], t);    // (broadcast reads)
-    uint32_t* cnt = s->cnt[round % 3];
-    if (c) atomicAdd(cnt + lane, (uint32_t)c);
+    shift = max(0, 22 - __clz((int)range));
+    for (int i = threadIdx.x; i < C; i += nt) {
+      const uint32_t d = k32[i] - lo;
+      if (d <= range) atomicAdd(&s->hist[d >> shift], 1u);
+    }
     __syncthreads();
-    select_tighten(b, t, (int)cnt[lane], n_sel);
-    if (b.c_lo - b.c_hi <= kSelList || b.hi - b.lo <= 1) break;
-    // still many (rare): thresholds at equal distances between the bounds
-    ++round;
-    if (warp == 0) s->cnt[(round + 1) % 3][lane] = 0;
-    t = b.lo + (uint32_t)(((unsigned long long)(b.hi - b.lo) * (unsigned)(lane + 1)) / 33u);
+    for (int w = warp; w < kSelBins / 32; w += nw) {
+      const uint32_t v = __reduce_add_sync(0xFFFFFFFFu, s->hist[w * 32 + lane]);
+      if (lane == 0) s->sum[w] = v;
+    }
+    __syncthreads();
+    // the last group of 32 bins, then the last bin, with at least `need` keys at or above it
+    int pos = 0, above = 0;
+    const uint32_t* v = s->sum;
+#pragma unroll 1
+    for (int level = 0; level < 2; ++level) {
+      const int own = (int)v[pos + lane];
+      int a = own;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_down_sync(0xFFFFFFFFu, a, o);
+        if (lane + o < 32) a += t;
+      }
+      const int l = __popc(__ballot_sync(0xFFFFFFFFu, a + above >= need)) - 1;
+      m = __shfl_sync(0xFFFFFFFFu, own, l);
+      above += __shfl_sync(0xFFFFFFFFu, a, l) - m;
+      pos = (pos + l) * 32;
+      v = s->hist;
+    }
+    pos >>= 5;
+    need -= above;
+    lo += (uint32_t)pos << shift;
+    range = (1u << shift) - 1u;
+    if (m <= kSelFew || shift == 0) break;
+    __syncthreads();
+    for (int i = threadIdx.x; i < kSelBins; i += nt) s->hist[i] = 0;
+    __syncthreads();
   }
-  int m = b.c_lo - b.c_hi;
   if (m > kSelList) {
-    const int need = n_sel - b.c_hi;
-    const Selection e = select_ties(sc, k32, b.lo, C, need, [&](auto pred) {
+    r = select_ties(sc, k32, lo, C, need, [&](auto pred) {
       __syncthreads();                                       // the previous count has been read
       if (threadIdx.x == 0) s->n_list = 0;
       __syncthreads();
@@ -121,67 +141,29 @@ __device__ Selection select_largest(const unsigned long long* sc, uint32_t* k32,
       return s->n_list;
     });
     __syncthreads();
-    return e;
+    return r;
   }
-  for (int i0 = warp * 32; i0 < C; i0 += nt) {
-    const uint32_t k = k32[i0 + lane];
-    const bool in = k >= b.lo && k < b.hi;
-    const uint32_t who = __ballot_sync(0xFFFFFFFFu, in);
-    if (who == 0) continue;
-    int base = 0;
-    if (lane == 0) base = atomicAdd(&s->n_list, __popc(who));
-    base = __shfl_sync(0xFFFFFFFFu, base, 0);
-    if (in) {
-      const int p = base + __popc(who & ((1u << lane) - 1u));
-      s->key[0][p] = k;
-      s->idx[0][p] = i0 + lane;
+  for (int i = threadIdx.x; i < C; i += nt)
+    if (k32[i] - lo <= range) {
+      const int p = atomicAdd(&s->n_list, 1);
+      s->list[p].key = sc[i];
+      s->list[p].idx = i;
     }
-  }
   __syncthreads();
-  if (warp == 0) {
-    int cur = 0;
-    while (m > 32) {
-      const uint32_t* lk = s->key[cur];
-      const int* li = s->idx[cur];
-      const uint32_t tt = lk[(lane * m) >> 5];
-      int c = 0;
-      for (int i = 0; i < m; ++i) c += lk[i] >= tt ? 1 : 0;
-      SelectBounds d{b.lo, b.hi, b.c_lo, b.c_hi};
-      select_tighten(d, tt, c + b.c_hi, n_sel);
-      const int left = d.c_lo - d.c_hi;
-      if (left == m) break;                                  // equal images: ranked in the loop below
-      int n = 0;
-      for (int i0 = 0; i0 < m; i0 += 32) {
-        const bool here = i0 + lane < m;
-        const uint32_t k = here ? lk[i0 + lane] : 0u;
-        const bool in = here && k >= d.lo && k < d.hi;
-        const uint32_t who = __ballot_sync(0xFFFFFFFFu, in);
-        if (in) {
-          const int p = n + __popc(who & ((1u << lane) - 1u));
-          s->key[cur ^ 1][p] = k;
-          s->idx[cur ^ 1][p] = li[i0 + lane];
-        }
-        n += __popc(who);
-      }
-      __syncwarp();
-      b = d;
-      m = left;
-      cur ^= 1;
+  // eight threads per candidate count the candidates selected before it; the boundary has need - 1 of them
+  for (int i0 = 0; i0 < m; i0 += nt >> 3) {
+    const int me = i0 + (threadIdx.x >> 3);
+    const SelectScratch::Entry e = s->list[min(me, m - 1)];
+    int rank = 0;
+#pragma unroll 4
+    for (int j = threadIdx.x & 7; j < m; j += 8) {
+      const SelectScratch::Entry o = s->list[j];
+      rank += (o.key > e.key ? 1 : 0) + ((o.key == e.key ? 1 : 0) & (o.idx < e.idx ? 1 : 0));
     }
-    const int* li = s->idx[cur];
-    const int need = n_sel - b.c_hi;                         // the boundary is the candidate with need - 1 before it
-    for (int i0 = 0; i0 < m; i0 += 32) {
-      const bool on = i0 + lane < m;
-      const int idx = on ? li[i0 + lane] : 0;
-      const unsigned long long k = sc[idx];
-      int rank = 0;
-      for (int j = 0; j < m; ++j) {
-        const int ij = li[j];
-        const unsigned long long kj = sc[ij];
-        rank += (kj > k || (kj == k && ij < idx)) ? 1 : 0;
-      }
-      if (on && rank == need - 1) { s->result.thr = k; s->result.tie_end = idx + 1; }
-    }
+    rank += __shfl_xor_sync(0xFFFFFFFFu, rank, 1);
+    rank += __shfl_xor_sync(0xFFFFFFFFu, rank, 2);
+    rank += __shfl_xor_sync(0xFFFFFFFFu, rank, 4);
+    if (me < m && rank == need - 1 && (threadIdx.x & 7) == 0) { s->result.thr = e.key; s->result.tie_end = e.idx + 1; }
   }
   __syncthreads();
   return s->result;

@@ -38,14 +38,15 @@ __device__ __forceinline__ uint32_t float_key(float v) {
   return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
-constexpr int kRouteWords = kSmallRouteMaxTokens / 32;     // 32-token words of the assignment bit matrix
+constexpr int kRouteThreads = 512;                         // 16 warps: a warp per token, four per scheduler
+constexpr int kRouteTokens = kRouteThreads / 32;           // tokens of a word of the assignment bit matrix
+constexpr int kRouteWords = kSmallRouteMaxTokens / kRouteTokens;
 
-// One warp per token (TW tokens: 32 of each word).  The assignments are a bit matrix, words[t / 32][expert]
-// bit t % 32: an expert's count is a population count over its words, and the row of token t inside an
+// One warp per token (TW tokens).  The assignments are a bit matrix, words[t / 16][expert] bit t % 16: an expert's count is a population count over its words, and the row of token t inside an
 // expert is the population count below bit t, which is the (expert, token, slot) order without a sort.
 // Every CTA sends its words to the others, then scans all experts for itself.
 template <int NJ, int TW>
-__global__ void __launch_bounds__(kSmallThreads)
+__global__ void __launch_bounds__(kRouteThreads)
 route_small_kernel(const SmallRouteArgs p) {
   pdl_sync();
   __shared__ uint32_t words[kRouteWords][kMaxExperts];
@@ -55,13 +56,13 @@ route_small_kernel(const SmallRouteArgs p) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int E = p.E, topk = p.topk;
   cluster_arrive();                                        // (waited for before the first remote store)
-  for (int i = threadIdx.x; i < TW * kMaxExperts; i += kSmallThreads) words[rank * TW + i / kMaxExperts][i % kMaxExperts] = 0;
+  for (int i = threadIdx.x; i < TW * kMaxExperts; i += kRouteThreads) words[rank * TW + i / kMaxExperts][i % kMaxExperts] = 0;
   // Top-k on order-preserving integer keys, two warp reductions per slot; softmax only for the chosen ones.
   float v[TW][NJ], my_w[TW];
   int my_id[TW];
 #pragma unroll
   for (int a = 0; a < TW; ++a) {
-    const int t = (rank * TW + a) * 32 + warp;
+    const int t = (rank * TW + a) * kRouteTokens + warp;
     my_w[a] = 0.f; my_id[a] = 0;
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
@@ -72,7 +73,7 @@ route_small_kernel(const SmallRouteArgs p) {
   __syncthreads();                                         // the words are zero
 #pragma unroll
   for (int a = 0; a < TW; ++a) {
-    const int t = (rank * TW + a) * 32 + warp;
+    const int t = (rank * TW + a) * kRouteTokens + warp;
     if (t >= p.T) continue;                                // (the whole warp)
     uint32_t key[NJ];
 #pragma unroll
@@ -112,7 +113,7 @@ route_small_kernel(const SmallRouteArgs p) {
   __syncthreads();
   cluster_wait();                                          // every CTA of the cluster has started
   if (n_cta > 1)
-    for (int i = threadIdx.x; i < TW * E * n_cta; i += kSmallThreads) {
+    for (int i = threadIdx.x; i < TW * E * n_cta; i += kRouteThreads) {
       const int c = i / (TW * E), k = i - c * (TW * E), a = k / E, e = k - a * E;
       if (c != rank) st_cluster_u32(map_to_cta(smem_u32(&words[rank * TW + a][e]), (uint32_t)c), words[rank * TW + a][e]);
     }
@@ -168,12 +169,12 @@ route_small_kernel(const SmallRouteArgs p) {
   // words of the call that start at zero: the status word and the column totals of site 2
   if (rank == n_cta - 1) {
     if (threadIdx.x < kHdrWords - kHdrStatus) p.header[kHdrStatus + threadIdx.x] = 0;
-    for (int i = threadIdx.x; i < p.n_zero; i += kSmallThreads) p.zero_u64[i] = 0ull;
+    for (int i = threadIdx.x; i < p.n_zero; i += kRouteThreads) p.zero_u64[i] = 0ull;
   }
   // ---- rows (and the stores that the barriers above would have waited for)
 #pragma unroll
   for (int a = 0; a < TW; ++a) {
-    const int t = (rank * TW + a) * 32 + warp;
+    const int t = (rank * TW + a) * kRouteTokens + warp;
     if (t >= p.T || lane >= topk) continue;
     const int flat = t * topk + lane;
     const int e = my_id[a];
@@ -206,8 +207,8 @@ front_small_kernel(const SmallFrontArgs p) {
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ uint32_t amax_all[16];
   __shared__ uint32_t wmax[32];
-  __shared__ float inv_lut[128];
   __shared__ SelectScratch scratch;
+  __shared__ double red2[8][128];
   __shared__ __align__(16) uint32_t nib[kSmallMaxUnits * 16];
   const int rank = (int)cluster_ctarank(), n_cta = (int)gridDim.x;
   const int T = p.T, H = p.H, units = H >> 7;
@@ -259,11 +260,9 @@ front_small_kernel(const SmallFrontArgs p) {
     if (p.gs_store) p.gs_store[0] = gs;
     if (!p.after_routing) p.header[kHdrStatus] = 0;
   }
-  if (threadIdx.x < 128) inv_lut[threadIdx.x] = quant_inv_entry(threadIdx.x, gs);
-  __syncthreads();
-  QuantCtx qc;
+  QuantCtx qc;                                             // (a reciprocal table costs more than a few blocks' divisions)
   quant_ctx_scalars(qc, gs);
-  qc.inv_lut = inv_lut;
+  qc.inv_lut = nullptr;
   if (!started) cluster_wait();
   const int n_warps = min(32, (T * 8 + 31) / 32);          // warps that hold rows
   for (int ui = 0; ui < n_my; ++ui) {
@@ -277,7 +276,7 @@ front_small_kernel(const SmallFrontArgs p) {
       float f[16];
       unpack8(v0, f);
       unpack8(v1, f + 8);
-      const BlockQ bq = quantize_block(f, qc);
+      const BlockQ bq = quantize_block<false>(f, qc);
       const int idx = ui * T + r;
       const size_t qo = (size_t)r * (H >> 1) + u * 64 + blk * 8, so = (size_t)r * (H >> 4) + u * 8 + blk;
       if (p.token_order) {
@@ -297,7 +296,7 @@ front_small_kernel(const SmallFrontArgs p) {
           o[i] = __fsub_rn(o[i], f[i]);
           acc[i] = __fmaf_rn(o[i], o[i], acc[i]);
         }
-        const BlockQ br = quantize_block(o, qc);
+        const BlockQ br = quantize_block<false>(o, qc);
         reinterpret_cast<uint2*>(st_r)[idx * 8 + blk] = make_uint2(br.lo, br.hi);
         if (p.token_order) p.rsf[so] = (uint8_t)br.sf8;
         else sf_r[idx * 8 + blk] = (uint8_t)br.sf8;
@@ -305,7 +304,7 @@ front_small_kernel(const SmallFrontArgs p) {
       }
     }
     if (p.n_sel > 0) {
-      // column scores: the four row groups of a warp, then the warps in order (float64)
+      // column scores: the four row groups of a warp, then (float64) four warps each, then the eight groups of warps
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
         acc[i] += __shfl_xor_sync(0xFFFFFFFFu, acc[i], 8);
@@ -319,9 +318,19 @@ front_small_kernel(const SmallFrontArgs p) {
         d[3] = make_float4(acc[12], acc[13], acc[14], acc[15]);
       }
       __syncthreads();
+      {
+        const int c = threadIdx.x & 127, w0 = (threadIdx.x >> 7) * 4;
+        double s = 0.0;
+#pragma unroll
+        for (int w = 0; w < 4; ++w)
+          if (w0 + w < n_warps) s += (double)red[(w0 + w) * 128 + c];
+        red2[w0 / 4][c] = s;
+      }
+      __syncthreads();
       if (threadIdx.x < 128) {
         double s = 0.0;
-        for (int w = 0; w < n_warps; ++w) s += (double)red[w * 128 + threadIdx.x];
+#pragma unroll
+        for (int w = 0; w < 8; ++w) s += red2[w][threadIdx.x];
         keys[u * 128 + threadIdx.x] = (unsigned long long)__double_as_longlong(s);   // order-preserving: s >= 0
       }
       __syncthreads();
@@ -433,25 +442,33 @@ int front_ctas(int H) {
   return n;
 }
 
+template <int NJ, int TW>
+quads_status launch_route_tw(const SmallRouteArgs& a, cudaStream_t st) {
+  static std::atomic<bool> wide[64];                       // clusters beyond the portable size allowed for this kernel
+  int n = 1, dev = 0;
+  while (n * TW * kRouteTokens < a.T) n *= 2;
+  if (n > 8) {
+    QUADS_CUDA_OK(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) return QUADS_ERR_CUDA;
+    if (!wide[dev].load()) {
+      QUADS_CUDA_OK(cudaFuncSetAttribute(route_small_kernel<NJ, TW>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      wide[dev].store(true);
+    }
+  }
+  QUADS_CUDA_OK(launch_cluster(route_small_kernel<NJ, TW>, n, kRouteThreads, 0, st, a));
+  return QUADS_OK;
+}
+
 template <int NJ>
 quads_status launch_route_nj(const SmallRouteArgs& a, cudaStream_t st) {
-  const int words = (a.T + 31) / 32;
-  int n = 1;
-  if (words <= 8) {
-    while (n < words) n *= 2;
-    QUADS_CUDA_OK(launch_cluster(route_small_kernel<NJ, 1>, n, kSmallThreads, 0, st, a));
-  } else {
-    while (n < (words + 1) / 2) n *= 2;
-    QUADS_CUDA_OK(launch_cluster(route_small_kernel<NJ, 2>, n, kSmallThreads, 0, st, a));
-  }
-  return QUADS_OK;
+  return a.T <= kRouteTokens * front_cluster_limit() ? launch_route_tw<NJ, 1>(a, st) : launch_route_tw<NJ, 2>(a, st);
 }
 
 }  // namespace
 
 bool front_small_fits(int T, int H, bool token_order) {
   const int n = front_ctas(H), upc = (H / 128 + n - 1) / n;
-  return T <= kSmallRouteMaxTokens && upc <= kSmallMaxUnits && front_small_smem(T, H, n, token_order) <= (size_t)kFrontMaxSmem;
+  return T <= 2 * kRouteTokens * front_cluster_limit() && upc <= kSmallMaxUnits && front_small_smem(T, H, n, token_order) <= (size_t)kFrontMaxSmem;
 }
 
 quads_status launch_route_small(const SmallRouteArgs& a, cudaStream_t st) {
