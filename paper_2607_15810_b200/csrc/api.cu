@@ -119,12 +119,12 @@ inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_
 
 // ------------------------------------------------------------------ workspace
 struct MoeLayout {
-  size_t header, amax, counters13, keys13, keys2, expert_total, ids, wts, chunk_counts, chunk_base, offsets, tile_prefix, tile_expert, tile_rows;
+  size_t header, amax, keys13, keys2, expert_total, ids, wts, chunk_counts, chunk_base, offsets, tile_prefix, tile_expert, tile_rows;
   size_t perm, pos_pad, row_token, row_weight;
-  size_t partials13, scores13, sel13, mask13, xq_tok, xsf_tok, rq_tok, rsf_tok, xq_pad, xsf, rq_pad, rsf;
-  size_t hq_pad, hsf, r2q_pad, r2sf, sel2, mask2, y_pad, dec;
+  size_t mask13, xq_tok, xsf_tok, rq_tok, rsf_tok, xq_pad, xsf, rq_pad, rsf;
+  size_t hq_pad, hsf, r2q_pad, r2sf, mask2, y_pad, dec;
   size_t total;
-  int n_chunks, m_tiles_max, stats_ctas, rows_per_cta;
+  int n_chunks, m_tiles_max;
 };
 
 MoeLayout moe_layout(int T, int H, int I, int E, int topk, int N) {
@@ -134,19 +134,12 @@ MoeLayout moe_layout(int T, int H, int I, int E, int topk, int N) {
   const int Ee = dense ? 1 : E;
   L.n_chunks = (T + kRouteTokensPerCta - 1) / kRouteTokensPerCta;
   L.m_tiles_max = ((int)(A / 256) + Ee) * 2;      // enough for either tile grouping (1 or 2)
-  L.stats_ctas = T < 592 * 4 ? (T + 3) / 4 : 592;
-  if (L.stats_ctas < 1) L.stats_ctas = 1;
-  L.rows_per_cta = (T + L.stats_ctas - 1) / L.stats_ctas;
-  if (L.rows_per_cta < 1) L.rows_per_cta = 1;
-  L.stats_ctas = (T + L.rows_per_cta - 1) / L.rows_per_cta;
-  if (L.stats_ctas < 1) L.stats_ctas = 1;
   const size_t pad_rows = (size_t)L.m_tiles_max * 128;
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
   L.header = take(kHdrWords * 4);
   L.amax = take((size_t)kAmaxPartsMax * 4);    // the amax word; also the quantizer's scratch in the one-sided modes
-  L.counters13 = take((size_t)((H + 31) / 32) * 4);
-  L.keys13 = take((size_t)H * 8);                  // integer column scores of site 13 (small batches), zeroed with the header
+  L.keys13 = take((size_t)H * 8);                  // integer column scores of site 13, zeroed with the header
   L.keys2 = take((size_t)I * 8);                   // zeroed with the header: the first projection's epilogue adds to it
   L.expert_total = take((size_t)Ee * 4);           // zeroed with the header: the routing kernel adds to it
   L.ids = take((size_t)A * 4);
@@ -161,9 +154,6 @@ MoeLayout moe_layout(int T, int H, int I, int E, int topk, int N) {
   L.pos_pad = take((size_t)A * 4);
   L.row_token = take(pad_rows * 4);
   L.row_weight = take(pad_rows * 4);
-  L.partials13 = take((size_t)L.stats_ctas * H * 4);
-  L.scores13 = take((size_t)H * 8 * kScoreSlices);
-  L.sel13 = take((size_t)H * 4);
   L.mask13 = take((size_t)H);
   L.xq_tok = take((size_t)T * (H / 2));
   L.xsf_tok = take((size_t)T * (H / 16));
@@ -178,7 +168,6 @@ MoeLayout moe_layout(int T, int H, int I, int E, int topk, int N) {
     L.hsf = take((size_t)L.m_tiles_max * (I / 64) * 512);
     L.r2q_pad = take(pad_rows * (I / 2));
     L.r2sf = take((size_t)L.m_tiles_max * (I / 64) * 512);
-    L.sel2 = take((size_t)I * 4);
     L.mask2 = take((size_t)I);
     L.y_pad = take(pad_rows * (size_t)H * 2);
   }
@@ -279,11 +268,10 @@ quads_status run_rank(const unsigned long long* keys, int C, int n_sel, uint8_t*
 }
 
 // Selection and masking of a code matrix in one launch (see select_mask_kernel).
-template <bool kDoubleKeys>
 quads_status run_select_mask(uint8_t* codes, int n_rows_fixed, uint32_t flip, const int32_t* header, const int32_t* tile_rows,
                              const unsigned long long* keys, int C, int n_sel, uint8_t* mask_out, int sm_count, cudaStream_t st) {
-  QUADS_CUDA_OK(set_max_dynamic_smem<select_mask_kernel<kDoubleKeys>>(16384 * 12 + 16384 / 2));
-  QUADS_CUDA_OK(launch_kernel(select_mask_kernel<kDoubleKeys>, dim3(sm_count), dim3(kSelectThreads), (size_t)C * 12 + C / 2, st, codes,
+  QUADS_CUDA_OK(set_max_dynamic_smem<select_mask_kernel>(16384 * 12 + 16384 / 2));
+  QUADS_CUDA_OK(launch_kernel(select_mask_kernel, dim3(sm_count), dim3(kSelectThreads), (size_t)C * 12 + C / 2, st, codes,
                               n_rows_fixed, flip, header, tile_rows, keys, C, n_sel, mask_out));
   return QUADS_OK;
 }
@@ -562,8 +550,7 @@ quads_status quads_rac_channel_scores(const void* x, int64_t T, int64_t H, const
   int rpc;
   const int ctas = score_stats_ctas(T, &rpc);
   uint8_t* ws = static_cast<uint8_t*>(workspace);
-  uint32_t* amax_bits = reinterpret_cast<uint32_t*>(ws);                 // [0, 256): amax word; [256, 512): status word
-  int32_t* status_word = reinterpret_cast<int32_t*>(ws + 256);
+  uint32_t* amax_bits = reinterpret_cast<uint32_t*>(ws);                 // [0, 256): amax word
   unsigned int* counters = reinterpret_cast<unsigned int*>(ws + 512);
   const size_t n_counter_bytes = align_up((size_t)((H + 31) / 32) * 4, 256);
   float* partials = reinterpret_cast<float*>(ws + 512 + n_counter_bytes);
@@ -576,10 +563,8 @@ quads_status quads_rac_channel_scores(const void* x, int64_t T, int64_t H, const
     QUADS_CUDA_OK(launch_kernel(amax_kernel, dim3(gx, 1), dim3(256), (size_t)0, st, xp, T, H, H, (int64_t)0, amax_bits));
   }
   const int block = H / 16 > 256 ? 256 : (int)((H / 16 + 31) / 32 * 32);
-  QUADS_CUDA_OK(launch_kernel(rac_quant_kernel, dim3(ctas), dim3(block), (size_t)0, st, xp, (int)T, (int)H, gs_in, amax_bits,
-                              (unsigned int*)nullptr, status_word, (float*)nullptr, rpc, 1, partials, (uint8_t*)nullptr,
-                              (uint8_t*)nullptr, (uint8_t*)nullptr, (uint8_t*)nullptr, (uint8_t*)nullptr, (uint8_t*)nullptr,
-                              (unsigned long long*)nullptr, 0, 0));
+  QUADS_CUDA_OK(launch_kernel(channel_stats_kernel, dim3(ctas), dim3(block), (size_t)0, st, xp, (int)T, (int)H, gs_in, amax_bits,
+                              rpc, partials));
   // the order-preserving 64-bit keys of non-negative scores are the scores' own bit patterns
   QUADS_CUDA_OK(launch_kernel(score_reduce_kernel, dim3((unsigned)((H + 31) / 32), kScoreSlices), dim3(256), (size_t)0, st,
                               (const float*)partials, (const int*)nullptr, 1, ctas, (int)H, slices, counters,
@@ -815,9 +800,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
       side_guard.arm(side, st);
       rs = side->stream;
     }
-    if (dense) {
-      QUADS_CUDA_OK(launch_kernel(dense_dispatch_kernel, dim3((T + 255) / 256), dim3(256), (size_t)(0), st, T, cta_group, pos_pad, row_token, row_weight, tile_expert, tile_rows, header));
-    } else {
+    if (!dense) {
       int32_t* chunk_counts = reinterpret_cast<int32_t*>(P(L.chunk_counts));
       int32_t* chunk_base = reinterpret_cast<int32_t*>(P(L.chunk_base));
       int32_t* expert_total = reinterpret_cast<int32_t*>(P(L.expert_total));
@@ -833,89 +816,67 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
     }
     trace_mark("permute", st);
 
-    // ---- per-tensor scale of x
-    // ---- per-tensor scale of x: folded into the quantization kernel (cooperative launch, grid
-    // barrier) when all of its CTAs fit on the GPU at once; else a kernel of its own
-    const int rq_block = H / 16 > 256 ? 256 : (H / 16 + 31) / 32 * 32;
-    static const bool no_fused_amax = getenv("QUADS_NO_FUSED_AMAX") != nullptr;
-    bool fused_amax = false;
-    if (!a->a13_gs && !no_fused_amax && !g_trace.enabled) {
-      // resident CTAs per SM for the two block sizes in use (128 and 256 threads); same on every sm_100 device
-      static std::atomic<int> per_sm_cache[2] = {{0}, {0}};
-      std::atomic<int>& slot = per_sm_cache[rq_block > 128 ? 1 : 0];
-      int per_sm = slot.load();
-      if (per_sm == 0) {
-        QUADS_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rac_quant_kernel, rq_block > 128 ? 256 : 128, 0));
-        slot.store(per_sm);
-      }
-      fused_amax = (int64_t)per_sm * di.sm_count >= L.stats_ctas;
-    }
-    if (!a->a13_gs && !fused_amax) {
-      const int64_t chunks = (int64_t)T * (H / 8);
-      int gx = (int)((chunks + 2047) / 2048);
-      if (gx > di.sm_count * 8) gx = di.sm_count * 8;
-      QUADS_CUDA_OK(launch_kernel(amax_kernel, dim3(gx, 1), dim3(256), (size_t)(0), st, x, T, H, H, 0, amax_bits));
-    }
-    trace_mark("amax", st);
-    // ---- site 13: quantize (+ residual + statistics), selection, dispatch scatter
-    const bool totals13 = (int64_t)L.stats_ctas * H <= ((int64_t)1 << 18);
+    // ---- site 13: per-tensor scale, quantization, residual and channel scores in one launch.  A dense projection's
+    // rows are its operand as they are (tiled scales); the others stay in token order.
+    unsigned long long* keys13 = reinterpret_cast<unsigned long long*>(P(L.keys13));
     {
-      const uint16_t* xp = x;
-      int Tt = T, Hh = H, rows_per_cta = L.rows_per_cta, with_res = nsel13 > 0 ? 1 : 0;
-      const float* gs13 = a->a13_gs;
-      unsigned int* arrivals = fused_amax ? reinterpret_cast<unsigned int*>(header + kHdrArrivals) : nullptr;
-      int32_t* status_word = header + kHdrStatus;
-      float* gs_store = a->a13_gs_out;
-      // Column scores of site 13: integer totals added by every CTA when there are few of them (the
-      // selection is then one ranking kernel; decode-sized batches), else one partial row per CTA and a
-      // reduction kernel (586 x 2048 integer reductions at the end of the kernel cost 20 us, the
-      // reduction kernel 9)
-      float* partials = totals13 ? nullptr : reinterpret_cast<float*>(P(L.partials13));
-      unsigned long long* totals = totals13 ? reinterpret_cast<unsigned long long*>(P(L.keys13)) : nullptr;
-      // a CTA's partial sum covers rows_per_cta rows (< rows * 2^18 in units of the squared scale); the
-      // stats_ctas partial sums of a column must fit 62 bits together
-      int cap_bits = 18, ctas_log2 = 0;
-      while ((1 << (cap_bits - 18)) < rows_per_cta) ++cap_bits;
-      while ((1 << ctas_log2) < L.stats_ctas) ++ctas_log2;
-      int score_bits = std::max(0, std::min(26, 62 - cap_bits - ctas_log2));
-      uint8_t *xq_tok = P(L.xq_tok), *xsf_tok = P(L.xsf_tok), *rq_tok = P(L.rq_tok), *rsf_tok = P(L.rsf_tok);
-      uint8_t *xq_exp = a->xq, *xsf_exp = a->xsf;
-      if (fused_amax) {
-        void* args[] = {&xp, &Tt, &Hh, &gs13, &amax_bits, &arrivals, &status_word, &gs_store, &rows_per_cta, &with_res,
-                        &partials, &xq_tok, &xsf_tok, &rq_tok, &rsf_tok, &xq_exp, &xsf_exp, &totals, &score_bits, &cap_bits};
-        QUADS_CUDA_OK(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(rac_quant_kernel), dim3(L.stats_ctas),
-                                                  dim3(rq_block), args, 0, st));
+      QuantRowsArgs q{};
+      q.x = x; q.T = T; q.H = H; q.with_residual = nsel13 > 0; q.sf_tiled = dense;
+      q.bw = (H / 16) % 32 == 0 ? 32 : ((H / 16) % 16 == 0 ? 16 : 8);
+      q.n_col = H / 16 / q.bw;
+      // as many row ranges as are resident at once, each at least a row per row lane
+      static std::atomic<int> per_sm_cache{0};       // same kernel and block size on every sm_100 device
+      int per_sm = per_sm_cache.load();
+      if (per_sm == 0) {
+        QUADS_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, quant_rows_kernel, 256, 0));
+        per_sm_cache.store(per_sm);
+      }
+      if (side) per_sm = std::min(per_sm, kQuantRowsPerSm - 1);   // room for the routing kernels beside it
+      const int lanes = 256 / q.bw;
+      const int n_rg = std::max(1, std::min(per_sm * di.sm_count / q.n_col, (T + lanes - 1) / lanes));
+      q.rows_per_cta = ((T + n_rg - 1) / n_rg + lanes - 1) / lanes * lanes;
+      const int n_used = (T + q.rows_per_cta - 1) / q.rows_per_cta;
+      q.gs_in = a->a13_gs; q.amax_bits = amax_bits;
+      q.arrivals = a->a13_gs ? nullptr : reinterpret_cast<unsigned int*>(header + kHdrArrivals);
+      q.status = header + kHdrStatus; q.gs_store = a->a13_gs_out;
+      q.xq = P(dense ? L.xq_pad : L.xq_tok); q.xsf = P(dense ? L.xsf : L.xsf_tok);
+      q.rq = P(dense ? L.rq_pad : L.rq_tok); q.rsf = P(dense ? L.rsf : L.rsf_tok);
+      q.xq_exp = a->xq; q.xsf_exp = a->xsf; q.rsf_exp = a->rsf;
+      q.totals = keys13;
+      // a CTA's sum covers rows_per_cta rows (< rows * 2^18 in units of the squared scale); the sums of
+      // all row ranges must fit 62 bits together
+      int cap_bits = 18, ranges_log2 = 0;
+      while ((1 << (cap_bits - 18)) < q.rows_per_cta) ++cap_bits;
+      while ((1 << ranges_log2) < n_used) ++ranges_log2;
+      q.cap_bits = cap_bits;
+      q.score_bits = std::max(0, std::min(26, 62 - cap_bits - ranges_log2));
+      const dim3 grid(n_used * q.n_col);
+      if (q.arrivals) {                               // its CTAs wait for one another
+        void* args[] = {&q};
+        QUADS_CUDA_OK(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(quant_rows_kernel), grid, dim3(256), args, 0, st));
         note_launch();
       } else {
-        QUADS_CUDA_OK(launch_kernel(rac_quant_kernel, dim3(L.stats_ctas), dim3(rq_block), (size_t)(0), st, xp, Tt, Hh, gs13,
-                                    amax_bits, arrivals, status_word, gs_store, rows_per_cta, with_res, partials, xq_tok,
-                                    xsf_tok, rq_tok, rsf_tok, xq_exp, xsf_exp, totals, score_bits, cap_bits));
+        QUADS_CUDA_OK(launch_kernel(quant_rows_kernel, grid, dim3(256), (size_t)0, st, q));
       }
     }
-    trace_mark("rac_stats", st);
-    unsigned long long* keys13 = reinterpret_cast<unsigned long long*>(P(L.keys13));
-    if (nsel13 > 0 && !totals13) {
-      QUADS_CUDA_OK(launch_kernel(score_reduce_kernel, dim3((H + 31) / 32, kScoreSlices), dim3(256), (size_t)0, st,
-                                  reinterpret_cast<float*>(P(L.partials13)), (const int*)nullptr, 1, L.stats_ctas, H,
-                                  reinterpret_cast<double*>(P(L.scores13)), reinterpret_cast<unsigned int*>(P(L.counters13)), keys13));
-    }
+    trace_mark("quant13", st);
     // verification exports of the selection and, from codes stored with `flip` applied, of the masked residual
-    auto export13 = [&](uint32_t flip) -> quads_status {
+    auto export13 = [&](const uint8_t* codes, uint32_t flip) -> quads_status {
       if (a->sel13) QUADS_CUDA_OK(launch_kernel(sel_list_kernel, dim3(1), dim3(1024), (size_t)0, st, mask13, H, a->sel13));
-      if (a->rq || a->rsf) {
+      if (a->rq) {
         const int64_t chunks = (int64_t)T * (H / 32);
         QUADS_CUDA_OK(launch_kernel(export_residual_kernel, dim3((unsigned)((chunks + 255) / 256)), dim3(256), (size_t)0, st, T, H,
-                                    mask13, flip, P(L.rq_tok), P(L.rsf_tok), a->rq, a->rsf));
+                                    mask13, flip, codes, a->rq));
       }
       return QUADS_OK;
     };
-    if (swapped) {
-      // the first projection gathers out of the token-order codes: the residual is masked and negated in place
+    if (swapped || dense) {
+      // the operand is in token order: the residual is masked and negated in place
       if (nsel13 > 0) {
+        uint8_t* rq = P(dense ? L.rq_pad : L.rq_tok);
         uint8_t* mask_out = (a->sel13 || a->rq) ? mask13 : nullptr;
-        s = totals13 ? run_select_mask<false>(P(L.rq_tok), T, 0x88888888u, header, tile_rows, keys13, H, nsel13, mask_out, di.sm_count, st)
-                     : run_select_mask<true>(P(L.rq_tok), T, 0x88888888u, header, tile_rows, keys13, H, nsel13, mask_out, di.sm_count, st);
-        if (s != QUADS_OK || (s = export13(0x88888888u)) != QUADS_OK) return s;
+        if ((s = run_select_mask(rq, T, 0x88888888u, header, tile_rows, keys13, H, nsel13, mask_out, di.sm_count, st)) != QUADS_OK) return s;
+        if ((s = export13(rq, 0x88888888u)) != QUADS_OK) return s;
       }
       trace_mark("select13+mask", st);
       if (side) {
@@ -942,7 +903,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
       }
       if (nsel13 > 0) {
         if ((s = run_rank(keys13, H, nsel13, mask13, st)) != QUADS_OK) return s;
-        if ((s = export13(0u)) != QUADS_OK) return s;
+        if ((s = export13(P(L.rq_tok), 0u)) != QUADS_OK) return s;
       }
       trace_mark("select13", st);
       if (split_scatter) {
@@ -1027,7 +988,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   if (nsel2 > 0) {
     // the scores are complete when the first projection ends (integer totals)
     const bool want_mask = a->sel2 || a->hq || a->hsf || a->r2q || a->r2sf;
-    if ((s = run_select_mask<false>(P(L.r2q_pad), 0, 0u, header, tile_rows, g.keys2, I, nsel2, want_mask ? mask2 : nullptr,
+    if ((s = run_select_mask(P(L.r2q_pad), 0, 0u, header, tile_rows, g.keys2, I, nsel2, want_mask ? mask2 : nullptr,
                                     di.sm_count, st)) != QUADS_OK)
       return s;
     if (a->sel2) QUADS_CUDA_OK(launch_kernel(sel_list_kernel, dim3(1), dim3(1024), (size_t)0, st, mask2, I, a->sel2));

@@ -37,27 +37,36 @@ __global__ void fake_quant_ring_kernel(const uint16_t* x, int64_t nblk, int64_t 
                                        int kt_count);
 __global__ void dequantize_kernel(const uint8_t* q, const uint8_t* sf, const float* gs, int n_tensors, int64_t nblk,
                                   uint32_t k16, int kt_count, int sf_tiled, int64_t sf_tensor_stride, uint16_t* out);
-__global__ void rac_quant_kernel(const uint16_t* x, int T, int H, const float* gs_in, uint32_t* amax_bits,
-                                 unsigned int* grid_arrivals, int32_t* status,
-                                 float* gs_store, int rows_per_cta, int with_residual, float* partials, uint8_t* xq,
-                                 uint8_t* xsf, uint8_t* rq, uint8_t* rsf, uint8_t* xq_exp, uint8_t* xsf_exp,
-                                 unsigned long long* score_totals /* or NULL: partial rows */, int score_bits,
-                                 int cap_bits);
+constexpr int kQuantRowsPerSm = 4;    // resident CTAs of quant_rows_kernel
+struct QuantRowsArgs {
+  const uint16_t* x;
+  int T, H, bw, n_col, rows_per_cta, with_residual, sf_tiled;
+  const float* gs_in;                 // per-tensor scale, or NULL: amax-derived (then the launch is cooperative)
+  uint32_t* amax_bits;
+  unsigned int* arrivals;             // NULL when gs_in is given; amax_bits and arrivals are zero on entry
+  int32_t* status;
+  float* gs_store;                    // exports, each may be NULL
+  uint8_t *xq, *xsf, *rq, *rsf;
+  uint8_t *xq_exp, *xsf_exp, *rsf_exp;
+  unsigned long long* totals;         // [H] integer channel scores, zero on entry
+  int score_bits, cap_bits;
+};
+__global__ void quant_rows_kernel(const QuantRowsArgs p);
+__global__ void channel_stats_kernel(const uint16_t* x, int T, int H, const float* gs_in, const uint32_t* amax_bits,
+                                     int rows_per_cta, float* partials);
 constexpr int kScoreSlices = 16;
 __global__ void score_reduce_kernel(const float* partials, const int* n_part_ptr, int n_part_mul,
                                     int n_part_fixed, int C, double* slice_sums, unsigned int* counters,
                                     unsigned long long* score_keys);
 __global__ void rank_select_kernel(const unsigned long long* score_keys, int C, int n_sel, uint8_t* mask);
 __global__ void sel_list_kernel(const uint8_t* mask, int C, int32_t* sel_export);
-__global__ void export_residual_kernel(int T, int H, const uint8_t* mask, uint32_t flip, const uint8_t* rq, const uint8_t* rsf,
-                                       uint8_t* rq_exp, uint8_t* rsf_exp);
+__global__ void export_residual_kernel(int T, int H, const uint8_t* mask, uint32_t flip, const uint8_t* rq, uint8_t* rq_exp);
 template <int kParts>   // bit 0: copies of Q(x), bit 1: masked, negated copies of the residual
 __global__ void rac_dispatch_kernel(int H, const uint8_t* mask, const int32_t* header,
                                     const int32_t* tile_rows, const int32_t* row_token, const uint8_t* xq,
                                     const uint8_t* xsf, const uint8_t* rq, const uint8_t* rsf, uint8_t* xq_pad,
                                     uint8_t* xsf_tiled, uint8_t* rq_pad, uint8_t* rsf_tiled);
 constexpr int kSelectThreads = 512;   // one CTA per SM: the CTAs of an SM would only repeat each other's search
-template <bool kDoubleKeys>
 __global__ void select_mask_kernel(uint8_t* codes, int n_rows_fixed, uint32_t flip, const int32_t* header, const int32_t* tile_rows,
                                    const unsigned long long* score_keys, int C, int n_sel, uint8_t* mask_out /* or NULL */);
 __global__ void combine_kernel(const uint16_t* y_pad, const int32_t* pos_pad, const float* wts, int T, int H,
@@ -82,8 +91,6 @@ __global__ void permute_kernel(int T, int E, int topk, int n_chunks, const int32
                                const int32_t* chunk_base, const int32_t* offsets, const int32_t* tile_prefix,
                                int32_t* perm, int32_t* pos_pad, int32_t* row_token, float* row_weight,
                                int32_t* perm_out, int e_lo, int e_hi);
-__global__ void dense_dispatch_kernel(int T, int tile_group, int32_t* pos_pad, int32_t* row_token, float* row_weight,
-                                      int32_t* tile_expert, int32_t* tile_rows, int32_t* header);
 
 // ---- small_batch.cu: the front of a call with few tokens, two kernels of one cluster each
 constexpr int kSmallThreads = 1024;

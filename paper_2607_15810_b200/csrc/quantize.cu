@@ -701,65 +701,133 @@ dequantize_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ sf,
 // ---------------------------------------------------------------------------
 // Site-13 quantization pass, token order.  For every row and 16-channel block:
 // Q_A(x) codes + scale; the residual Q_A(x) - x in float32 (Eq. residual-def);
-// its squared sum per channel over the rows this CTA owns (Eq. channel-score,
-// one partial row per CTA, reduced later in a fixed order); and the residual's
-// own quantization with the same per-tensor scale (the mask of Eq.
-// residual-recon is applied later, when rows are copied into dispatch order:
-// quantizing the residual does not depend on the selection).
+// its squared sum per channel (Eq. channel-score); and the residual's own
+// quantization with the same per-tensor scale (the mask of Eq. residual-recon is
+// applied later: quantizing the residual does not depend on the selection).
+//
+// A CTA owns bw blocks of 16 channels (8, 16 or 32, whatever divides the row) for a range of rows;
+// thread = (block, row lane).  The grid is what is resident at once, so that the amax of x can be the
+// first phase of the same launch: the CTAs meet at a counter (bounded wait) and read their rows again, out of L2.
+// A CTA adds its row lanes' column sums up in shared memory and adds one 64-bit integer per channel to the
+// channel's total, which is complete when the kernel ends: with CTAs that own whole rows, four times as
+// many reductions arrive together (20 us at 8192 x 2048), and partial rows need a kernel to add them up.
+// Issue-bound: about 400 issue cycles per warp and block, 128 of them in the two conversions to E2M1.
+// Dense projection 8192 x 4096 -> 4096: amax, quantization, score reduction, ranking and copy took 16 + 27 + 12 +
+// 12 + 28 us as kernels of their own; this one takes 39.8 and the in-place mask behind it 10 (whole call
+// 205 -> 165 us).
+// Scales are stored linear [T, H/16], or tiled when the rows are a dense projection's operand as they are.
 // ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256, kQuantRowsPerSm)
+quant_rows_kernel(const QuantRowsArgs p) {
+  pdl_sync();
+  __shared__ float gs_sh;
+  __shared__ uint32_t wmax[8];
+  __shared__ float inv_lut[128];
+  __shared__ __align__(16) float red[256 * 16];
+  const int H = p.H, k16 = H >> 4;
+  const int col = blockIdx.x % p.n_col, rg = blockIdx.x / p.n_col;
+  const int blk = threadIdx.x % p.bw, lane_r = threadIdx.x / p.bw, lanes = 256 / p.bw;
+  const int kb = col * p.bw + blk;
+  const int r0 = rg * p.rows_per_cta + lane_r, r1 = min(p.T, (rg + 1) * p.rows_per_cta);
+  const uint16_t* xk = p.x + kb * 16;
+  if (p.arrivals) {
+    uint32_t m = 0;
+    int r = r0;
+    for (; r + 3 * lanes < r1; r += 4 * lanes) {
+      uint4 v[8];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) ldg256_keep(xk + (size_t)(r + u * lanes) * H, v[2 * u], v[2 * u + 1]);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) m = __vmaxu2(m, absmax8(v[u]));
+    }
+    for (; r < r1; r += lanes) {
+      uint4 v0, v1;
+      ldg256_keep(xk + (size_t)r * H, v0, v1);
+      m = __vmaxu2(m, __vmaxu2(absmax8(v0), absmax8(v1)));
+    }
+    m = __reduce_max_sync(0xFFFFFFFFu, max(m & 0xFFFFu, m >> 16));
+    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      uint32_t tm = 0;
+      for (int i = 0; i < 8; ++i) tm = max(tm, wmax[i]);
+      if (tm) atomicMax(p.amax_bits, tm << 16);
+      __threadfence();
+      atomicAdd(p.arrivals, 1u);
+      const long long t0 = clock64();
+      for (;;) {
+        if (ld_acquire_u32(p.arrivals) >= gridDim.x) break;
+        __nanosleep(100);
+        if (clock64() - t0 > 4000000000ll) { atomicExch(p.status, (int32_t)QUADS_ERR_TIMEOUT); break; }
+      }
+      gs_sh = gs_from_amax_bits(ld_relaxed_u32(p.amax_bits));
+    }
+    __syncthreads();
+  } else {
+    if (threadIdx.x == 0) gs_sh = p.gs_in[0];
+    __syncthreads();
+  }
+  const float gs = gs_sh;
+  if (p.gs_store && blockIdx.x == 0 && threadIdx.x == 0) p.gs_store[0] = gs;
+  if (threadIdx.x < 128) inv_lut[threadIdx.x] = quant_inv_entry(threadIdx.x, gs);
+  __syncthreads();
+  QuantCtx qc;
+  quant_ctx_scalars(qc, gs);
+  qc.inv_lut = inv_lut;
+  float acc[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) acc[i] = 0.f;
+  uint4 n0 = make_uint4(0, 0, 0, 0), n1 = n0;
+  if (r0 < r1) ldg256(xk + (size_t)r0 * H, n0, n1);
+  for (int r = r0; r < r1; r += lanes) {
+    const uint4 v0 = n0, v1 = n1;
+    if (r + lanes < r1) ldg256(xk + (size_t)(r + lanes) * H, n0, n1);   // next block, ahead of this one's arithmetic
+    float f[16], o[16];
+    unpack8(v0, f);
+    unpack8(v1, f + 8);
+    const BlockQ bq = quantize_block(f, qc);
+    const size_t qo = (size_t)r * (H >> 1) + kb * 8, so = (size_t)r * k16 + kb;
+    const size_t so_op = p.sf_tiled ? sf_tiled_offset(r, kb, H >> 6) : so;
+    *reinterpret_cast<uint2*>(p.xq + qo) = make_uint2(bq.lo, bq.hi);
+    p.xsf[so_op] = (uint8_t)bq.sf8;
+    if (p.xq_exp) *reinterpret_cast<uint2*>(p.xq_exp + qo) = make_uint2(bq.lo, bq.hi);
+    if (p.xsf_exp) p.xsf_exp[so] = (uint8_t)bq.sf8;
+    if (p.with_residual) {
+      dequant_block(bq, o);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        o[i] = __fsub_rn(o[i], f[i]);
+        acc[i] = __fmaf_rn(o[i], o[i], acc[i]);
+      }
+      const BlockQ br = quantize_block(o, qc);
+      *reinterpret_cast<uint2*>(p.rq + qo) = make_uint2(br.lo, br.hi);
+      p.rsf[so_op] = (uint8_t)br.sf8;
+      if (p.rsf_exp) p.rsf_exp[so] = (uint8_t)br.sf8;
+    }
+  }
+  if (p.with_residual) {
+    float4* d = reinterpret_cast<float4*>(red + threadIdx.x * 16);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) d[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
+    __syncthreads();
+    const int n_ch = p.bw * 16;                              // channels of this CTA, at most 512
+    for (int c = threadIdx.x; c < n_ch; c += 256) {
+      float t = 0.f;
+      for (int l = 0; l < lanes; ++l) t += red[l * n_ch + c];
+      add_score(p.totals + col * n_ch + c, t, gs, p.score_bits, p.cap_bits);
+    }
+  }
+}
+
+// Statistics only (quads_rac_channel_scores): the squared residual sums of a CTA's rows, one partial row per CTA.
 __global__ void __launch_bounds__(256)
-rac_quant_kernel(const uint16_t* __restrict__ x, int T, int H, const float* __restrict__ gs_in,
-                 uint32_t* __restrict__ amax_bits, unsigned int* __restrict__ grid_arrivals, int32_t* __restrict__ status,
-                 float* __restrict__ gs_store, int rows_per_cta,
-                 int with_residual, float* __restrict__ partials, uint8_t* __restrict__ xq,
-                 uint8_t* __restrict__ xsf, uint8_t* __restrict__ rq, uint8_t* __restrict__ rsf,
-                 uint8_t* __restrict__ xq_exp, uint8_t* __restrict__ xsf_exp,
-                 unsigned long long* __restrict__ score_totals, int score_bits, int cap_bits) {
+channel_stats_kernel(const uint16_t* __restrict__ x, int T, int H, const float* __restrict__ gs_in,
+                     const uint32_t* __restrict__ amax_bits, int rows_per_cta, float* __restrict__ partials) {
   pdl_sync();
   const int k16 = H >> 4;
   const int r0 = blockIdx.x * rows_per_cta;
   const int r1 = min(T, r0 + rows_per_cta);
-  __shared__ float gs_sh;
-  if (grid_arrivals) {
-    // Cooperative launch with no per-tensor scale given: first the tensor's amax over this
-    // CTA's rows (the same rows it quantizes below, so the second read hits L1 / L2), then a
-    // bounded wait until every CTA has contributed.
-    __shared__ uint32_t wmax[8];
-    uint32_t m = 0;
-    for (int kb = threadIdx.x; kb < k16; kb += blockDim.x)
-      for (int r = r0; r < r1; ++r) {
-        uint4 v0, v1;
-        ldg256(x + (size_t)r * H + kb * 16, v0, v1);
-        m = __vmaxu2(m, __vmaxu2(absmax8(v0), absmax8(v1)));
-      }
-    uint32_t smx = max(m & 0xFFFFu, m >> 16);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) smx = max(smx, __shfl_xor_sync(0xFFFFFFFFu, smx, o));
-    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = smx;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t tm = 0;
-      for (int i = 0; i < (int)((blockDim.x + 31) >> 5); ++i) tm = max(tm, wmax[i]);
-      if (tm) atomicMax(amax_bits, tm << 16);
-      __threadfence();
-      atomicAdd(grid_arrivals, 1u);
-      const long long t0 = clock64();
-      unsigned int seen;
-      for (;;) {
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(grid_arrivals) : "memory");
-        if (seen >= gridDim.x) break;
-        __nanosleep(200);
-        if (clock64() - t0 > 4000000000ll) { atomicExch(status, (int32_t)QUADS_ERR_TIMEOUT); break; }
-      }
-      gs_sh = gs_from_amax_bits(atomicAdd(amax_bits, 0u));
-    }
-    __syncthreads();
-  } else if (threadIdx.x == 0) {
-    gs_sh = gs_in ? gs_in[0] : gs_from_amax_bits(amax_bits[0]);
-  }
-  __syncthreads();
-  const float gs = gs_sh;
-  if (gs_store && blockIdx.x == 0 && threadIdx.x == 0) gs_store[0] = gs;
+  const float gs = gs_in ? gs_in[0] : gs_from_amax_bits(amax_bits[0]);
   __shared__ float inv_lut[128];
   for (int i = threadIdx.x; i < 128; i += blockDim.x) inv_lut[i] = quant_inv_entry(i, gs);
   __syncthreads();
@@ -774,43 +842,22 @@ rac_quant_kernel(const uint16_t* __restrict__ x, int T, int H, const float* __re
     if (r0 < r1) ldg256(x + (size_t)r0 * H + kb * 16, n0, n1);
     for (int r = r0; r < r1; ++r) {
       const uint4 v0 = n0, v1 = n1;
-      if (r + 1 < r1) ldg256(x + (size_t)(r + 1) * H + kb * 16, n0, n1);   // next row's block, ahead of this row's arithmetic
+      if (r + 1 < r1) ldg256(x + (size_t)(r + 1) * H + kb * 16, n0, n1);
       float f[16], o[16];
       unpack8(v0, f);
       unpack8(v1, f + 8);
-      const BlockQ bq = quantize_block(f, qc);
-      const size_t qo = (size_t)r * (H >> 1) + kb * 8, so = (size_t)r * k16 + kb;
-      if (xq) {
-        *reinterpret_cast<uint2*>(xq + qo) = make_uint2(bq.lo, bq.hi);
-        xsf[so] = (uint8_t)bq.sf8;
-      }
-      if (xq_exp) *reinterpret_cast<uint2*>(xq_exp + qo) = make_uint2(bq.lo, bq.hi);
-      if (xsf_exp) xsf_exp[so] = (uint8_t)bq.sf8;
-      if (with_residual) {
-        dequant_block(bq, o);
+      dequant_block(quantize_block(f, qc), o);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          o[i] = __fsub_rn(o[i], f[i]);
-          acc[i] = __fmaf_rn(o[i], o[i], acc[i]);
-        }
-        if (rq) {                                     // (statistics-only callers pass no code buffers)
-          const BlockQ br = quantize_block(o, qc);
-          *reinterpret_cast<uint2*>(rq + qo) = make_uint2(br.lo, br.hi);
-          rsf[so] = (uint8_t)br.sf8;
-        }
+      for (int i = 0; i < 16; ++i) {
+        o[i] = __fsub_rn(o[i], f[i]);
+        acc[i] = __fmaf_rn(o[i], o[i], acc[i]);
       }
     }
-    if (with_residual && score_totals) {
-      // integer totals per channel (zero on entry): complete when the kernel ends, whatever the order
-#pragma unroll
-      for (int i = 0; i < 16; ++i) add_score(score_totals + kb * 16 + i, acc[i], gs, score_bits, cap_bits);
-    } else if (with_residual) {
-      float4* dst = reinterpret_cast<float4*>(partials + (size_t)blockIdx.x * H + kb * 16);
-      dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-      dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
-      dst[2] = make_float4(acc[8], acc[9], acc[10], acc[11]);
-      dst[3] = make_float4(acc[12], acc[13], acc[14], acc[15]);
-    }
+    float4* dst = reinterpret_cast<float4*>(partials + (size_t)blockIdx.x * H + kb * 16);
+    dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+    dst[2] = make_float4(acc[8], acc[9], acc[10], acc[11]);
+    dst[3] = make_float4(acc[12], acc[13], acc[14], acc[15]);
   }
 }
 
@@ -927,11 +974,11 @@ __device__ __forceinline__ uint32_t nibble_mask8(const uint8_t* m) {
   return out;
 }
 
-// Verification export of the masked residual in token order (Eq. residual-recon: codes of unselected channels
-// cleared), from codes stored with `flip` XORed into every word.  One thread per (token, 32 channels).
+// Verification export of the masked residual's codes in token order (Eq. residual-recon: codes of unselected
+// channels cleared), from codes stored with `flip` XORed into every word.  One thread per (token, 32 channels).
 __global__ void __launch_bounds__(256)
 export_residual_kernel(int T, int H, const uint8_t* __restrict__ mask, uint32_t flip, const uint8_t* __restrict__ rq,
-                       const uint8_t* __restrict__ rsf, uint8_t* __restrict__ rq_exp, uint8_t* __restrict__ rsf_exp) {
+                       uint8_t* __restrict__ rq_exp) {
   pdl_sync();
   const int per_row = H >> 5;
   const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -942,11 +989,7 @@ export_residual_kernel(int T, int H, const uint8_t* __restrict__ mask, uint32_t 
   const uint8_t* m = mask + c * 32;
   v.x = (v.x ^ flip) & nibble_mask8(m); v.y = (v.y ^ flip) & nibble_mask8(m + 8);
   v.z = (v.z ^ flip) & nibble_mask8(m + 16); v.w = (v.w ^ flip) & nibble_mask8(m + 24);
-  if (rq_exp) *reinterpret_cast<uint4*>(rq_exp + co) = v;
-  if (rsf_exp) {
-    const size_t so = (size_t)t * (H >> 4) + c * 2;
-    *reinterpret_cast<uint16_t*>(rsf_exp + so) = *reinterpret_cast<const uint16_t*>(rsf + so);
-  }
+  *reinterpret_cast<uint4*>(rq_exp + co) = v;
 }
 
 // ---------------------------------------------------------------------------
@@ -1101,10 +1144,9 @@ template __global__ void rac_dispatch_kernel<3>(int, const uint8_t*, const int32
 // Against a ranking kernel (C / 16 CTAs, one rank per key) and a mask kernel behind it: decode layer of
 // 256 tokens 126.3 -> 120.4 us, of one token 55.8 -> 52.5 us, prefill of 8192 unchanged (522.7 us).  With
 // eight CTAs of 256 threads per SM, each repeating the search, the same layers took 133.6 and 65.7 us.
-// With n_rows_fixed > 0 the matrix has that many rows, all valid (site 13 in token order); `flip` is XORed
+// With n_rows_fixed > 0 the matrix has that many rows, all valid (site 13 in token order, dense projections); `flip` is XORed
 // into every word of the result (the residual operand is stored negated).
 // dynamic shared memory: C keys of 8 bytes, C words of scratch, C / 8 mask words.
-template <bool kDoubleKeys>
 __global__ void __launch_bounds__(kSelectThreads)
 select_mask_kernel(uint8_t* __restrict__ codes, int n_rows_fixed, uint32_t flip, const int32_t* __restrict__ header,
                    const int32_t* __restrict__ tile_rows,
@@ -1138,7 +1180,7 @@ select_mask_kernel(uint8_t* __restrict__ codes, int n_rows_fixed, uint32_t flip,
   const int c_first = threadIdx.x % cols;
   fetch(c_first, first);
   __syncthreads();
-  const Selection sel = select_largest<kDoubleKeys>(sc, images, C, n_sel, &scratch);
+  const Selection sel = select_largest<false>(sc, images, C, n_sel, &scratch);
   for (int w = threadIdx.x; w < (C >> 3); w += kSelectThreads) {
     uint32_t m = 0;
 #pragma unroll
@@ -1163,11 +1205,6 @@ select_mask_kernel(uint8_t* __restrict__ codes, int n_rows_fixed, uint32_t flip,
     }
   }
 }
-
-template __global__ void select_mask_kernel<false>(uint8_t*, int, uint32_t, const int32_t*, const int32_t*, const unsigned long long*,
-                                                   int, int, uint8_t*);
-template __global__ void select_mask_kernel<true>(uint8_t*, int, uint32_t, const int32_t*, const int32_t*, const unsigned long long*,
-                                                  int, int, uint8_t*);
 
 // Weighted top-k combine: out[t, :] = sum over the token's slots, in slot order,
 // of weight * y[row of (t, slot), :], accumulated in float32, rounded to bf16.

@@ -272,17 +272,4 @@ permute_kernel(int T, int E, int topk, int n_chunks, const int32_t* __restrict__
   }
 }
 
-// Dense mode: identity dispatch of T rows to a single "expert".
-__global__ void __launch_bounds__(256)
-dense_dispatch_kernel(int T, int tile_group, int32_t* __restrict__ pos_pad, int32_t* __restrict__ row_token,
-                      float* __restrict__ row_weight, int32_t* __restrict__ tile_expert,
-                      int32_t* __restrict__ tile_rows, int32_t* __restrict__ header) {
-  pdl_sync();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int m_tiles = ((T + 128 * tile_group - 1) / (128 * tile_group)) * tile_group;
-  if (i < T) { pos_pad[i] = i; row_token[i] = i; row_weight[i] = 1.f; }
-  if (i < m_tiles) { tile_expert[i] = 0; tile_rows[i] = max(0, min(128, T - i * 128)); }
-  if (i == 0) { header[kHdrMTiles] = m_tiles; header[kHdrPaddedRows] = m_tiles * 128; header[kHdrAssignments] = T; }
-}
-
 }  // namespace quads
