@@ -85,8 +85,12 @@ def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
+# The current stream's handle without a torch.cuda.Stream object around it (0.2 us instead of 3.2 us per call).
+_raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+
+
 def _stream():
-    return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_current_device())
 
 
 def sf_tiled_bytes(rows, K):
@@ -108,10 +112,10 @@ def quantize_nvfp4(x, gs=None, sf_layout=SF_LINEAR, out=None, workspace=None):
     dev = x.device
     if out is None:
         q = torch.empty(rows, K // 2, dtype=torch.uint8, device=dev)
-        n_sf = sf_tiled_bytes(rows, K) if sf_layout == SF_TILED else rows * (K // 16)
-        sf = torch.empty(n_sf, dtype=torch.uint8, device=dev)
         if sf_layout == SF_LINEAR:
-            sf = sf.view(rows, K // 16)
+            sf = torch.empty(rows, K // 16, dtype=torch.uint8, device=dev)
+        else:
+            sf = torch.empty(sf_tiled_bytes(rows, K), dtype=torch.uint8, device=dev)
         gs_out = torch.empty(1, dtype=torch.float32, device=dev)
     else:
         q, sf, gs_out = out
