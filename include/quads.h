@@ -214,20 +214,15 @@ quads_status quads_fake_quant_weights_noalloc(const void* w, int64_t n_tensors, 
  * Limits: E <= 256, topk <= 16 and <= E, H <= 16384, I <= 16384; a size outside
  * them returns QUADS_ERR_SHAPE before anything is launched.
  *
- * The call allocates nothing and never synchronises the host.  Part of the
- * work (routing, the dispatched copies of Q_A(X)) is enqueued on a second
- * stream of the library's own, forked from and joined back into the caller's
- * stream with events, so the call as a whole is ordered like any other work on
- * `cuda_stream` and can be captured into a CUDA graph (make one ordinary call
- * first: kernel attributes are set on first use).  Device-side waits are bounded;
- * one that gives up writes QUADS_ERR_TIMEOUT to a status word in the workspace,
- * read with quads_moe_async_status().  Every call resets that word on its stream
- * before its first kernel: poll after each call whose status matters.
- * One side stream per device serves all callers: calls on one device are
- * serialised on the host by a lock while they enqueue, and a CUDA-graph capture
- * of a call must not overlap, in time, other MoE calls on the same device (they
- * would enqueue into the capturing side stream).  The timing and trace aids
- * below keep process-wide state and are not thread-safe.
+ * The call allocates nothing, never synchronises the host and enqueues all of
+ * its work on `cuda_stream`, so it can be captured into a CUDA graph (make one
+ * ordinary call first: kernel attributes are set on first use).  Beyond a few
+ * hundred tokens its first kernel is a cooperative launch whose thread blocks
+ * meet at counters.  Device-side waits are bounded; one that gives up writes
+ * QUADS_ERR_TIMEOUT to a status word in the workspace, read with
+ * quads_moe_async_status().  Every call resets that word on its stream before
+ * its first kernel or in it: poll after each call whose status matters.  The
+ * timing and trace aids below keep process-wide state and are not thread-safe.
  */
 enum {
   QUADS_W4A4 = 0,   /* both operands NVFP4, block-scaled FP4 tensor-core product (+ RAC) */

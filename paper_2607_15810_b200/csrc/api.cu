@@ -119,12 +119,12 @@ inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_
 
 // ------------------------------------------------------------------ workspace
 struct MoeLayout {
-  size_t header, amax, keys13, keys2, expert_total, ids, wts, chunk_counts, chunk_base, offsets, tile_prefix, tile_expert, tile_rows;
-  size_t perm, pos_pad, row_token, row_weight;
+  size_t header, amax, keys13, keys2, ids, wts, route_counts, offsets, tile_prefix, tile_expert, tile_rows;
+  size_t perm, pos_pad, row_token;
   size_t mask13, xq_tok, xsf_tok, rq_tok, rsf_tok, xq_pad, xsf, rq_pad, rsf;
   size_t hq_pad, hsf, r2q_pad, r2sf, mask2, y_pad, dec;
   size_t total;
-  int n_chunks, m_tiles_max;
+  int m_tiles_max;
 };
 
 MoeLayout moe_layout(int T, int H, int I, int E, int topk, int N) {
@@ -132,7 +132,6 @@ MoeLayout moe_layout(int T, int H, int I, int E, int topk, int N) {
   const bool dense = (I == 0);
   const int64_t A = dense ? T : (int64_t)T * topk;
   const int Ee = dense ? 1 : E;
-  L.n_chunks = (T + kRouteTokensPerCta - 1) / kRouteTokensPerCta;
   L.m_tiles_max = ((int)(A / 256) + Ee) * 2;      // enough for either tile grouping (1 or 2)
   const size_t pad_rows = (size_t)L.m_tiles_max * 128;
   size_t o = 0;
@@ -141,11 +140,9 @@ MoeLayout moe_layout(int T, int H, int I, int E, int topk, int N) {
   L.amax = take((size_t)kAmaxPartsMax * 4);    // the amax word; also the quantizer's scratch in the one-sided modes
   L.keys13 = take((size_t)H * 8);                  // integer column scores of site 13, zeroed with the header
   L.keys2 = take((size_t)I * 8);                   // zeroed with the header: the first projection's epilogue adds to it
-  L.expert_total = take((size_t)Ee * 4);           // zeroed with the header: the routing kernel adds to it
+  L.route_counts = take(dense ? 0 : (size_t)kRouteCtasMax * Ee * 4);   // zeroed with the header
   L.ids = take((size_t)A * 4);
   L.wts = take((size_t)A * 4);
-  L.chunk_counts = take((size_t)L.n_chunks * Ee * 4);
-  L.chunk_base = take((size_t)L.n_chunks * Ee * 4);
   L.offsets = take((size_t)(Ee + 1) * 4);
   L.tile_prefix = take((size_t)(Ee + 1) * 4);
   L.tile_expert = take((size_t)L.m_tiles_max * 4);
@@ -153,7 +150,6 @@ MoeLayout moe_layout(int T, int H, int I, int E, int topk, int N) {
   L.perm = take((size_t)A * 4);
   L.pos_pad = take((size_t)A * 4);
   L.row_token = take(pad_rows * 4);
-  L.row_weight = take(pad_rows * 4);
   L.mask13 = take((size_t)H);
   L.xq_tok = take((size_t)T * (H / 2));
   L.xsf_tok = take((size_t)T * (H / 16));
@@ -201,49 +197,6 @@ inline void trace_mark(const char* name, cudaStream_t st) {
   ++g_trace.n;
 }
 
-// Side stream on which the routing chain (route -> scan -> permute) runs next to the
-// activation chain (amax -> quantize -> select); both are joined before the dispatch copy.
-struct SideStream {
-  cudaStream_t stream = nullptr;
-  cudaEvent_t fork = nullptr, mid = nullptr, tables = nullptr, join = nullptr;
-  bool ok = false;
-};
-std::mutex g_side_mu;
-// Call with g_side_mu held (the per-device objects are created on first use).
-SideStream* side_stream() {
-  static SideStream per_device[64];
-  static const bool disabled = [] { const char* e = getenv("QUADS_NO_OVERLAP"); return e && e[0] == '1'; }();
-  if (disabled) return nullptr;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-  SideStream& s = per_device[dev];
-  if (!s.ok) {
-    if (cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking) != cudaSuccess) return nullptr;
-    if (cudaEventCreateWithFlags(&s.fork, cudaEventDisableTiming) != cudaSuccess) return nullptr;
-    if (cudaEventCreateWithFlags(&s.mid, cudaEventDisableTiming) != cudaSuccess) return nullptr;
-    if (cudaEventCreateWithFlags(&s.tables, cudaEventDisableTiming) != cudaSuccess) return nullptr;
-    if (cudaEventCreateWithFlags(&s.join, cudaEventDisableTiming) != cudaSuccess) return nullptr;
-    s.ok = true;
-  }
-  return &s;
-}
-
-// Joins the side stream back into the caller's stream when the scope is left before the regular
-// join (an error return between fork and join): without it the side stream would stay forked
-// and, under stream capture, the captured graph would be left with an unjoined branch.
-struct SideJoinGuard {
-  SideStream* side = nullptr;
-  cudaStream_t main = nullptr;
-  bool joined = true;
-  void arm(SideStream* s, cudaStream_t st) { side = s; main = st; joined = false; }
-  void join() {
-    if (joined || !side) return;
-    joined = true;
-    if (cudaEventRecord(side->join, side->stream) == cudaSuccess) cudaStreamWaitEvent(main, side->join, 0);
-  }
-  ~SideJoinGuard() { join(); }
-};
-
 // GEMM variant of a call.  1: single-CTA tiles of 128 x 256; 2: CTA pairs computing 256 x 256
 // tiles with cta_group::2 MMAs: about 7 % (first projection) / 5 % (second) faster per tile, but
 // every expert's rows are then padded to a multiple of 256, i.e. half a tile more per expert on
@@ -260,19 +213,12 @@ int gemm_cta_group_for(int64_t rows, int experts) {
   return rows >= (int64_t)1024 * (experts > 0 ? experts : 1) ? 2 : 1;
 }
 
-// Ranking of C order-preserving 64-bit score keys: mask of the n_sel largest.
-quads_status run_rank(const unsigned long long* keys, int C, int n_sel, uint8_t* mask, cudaStream_t st) {
-  QUADS_CUDA_OK(set_max_dynamic_smem<rank_select_kernel>(128 * 1024));
-  QUADS_CUDA_OK(launch_kernel(rank_select_kernel, dim3((C + 15) / 16), dim3(256), (size_t)((size_t)C * 8), st, keys, C, n_sel, mask));
-  return QUADS_OK;
-}
-
 // Selection and masking of a code matrix in one launch (see select_mask_kernel).
-quads_status run_select_mask(uint8_t* codes, int n_rows_fixed, uint32_t flip, const int32_t* header, const int32_t* tile_rows,
-                             const unsigned long long* keys, int C, int n_sel, uint8_t* mask_out, int sm_count, cudaStream_t st) {
+quads_status launch_select_mask(uint8_t* codes, int n_rows_fixed, uint32_t flip, const int32_t* header, const int32_t* tile_rows,
+                                const unsigned long long* keys, int C, int n_sel, uint8_t* mask_out, int sm_count, cudaStream_t st) {
   QUADS_CUDA_OK(set_max_dynamic_smem<select_mask_kernel>(16384 * 12 + 16384 / 2));
-  QUADS_CUDA_OK(launch_kernel(select_mask_kernel, dim3(sm_count), dim3(kSelectThreads), (size_t)C * 12 + C / 2, st, codes,
-                              n_rows_fixed, flip, header, tile_rows, keys, C, n_sel, mask_out));
+  QUADS_CUDA_OK(launch_kernel(select_mask_kernel, dim3(sm_count), dim3(kSelectThreads), (size_t)C * 12 + C / 2, st, codes, n_rows_fixed,
+                              flip, header, tile_rows, keys, C, n_sel, mask_out));
   return QUADS_OK;
 }
 
@@ -707,7 +653,6 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   int32_t* perm = reinterpret_cast<int32_t*>(P(L.perm));
   int32_t* pos_pad = reinterpret_cast<int32_t*>(P(L.pos_pad));
   int32_t* row_token = reinterpret_cast<int32_t*>(P(L.row_token));
-  float* row_weight = reinterpret_cast<float*>(P(L.row_weight));
   const uint16_t* x = static_cast<const uint16_t*>(a->x);
   const int A = T * topk;
   const size_t pad_rows = (size_t)L.m_tiles_max * 128;
@@ -761,7 +706,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
       r.logits = a->router_logits;
       r.T = T; r.E = E; r.topk = topk; r.renormalize = a->renormalize; r.e_lo = e_lo; r.e_hi = e_lo + e_cnt;
       r.wts = wts; r.offsets = offsets; r.tile_prefix = tile_prefix; r.tile_expert = tile_expert; r.tile_rows = tile_rows;
-      r.header = header; r.perm = perm; r.pos_pad = pos_pad; r.row_token = row_token; r.row_weight = row_weight;
+      r.header = header; r.perm = perm; r.pos_pad = pos_pad; r.row_token = row_token;
       r.zero_u64 = reinterpret_cast<unsigned long long*>(P(L.keys2)); r.n_zero = I;
       r.ids_out = a->topk_ids; r.wts_out = a->topk_w; r.offsets_out = a->expert_offsets; r.perm_out = a->perm;
       if ((s = launch_route_small(r, st)) != QUADS_OK) return s;
@@ -782,143 +727,58 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
     trace_mark("front", st);
   }
 
-  // ---- routing and dispatch order: on a side stream, next to the activation chain below
-  // (declared in this order: on an early return the guard joins first, then the lock is released)
-  std::unique_lock<std::mutex> side_lock(g_side_mu, std::defer_lock);
-  SideJoinGuard side_guard;
-  SideStream* side = nullptr;
   if (!small) {
-    if (!dense && !g_trace.enabled) {
-      side_lock.lock();                       // event record / wait pairs of two host threads must not interleave
-      side = side_stream();
-      if (!side) side_lock.unlock();
-    }
-    cudaStream_t rs = st;
-    if (side) {
-      QUADS_CUDA_OK(cudaEventRecord(side->fork, st));
-      QUADS_CUDA_OK(cudaStreamWaitEvent(side->stream, side->fork, 0));
-      side_guard.arm(side, st);
-      rs = side->stream;
-    }
-    if (!dense) {
-      int32_t* chunk_counts = reinterpret_cast<int32_t*>(P(L.chunk_counts));
-      int32_t* chunk_base = reinterpret_cast<int32_t*>(P(L.chunk_base));
-      int32_t* expert_total = reinterpret_cast<int32_t*>(P(L.expert_total));
-      {
-        auto route = E <= 32 ? route_kernel_t<1> : (E <= 64 ? route_kernel_t<2> : (E <= 128 ? route_kernel_t<4> : route_kernel_t<8>));
-        QUADS_CUDA_OK(launch_kernel(route, dim3(L.n_chunks), dim3(256), (size_t)(0), rs, a->router_logits, T, E, topk,
-                                    a->renormalize, ids, wts, chunk_counts, expert_total, a->topk_ids, a->topk_w, e_lo, e_lo + e_cnt));
-      }
-      trace_mark("route", st);
-      QUADS_CUDA_OK(launch_kernel(scan_kernel, dim3(E), dim3(256), (size_t)(0), rs, E, L.n_chunks, cta_group, chunk_counts, expert_total, chunk_base, offsets, tile_prefix, tile_expert, tile_rows, header, a->expert_offsets));
-      trace_mark("scan", st);
-      QUADS_CUDA_OK(launch_kernel(permute_kernel, dim3(L.n_chunks), dim3(128), (size_t)(0), rs, T, E, topk, L.n_chunks, ids, wts, chunk_base, offsets, tile_prefix, perm, pos_pad, row_token, row_weight, a->perm, e_lo, e_lo + e_cnt));
-    }
-    trace_mark("permute", st);
-
-    // ---- site 13: per-tensor scale, quantization, residual and channel scores in one launch.  A dense projection's
-    // rows are its operand as they are (tiled scales); the others stay in token order.
+    // ---- site 13: per-tensor scale, quantization, residual and channel scores in one launch, with the routing of a
+    // MoE call as a second role beside it.  A dense projection's rows are its operand as they are (tiled scales);
+    // the others stay in token order.
     unsigned long long* keys13 = reinterpret_cast<unsigned long long*>(P(L.keys13));
-    {
-      QuantRowsArgs q{};
-      q.x = x; q.T = T; q.H = H; q.with_residual = nsel13 > 0; q.sf_tiled = dense;
-      q.bw = (H / 16) % 32 == 0 ? 32 : ((H / 16) % 16 == 0 ? 16 : 8);
-      q.n_col = H / 16 / q.bw;
-      // as many row ranges as are resident at once, each at least a row per row lane
-      static std::atomic<int> per_sm_cache{0};       // same kernel and block size on every sm_100 device
-      int per_sm = per_sm_cache.load();
-      if (per_sm == 0) {
-        QUADS_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, quant_rows_kernel, 256, 0));
-        per_sm_cache.store(per_sm);
-      }
-      if (side) per_sm = std::min(per_sm, kQuantRowsPerSm - 1);   // room for the routing kernels beside it
-      const int lanes = 256 / q.bw;
-      const int n_rg = std::max(1, std::min(per_sm * di.sm_count / q.n_col, (T + lanes - 1) / lanes));
-      q.rows_per_cta = ((T + n_rg - 1) / n_rg + lanes - 1) / lanes * lanes;
-      const int n_used = (T + q.rows_per_cta - 1) / q.rows_per_cta;
-      q.gs_in = a->a13_gs; q.amax_bits = amax_bits;
-      q.arrivals = a->a13_gs ? nullptr : reinterpret_cast<unsigned int*>(header + kHdrArrivals);
-      q.status = header + kHdrStatus; q.gs_store = a->a13_gs_out;
-      q.xq = P(dense ? L.xq_pad : L.xq_tok); q.xsf = P(dense ? L.xsf : L.xsf_tok);
-      q.rq = P(dense ? L.rq_pad : L.rq_tok); q.rsf = P(dense ? L.rsf : L.rsf_tok);
-      q.xq_exp = a->xq; q.xsf_exp = a->xsf; q.rsf_exp = a->rsf;
-      q.totals = keys13;
-      // a CTA's sum covers rows_per_cta rows (< rows * 2^18 in units of the squared scale); the sums of
-      // all row ranges must fit 62 bits together
-      int cap_bits = 18, ranges_log2 = 0;
-      while ((1 << (cap_bits - 18)) < q.rows_per_cta) ++cap_bits;
-      while ((1 << ranges_log2) < n_used) ++ranges_log2;
-      q.cap_bits = cap_bits;
-      q.score_bits = std::max(0, std::min(26, 62 - cap_bits - ranges_log2));
-      const dim3 grid(n_used * q.n_col);
-      if (q.arrivals) {                               // its CTAs wait for one another
-        void* args[] = {&q};
-        QUADS_CUDA_OK(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(quant_rows_kernel), grid, dim3(256), args, 0, st));
-        note_launch();
-      } else {
-        QUADS_CUDA_OK(launch_kernel(quant_rows_kernel, grid, dim3(256), (size_t)0, st, q));
-      }
+    QuantRowsArgs q{};
+    q.x = x; q.T = T; q.H = H; q.with_residual = nsel13 > 0; q.sf_tiled = dense;
+    q.gs_in = a->a13_gs; q.amax_bits = amax_bits;
+    q.arrivals = reinterpret_cast<unsigned int*>(header + kHdrArrivals);
+    q.status = header + kHdrStatus; q.gs_store = a->a13_gs_out;
+    q.xq = P(dense ? L.xq_pad : L.xq_tok); q.xsf = P(dense ? L.xsf : L.xsf_tok);
+    q.rq = P(dense ? L.rq_pad : L.rq_tok); q.rsf = P(dense ? L.rsf : L.rsf_tok);
+    q.xq_exp = a->xq; q.xsf_exp = a->xsf; q.rsf_exp = a->rsf;
+    q.totals = keys13;
+    if (dense) {
+      s = launch_quant_rows(q, di.sm_count, st);
+    } else {
+      RouteArgs r{};
+      r.logits = a->router_logits;
+      r.T = T; r.E = E; r.topk = topk; r.renormalize = a->renormalize; r.e_lo = e_lo; r.e_hi = e_lo + e_cnt;
+      r.slot_rows = 128; r.tile_group = cta_group;
+      r.ids = ids; r.wts = wts; r.counts = reinterpret_cast<int32_t*>(P(L.route_counts));
+      r.arrivals = reinterpret_cast<unsigned int*>(header + kHdrRouteArrivals); r.status = header + kHdrStatus;
+      r.offsets = offsets; r.tile_prefix = tile_prefix; r.tile_expert = tile_expert; r.tile_rows = tile_rows; r.header = header;
+      r.perm = perm; r.pos_pad = pos_pad; r.row_token = row_token;
+      r.ids_out = a->topk_ids; r.wts_out = a->topk_w; r.offsets_out = a->expert_offsets; r.perm_out = a->perm;
+      s = launch_front(q, r, di.sm_count, st);
     }
-    trace_mark("quant13", st);
-    // verification exports of the selection and, from codes stored with `flip` applied, of the masked residual
-    auto export13 = [&](const uint8_t* codes, uint32_t flip) -> quads_status {
+    if (s != QUADS_OK) return s;
+    trace_mark("route+quantize", st);
+    const bool in_place = swapped || dense;           // the operand is in token order: the residual is masked and negated there
+    if (!in_place) {
+      DispatchArgs d{};
+      d.H = H; d.n_sel = nsel13; d.keys = keys13; d.mask = mask13;
+      d.header = header; d.tile_rows = tile_rows; d.row_token = row_token;
+      d.xq = q.xq; d.xsf = q.xsf; d.rq = q.rq; d.rsf = q.rsf;
+      d.xq_pad = P(L.xq_pad); d.xsf_tiled = P(L.xsf); d.rq_pad = P(L.rq_pad); d.rsf_tiled = P(L.rsf);
+      if ((s = launch_dispatch(d, L.m_tiles_max, di.sm_count, st)) != QUADS_OK) return s;
+    } else if (nsel13 > 0) {
+      s = launch_select_mask(q.rq, T, 0x88888888u, header, tile_rows, keys13, H, nsel13, (a->sel13 || a->rq) ? mask13 : nullptr,
+                             di.sm_count, st);
+      if (s != QUADS_OK) return s;
+    }
+    if (nsel13 > 0) {                                 // verification exports
       if (a->sel13) QUADS_CUDA_OK(launch_kernel(sel_list_kernel, dim3(1), dim3(1024), (size_t)0, st, mask13, H, a->sel13));
       if (a->rq) {
         const int64_t chunks = (int64_t)T * (H / 32);
         QUADS_CUDA_OK(launch_kernel(export_residual_kernel, dim3((unsigned)((chunks + 255) / 256)), dim3(256), (size_t)0, st, T, H,
-                                    mask13, flip, codes, a->rq));
-      }
-      return QUADS_OK;
-    };
-    if (swapped || dense) {
-      // the operand is in token order: the residual is masked and negated in place
-      if (nsel13 > 0) {
-        uint8_t* rq = P(dense ? L.rq_pad : L.rq_tok);
-        uint8_t* mask_out = (a->sel13 || a->rq) ? mask13 : nullptr;
-        if ((s = run_select_mask(rq, T, 0x88888888u, header, tile_rows, keys13, H, nsel13, mask_out, di.sm_count, st)) != QUADS_OK) return s;
-        if ((s = export13(rq, 0x88888888u)) != QUADS_OK) return s;
-      }
-      trace_mark("select13+mask", st);
-      if (side) {
-        side_guard.join();
-        side_lock.unlock();
-      }
-    } else {
-      // The dispatched copies of Q(x) need only the dispatch order and the codes: with a side stream
-      // they are written there, next to the channel selection; the residual copies (which need the
-      // selection and the dispatch tables, not the other copies) follow on the main stream and may run
-      // beside them: the two streams meet again only in front of the first projection.
-      const bool split_scatter = side != nullptr && nsel13 > 0;
-      auto dispatch = [&](int parts, cudaStream_t s_) {
-        auto k = parts == 1 ? rac_dispatch_kernel<1> : (parts == 2 ? rac_dispatch_kernel<2> : rac_dispatch_kernel<3>);
-        return launch_kernel(k, dim3(L.m_tiles_max), dim3(256), (size_t)(0), s_, H, mask13, header,
-                             tile_rows, row_token, P(L.xq_tok), P(L.xsf_tok), P(L.rq_tok), P(L.rsf_tok), P(L.xq_pad),
-                             P(L.xsf), P(L.rq_pad), P(L.rsf));
-      };
-      if (split_scatter) {
-        QUADS_CUDA_OK(cudaEventRecord(side->tables, side->stream));      // routing tables complete
-        QUADS_CUDA_OK(cudaEventRecord(side->mid, st));
-        QUADS_CUDA_OK(cudaStreamWaitEvent(side->stream, side->mid, 0));
-        QUADS_CUDA_OK(dispatch(1, side->stream));
-      }
-      if (nsel13 > 0) {
-        if ((s = run_rank(keys13, H, nsel13, mask13, st)) != QUADS_OK) return s;
-        if ((s = export13(P(L.rq_tok), 0u)) != QUADS_OK) return s;
-      }
-      trace_mark("select13", st);
-      if (split_scatter) {
-        QUADS_CUDA_OK(cudaStreamWaitEvent(st, side->tables, 0));
-      } else if (side) {
-        side_guard.join();
-        side_lock.unlock();
-      }
-      QUADS_CUDA_OK(dispatch(split_scatter ? 2 : (nsel13 > 0 ? 3 : 1), st));
-      if (split_scatter) {
-        side_guard.join();
-        side_lock.unlock();
+                                    mask13, in_place ? 0x88888888u : 0u, q.rq, a->rq));
       }
     }
-    trace_mark("rac_dispatch", st);
+    trace_mark("select+dispatch", st);
   }
   // ---- tensor maps
   const uint32_t act_box = swapped ? 16 : 128;
@@ -941,6 +801,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   GemmParams g{};
   g.K = H;
   g.has_resid = nsel13 > 0;
+  g.tables_late = swapped && !small && nsel13 == 0; // front kernel, then the first projection
   g.header = header; g.tile_expert = tile_expert; g.tile_rows = tile_rows;
   g.a_sf = P(L.xsf); g.r_sf = P(L.rsf);
   g.b_sf = a->w13_sf; g.b_sf_expert_stride = quads_sf_tiled_bytes(N1, H);
@@ -988,8 +849,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   if (nsel2 > 0) {
     // the scores are complete when the first projection ends (integer totals)
     const bool want_mask = a->sel2 || a->hq || a->hsf || a->r2q || a->r2sf;
-    if ((s = run_select_mask(P(L.r2q_pad), 0, 0u, header, tile_rows, g.keys2, I, nsel2, want_mask ? mask2 : nullptr,
-                                    di.sm_count, st)) != QUADS_OK)
+    if ((s = launch_select_mask(P(L.r2q_pad), 0, 0u, header, tile_rows, g.keys2, I, nsel2, want_mask ? mask2 : nullptr, di.sm_count, st)) != QUADS_OK)
       return s;
     if (a->sel2) QUADS_CUDA_OK(launch_kernel(sel_list_kernel, dim3(1), dim3(1024), (size_t)0, st, mask2, I, a->sel2));
   } else if (a->r2q) {
@@ -1016,6 +876,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   GemmParams g2 = g;
   g2.K = I;
   g2.has_resid = nsel2 > 0;
+  g2.tables_late = 0;
   g2.a_sf = P(L.hsf); g2.r_sf = P(L.r2sf);
   g2.b_sf = a->w2_sf; g2.b_sf_expert_stride = quads_sf_tiled_bytes(H, I);
   g2.b_gs = a->w2_gs; g2.a_gs = a->a2_gs; g2.a_amax_bits = nullptr;
@@ -1046,24 +907,21 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
 // ---------------------------------------------------------------------------
 namespace {
 struct Fp8Layout {
-  size_t header, expert_total, ids, wts, chunk_counts, chunk_base, offsets, tile_prefix, tile_expert, tile_rows;
-  size_t perm, pos_pad, row_token, row_weight, xq_tok, xe_tok, xq_pad, xsf, hq_pad, hsf, y_pad, total;
-  int n_chunks, m_tiles_max;
+  size_t header, ids, wts, route_counts, offsets, tile_prefix, tile_expert, tile_rows;
+  size_t perm, pos_pad, row_token, xq_tok, xe_tok, xq_pad, xsf, hq_pad, hsf, y_pad, total;
+  int m_tiles_max;
 };
 Fp8Layout fp8_layout(int T, int H, int I, int E, int topk) {
   Fp8Layout L{};
   const int64_t A = (int64_t)T * topk;
-  L.n_chunks = (T + kRouteTokensPerCta - 1) / kRouteTokensPerCta;
   L.m_tiles_max = (int)(A / 128) + E;
   const size_t pad_rows = (size_t)L.m_tiles_max * 128;
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
   L.header = take(kHdrWords * 4);
-  L.expert_total = take((size_t)E * 4);
+  L.route_counts = take((size_t)kRouteCtasMax * E * 4);   // zeroed with the header
   L.ids = take((size_t)A * 4);
   L.wts = take((size_t)A * 4);
-  L.chunk_counts = take((size_t)L.n_chunks * E * 4);
-  L.chunk_base = take((size_t)L.n_chunks * E * 4);
   L.offsets = take((size_t)(E + 1) * 4);
   L.tile_prefix = take((size_t)(E + 1) * 4);
   L.tile_expert = take((size_t)L.m_tiles_max * 4);
@@ -1071,7 +929,6 @@ Fp8Layout fp8_layout(int T, int H, int I, int E, int topk) {
   L.perm = take((size_t)A * 4);
   L.pos_pad = take((size_t)A * 4);
   L.row_token = take(pad_rows * 4);
-  L.row_weight = take(pad_rows * 4);
   L.xq_tok = take((size_t)T * H);
   L.xe_tok = take((size_t)T * (H / 128));
   L.xq_pad = take(pad_rows * (size_t)H);
@@ -1132,9 +989,6 @@ quads_status quads_moe_fp8_w8a8(const quads_moe_fp8_args* a, void* cuda_stream) 
   int32_t* header = reinterpret_cast<int32_t*>(P(L.header));
   int32_t* ids = reinterpret_cast<int32_t*>(P(L.ids));
   float* wts = reinterpret_cast<float*>(P(L.wts));
-  int32_t* chunk_counts = reinterpret_cast<int32_t*>(P(L.chunk_counts));
-  int32_t* chunk_base = reinterpret_cast<int32_t*>(P(L.chunk_base));
-  int32_t* expert_total = reinterpret_cast<int32_t*>(P(L.expert_total));
   int32_t* offsets = reinterpret_cast<int32_t*>(P(L.offsets));
   int32_t* tile_prefix = reinterpret_cast<int32_t*>(P(L.tile_prefix));
   int32_t* tile_expert = reinterpret_cast<int32_t*>(P(L.tile_expert));
@@ -1142,27 +996,22 @@ quads_status quads_moe_fp8_w8a8(const quads_moe_fp8_args* a, void* cuda_stream) 
   int32_t* perm = reinterpret_cast<int32_t*>(P(L.perm));
   int32_t* pos_pad = reinterpret_cast<int32_t*>(P(L.pos_pad));
   int32_t* row_token = reinterpret_cast<int32_t*>(P(L.row_token));
-  float* row_weight = reinterpret_cast<float*>(P(L.row_weight));
   const size_t pad_rows = (size_t)L.m_tiles_max * 128;
-  QUADS_CUDA_OK(cudaMemsetAsync(ws, 0, L.ids, st));            // header, status word, per-expert totals
-  // ---- routing and dispatch order (the NVFP4 path's kernels)
-  {
-    auto route = E <= 32 ? route_kernel_t<1> : (E <= 64 ? route_kernel_t<2> : (E <= 128 ? route_kernel_t<4> : route_kernel_t<8>));
-    QUADS_CUDA_OK(launch_kernel(route, dim3(L.n_chunks), dim3(256), (size_t)0, st, a->router_logits, T, E, topk, a->renormalize,
-                                ids, wts, chunk_counts, expert_total, a->topk_ids, (float*)nullptr, 0, E));
-  }
-  QUADS_CUDA_OK(launch_kernel(scan_kernel, dim3(E), dim3(256), (size_t)0, st, E, L.n_chunks, 1, chunk_counts, expert_total,
-                              chunk_base, offsets, tile_prefix, tile_expert, tile_rows, header, (int32_t*)nullptr));
-  QUADS_CUDA_OK(launch_kernel(permute_kernel, dim3(L.n_chunks), dim3(128), (size_t)0, st, T, E, topk, L.n_chunks, ids, wts,
-                              chunk_base, offsets, tile_prefix, perm, pos_pad, row_token, row_weight, a->perm, 0, E));
-  // ---- activation quantization (token order) and dispatch
+  QUADS_CUDA_OK(cudaMemsetAsync(ws, 0, L.ids, st));            // header, status word, route counts
+  // ---- routing, dispatch order and activation quantization (token order), then the dispatched copies
   uint8_t* xq_tok = a->xq ? a->xq : P(L.xq_tok);
   uint8_t* xe_tok = a->xexp ? a->xexp : P(L.xe_tok);
   {
-    const int64_t tiles = (int64_t)T * (H / 128);
-    const unsigned grid = (unsigned)std::min<int64_t>((tiles + 7) / 8, (int64_t)di.sm_count * 16);
-    QUADS_CUDA_OK(launch_kernel(fp8_quantize_act_kernel, dim3(grid), dim3(256), (size_t)0, st, static_cast<const uint16_t*>(a->x),
-                                (int64_t)T, H, xq_tok, xe_tok));
+    RouteArgs r{};
+    r.logits = a->router_logits;
+    r.T = T; r.E = E; r.topk = topk; r.renormalize = a->renormalize; r.e_lo = 0; r.e_hi = E;
+    r.slot_rows = 128; r.tile_group = 1;
+    r.ids = ids; r.wts = wts; r.counts = reinterpret_cast<int32_t*>(P(L.route_counts));
+    r.arrivals = reinterpret_cast<unsigned int*>(header + kHdrRouteArrivals); r.status = header + kHdrStatus;
+    r.offsets = offsets; r.tile_prefix = tile_prefix; r.tile_expert = tile_expert; r.tile_rows = tile_rows; r.header = header;
+    r.perm = perm; r.pos_pad = pos_pad; r.row_token = row_token;
+    r.ids_out = a->topk_ids; r.perm_out = a->perm;
+    if ((s = launch_fp8_front(static_cast<const uint16_t*>(a->x), T, H, xq_tok, xe_tok, r, di.sm_count, st)) != QUADS_OK) return s;
   }
   QUADS_CUDA_OK(launch_kernel(fp8_dispatch_kernel, dim3(L.m_tiles_max), dim3(256), (size_t)0, st, H, header, tile_rows, row_token,
                               xq_tok, xe_tok, P(L.xq_pad), P(L.xsf)));

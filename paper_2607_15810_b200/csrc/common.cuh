@@ -101,6 +101,39 @@ __device__ __forceinline__ void ldg256(const void* p, uint4& a, uint4& b) {
                : "l"(p));
 }
 
+// The same, asking L2 to keep the lines for a second pass (evict_last) or to drop them (evict_first).
+__device__ __forceinline__ void ldg256_keep(const void* p, uint4& a, uint4& b) {
+  asm volatile("ld.global.L2::evict_last.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(p));
+}
+__device__ __forceinline__ void ldg256_stream(const void* p, uint4& a, uint4& b) {
+  asm volatile("ld.global.L2::evict_first.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(p));
+}
+// Largest magnitudes of eight bf16 values, two per word.
+__device__ __forceinline__ uint32_t absmax8(const uint4& v) {
+  return __vmaxu2(__vmaxu2(v.x & 0x7FFF7FFFu, v.y & 0x7FFF7FFFu), __vmaxu2(v.z & 0x7FFF7FFFu, v.w & 0x7FFF7FFFu));
+}
+// Order-preserving map float -> uint32 (larger float <=> larger uint).
+__device__ __forceinline__ uint32_t float_key(float v) {
+  const uint32_t b = __float_as_uint(v);
+  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+__device__ __forceinline__ uint32_t ld_acquire_u32(const void* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t ld_relaxed_u32(const void* p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ float gs_from_amax_bits(uint32_t bits) {
+  const float amax = __uint_as_float(bits);
+  return amax > 0.f ? __fdiv_rn(amax, kGlobalDiv) : 1.0f;
+}
+
 // float -> E4M3 byte, round-to-nearest-even, saturating to 448.
 __device__ __forceinline__ uint32_t f32_to_e4m3(float v) {
   uint16_t r;
@@ -207,6 +240,18 @@ __device__ __forceinline__ uint32_t f32x2_to_bf16x2(float lo, float hi) {
   __nv_bfloat162 b = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&b);
 }
+
+// Mask bytes m[0..7] in {0, 1} -> 0xF per selected nibble.
+__device__ __forceinline__ uint32_t nibble_mask8(const uint2& v) {
+  uint32_t out = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    out |= ((v.x >> (8 * i)) & 1u) * (0xFu << (4 * i));
+    out |= ((v.y >> (8 * i)) & 1u) * (0xFu << (16 + 4 * i));
+  }
+  return out;
+}
+__device__ __forceinline__ uint32_t nibble_mask8(const uint8_t* m) { return nibble_mask8(*reinterpret_cast<const uint2*>(m)); }
 
 // Byte offset of scale (row, blk) in the tiled layout with kt_count = ceil(K/64) atoms per row tile.
 __host__ __device__ __forceinline__ size_t sf_tiled_offset(int64_t row, int64_t blk, int64_t kt_count) {

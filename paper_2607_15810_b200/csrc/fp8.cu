@@ -4,7 +4,10 @@
 // (tcgen05.mma.kind::mxf8f6f4, one UE8M0 scale byte per 32 elements: a tile's scale is repeated).
 // Same layer, routing, dispatch order and combine as the NVFP4 path; no RAC (there is none in FP8).
 // It exists so that the W4A4 / FP8 relations the paper reports can be restated on one layer.
-#include "kernels.cuh"
+#include <algorithm>
+#include <atomic>
+
+#include "routing.cuh"
 #include "tcgen05.cuh"
 
 namespace quads {
@@ -29,14 +32,12 @@ __device__ __forceinline__ uint32_t f32x4_to_e4m3x4(float a, float b, float c, f
 
 // Activation quantizer: one warp per (row, 128-channel tile), a lane holds 4 consecutive values.
 // codes [rows, K] u8, exps [rows, K/128] u8 (e + 127).
-__global__ void __launch_bounds__(256)
-fp8_quantize_act_kernel(const uint16_t* __restrict__ x, int64_t rows, int K, uint8_t* __restrict__ codes,
-                        uint8_t* __restrict__ exps) {
-  pdl_sync();
+__device__ __forceinline__ void fp8_quantize_act(const uint16_t* __restrict__ x, int64_t rows, int K, uint8_t* __restrict__ codes,
+                                                 uint8_t* __restrict__ exps, int cta, int n_cta) {
   const int kt = K >> 7;
   const int64_t n_tiles = rows * kt;
   const int lane = threadIdx.x & 31;
-  for (int64_t w = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); w < n_tiles; w += (int64_t)gridDim.x * 8) {
+  for (int64_t w = (int64_t)cta * 8 + (threadIdx.x >> 5); w < n_tiles; w += (int64_t)n_cta * 8) {
     const int64_t r = w / kt;
     const int t = (int)(w - r * kt);
     const uint2 v = __ldg(reinterpret_cast<const uint2*>(x + r * K + t * 128) + lane);
@@ -49,6 +50,47 @@ fp8_quantize_act_kernel(const uint16_t* __restrict__ x, int64_t rows, int K, uin
         f32x4_to_e4m3x4(ldexpf(f0, -e), ldexpf(f1, -e), ldexpf(f2, -e), ldexpf(f3, -e));
     if (lane == 0) exps[r * kt + t] = (uint8_t)code;
   }
+}
+
+// All CTAs route a few tokens; then the first n_groups hand out the rows (they wait for the others: cooperative
+// launch) while the others quantize.
+template <int NJ>
+__global__ void __launch_bounds__(256)
+fp8_front_kernel(const uint16_t* __restrict__ x, int64_t rows, int K, uint8_t* __restrict__ codes, uint8_t* __restrict__ exps,
+                 const RouteArgs r, int n_groups) {
+  pdl_sync();
+  __shared__ RouteShared s;
+  route_part1<NJ>(r, (int)blockIdx.x, (int)gridDim.x, n_groups);
+  if ((int)blockIdx.x < n_groups) route_part2<NJ>(r, (int)blockIdx.x, n_groups, gridDim.x, &s);
+  else fp8_quantize_act(x, rows, K, codes, exps, (int)blockIdx.x - n_groups, (int)gridDim.x - n_groups);
+}
+
+namespace {
+template <int NJ>
+quads_status launch_fp8_front_nj(const uint16_t* x, int64_t rows, int K, uint8_t* codes, uint8_t* exps, RouteArgs r, int sm_count,
+                                 cudaStream_t st) {
+  static std::atomic<int> cache{0};                    // resident CTAs per SM (same on every sm_100 device)
+  int per_sm = cache.load();
+  if (per_sm == 0) {
+    QUADS_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fp8_front_kernel<NJ>, 256, 0));
+    cache.store(per_sm);
+  }
+  if (per_sm < 2) return QUADS_ERR_CUDA;
+  int n_groups = std::min(std::min(sm_count, kRouteCtasMax), (r.T + kRouteWarps - 1) / kRouteWarps);
+  const int n_quant = (int)std::max<int64_t>(1, std::min<int64_t>((rows * (K / 128) + 7) / 8, (int64_t)(per_sm - 1) * sm_count));
+  void* args[] = {&x, &rows, &K, &codes, &exps, &r, &n_groups};
+  QUADS_CUDA_OK(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(fp8_front_kernel<NJ>), dim3(n_groups + n_quant), dim3(256), args, 0, st));
+  note_launch();
+  return QUADS_OK;
+}
+}  // namespace
+
+quads_status launch_fp8_front(const uint16_t* x, int64_t rows, int K, uint8_t* codes, uint8_t* exps, const RouteArgs& r, int sm_count,
+                              cudaStream_t st) {
+  return r.E <= 32 ? launch_fp8_front_nj<1>(x, rows, K, codes, exps, r, sm_count, st)
+                   : (r.E <= 64 ? launch_fp8_front_nj<2>(x, rows, K, codes, exps, r, sm_count, st)
+                                : (r.E <= 128 ? launch_fp8_front_nj<4>(x, rows, K, codes, exps, r, sm_count, st)
+                                              : launch_fp8_front_nj<8>(x, rows, K, codes, exps, r, sm_count, st)));
 }
 
 // Weight quantizer: one CTA per 128 x 128 tile (256 threads, 64 values each: half a row).

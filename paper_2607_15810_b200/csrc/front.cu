@@ -1,0 +1,361 @@
+// The front of a MoE call or a dense projection of more than a few tokens (small_batch.cu has the others):
+//   front_kernel        routing and quantization, two independent roles of one cooperative launch;
+//   quant_rows_kernel   the quantization role alone (dense projections have no routing);
+//   dispatch_kernel     the copies of codes and scales in dispatch order, and the channel selection.
+#include <algorithm>
+#include <atomic>
+
+#include "routing.cuh"
+
+namespace quads {
+
+// ---------------------------------------------------------------------------
+// Site-13 quantization pass, token order.  For every row and 16-channel block:
+// Q_A(x) codes + scale; the residual Q_A(x) - x in float32 (Eq. residual-def);
+// its squared sum per channel (Eq. channel-score); and the residual's own
+// quantization with the same per-tensor scale (the mask of Eq. residual-recon is
+// applied later: quantizing the residual does not depend on the selection).
+//
+// A CTA owns bw blocks of 16 channels (8, 16 or 32, whatever divides the row) for a range of rows;
+// thread = (block, row lane).  The grid is what is resident at once, so that the amax of x can be the
+// first phase of the same launch: the CTAs meet at a counter (bounded wait) and read their rows again, out of L2.
+// A CTA adds its row lanes' column sums up in shared memory and adds one 64-bit integer per channel to the
+// channel's total, which is complete when the kernel ends: with CTAs that own whole rows, four times as
+// many reductions arrive together (20 us at 8192 x 2048), and partial rows need a kernel to add them up.
+// Issue-bound: about 400 issue cycles per warp and block, 128 of them in the two conversions to E2M1.
+// Dense projection 8192 x 4096 -> 4096: amax, quantization, score reduction, ranking and copy took 16 + 27 + 12 +
+// 12 + 28 us as kernels of their own; this one takes 39.8 and the in-place mask behind it 10 (whole call
+// 205 -> 165 us).
+// Scales are stored linear [T, H/16], or tiled when the rows are a dense projection's operand as they are.
+// ---------------------------------------------------------------------------
+struct QuantShared {
+  float gs;
+  uint32_t wmax[8];
+  float inv_lut[128];
+  __align__(16) float red[256 * 16];
+};
+
+// CTA `cta` of `n_cta`.
+__device__ __forceinline__ void quant_role(const QuantRowsArgs& p, int cta, int n_cta, QuantShared* s) {
+  const int H = p.H, k16 = H >> 4;
+  const int col = cta % p.n_col, rg = cta / p.n_col;
+  const int blk = threadIdx.x % p.bw, lane_r = threadIdx.x / p.bw, lanes = 256 / p.bw;
+  const int kb = col * p.bw + blk;
+  const int r0 = rg * p.rows_per_cta + lane_r, r1 = min(p.T, (rg + 1) * p.rows_per_cta);
+  const uint16_t* xk = p.x + kb * 16;
+  if (!p.gs_in) {
+    uint32_t m = 0;
+    int r = r0;
+    for (; r + 3 * lanes < r1; r += 4 * lanes) {
+      uint4 v[8];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) ldg256_keep(xk + (size_t)(r + u * lanes) * H, v[2 * u], v[2 * u + 1]);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) m = __vmaxu2(m, absmax8(v[u]));
+    }
+    for (; r < r1; r += lanes) {
+      uint4 v0, v1;
+      ldg256_keep(xk + (size_t)r * H, v0, v1);
+      m = __vmaxu2(m, __vmaxu2(absmax8(v0), absmax8(v1)));
+    }
+    m = __reduce_max_sync(0xFFFFFFFFu, max(m & 0xFFFFu, m >> 16));
+    if ((threadIdx.x & 31) == 0) s->wmax[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      uint32_t tm = 0;
+      for (int i = 0; i < 8; ++i) tm = max(tm, s->wmax[i]);
+      if (tm) atomicMax(p.amax_bits, tm << 16);
+      __threadfence();
+      atomicAdd(p.arrivals, 1u);
+      grid_wait(p.arrivals, (uint32_t)n_cta, p.status);
+      s->gs = gs_from_amax_bits(ld_relaxed_u32(p.amax_bits));
+    }
+    __syncthreads();
+  } else {
+    if (threadIdx.x == 0) s->gs = p.gs_in[0];
+    __syncthreads();
+  }
+  const float gs = s->gs;
+  if (p.gs_store && cta == 0 && threadIdx.x == 0) p.gs_store[0] = gs;
+  if (threadIdx.x < 128) s->inv_lut[threadIdx.x] = quant_inv_entry(threadIdx.x, gs);
+  __syncthreads();
+  QuantCtx qc;
+  quant_ctx_scalars(qc, gs);
+  qc.inv_lut = s->inv_lut;
+  float acc[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) acc[i] = 0.f;
+  uint4 n0 = make_uint4(0, 0, 0, 0), n1 = n0;
+  if (r0 < r1) ldg256(xk + (size_t)r0 * H, n0, n1);
+  for (int r = r0; r < r1; r += lanes) {
+    const uint4 v0 = n0, v1 = n1;
+    if (r + lanes < r1) ldg256(xk + (size_t)(r + lanes) * H, n0, n1);   // next block, ahead of this one's arithmetic
+    float f[16], o[16];
+    unpack8(v0, f);
+    unpack8(v1, f + 8);
+    const BlockQ bq = quantize_block(f, qc);
+    const size_t qo = (size_t)r * (H >> 1) + kb * 8, so = (size_t)r * k16 + kb;
+    const size_t so_op = p.sf_tiled ? sf_tiled_offset(r, kb, H >> 6) : so;
+    *reinterpret_cast<uint2*>(p.xq + qo) = make_uint2(bq.lo, bq.hi);
+    p.xsf[so_op] = (uint8_t)bq.sf8;
+    if (p.xq_exp) *reinterpret_cast<uint2*>(p.xq_exp + qo) = make_uint2(bq.lo, bq.hi);
+    if (p.xsf_exp) p.xsf_exp[so] = (uint8_t)bq.sf8;
+    if (p.with_residual) {
+      dequant_block(bq, o);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        o[i] = __fsub_rn(o[i], f[i]);
+        acc[i] = __fmaf_rn(o[i], o[i], acc[i]);
+      }
+      const BlockQ br = quantize_block(o, qc);
+      *reinterpret_cast<uint2*>(p.rq + qo) = make_uint2(br.lo, br.hi);
+      p.rsf[so_op] = (uint8_t)br.sf8;
+      if (p.rsf_exp) p.rsf_exp[so] = (uint8_t)br.sf8;
+    }
+  }
+  if (!p.with_residual) return;
+  {
+    float4* d = reinterpret_cast<float4*>(s->red + threadIdx.x * 16);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) d[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
+    __syncthreads();
+    const int n_ch = p.bw * 16;                              // channels of this CTA, at most 512
+    for (int c = threadIdx.x; c < n_ch; c += 256) {
+      float t = 0.f;
+      for (int l = 0; l < lanes; ++l) t += s->red[l * n_ch + c];
+      add_score(p.totals + col * n_ch + c, t, gs, p.score_bits, p.cap_bits);
+    }
+  }
+}
+
+// Asks L2 for the rows of quant_role's CTA.
+__device__ __forceinline__ void quant_prefetch(const QuantRowsArgs& p, int cta) {
+  const int col = cta % p.n_col, rg = cta / p.n_col;
+  const int r0 = rg * p.rows_per_cta, n_rows = min(p.T, r0 + p.rows_per_cta) - r0, lines = p.bw >> 2;   // of 128 bytes per row
+  const uint8_t* base = reinterpret_cast<const uint8_t*>(p.x + (size_t)col * p.bw * 16);
+  for (int i = threadIdx.x; i < n_rows * lines; i += 256) {
+    const int r = i / lines;
+    asm volatile("prefetch.global.L2::evict_last [%0];" ::"l"(base + (size_t)(r0 + r) * p.H * 2 + (size_t)(i - r * lines) * 128));
+  }
+}
+
+__global__ void __launch_bounds__(256, kQuantRowsPerSm) quant_rows_kernel(const QuantRowsArgs p) {
+  pdl_sync();
+  __shared__ QuantShared s;
+  quant_role(p, (int)blockIdx.x, (int)gridDim.x, &s);
+}
+
+// All CTAs route a few tokens first; then the first n_groups (one per SM) hand out the rows while the others, three
+// per SM beside them, quantize: the roles need nothing of one another, each has its own counters to meet at.
+// As five kernels on two streams (route, scan, permute beside quantize, rank) the last of them ended 44 us after
+// the call's start at 8192 tokens, because the quantization held the SMs; here codes, scores and tables are
+// there after 30 us (1500 tokens: 14 instead of 30).
+template <int NJ>
+__global__ void __launch_bounds__(256, kQuantRowsPerSm)
+front_kernel(const QuantRowsArgs q, const RouteArgs r, int n_groups) {
+  pdl_sync();
+  __shared__ union { QuantShared q; RouteShared r; } s;
+  if ((int)blockIdx.x >= n_groups) quant_prefetch(q, (int)blockIdx.x - n_groups);   // x arrives while the tokens are routed
+  route_part1<NJ>(r, (int)blockIdx.x, (int)gridDim.x, n_groups);
+  if ((int)blockIdx.x < n_groups) route_part2<NJ>(r, (int)blockIdx.x, n_groups, gridDim.x, &s.r);
+  else quant_role(q, (int)blockIdx.x - n_groups, (int)gridDim.x - n_groups, &s.q);
+}
+
+// ---------------------------------------------------------------------------
+// Site-13 dispatch, driven by the DESTINATION: the tiles of the padded dispatch order are cut into slabs of 512
+// channels; a CTA gathers a slab's rows from the token-order arrays (which stay in L2: every token row is
+// read top-k times) and writes its codes and its eight scale atoms as whole regions.  Written from the
+// source side instead (one thread per token chunk), every 512-byte scale atom is touched by 128 different
+// tokens at 128 different times, 4 bytes each: partially written sectors get evicted and the memory system
+// pays for them.
+// kResid = false copies Q(x), and ranks the channels on the side (every CTA a few of them), so that the mask is there
+// for kResid = true, which copies the residual: masked on the way (Eq. residual-recon: codes of unselected
+// channels are cleared) and stored NEGATED (sign bits flipped), so that the GEMM can accumulate
+// W Q(x) + W (-M Q(dx)) with two plain MMAs.
+// Bound by the writes (75 MB each at 8192 tokens x 8 x 2048 channels).  A ranking kernel and copies with one CTA
+// per tile (half of the last wave idle) took 6 + 21 + 21 us; these are 18 (ranking included) + 16.
+// dynamic shared memory: two sets of eight scale atoms, H / 8 mask words.
+// ---------------------------------------------------------------------------
+constexpr int kSlabChunks = 16;                      // 16-byte chunks of codes (32 channels each) per row and slab
+constexpr int kSlabAtoms = 8;
+constexpr int kRankBatch = 4;                        // channels a CTA ranks in one pass over the scores
+
+// rank_j = #{i : s_i > s_j, or s_i == s_j and i < j}; channel j is selected iff rank_j < n_sel (the n_sel largest, ties
+// to the lower index; Eq. channel-select).
+__device__ __forceinline__ void rank_channels(const DispatchArgs& p, int* rank_sh) {
+  const int H = p.H;
+  if (threadIdx.x < kRankBatch) rank_sh[threadIdx.x] = 0;
+  __syncthreads();
+  for (int j0 = blockIdx.x * kRankBatch; j0 < H; j0 += gridDim.x * kRankBatch) {
+    unsigned long long mine[kRankBatch];
+    int cnt[kRankBatch];
+#pragma unroll
+    for (int k = 0; k < kRankBatch; ++k) {
+      mine[k] = __ldcg(p.keys + j0 + k);             // (H is a multiple of 128)
+      cnt[k] = 0;
+    }
+#pragma unroll 4
+    for (int i = threadIdx.x; i < H; i += kDispatchThreads) {
+      const unsigned long long si = __ldcg(p.keys + i);
+#pragma unroll
+      for (int k = 0; k < kRankBatch; ++k) cnt[k] += (si > mine[k] || (si == mine[k] && i < j0 + k)) ? 1 : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < kRankBatch; ++k) {
+      const int t = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)cnt[k]);
+      if ((threadIdx.x & 31) == 0 && t) atomicAdd(rank_sh + k, t);
+    }
+    __syncthreads();
+    if (threadIdx.x < kRankBatch) {
+      p.mask[j0 + threadIdx.x] = rank_sh[threadIdx.x] < p.n_sel ? 1 : 0;
+      rank_sh[threadIdx.x] = 0;
+    }
+    __syncthreads();
+  }
+}
+
+template <bool kResid>
+__global__ void __launch_bounds__(kDispatchThreads, kDispatchPerSm)
+dispatch_kernel(const DispatchArgs p) {
+  static_assert(kDispatchThreads == 512, "four 16-byte chunks and one 8-byte piece of scales per thread");
+  pdl_sync();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int tok[2][128];
+  __shared__ int rank_sh[kRankBatch];
+  const int H = p.H, per_row = H >> 5, kt_count = H >> 6;
+  uint32_t* nib = reinterpret_cast<uint32_t*>(smem_raw + 2 * kSlabAtoms * 512);
+  if (kResid) {
+    for (int w = threadIdx.x; w < (H >> 3); w += kDispatchThreads)
+      nib[w] = nibble_mask8(__ldg(reinterpret_cast<const uint2*>(p.mask) + w));
+  } else if (p.n_sel > 0) {
+    rank_channels(p, rank_sh);
+  }
+  const uint8_t *src = kResid ? p.rq : p.xq, *src_sf = kResid ? p.rsf : p.xsf;
+  uint8_t *dst = kResid ? p.rq_pad : p.xq_pad, *dst_sf = kResid ? p.rsf_tiled : p.xsf_tiled;
+  const int n_slabs = (per_row + kSlabChunks - 1) / kSlabChunks;
+  const int n_items = p.header[kHdrMTiles] * n_slabs;
+  int buf = 0;
+  for (int item = blockIdx.x; item < n_items; item += gridDim.x, buf ^= 1) {
+    const int mt = item / n_slabs, sl = item - mt * n_slabs;
+    const int n_rows = p.tile_rows[mt];
+    if (threadIdx.x < 128) tok[buf][threadIdx.x] = threadIdx.x < n_rows ? p.row_token[mt * 128 + threadIdx.x] : -1;
+    __syncthreads();                                 // (and the atoms of two items ago have been written out)
+    const int c0 = sl * kSlabChunks, nc = min(kSlabChunks, per_row - c0), k0 = sl * kSlabAtoms, nk = nc >> 1;
+    // ---- loads: codes (thread = chunk threadIdx % 16 of rows threadIdx / 16 + 32 u), scales (two atoms of a row)
+    const int c = threadIdx.x & 15, r_of = threadIdx.x >> 4;
+    uint4 v[4];
+    bool on[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int t = tok[buf][r_of + 32 * u];
+      on[u] = t >= 0 && c < nc;
+      if (on[u]) v[u] = __ldg(reinterpret_cast<const uint4*>(src + (size_t)t * (H >> 1) + (size_t)(c0 + c) * 16));
+    }
+    const int sr = threadIdx.x >> 2, pc = threadIdx.x & 3, st = tok[buf][sr];
+    uint2 sv = make_uint2(0, 0);                     // (padding rows get zero scales)
+    if (st >= 0 && 2 * pc < nk) sv = __ldg(reinterpret_cast<const uint2*>(src_sf + (size_t)st * (H >> 4) + (size_t)(k0 + 2 * pc) * 4));
+    uint8_t* atoms = smem_raw + buf * (kSlabAtoms * 512);
+    {
+      uint32_t* a = reinterpret_cast<uint32_t*>(atoms + 2 * pc * 512 + (sr & 31) * 16 + (sr >> 5) * 4);
+      a[0] = sv.x; a[128] = sv.y;
+    }
+    __syncthreads();
+    // ---- stores
+    if (threadIdx.x < nk * 32)
+      __stcs(reinterpret_cast<uint4*>(dst_sf + ((size_t)mt * kt_count + k0) * 512u) + threadIdx.x, reinterpret_cast<const uint4*>(atoms)[threadIdx.x]);
+    uint4 m = make_uint4(0, 0, 0, 0);
+    if (kResid && c < nc) m = reinterpret_cast<const uint4*>(nib)[c0 + c];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (on[u]) {
+        if (kResid) {
+          v[u].x = (v[u].x & m.x) ^ 0x88888888u; v[u].y = (v[u].y & m.y) ^ 0x88888888u;
+          v[u].z = (v[u].z & m.z) ^ 0x88888888u; v[u].w = (v[u].w & m.w) ^ 0x88888888u;
+        }
+        __stcs(reinterpret_cast<uint4*>(dst + (size_t)(mt * 128 + r_of + 32 * u) * (H >> 1) + (size_t)(c0 + c) * 16), v[u]);
+      }
+  }
+}
+
+namespace {
+
+// Resident CTAs per SM of a kernel (same on every sm_100 device).
+template <typename K>
+cudaError_t resident_per_sm(K kernel, int threads, std::atomic<int>* cache, int* out) {
+  int v = cache->load();
+  if (v == 0) {
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kernel, threads, 0);
+    if (e != cudaSuccess) return e;
+    if (v < 1) return cudaErrorLaunchOutOfResources;
+    cache->store(v);
+  }
+  *out = v;
+  return cudaSuccess;
+}
+
+// Row ranges of the quantization role on at most `ctas` CTAs; returns the CTAs used.
+int plan_quant(QuantRowsArgs* q, int ctas) {
+  q->bw = (q->H / 16) % 32 == 0 ? 32 : ((q->H / 16) % 16 == 0 ? 16 : 8);
+  q->n_col = q->H / 16 / q->bw;
+  const int lanes = 256 / q->bw;                    // each range at least a row per row lane
+  const int n_rg = std::max(1, std::min(ctas / q->n_col, (q->T + lanes - 1) / lanes));
+  q->rows_per_cta = ((q->T + n_rg - 1) / n_rg + lanes - 1) / lanes * lanes;
+  const int n_used = (q->T + q->rows_per_cta - 1) / q->rows_per_cta;
+  // a CTA's column sum covers rows_per_cta rows (< rows * 2^18 in units of the squared scale); the sums of
+  // all row ranges must fit 62 bits together
+  int cap_bits = 18, ranges_log2 = 0;
+  while ((1 << (cap_bits - 18)) < q->rows_per_cta) ++cap_bits;
+  while ((1 << ranges_log2) < n_used) ++ranges_log2;
+  q->cap_bits = cap_bits;
+  q->score_bits = std::max(0, std::min(26, 62 - cap_bits - ranges_log2));
+  return n_used * q->n_col;
+}
+
+template <int NJ>
+quads_status launch_front_nj(QuantRowsArgs q, RouteArgs r, int sm_count, cudaStream_t st) {
+  static std::atomic<int> cache{0};
+  int per_sm = 0;
+  QUADS_CUDA_OK(resident_per_sm(front_kernel<NJ>, 256, &cache, &per_sm));
+  if (per_sm < 2) return QUADS_ERR_CUDA;
+  int n_groups = std::min(std::min(sm_count, kRouteCtasMax), (r.T + kRouteWarps - 1) / kRouteWarps);
+  const int n_quant = plan_quant(&q, (per_sm - 1) * sm_count);
+  void* args[] = {&q, &r, &n_groups};
+  QUADS_CUDA_OK(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(front_kernel<NJ>), dim3(n_groups + n_quant), dim3(256), args, 0, st));
+  note_launch();
+  return QUADS_OK;
+}
+
+}  // namespace
+
+quads_status launch_front(const QuantRowsArgs& q, const RouteArgs& r, int sm_count, cudaStream_t st) {
+  return r.E <= 32 ? launch_front_nj<1>(q, r, sm_count, st)
+                   : (r.E <= 64 ? launch_front_nj<2>(q, r, sm_count, st)
+                                : (r.E <= 128 ? launch_front_nj<4>(q, r, sm_count, st) : launch_front_nj<8>(q, r, sm_count, st)));
+}
+
+quads_status launch_quant_rows(const QuantRowsArgs& args, int sm_count, cudaStream_t st) {
+  static std::atomic<int> cache{0};
+  QuantRowsArgs q = args;
+  int per_sm = 0;
+  QUADS_CUDA_OK(resident_per_sm(quant_rows_kernel, 256, &cache, &per_sm));
+  const int n = plan_quant(&q, per_sm * sm_count);
+  if (!q.gs_in) {                                    // its CTAs wait for one another
+    void* kargs[] = {&q};
+    QUADS_CUDA_OK(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(quant_rows_kernel), dim3(n), dim3(256), kargs, 0, st));
+    note_launch();
+  } else {
+    QUADS_CUDA_OK(launch_kernel(quant_rows_kernel, dim3(n), dim3(256), (size_t)0, st, q));
+  }
+  return QUADS_OK;
+}
+
+quads_status launch_dispatch(const DispatchArgs& p, int m_tiles_max, int sm_count, cudaStream_t st) {
+  const int64_t items = (int64_t)m_tiles_max * ((p.H / 32 + kSlabChunks - 1) / kSlabChunks);
+  const int grid = (int)std::min<int64_t>(items, kDispatchPerSm * sm_count);
+  const int atoms = 2 * kSlabAtoms * 512;
+  QUADS_CUDA_OK(launch_kernel(dispatch_kernel<false>, dim3(grid), dim3(kDispatchThreads), (size_t)atoms, st, p));
+  if (p.n_sel > 0) QUADS_CUDA_OK(launch_kernel(dispatch_kernel<true>, dim3(grid), dim3(kDispatchThreads), (size_t)(atoms + p.H / 2), st, p));
+  return QUADS_OK;
+}
+
+}  // namespace quads

@@ -160,6 +160,7 @@ gemm_swapped_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_x
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
 
+  if (p.tables_late) asm volatile("griddepcontrol.wait;" ::: "memory");
   // ---- per-CTA tables: slot -> expert / valid rows, expert -> weight scale, and the compact
   // list of non-empty (slot, chunk) pairs in slot order (every CTA builds the same list)
   const int m_slots = p.header[kHdrMTiles];

@@ -6,12 +6,11 @@
 
 namespace quads {
 
-constexpr int kRouteTokensPerCta = 32;
 constexpr int kMaxTopk = 16;
 constexpr int kMaxExperts = 256;
 
 // header words written by the scan (device side sizes of the dispatch)
-enum { kHdrMTiles = 0, kHdrPaddedRows = 1, kHdrAssignments = 2, kHdrStatus = 3, kHdrArrivals = 4, kHdrWords = 8 };
+enum { kHdrMTiles = 0, kHdrPaddedRows = 1, kHdrAssignments = 2, kHdrStatus = 3, kHdrArrivals = 4, kHdrRouteArrivals = 5, kHdrWords = 8 };
 
 constexpr int kAmaxPartsMax = 2048;   // partial maxima left by the first pass of the single-tensor quantizer
 
@@ -37,35 +36,14 @@ __global__ void fake_quant_ring_kernel(const uint16_t* x, int64_t nblk, int64_t 
                                        int kt_count);
 __global__ void dequantize_kernel(const uint8_t* q, const uint8_t* sf, const float* gs, int n_tensors, int64_t nblk,
                                   uint32_t k16, int kt_count, int sf_tiled, int64_t sf_tensor_stride, uint16_t* out);
-constexpr int kQuantRowsPerSm = 4;    // resident CTAs of quant_rows_kernel
-struct QuantRowsArgs {
-  const uint16_t* x;
-  int T, H, bw, n_col, rows_per_cta, with_residual, sf_tiled;
-  const float* gs_in;                 // per-tensor scale, or NULL: amax-derived (then the launch is cooperative)
-  uint32_t* amax_bits;
-  unsigned int* arrivals;             // NULL when gs_in is given; amax_bits and arrivals are zero on entry
-  int32_t* status;
-  float* gs_store;                    // exports, each may be NULL
-  uint8_t *xq, *xsf, *rq, *rsf;
-  uint8_t *xq_exp, *xsf_exp, *rsf_exp;
-  unsigned long long* totals;         // [H] integer channel scores, zero on entry
-  int score_bits, cap_bits;
-};
-__global__ void quant_rows_kernel(const QuantRowsArgs p);
 __global__ void channel_stats_kernel(const uint16_t* x, int T, int H, const float* gs_in, const uint32_t* amax_bits,
                                      int rows_per_cta, float* partials);
 constexpr int kScoreSlices = 16;
 __global__ void score_reduce_kernel(const float* partials, const int* n_part_ptr, int n_part_mul,
                                     int n_part_fixed, int C, double* slice_sums, unsigned int* counters,
                                     unsigned long long* score_keys);
-__global__ void rank_select_kernel(const unsigned long long* score_keys, int C, int n_sel, uint8_t* mask);
 __global__ void sel_list_kernel(const uint8_t* mask, int C, int32_t* sel_export);
 __global__ void export_residual_kernel(int T, int H, const uint8_t* mask, uint32_t flip, const uint8_t* rq, uint8_t* rq_exp);
-template <int kParts>   // bit 0: copies of Q(x), bit 1: masked, negated copies of the residual
-__global__ void rac_dispatch_kernel(int H, const uint8_t* mask, const int32_t* header,
-                                    const int32_t* tile_rows, const int32_t* row_token, const uint8_t* xq,
-                                    const uint8_t* xsf, const uint8_t* rq, const uint8_t* rsf, uint8_t* xq_pad,
-                                    uint8_t* xsf_tiled, uint8_t* rq_pad, uint8_t* rsf_tiled);
 constexpr int kSelectThreads = 512;   // one CTA per SM: the CTAs of an SM would only repeat each other's search
 __global__ void select_mask_kernel(uint8_t* codes, int n_rows_fixed, uint32_t flip, const int32_t* header, const int32_t* tile_rows,
                                    const unsigned long long* score_keys, int C, int n_sel, uint8_t* mask_out /* or NULL */);
@@ -79,18 +57,49 @@ __global__ void export_site2_kernel(int A, const int32_t* n_rows_ptr, int I, con
 __global__ void mismatch_norms_kernel(const uint16_t* a, const uint16_t* b, int64_t n, double* partials,
                                       unsigned int* counter, double* out);
 
-// ---- routing.cu
-template <int NJ>
-__global__ void route_kernel_t(const float* logits, int T, int E, int topk, int renormalize, int32_t* ids,
-                               float* wts, int32_t* chunk_counts, int32_t* expert_total, int32_t* ids_out,
-                               float* wts_out, int e_lo, int e_hi);
-__global__ void scan_kernel(int E, int n_chunks, int tile_group, const int32_t* chunk_counts,
-                            const int32_t* expert_total, int32_t* chunk_base, int32_t* offsets, int32_t* tile_prefix,
-                            int32_t* tile_expert, int32_t* tile_rows, int32_t* header, int32_t* offsets_out);
-__global__ void permute_kernel(int T, int E, int topk, int n_chunks, const int32_t* ids, const float* wts,
-                               const int32_t* chunk_base, const int32_t* offsets, const int32_t* tile_prefix,
-                               int32_t* perm, int32_t* pos_pad, int32_t* row_token, float* row_weight,
-                               int32_t* perm_out, int e_lo, int e_hi);
+// ---- front.cu
+constexpr int kQuantRowsPerSm = 4;    // resident CTAs of the front kernels
+struct QuantRowsArgs {
+  const uint16_t* x;
+  int T, H, with_residual, sf_tiled;
+  const float* gs_in;                 // per-tensor scale, or NULL: amax-derived (then the launch is cooperative)
+  uint32_t* amax_bits;
+  unsigned int* arrivals;             // it and amax_bits are zero on entry
+  int32_t* status;
+  float* gs_store;                    // exports, each may be NULL
+  uint8_t *xq, *xsf, *rq, *rsf;
+  uint8_t *xq_exp, *xsf_exp, *rsf_exp;
+  unsigned long long* totals;         // [H] integer channel scores, zero on entry
+  int bw, n_col, rows_per_cta, score_bits, cap_bits;   // filled in at launch
+};
+// Top-k routing and dispatch order (routing.cuh).
+constexpr int kRouteCtasMax = 256;
+struct RouteArgs {
+  const float* logits;
+  int T, E, topk, renormalize, e_lo, e_hi;
+  int slot_rows, tile_group;          // valid rows of a 128-row tile at most; tiles per expert are a multiple of tile_group
+  int32_t* ids;
+  float* wts;
+  int32_t* counts;                    // [kRouteCtasMax][E], zero on entry
+  unsigned int* arrivals;             // zero on entry
+  int32_t* status;
+  int32_t *offsets, *tile_prefix, *tile_expert, *tile_rows, *header, *perm, *pos_pad, *row_token;
+  int32_t* ids_out;                   // exports, each may be NULL
+  float* wts_out;
+  int32_t *offsets_out, *perm_out;
+};
+quads_status launch_front(const QuantRowsArgs& q, const RouteArgs& r, int sm_count, cudaStream_t st);
+quads_status launch_quant_rows(const QuantRowsArgs& q, int sm_count, cudaStream_t st);
+constexpr int kDispatchThreads = 512, kDispatchPerSm = 3;
+struct DispatchArgs {
+  int H, n_sel;                       // n_sel == 0: no residual
+  const unsigned long long* keys;     // [H] channel scores
+  uint8_t* mask;                      // [H] out: 1 for the selected channels
+  const int32_t *header, *tile_rows, *row_token;
+  const uint8_t *xq, *xsf, *rq, *rsf; // token order, linear scales
+  uint8_t *xq_pad, *xsf_tiled, *rq_pad, *rsf_tiled;
+};
+quads_status launch_dispatch(const DispatchArgs& p, int m_tiles_max, int sm_count, cudaStream_t st);
 
 // ---- small_batch.cu: the front of a call with few tokens, two kernels of one cluster each
 constexpr int kSmallThreads = 1024;
@@ -101,7 +110,6 @@ struct SmallRouteArgs {
   int T, E, topk, renormalize, e_lo, e_hi;
   float* wts;
   int32_t *offsets, *tile_prefix, *tile_expert, *tile_rows, *header, *perm, *pos_pad, *row_token;
-  float* row_weight;
   unsigned long long* zero_u64;       // n_zero words cleared for the kernels that follow
   int n_zero;
   int32_t* ids_out;                   // exports, each may be NULL
@@ -141,6 +149,7 @@ struct GemmParams {
   int half1_row_offset;  // weight-row distance from the tile's first half to its second half
   int has_resid;         // 1: also accumulate the (negated, masked) residual operand
   int dense_rows;        // > 0: one weight and this many activation rows in token order, no routing tables
+  int tables_late;       // the preceding kernel wrote the routing tables (operand-swapped first projection)
   int n_experts;         // entries of b_gs (the experts whose weights this call holds)
   int expert_lo;         // global id of the first of them: weights / scales are indexed by (expert - expert_lo)
   const int32_t* header;
@@ -217,7 +226,8 @@ struct Fp8GemmParams {
   const int32_t* offsets;
   int32_t* status;
 };
-__global__ void fp8_quantize_act_kernel(const uint16_t* x, int64_t rows, int K, uint8_t* codes, uint8_t* exps);
+quads_status launch_fp8_front(const uint16_t* x, int64_t rows, int K, uint8_t* codes, uint8_t* exps, const RouteArgs& r, int sm_count,
+                              cudaStream_t st);
 __global__ void fp8_quantize_weight_kernel(const uint16_t* w, int N, int K, uint8_t* codes, uint8_t* exps, uint8_t* atoms);
 __global__ void fp8_dispatch_kernel(int H, const int32_t* header, const int32_t* tile_rows, const int32_t* row_token,
                                     const uint8_t* xq, const uint8_t* xe, uint8_t* xq_pad, uint8_t* xsf_atoms);

@@ -62,11 +62,6 @@ __global__ void __launch_bounds__(256) amax_kernel(const uint16_t* __restrict__ 
   }
 }
 
-__device__ __forceinline__ float gs_from_amax_bits(uint32_t bits) {
-  const float amax = __uint_as_float(bits);
-  return amax > 0.f ? __fdiv_rn(amax, kGlobalDiv) : 1.0f;
-}
-
 // ---------------------------------------------------------------------------
 // Fused amax + NVFP4 quantize / fake-quant in ONE cooperative launch.
 // The CTAs form `n_groups` groups (CTA c belongs to group c % n_groups, so every
@@ -79,18 +74,6 @@ __device__ __forceinline__ float gs_from_amax_bits(uint32_t bits) {
 // each input byte once: 2 B read + the outputs per element.
 // `amax_bits` and `counters` (one word each per tensor) must be zero on entry.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void ldg256_keep(const void* p, uint4& a, uint4& b) {
-  asm volatile("ld.global.L2::evict_last.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(p));
-}
-__device__ __forceinline__ void ldg256_stream(const void* p, uint4& a, uint4& b) {
-  asm volatile("ld.global.L2::evict_first.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(p));
-}
-__device__ __forceinline__ uint32_t absmax8(const uint4& v) {
-  return __vmaxu2(__vmaxu2(v.x & 0x7FFF7FFFu, v.y & 0x7FFF7FFFu), __vmaxu2(v.z & 0x7FFF7FFFu, v.w & 0x7FFF7FFFu));
-}
-
 // First pass of the single-tensor quantizer: CTA b leaves the |x| maximum of its share in
 // partials[b] (every CTA stores, so the array needs no initialisation and there is no atomic);
 // the 32-byte loads ask L2 to keep the lines for the pass that follows.
@@ -367,19 +350,6 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
                : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
-// Acquire load of a tensor's arrival word.  A CTA publishes its maximum (atomicMax), fences, then
-// counts itself in: once this load shows every arrival, a later load of the amax word returns the
-// final maximum.
-__device__ __forceinline__ uint32_t ld_acquire_u32(const void* p) {
-  uint32_t v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ uint32_t ld_relaxed_u32(const void* p) {
-  uint32_t v;
-  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
 __device__ __forceinline__ void bulk_load_hint(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar,
                                                uint64_t policy) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
@@ -515,6 +485,8 @@ fake_quant_ring_kernel(const uint16_t* __restrict__ x, int64_t nblk, int64_t ten
         asked = false;
         if (watch >= n_tensors) return;
       }
+      // (a CTA publishes its maximum, fences, then counts itself in: once this acquire load shows every arrival, a
+      // later load of the amax word returns the final maximum)
       seen = ld_acquire_u32(pair + 2 * glob(watch) + 1);
       asked = true;
       asked_at = clock64();
@@ -698,127 +670,6 @@ dequantize_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ sf,
   }
 }
 
-// ---------------------------------------------------------------------------
-// Site-13 quantization pass, token order.  For every row and 16-channel block:
-// Q_A(x) codes + scale; the residual Q_A(x) - x in float32 (Eq. residual-def);
-// its squared sum per channel (Eq. channel-score); and the residual's own
-// quantization with the same per-tensor scale (the mask of Eq. residual-recon is
-// applied later: quantizing the residual does not depend on the selection).
-//
-// A CTA owns bw blocks of 16 channels (8, 16 or 32, whatever divides the row) for a range of rows;
-// thread = (block, row lane).  The grid is what is resident at once, so that the amax of x can be the
-// first phase of the same launch: the CTAs meet at a counter (bounded wait) and read their rows again, out of L2.
-// A CTA adds its row lanes' column sums up in shared memory and adds one 64-bit integer per channel to the
-// channel's total, which is complete when the kernel ends: with CTAs that own whole rows, four times as
-// many reductions arrive together (20 us at 8192 x 2048), and partial rows need a kernel to add them up.
-// Issue-bound: about 400 issue cycles per warp and block, 128 of them in the two conversions to E2M1.
-// Dense projection 8192 x 4096 -> 4096: amax, quantization, score reduction, ranking and copy took 16 + 27 + 12 +
-// 12 + 28 us as kernels of their own; this one takes 39.8 and the in-place mask behind it 10 (whole call
-// 205 -> 165 us).
-// Scales are stored linear [T, H/16], or tiled when the rows are a dense projection's operand as they are.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256, kQuantRowsPerSm)
-quant_rows_kernel(const QuantRowsArgs p) {
-  pdl_sync();
-  __shared__ float gs_sh;
-  __shared__ uint32_t wmax[8];
-  __shared__ float inv_lut[128];
-  __shared__ __align__(16) float red[256 * 16];
-  const int H = p.H, k16 = H >> 4;
-  const int col = blockIdx.x % p.n_col, rg = blockIdx.x / p.n_col;
-  const int blk = threadIdx.x % p.bw, lane_r = threadIdx.x / p.bw, lanes = 256 / p.bw;
-  const int kb = col * p.bw + blk;
-  const int r0 = rg * p.rows_per_cta + lane_r, r1 = min(p.T, (rg + 1) * p.rows_per_cta);
-  const uint16_t* xk = p.x + kb * 16;
-  if (p.arrivals) {
-    uint32_t m = 0;
-    int r = r0;
-    for (; r + 3 * lanes < r1; r += 4 * lanes) {
-      uint4 v[8];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) ldg256_keep(xk + (size_t)(r + u * lanes) * H, v[2 * u], v[2 * u + 1]);
-#pragma unroll
-      for (int u = 0; u < 8; ++u) m = __vmaxu2(m, absmax8(v[u]));
-    }
-    for (; r < r1; r += lanes) {
-      uint4 v0, v1;
-      ldg256_keep(xk + (size_t)r * H, v0, v1);
-      m = __vmaxu2(m, __vmaxu2(absmax8(v0), absmax8(v1)));
-    }
-    m = __reduce_max_sync(0xFFFFFFFFu, max(m & 0xFFFFu, m >> 16));
-    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t tm = 0;
-      for (int i = 0; i < 8; ++i) tm = max(tm, wmax[i]);
-      if (tm) atomicMax(p.amax_bits, tm << 16);
-      __threadfence();
-      atomicAdd(p.arrivals, 1u);
-      const long long t0 = clock64();
-      for (;;) {
-        if (ld_acquire_u32(p.arrivals) >= gridDim.x) break;
-        __nanosleep(100);
-        if (clock64() - t0 > 4000000000ll) { atomicExch(p.status, (int32_t)QUADS_ERR_TIMEOUT); break; }
-      }
-      gs_sh = gs_from_amax_bits(ld_relaxed_u32(p.amax_bits));
-    }
-    __syncthreads();
-  } else {
-    if (threadIdx.x == 0) gs_sh = p.gs_in[0];
-    __syncthreads();
-  }
-  const float gs = gs_sh;
-  if (p.gs_store && blockIdx.x == 0 && threadIdx.x == 0) p.gs_store[0] = gs;
-  if (threadIdx.x < 128) inv_lut[threadIdx.x] = quant_inv_entry(threadIdx.x, gs);
-  __syncthreads();
-  QuantCtx qc;
-  quant_ctx_scalars(qc, gs);
-  qc.inv_lut = inv_lut;
-  float acc[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-  uint4 n0 = make_uint4(0, 0, 0, 0), n1 = n0;
-  if (r0 < r1) ldg256(xk + (size_t)r0 * H, n0, n1);
-  for (int r = r0; r < r1; r += lanes) {
-    const uint4 v0 = n0, v1 = n1;
-    if (r + lanes < r1) ldg256(xk + (size_t)(r + lanes) * H, n0, n1);   // next block, ahead of this one's arithmetic
-    float f[16], o[16];
-    unpack8(v0, f);
-    unpack8(v1, f + 8);
-    const BlockQ bq = quantize_block(f, qc);
-    const size_t qo = (size_t)r * (H >> 1) + kb * 8, so = (size_t)r * k16 + kb;
-    const size_t so_op = p.sf_tiled ? sf_tiled_offset(r, kb, H >> 6) : so;
-    *reinterpret_cast<uint2*>(p.xq + qo) = make_uint2(bq.lo, bq.hi);
-    p.xsf[so_op] = (uint8_t)bq.sf8;
-    if (p.xq_exp) *reinterpret_cast<uint2*>(p.xq_exp + qo) = make_uint2(bq.lo, bq.hi);
-    if (p.xsf_exp) p.xsf_exp[so] = (uint8_t)bq.sf8;
-    if (p.with_residual) {
-      dequant_block(bq, o);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        o[i] = __fsub_rn(o[i], f[i]);
-        acc[i] = __fmaf_rn(o[i], o[i], acc[i]);
-      }
-      const BlockQ br = quantize_block(o, qc);
-      *reinterpret_cast<uint2*>(p.rq + qo) = make_uint2(br.lo, br.hi);
-      p.rsf[so_op] = (uint8_t)br.sf8;
-      if (p.rsf_exp) p.rsf_exp[so] = (uint8_t)br.sf8;
-    }
-  }
-  if (p.with_residual) {
-    float4* d = reinterpret_cast<float4*>(red + threadIdx.x * 16);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) d[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
-    __syncthreads();
-    const int n_ch = p.bw * 16;                              // channels of this CTA, at most 512
-    for (int c = threadIdx.x; c < n_ch; c += 256) {
-      float t = 0.f;
-      for (int l = 0; l < lanes; ++l) t += red[l * n_ch + c];
-      add_score(p.totals + col * n_ch + c, t, gs, p.score_bits, p.cap_bits);
-    }
-  }
-}
-
 // Statistics only (quads_rac_channel_scores): the squared residual sums of a CTA's rows, one partial row per CTA.
 __global__ void __launch_bounds__(256)
 channel_stats_kernel(const uint16_t* __restrict__ x, int T, int H, const float* __restrict__ gs_in,
@@ -904,42 +755,6 @@ score_reduce_kernel(const float* __restrict__ partials, const int* __restrict__ 
   }
 }
 
-// Channel selection (Eq. channel-select): rank_j = #{i : s_i > s_j, or s_i ==
-// s_j and i < j}; channel j is selected iff rank_j < n_sel (the n_sel largest,
-// ties to the lower index).  Every CTA loads all C score keys into shared
-// memory and ranks 16 channels with 16 threads each.
-// grid = ceil(C/16), 256 threads, smem = C * 8 bytes.
-__global__ void __launch_bounds__(256)
-rank_select_kernel(const unsigned long long* __restrict__ score_keys, int C, int n_sel, uint8_t* __restrict__ mask) {
-  pdl_sync();
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned long long* sc = reinterpret_cast<unsigned long long*>(smem_raw);
-  for (int i0 = threadIdx.x; i0 < C; i0 += 8 * 256) {      // eight loads in flight per thread, then the stores
-    unsigned long long k[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (i0 + u * 256 < C) k[u] = __ldcg(score_keys + i0 + u * 256);
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (i0 + u * 256 < C) sc[i0 + u * 256] = k[u];
-  }
-  __syncthreads();
-  const int j = blockIdx.x * 16 + (threadIdx.x >> 4);
-  const int sub = threadIdx.x & 15;
-  int rank = 0;
-  if (j < C) {
-    const unsigned long long sj = sc[j];
-#pragma unroll 8
-    for (int i = sub; i < C; i += 16) {
-      const unsigned long long si = sc[i];
-      rank += (si > sj || (si == sj && i < j)) ? 1 : 0;
-    }
-  }
-#pragma unroll
-  for (int o = 1; o < 16; o <<= 1) rank += __shfl_xor_sync(0xFFFFFFFFu, rank, o);
-  if (j < C && sub == 0) mask[j] = rank < n_sel ? 1 : 0;
-}
-
 // Ascending list of the selected channels (verification export only).  One CTA.
 __global__ void __launch_bounds__(1024)
 sel_list_kernel(const uint8_t* __restrict__ mask, int C, int32_t* __restrict__ sel_export) {
@@ -962,18 +777,6 @@ sel_list_kernel(const uint8_t* __restrict__ mask, int C, int32_t* __restrict__ s
     if (mask[i]) sel_export[pos++] = i;
 }
 
-__device__ __forceinline__ uint32_t nibble_mask8(const uint8_t* m) {
-  // m[0..7] in {0,1} -> 0xF per selected nibble
-  const uint2 v = *reinterpret_cast<const uint2*>(m);
-  uint32_t out = 0;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    out |= ((v.x >> (8 * i)) & 1u) * (0xFu << (4 * i));
-    out |= ((v.y >> (8 * i)) & 1u) * (0xFu << (16 + 4 * i));
-  }
-  return out;
-}
-
 // Verification export of the masked residual's codes in token order (Eq. residual-recon: codes of unselected
 // channels cleared), from codes stored with `flip` XORed into every word.  One thread per (token, 32 channels).
 __global__ void __launch_bounds__(256)
@@ -991,149 +794,6 @@ export_residual_kernel(int T, int H, const uint8_t* __restrict__ mask, uint32_t 
   v.z = (v.z ^ flip) & nibble_mask8(m + 16); v.w = (v.w ^ flip) & nibble_mask8(m + 24);
   *reinterpret_cast<uint4*>(rq_exp + co) = v;
 }
-
-// ---------------------------------------------------------------------------
-// Site-13 dispatch, driven by the DESTINATION: one CTA per 128-row tile of the padded dispatch
-// order gathers its rows' codes and scales from the token-order arrays (which stay in L2: every
-// token row is read top-k times) and writes the tile's 128 x H/2 code bytes and its scale atoms
-// as whole, contiguous regions.  Written from the source side instead (one thread per token
-// chunk), every 512-byte scale atom is touched by 128 different tokens at 128 different times,
-// 4 bytes each: partially written sectors get evicted and the memory system pays for them.
-// The residual is masked on the way (Eq. residual-recon: codes of unselected channels are cleared) and
-// stored NEGATED (sign bits flipped), so that the GEMM can accumulate W Q(x) + W (-M Q(dx)) with two
-// plain MMAs.
-// grid = upper bound of the tile count (tiles beyond header[kHdrMTiles] leave at once), 256 threads.
-// ---------------------------------------------------------------------------
-constexpr int kDispatchSlab = 32;                   // scale atoms (K = 64 each) staged per pass
-constexpr int kDispatchRows = 8;                    // rows (16-byte loads) in flight per thread (4: 2 us slower per half, 16: spills)
-template <int kParts>
-__global__ void __launch_bounds__(256, 4)
-rac_dispatch_kernel(int H, const uint8_t* __restrict__ mask, const int32_t* __restrict__ header,
-                    const int32_t* __restrict__ tile_rows, const int32_t* __restrict__ row_token,
-                    const uint8_t* __restrict__ xq, const uint8_t* __restrict__ xsf, const uint8_t* __restrict__ rq,
-                    const uint8_t* __restrict__ rsf, uint8_t* __restrict__ xq_pad, uint8_t* __restrict__ xsf_tiled,
-                    uint8_t* __restrict__ rq_pad, uint8_t* __restrict__ rsf_tiled) {
-  pdl_sync();
-  const int mt = blockIdx.x;
-  if (mt >= header[kHdrMTiles]) return;
-  const int n_rows = tile_rows[mt];
-  __shared__ int tok[128];
-  __shared__ __align__(16) uint8_t atoms[kParts == 3 ? 2 : 1][kDispatchSlab * 512];
-  if (threadIdx.x < 128) tok[threadIdx.x] = threadIdx.x < n_rows ? row_token[mt * 128 + threadIdx.x] : -1;
-  __syncthreads();
-  constexpr bool do_x = (kParts & 1) != 0, do_r = (kParts & 2) != 0;
-  constexpr int kRows = kParts == 3 ? kDispatchRows / 2 : kDispatchRows;   // the same number of loads in flight
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int per_row = H >> 5;                         // 16-byte chunks of codes per row
-  const size_t row_bytes = (size_t)(H >> 1);
-  // ---- codes: a warp walks rows warp, warp + 8, ...; its lanes take consecutive 16-byte chunks
-  for (int c = lane; c < per_row; c += 32) {
-    uint32_t m0 = 0, m1 = 0, m2 = 0, m3 = 0;
-    if (do_r) {
-      const uint8_t* m = mask + c * 32;
-      m0 = nibble_mask8(m); m1 = nibble_mask8(m + 8); m2 = nibble_mask8(m + 16); m3 = nibble_mask8(m + 24);
-    }
-    for (int r0 = warp; r0 < n_rows; r0 += 8 * kRows) {   // kRows rows in flight per thread
-      uint4 xv[do_x ? kRows : 1], rv[do_r ? kRows : 1];
-#pragma unroll
-      for (int j = 0; j < kRows; ++j) {
-        const int r = r0 + 8 * j;
-        if (r < n_rows) {
-          const size_t so = (size_t)tok[r] * row_bytes + (size_t)c * 16;
-          if (do_x) xv[do_x ? j : 0] = __ldg(reinterpret_cast<const uint4*>(xq + so));
-          if (do_r) rv[do_r ? j : 0] = __ldg(reinterpret_cast<const uint4*>(rq + so));
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < kRows; ++j) {
-        const int r = r0 + 8 * j;
-        if (r < n_rows) {
-          const size_t po = (size_t)(mt * 128 + r) * row_bytes + (size_t)c * 16;
-          if (do_x) __stcs(reinterpret_cast<uint4*>(xq_pad + po), xv[do_x ? j : 0]);
-          if (do_r) {
-            uint4 v = rv[do_r ? j : 0];
-            v.x = (v.x & m0) ^ 0x88888888u; v.y = (v.y & m1) ^ 0x88888888u;
-            v.z = (v.z & m2) ^ 0x88888888u; v.w = (v.w & m3) ^ 0x88888888u;
-            __stcs(reinterpret_cast<uint4*>(rq_pad + po), v);
-          }
-        }
-      }
-    }
-  }
-  // ---- scales: the rows' linear scale bytes are transposed into whole atoms through shared memory
-  const int kt_count = H >> 6;
-  const size_t sf_row = (size_t)(H >> 4);
-  for (int k0 = 0; k0 < kt_count; k0 += kDispatchSlab) {
-    const int nk = min(kDispatchSlab, kt_count - k0);
-    __syncthreads();                                  // the previous slab has been written out
-    for (int i = threadIdx.x; i < nk * 32; i += blockDim.x) {
-      if (do_x) reinterpret_cast<uint4*>(atoms[0])[i] = make_uint4(0, 0, 0, 0);
-      if (do_r) reinterpret_cast<uint4*>(atoms[kParts == 3 ? 1 : 0])[i] = make_uint4(0, 0, 0, 0);
-    }
-    __syncthreads();
-    // a thread moves 16 bytes = four atoms' worth of one row; consecutive threads take consecutive pieces;
-    // at most 128 rows x 8 pieces = four per thread, all fetched before the first is stored
-    const int pieces = (nk + 3) >> 2;
-    const int n_items = n_rows * pieces;
-    auto fetch = [&](const uint8_t* src, size_t so, int n4, bool wide) -> uint4 {
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (wide) {
-        v = __ldg(reinterpret_cast<const uint4*>(src + so));
-      } else {                                           // word loads (row tails, rows that are not 16-byte aligned)
-        const uint32_t* s = reinterpret_cast<const uint32_t*>(src + so);
-        if (n4 > 0) v.x = __ldg(s);
-        if (n4 > 1) v.y = __ldg(s + 1);
-        if (n4 > 2) v.z = __ldg(s + 2);
-        if (n4 > 3) v.w = __ldg(s + 3);
-      }
-      return v;
-    };
-    auto put = [&](uint8_t* atom, int pc, int dst, int n4, const uint4& v) {
-      uint32_t* a = reinterpret_cast<uint32_t*>(atom + (4 * pc) * 512 + dst);
-      if (n4 > 0) a[0] = v.x;
-      if (n4 > 1) a[128] = v.y;
-      if (n4 > 2) a[256] = v.z;
-      if (n4 > 3) a[384] = v.w;
-    };
-    uint4 xw[do_x ? 4 : 1], rw[do_r ? 4 : 1];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int i = threadIdx.x + u * 256;
-      if (i < n_items) {
-        const int r = i / pieces, pc = i - r * pieces;
-        const size_t so = (size_t)tok[r] * sf_row + (size_t)(k0 + 4 * pc) * 4;
-        const int n4 = min(4, nk - 4 * pc);
-        const bool wide = n4 == 4 && (sf_row & 15) == 0;
-        if (do_x) xw[do_x ? u : 0] = fetch(xsf, so, n4, wide);
-        if (do_r) rw[do_r ? u : 0] = fetch(rsf, so, n4, wide);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int i = threadIdx.x + u * 256;
-      if (i < n_items) {
-        const int r = i / pieces, pc = i - r * pieces;
-        const int dst = (r & 31) * 16 + (r >> 5) * 4;
-        const int n4 = min(4, nk - 4 * pc);
-        if (do_x) put(atoms[0], pc, dst, n4, xw[do_x ? u : 0]);
-        if (do_r) put(atoms[kParts == 3 ? 1 : 0], pc, dst, n4, rw[do_r ? u : 0]);
-      }
-    }
-    __syncthreads();
-    const size_t ao = ((size_t)mt * kt_count + k0) * 512u;
-    for (int i = threadIdx.x; i < nk * 32; i += blockDim.x) {
-      if (do_x) __stcs(reinterpret_cast<uint4*>(xsf_tiled + ao) + i, reinterpret_cast<const uint4*>(atoms[0])[i]);
-      if (do_r) __stcs(reinterpret_cast<uint4*>(rsf_tiled + ao) + i, reinterpret_cast<const uint4*>(atoms[kParts == 3 ? 1 : 0])[i]);
-    }
-  }
-}
-
-template __global__ void rac_dispatch_kernel<1>(int, const uint8_t*, const int32_t*, const int32_t*, const int32_t*, const uint8_t*,
-                                                const uint8_t*, const uint8_t*, const uint8_t*, uint8_t*, uint8_t*, uint8_t*, uint8_t*);
-template __global__ void rac_dispatch_kernel<2>(int, const uint8_t*, const int32_t*, const int32_t*, const int32_t*, const uint8_t*,
-                                                const uint8_t*, const uint8_t*, const uint8_t*, uint8_t*, uint8_t*, uint8_t*, uint8_t*);
-template __global__ void rac_dispatch_kernel<3>(int, const uint8_t*, const int32_t*, const int32_t*, const int32_t*, const uint8_t*,
-                                                const uint8_t*, const uint8_t*, const uint8_t*, uint8_t*, uint8_t*, uint8_t*, uint8_t*);
 
 // Site-2 selection and masking in one launch: every CTA finds the selection's threshold for itself (C
 // integer totals, 8 C bytes out of L2), turns it into nibble masks in shared memory and clears, in place,

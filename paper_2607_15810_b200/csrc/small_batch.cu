@@ -5,8 +5,7 @@
 //   front_small_kernel  tensor amax, quantization of x and of its residual, channel scores, selection,
 //                       masked copies in dispatch order.
 // What bounds them is latency: at decode sizes they move a few megabytes at most, which stay in L2 and
-// shared memory.  Larger batches use the grid-wide kernels of routing.cu / quantize.cu (api.cu holds
-// the rule): a cluster is 16 of the 148 SMs.
+// shared memory.  Larger batches use the grid-wide kernels of front.cu (api.cu holds the rule): a cluster is 16 of the 148 SMs.
 #include <algorithm>
 #include <atomic>
 
@@ -30,23 +29,16 @@ __device__ __forceinline__ void ldg256_l1(const void* p, uint4& a, uint4& b) {
   asm volatile("ld.global.nc.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(p));
 }
-__device__ __forceinline__ uint32_t absmax8(const uint4& v) {
-  return __vmaxu2(__vmaxu2(v.x & 0x7FFF7FFFu, v.y & 0x7FFF7FFFu), __vmaxu2(v.z & 0x7FFF7FFFu, v.w & 0x7FFF7FFFu));
-}
-__device__ __forceinline__ uint32_t float_key(float v) {
-  const uint32_t b = __float_as_uint(v);
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-
-constexpr int kRouteThreads = 512;                         // 16 warps: a warp per token, four per scheduler
-constexpr int kRouteTokens = kRouteThreads / 32;           // tokens of a word of the assignment bit matrix
+constexpr int kSmallRouteThreads = 512;                         // 16 warps: a warp per token, four per scheduler
+constexpr int kRouteTokens = kSmallRouteThreads / 32;           // tokens of a word of the assignment bit matrix
 constexpr int kRouteWords = kSmallRouteMaxTokens / kRouteTokens;
 
-// One warp per token (TW tokens).  The assignments are a bit matrix, words[t / 16][expert] bit t % 16: an expert's count is a population count over its words, and the row of token t inside an
-// expert is the population count below bit t, which is the (expert, token, slot) order without a sort.
+// One warp per token (TW tokens).  The assignments are a bit matrix, words[t / 16][expert] bit t % 16: an expert's
+// count is a population count over its words, and the row of token t inside an expert is the population count
+// below bit t, which is the (expert, token, slot) order without a sort.
 // Every CTA sends its words to the others, then scans all experts for itself.
 template <int NJ, int TW>
-__global__ void __launch_bounds__(kRouteThreads)
+__global__ void __launch_bounds__(kSmallRouteThreads)
 route_small_kernel(const SmallRouteArgs p) {
   pdl_sync();
   __shared__ uint32_t words[kRouteWords][kMaxExperts];
@@ -56,7 +48,7 @@ route_small_kernel(const SmallRouteArgs p) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int E = p.E, topk = p.topk;
   cluster_arrive();                                        // (waited for before the first remote store)
-  for (int i = threadIdx.x; i < TW * kMaxExperts; i += kRouteThreads) words[rank * TW + i / kMaxExperts][i % kMaxExperts] = 0;
+  for (int i = threadIdx.x; i < TW * kMaxExperts; i += kSmallRouteThreads) words[rank * TW + i / kMaxExperts][i % kMaxExperts] = 0;
   // Top-k on order-preserving integer keys, two warp reductions per slot; softmax only for the chosen ones.
   float v[TW][NJ], my_w[TW];
   int my_id[TW];
@@ -113,7 +105,7 @@ route_small_kernel(const SmallRouteArgs p) {
   __syncthreads();
   cluster_wait();                                          // every CTA of the cluster has started
   if (n_cta > 1)
-    for (int i = threadIdx.x; i < TW * E * n_cta; i += kRouteThreads) {
+    for (int i = threadIdx.x; i < TW * E * n_cta; i += kSmallRouteThreads) {
       const int c = i / (TW * E), k = i - c * (TW * E), a = k / E, e = k - a * E;
       if (c != rank) st_cluster_u32(map_to_cta(smem_u32(&words[rank * TW + a][e]), (uint32_t)c), words[rank * TW + a][e]);
     }
@@ -169,7 +161,7 @@ route_small_kernel(const SmallRouteArgs p) {
   // words of the call that start at zero: the status word and the column totals of site 2
   if (rank == n_cta - 1) {
     if (threadIdx.x < kHdrWords - kHdrStatus) p.header[kHdrStatus + threadIdx.x] = 0;
-    for (int i = threadIdx.x; i < p.n_zero; i += kRouteThreads) p.zero_u64[i] = 0ull;
+    for (int i = threadIdx.x; i < p.n_zero; i += kSmallRouteThreads) p.zero_u64[i] = 0ull;
   }
   // ---- rows (and the stores that the barriers above would have waited for)
 #pragma unroll
@@ -191,7 +183,6 @@ route_small_kernel(const SmallRouteArgs p) {
     if (p.perm_out) p.perm_out[row] = flat;
     p.pos_pad[flat] = pos;
     p.row_token[pos] = t;
-    p.row_weight[pos] = my_w[a];
   }
 }
 
@@ -455,7 +446,7 @@ quads_status launch_route_tw(const SmallRouteArgs& a, cudaStream_t st) {
       wide[dev].store(true);
     }
   }
-  QUADS_CUDA_OK(launch_cluster(route_small_kernel<NJ, TW>, n, kRouteThreads, 0, st, a));
+  QUADS_CUDA_OK(launch_cluster(route_small_kernel<NJ, TW>, n, kSmallRouteThreads, 0, st, a));
   return QUADS_OK;
 }
 
