@@ -705,6 +705,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
       SmallRouteArgs r{};
       r.logits = a->router_logits;
       r.T = T; r.E = E; r.topk = topk; r.renormalize = a->renormalize; r.e_lo = e_lo; r.e_hi = e_lo + e_cnt;
+      r.slot_rows = 128;
       r.wts = wts; r.offsets = offsets; r.tile_prefix = tile_prefix; r.tile_expert = tile_expert; r.tile_rows = tile_rows;
       r.header = header; r.perm = perm; r.pos_pad = pos_pad; r.row_token = row_token;
       r.zero_u64 = reinterpret_cast<unsigned long long*>(P(L.keys2)); r.n_zero = I;
@@ -911,10 +912,12 @@ struct Fp8Layout {
   size_t perm, pos_pad, row_token, xq_tok, xe_tok, xq_pad, xsf, hq_pad, hsf, y_pad, total;
   int m_tiles_max;
 };
+// Few rows per expert (decode-sized batches): at most 32 rows per 128-row tile, see fp8.cu.
+bool fp8_few_rows(int T, int E, int topk) { return (int64_t)T * topk <= (int64_t)E * 32; }
 Fp8Layout fp8_layout(int T, int H, int I, int E, int topk) {
   Fp8Layout L{};
   const int64_t A = (int64_t)T * topk;
-  L.m_tiles_max = (int)(A / 128) + E;
+  L.m_tiles_max = (int)(A / (fp8_few_rows(T, E, topk) ? 32 : 128)) + E;
   const size_t pad_rows = (size_t)L.m_tiles_max * 128;
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
@@ -997,27 +1000,40 @@ quads_status quads_moe_fp8_w8a8(const quads_moe_fp8_args* a, void* cuda_stream) 
   int32_t* pos_pad = reinterpret_cast<int32_t*>(P(L.pos_pad));
   int32_t* row_token = reinterpret_cast<int32_t*>(P(L.row_token));
   const size_t pad_rows = (size_t)L.m_tiles_max * 128;
-  QUADS_CUDA_OK(cudaMemsetAsync(ws, 0, L.ids, st));            // header, status word, route counts
+  const bool few = fp8_few_rows(T, E, topk), small = few && route_small_fits(T);
   // ---- routing, dispatch order and activation quantization (token order), then the dispatched copies
   uint8_t* xq_tok = a->xq ? a->xq : P(L.xq_tok);
   uint8_t* xe_tok = a->xexp ? a->xexp : P(L.xe_tok);
-  {
+  const uint16_t* x = static_cast<const uint16_t*>(a->x);
+  if (small) {
+    SmallRouteArgs r{};
+    r.logits = a->router_logits;
+    r.T = T; r.E = E; r.topk = topk; r.renormalize = a->renormalize; r.e_lo = 0; r.e_hi = E; r.slot_rows = 32;
+    r.wts = wts; r.offsets = offsets; r.tile_prefix = tile_prefix; r.tile_expert = tile_expert; r.tile_rows = tile_rows;
+    r.header = header; r.perm = perm; r.pos_pad = pos_pad; r.row_token = row_token;
+    r.ids_out = a->topk_ids; r.perm_out = a->perm;
+    if ((s = launch_route_small(r, st)) != QUADS_OK) return s;
+    if ((s = launch_fp8_quantize_act(x, T, H, xq_tok, xe_tok, di.sm_count, st)) != QUADS_OK) return s;
+  } else {
+    QUADS_CUDA_OK(cudaMemsetAsync(ws, 0, L.ids, st));          // header, status word, route counts
     RouteArgs r{};
     r.logits = a->router_logits;
     r.T = T; r.E = E; r.topk = topk; r.renormalize = a->renormalize; r.e_lo = 0; r.e_hi = E;
-    r.slot_rows = 128; r.tile_group = 1;
+    r.slot_rows = few ? 32 : 128; r.tile_group = 1;
     r.ids = ids; r.wts = wts; r.counts = reinterpret_cast<int32_t*>(P(L.route_counts));
     r.arrivals = reinterpret_cast<unsigned int*>(header + kHdrRouteArrivals); r.status = header + kHdrStatus;
     r.offsets = offsets; r.tile_prefix = tile_prefix; r.tile_expert = tile_expert; r.tile_rows = tile_rows; r.header = header;
     r.perm = perm; r.pos_pad = pos_pad; r.row_token = row_token;
     r.ids_out = a->topk_ids; r.perm_out = a->perm;
-    if ((s = launch_fp8_front(static_cast<const uint16_t*>(a->x), T, H, xq_tok, xe_tok, r, di.sm_count, st)) != QUADS_OK) return s;
+    if ((s = launch_fp8_front(x, T, H, xq_tok, xe_tok, r, di.sm_count, st)) != QUADS_OK) return s;
   }
-  QUADS_CUDA_OK(launch_kernel(fp8_dispatch_kernel, dim3(L.m_tiles_max), dim3(256), (size_t)0, st, H, header, tile_rows, row_token,
-                              xq_tok, xe_tok, P(L.xq_pad), P(L.xsf)));
+  if (!few)
+    QUADS_CUDA_OK(launch_kernel(fp8_dispatch_kernel, dim3(L.m_tiles_max), dim3(256), (size_t)0, st, H, header, tile_rows, row_token,
+                                xq_tok, xe_tok, P(L.xq_pad), P(L.xsf)));
   // ---- first projection: W13, SwiGLU, requantize
   CUtensorMap ma, mb;
-  if ((s = make_codes_map(&ma, P(L.xq_pad), pad_rows, (uint64_t)H)) != QUADS_OK) return s;
+  if ((s = few ? make_gather_map(&ma, xq_tok, (uint64_t)T, (uint64_t)H) : make_codes_map(&ma, P(L.xq_pad), pad_rows, (uint64_t)H)) != QUADS_OK)
+    return s;
   if ((s = make_codes_map(&mb, a->w13_q, (uint64_t)E * 2 * I, (uint64_t)H)) != QUADS_OK) return s;
   Fp8GemmParams g{};
   g.K = H; g.n_tiles_n = I / 128; g.n_out = I; g.b_rows_per_expert = 2 * I; g.half1_row_offset = I;
@@ -1026,21 +1042,23 @@ quads_status quads_moe_fp8_w8a8(const quads_moe_fp8_args* a, void* cuda_stream) 
   g.hq_pad = P(L.hq_pad); g.hsf_atoms = P(L.hsf);
   g.h_export = static_cast<uint16_t*>(a->h_bf16); g.hq_export = a->hq; g.hexp_export = a->hexp;
   g.tile_prefix = tile_prefix; g.offsets = offsets; g.status = header + kHdrStatus;
+  g.row_token = row_token; g.xe_tok = xe_tok; g.tables_late = few && !small;
   const bool timing = g_timers.enabled && g_timers.created;
   if (timing) QUADS_CUDA_OK(cudaEventRecord(g_timers.ev[0], st));
-  if ((s = launch_gemm_fp8(kEpiSwiGLU, g, ma, mb, di.sm_count, st)) != QUADS_OK) return s;
+  if ((s = launch_gemm_fp8(kEpiSwiGLU, few, g, ma, mb, di.sm_count, st)) != QUADS_OK) return s;
   if (timing) QUADS_CUDA_OK(cudaEventRecord(g_timers.ev[1], st));
   // ---- second projection and weighted combine
   CUtensorMap m2a, m2b;
-  if ((s = make_codes_map(&m2a, P(L.hq_pad), pad_rows, (uint64_t)I)) != QUADS_OK) return s;
+  if ((s = make_codes_map(&m2a, P(L.hq_pad), pad_rows, (uint64_t)I, few ? 32 : 128)) != QUADS_OK) return s;
   if ((s = make_codes_map(&m2b, a->w2_q, (uint64_t)E * H, (uint64_t)I)) != QUADS_OK) return s;
   Fp8GemmParams g2 = g;
   g2.K = I; g2.n_tiles_n = (H + 255) / 256; g2.n_out = H; g2.b_rows_per_expert = H; g2.half1_row_offset = 128;
   g2.a_sf = P(L.hsf); g2.b_sf = a->w2_atoms; g2.b_sf_expert_stride = (size_t)(H / 128) * (I / 128) * 512;
   g2.y_pad = reinterpret_cast<uint16_t*>(P(L.y_pad));
   g2.h_export = nullptr;
+  g2.tables_late = 0;
   if (timing) QUADS_CUDA_OK(cudaEventRecord(g_timers.ev[2], st));
-  if ((s = launch_gemm_fp8(kEpiCombine, g2, m2a, m2b, di.sm_count, st)) != QUADS_OK) return s;
+  if ((s = launch_gemm_fp8(kEpiCombine, few, g2, m2a, m2b, di.sm_count, st)) != QUADS_OK) return s;
   if (timing) {
     QUADS_CUDA_OK(cudaEventRecord(g_timers.ev[3], st));
     g_timers.valid = true;

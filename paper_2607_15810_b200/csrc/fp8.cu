@@ -23,6 +23,12 @@ __device__ __forceinline__ uint32_t fp8_scale_code(float amax) {
   return (uint32_t)(e + 127);
 }
 
+// 2^-e of a scale byte e + 127 (0..254), exact: multiplying by it is what __fmul_rn(x, sc) does, in one instruction.
+__device__ __forceinline__ float fp8_inv_scale(uint32_t code) {
+  const uint32_t k = 254u - code;
+  return __uint_as_float(k == 0 ? 0x00400000u : k << 23);
+}
+
 __device__ __forceinline__ uint32_t f32x4_to_e4m3x4(float a, float b, float c, float d) {
   uint16_t lo, hi;
   asm("cvt.rn.satfinite.e4m3x2.f32 %0, %2, %1;" : "=h"(lo) : "f"(a), "f"(b));
@@ -45,11 +51,19 @@ __device__ __forceinline__ void fp8_quantize_act(const uint16_t* __restrict__ x,
     const float f2 = __uint_as_float(v.y << 16), f3 = __uint_as_float(v.y & 0xFFFF0000u);
     const float a = warp_max(fmaxf(fmaxf(fabsf(f0), fabsf(f1)), fmaxf(fabsf(f2), fabsf(f3))));
     const uint32_t code = fp8_scale_code(a);
-    const int e = (int)code - 127;
+    const float sc = fp8_inv_scale(code);
     reinterpret_cast<uint32_t*>(codes + r * K + t * 128)[lane] =
-        f32x4_to_e4m3x4(ldexpf(f0, -e), ldexpf(f1, -e), ldexpf(f2, -e), ldexpf(f3, -e));
+        f32x4_to_e4m3x4(__fmul_rn(f0, sc), __fmul_rn(f1, sc), __fmul_rn(f2, sc), __fmul_rn(f3, sc));
     if (lane == 0) exps[r * kt + t] = (uint8_t)code;
   }
+}
+
+// Few tokens: quantization alone, behind route_small_kernel, which has itself waited for whatever produced x: only
+// the kernels that follow need the routing.
+__global__ void __launch_bounds__(256)
+fp8_quantize_act_kernel(const uint16_t* __restrict__ x, int64_t rows, int K, uint8_t* __restrict__ codes, uint8_t* __restrict__ exps) {
+  fp8_quantize_act(x, rows, K, codes, exps, (int)blockIdx.x, (int)gridDim.x);
+  pdl_sync();
 }
 
 // All CTAs route a few tokens; then the first n_groups hand out the rows (they wait for the others: cooperative
@@ -84,6 +98,13 @@ quads_status launch_fp8_front_nj(const uint16_t* x, int64_t rows, int K, uint8_t
   return QUADS_OK;
 }
 }  // namespace
+
+quads_status launch_fp8_quantize_act(const uint16_t* x, int64_t rows, int K, uint8_t* codes, uint8_t* exps, int sm_count, cudaStream_t st) {
+  const int64_t want = (rows * (K / 128) + 7) / 8;
+  QUADS_CUDA_OK(launch_kernel(fp8_quantize_act_kernel, dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)sm_count * 8))),
+                              dim3(256), (size_t)0, st, x, rows, K, codes, exps));
+  return QUADS_OK;
+}
 
 quads_status launch_fp8_front(const uint16_t* x, int64_t rows, int K, uint8_t* codes, uint8_t* exps, const RouteArgs& r, int sm_count,
                               cudaStream_t st) {
@@ -126,17 +147,17 @@ fp8_quantize_weight_kernel(const uint16_t* __restrict__ w, int N, int K, uint8_t
   }
   __syncthreads();
   const uint32_t code = code_sh;
-  const int e = (int)code - 127;
+  const float sc = fp8_inv_scale(code);
 #pragma unroll
   for (int i = 0; i < 8; i += 2) {
     float f[16];
     unpack8(v[i], f);
     unpack8(v[i + 1], f + 8);
     uint4 o;
-    o.x = f32x4_to_e4m3x4(ldexpf(f[0], -e), ldexpf(f[1], -e), ldexpf(f[2], -e), ldexpf(f[3], -e));
-    o.y = f32x4_to_e4m3x4(ldexpf(f[4], -e), ldexpf(f[5], -e), ldexpf(f[6], -e), ldexpf(f[7], -e));
-    o.z = f32x4_to_e4m3x4(ldexpf(f[8], -e), ldexpf(f[9], -e), ldexpf(f[10], -e), ldexpf(f[11], -e));
-    o.w = f32x4_to_e4m3x4(ldexpf(f[12], -e), ldexpf(f[13], -e), ldexpf(f[14], -e), ldexpf(f[15], -e));
+    o.x = f32x4_to_e4m3x4(__fmul_rn(f[0], sc), __fmul_rn(f[1], sc), __fmul_rn(f[2], sc), __fmul_rn(f[3], sc));
+    o.y = f32x4_to_e4m3x4(__fmul_rn(f[4], sc), __fmul_rn(f[5], sc), __fmul_rn(f[6], sc), __fmul_rn(f[7], sc));
+    o.z = f32x4_to_e4m3x4(__fmul_rn(f[8], sc), __fmul_rn(f[9], sc), __fmul_rn(f[10], sc), __fmul_rn(f[11], sc));
+    o.w = f32x4_to_e4m3x4(__fmul_rn(f[12], sc), __fmul_rn(f[13], sc), __fmul_rn(f[14], sc), __fmul_rn(f[15], sc));
     reinterpret_cast<uint4*>(codes + off)[i >> 1] = o;
   }
   const size_t ti = ((size_t)tensor * nt + tn) * kt + tk;
@@ -195,19 +216,35 @@ namespace {
 
 constexpr int k8BM = 128, k8BN = 256;
 constexpr int k8TileA = k8BM * 128, k8TileB = k8BN * 128;
-constexpr int k8OffB = k8TileA;
-constexpr int k8OffSfA = k8OffB + k8TileB;
-constexpr int k8OffSfB = k8OffSfA + 512;
-constexpr int k8StageBytes = k8OffSfB + 1024 + 512;      // 51200 (1 KB multiple)
-constexpr int k8Stages = 4;
-constexpr int k8Threads = 576;
-constexpr int k8EpiWarps = 16;
-constexpr int k8BarOffset = k8Stages * k8StageBytes;
-constexpr int k8SmemBytes = k8BarOffset + 256 + 2 * 128 * 4 * 4 + 1024;
+constexpr int k8ActWarp = 3;                             // loads the activation side of the few-rows form
+constexpr int k8FewRows = 32;                            // rows of a tile in that form
+constexpr int k8MaxStages = 5;
+
+// kFew: few rows per expert (decode-sized batches; the routing then puts at most 32 rows into a 128-row tile).  All
+// that matters there is the stream of weights: the activation operand takes 4 KB of a stage instead of 16 (the
+// MMA still reads 128 rows; what it finds behind the 32 gives accumulator rows nobody reads), which makes room for
+// a fifth stage; the first projection gathers its rows and scales out of the token-order arrays instead of
+// reading copies of them; and the weights and routing tables are older than the preceding kernel, so the ring
+// fills while that one still runs.  Layer of 256 tokens (645 MB of weights and scale atoms): 164.9 -> 130.0 us; the
+// two GEMMs stream at 5.9 and 6.1 TB/s (4.7 and 5.5 with 128-row tiles, four stages and copied rows).
+template <bool kFew>
+struct F8Cfg {
+  static constexpr int kOffB = kFew ? k8FewRows * 128 : k8TileA;
+  static constexpr int kOffSfA = kOffB + k8TileB;
+  static constexpr int kOffSfB = kOffSfA + 512;
+  static constexpr int kStageBytes = (kOffSfB + 1024 + 1023) / 1024 * 1024;      // 51200 / 38912
+  static constexpr int kStages = kFew ? 5 : 4;
+  static constexpr int kThreads = kFew ? 416 : 576;
+  static constexpr int kLoadWarp = kFew ? 1 : 0, kMmaWarp = kFew ? 2 : 1;
+  static constexpr int kEpiWarps = kFew ? 4 : 16;        // the warps whose tensor-memory lanes hold rows (few: 0, 4, 8, 12)
+  static constexpr int kBarOffset = kStages * kStageBytes;
+  static constexpr int kSmemBytes = kBarOffset + 256 + 2 * 128 * 4 * 4 + 1024;
+  static_assert(kSmemBytes <= 232448 && kStages <= k8MaxStages, "shared memory");
+};
 
 struct __align__(8) F8Barriers {
-  uint64_t full[k8Stages];
-  uint64_t empty[k8Stages];
+  uint64_t full[k8MaxStages];
+  uint64_t empty[k8MaxStages];
   uint64_t tmem_full;
   uint64_t tmem_empty;
   uint32_t tmem_base;
@@ -222,20 +259,30 @@ __device__ __forceinline__ void tc_mma_mxf8(uint32_t d_tmem, uint64_t adesc, uin
       ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(sfa_tmem), "r"(sfb_tmem), "r"(accumulate) : "memory");
 }
 
-template <int EPI>
-__global__ void __launch_bounds__(k8Threads, 1)
+// Four rows of the tensor map (box: one row) into 4 x 128 bytes, swizzled like a tile.
+__device__ __forceinline__ void tma_gather4_rows(uint32_t dst, const CUtensorMap* map, int x, int y0, int y1, int y2, int y3, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cta.global.tile::gather4.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
+      ::"r"(dst), "l"(map), "r"(x), "r"(y0), "r"(y1), "r"(y2), "r"(y3), "r"(bar) : "memory");
+}
+
+template <int EPI, bool kFew>
+__global__ void __launch_bounds__(F8Cfg<kFew>::kThreads, 1)
 gemm_fp8_kernel(const Fp8GemmParams p, const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b) {
+  using C = F8Cfg<kFew>;
+  constexpr int k8Stages = C::kStages, k8StageBytes = C::kStageBytes, k8OffB = C::kOffB, k8OffSfA = C::kOffSfA,
+                k8OffSfB = C::kOffSfB, k8EpiWarps = C::kEpiWarps;
   extern __shared__ uint8_t smem_dyn[];
   const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   uint8_t* smem_gen = smem_dyn + (smem_base - smem_u32(smem_dyn));
-  F8Barriers* bars = reinterpret_cast<F8Barriers*>(smem_gen + k8BarOffset);
-  float* row_amax = reinterpret_cast<float*>(smem_gen + k8BarOffset + 256);     // [2][128][4]
+  F8Barriers* bars = reinterpret_cast<F8Barriers*>(smem_gen + C::kBarOffset);
+  float* row_amax = reinterpret_cast<float*>(smem_gen + C::kBarOffset + 256);   // [2][128][4]
   const uint32_t bar_full = smem_u32(&bars->full[0]), bar_empty = smem_u32(&bars->empty[0]);
   const uint32_t bar_tfull = smem_u32(&bars->tmem_full), bar_tempty = smem_u32(&bars->tmem_empty);
   volatile int* abort_flag = &bars->abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < k8Stages; ++s) { mbar_init(bar_full + 8 * s, 1); mbar_init(bar_empty + 8 * s, 1); }
+    for (int s = 0; s < k8Stages; ++s) { mbar_init(bar_full + 8 * s, kFew ? 2 : 1); mbar_init(bar_empty + 8 * s, 1); }
     mbar_init(bar_tfull, 1);
     mbar_init(bar_tempty, k8EpiWarps);
     bars->abort_flag = 0;
@@ -243,18 +290,21 @@ gemm_fp8_kernel(const Fp8GemmParams p, const __grid_constant__ CUtensorMap tm_a,
     prefetch_tmap(&tm_a);
     prefetch_tmap(&tm_b);
   }
-  if (warp == 1) tmem_alloc<1>(smem_u32(&bars->tmem_base), 512);
+  if (warp == C::kMmaWarp) tmem_alloc<1>(smem_u32(&bars->tmem_base), 512);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
-  pdl_sync();
+  // (few rows: the weight loader and the MMA issuer read nothing of the preceding kernel, unless that is the one
+  // that made the routing tables)
+  if (!kFew || p.tables_late || (warp != C::kLoadWarp && warp != C::kMmaWarp)) pdl_sync();
+  else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   const int m_tiles = p.header[kHdrMTiles];
   const int total_tiles = m_tiles * p.n_tiles_n;
   const int k_stages = p.K >> 7;
 
-  if (warp == 0) {
+  if (warp == C::kLoadWarp) {
     // ------------------------------------------------------------ producer
     const bool issuer = elect_one();
     uint32_t stage = 0, phase = 0;
@@ -273,11 +323,11 @@ gemm_fp8_kernel(const Fp8GemmParams p, const __grid_constant__ CUtensorMap tm_a,
         if (!ok) break;
         if (issuer) {
           const uint32_t sb = smem_base + stage * k8StageBytes, full = bar_full + 8 * stage;
-          mbar_expect_tx(full, (uint32_t)(k8TileA + (half1 ? k8TileB : k8TileB / 2) + 512 + (half1 ? 1024 : 512)));
-          tma_load_2d(sb, &tm_a, ks * 128, mt * k8BM, full);
+          mbar_expect_tx(full, (uint32_t)((kFew ? 0 : k8TileA + 512) + (half1 ? k8TileB + 1024 : k8TileB / 2 + 512)));
+          if (!kFew) tma_load_2d(sb, &tm_a, ks * 128, mt * k8BM, full);
           tma_load_2d(sb + k8OffB, &tm_b, ks * 128, brow0, full);
           if (half1) tma_load_2d(sb + k8OffB + k8TileA, &tm_b, ks * 128, brow1, full);
-          bulk_load(sb + k8OffSfA, asf + (size_t)ks * 512u, 512u, full);
+          if (!kFew) bulk_load(sb + k8OffSfA, asf + (size_t)ks * 512u, 512u, full);
           bulk_load(sb + k8OffSfB, bsf + ((size_t)rt0 * k_stages + ks) * 512u, 512u, full);
           if (half1) bulk_load(sb + k8OffSfB + 512, bsf + ((size_t)rt1 * k_stages + ks) * 512u, 512u, full);
         }
@@ -289,7 +339,53 @@ gemm_fp8_kernel(const Fp8GemmParams p, const __grid_constant__ CUtensorMap tm_a,
       ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, p.status);
       if (++stage == k8Stages) { stage = 0; phase ^= 1u; }
     }
-  } else if (warp == 1) {
+  } else if (kFew && warp == k8ActWarp) {
+    // ------------------------------------------------------------ activation loader of the few-rows form
+    uint32_t stage = 0, phase = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+      const int mt = tile / p.n_tiles_n;
+      const int n_rows = p.tile_rows[mt];
+      if (EPI == kEpiSwiGLU) {
+        // lane = row of the tile (rows beyond the valid ones repeat the last); lanes 0..7 gather four rows each
+        const int tok = p.row_token[mt * 128 + min(lane, n_rows - 1)];
+        const int g4 = (lane & 7) * 4;
+        const int y0 = __shfl_sync(0xFFFFFFFFu, tok, g4), y1 = __shfl_sync(0xFFFFFFFFu, tok, g4 + 1);
+        const int y2 = __shfl_sync(0xFFFFFFFFu, tok, g4 + 2), y3 = __shfl_sync(0xFFFFFFFFu, tok, g4 + 3);
+        const bool gathers = lane < 8 && g4 < n_rows;
+        const uint32_t bytes = (uint32_t)((n_rows + 3) / 4) * 512u;
+        const uint8_t* xe = p.xe_tok + (size_t)tok * k_stages;
+        uint32_t code = __ldg(xe);
+        for (int ks = 0; ks < k_stages; ++ks) {
+          ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, p.status);
+          if (!ok) break;
+          const uint32_t sb = smem_base + stage * k8StageBytes, full = bar_full + 8 * stage;
+          if (gathers) tma_gather4_rows(sb + (uint32_t)g4 * 128u, &tm_a, ks * 128, y0, y1, y2, y3, full);
+          asm volatile("st.shared.u32 [%0], %1;" ::"r"(sb + k8OffSfA + lane * 16), "r"(code * 0x01010101u) : "memory");
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // the copy to tensor memory reads these words
+          __syncwarp();
+          if (lane == 0) mbar_expect_tx(full, bytes);
+          if (ks + 1 < k_stages) code = __ldg(xe + ks + 1);                 // a stage ahead of its use
+          if (++stage == k8Stages) { stage = 0; phase ^= 1u; }
+        }
+      } else {
+        const bool issuer = elect_one();
+        const uint8_t* asf = p.a_sf + (size_t)mt * k_stages * 512u;
+        for (int ks = 0; ks < k_stages; ++ks) {
+          ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, p.status);
+          if (!ok) break;
+          if (issuer) {
+            const uint32_t sb = smem_base + stage * k8StageBytes, full = bar_full + 8 * stage;
+            mbar_expect_tx(full, (uint32_t)(k8FewRows * 128 + 512));
+            tma_load_2d(sb, &tm_a, ks * 128, mt * k8BM, full);
+            bulk_load(sb + k8OffSfA, asf + (size_t)ks * 512u, 512u, full);
+          }
+          __syncwarp();
+          if (++stage == k8Stages) { stage = 0; phase ^= 1u; }
+        }
+      }
+    }
+  } else if (warp == C::kMmaWarp) {
     // ------------------------------------------------------------ MMA issuer
     const bool issuer = elect_one();
     uint32_t stage = 0, phase = 0, kcount = 0;
@@ -328,9 +424,9 @@ gemm_fp8_kernel(const Fp8GemmParams p, const __grid_constant__ CUtensorMap tm_a,
       if (ok && issuer) tc_commit<1>(bar_tfull);
       __syncwarp();
     }
-  } else {
+  } else if (!kFew || (warp & 3) == 0) {
     // ------------------------------------------------------------ epilogue
-    const int q = warp & 3, cq = (warp - 2) >> 2;
+    const int q = warp & 3, cq = kFew ? warp >> 2 : (warp - 2) >> 2;
     const int row_in_tile = q * 32 + lane;
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
     int it = 0;
@@ -373,13 +469,13 @@ gemm_fp8_kernel(const Fp8GemmParams p, const __grid_constant__ CUtensorMap tm_a,
         asm volatile("bar.sync 1, %0;" ::"n"(32 * k8EpiWarps) : "memory");
         const float4 m4 = *reinterpret_cast<const float4*>(slot + row_in_tile * 4);
         const uint32_t code = fp8_scale_code(fmaxf(fmaxf(m4.x, m4.y), fmaxf(m4.z, m4.w)));
-        const int ex = (int)code - 127;
+        const float sc = fp8_inv_scale(code);
         if (ok && valid) {
           uint32_t w8[8];
 #pragma unroll
           for (int i = 0; i < 8; ++i)
-            w8[i] = f32x4_to_e4m3x4(ldexpf(hb[4 * i], -ex), ldexpf(hb[4 * i + 1], -ex), ldexpf(hb[4 * i + 2], -ex),
-                                    ldexpf(hb[4 * i + 3], -ex));
+            w8[i] = f32x4_to_e4m3x4(__fmul_rn(hb[4 * i], sc), __fmul_rn(hb[4 * i + 1], sc), __fmul_rn(hb[4 * i + 2], sc),
+                                    __fmul_rn(hb[4 * i + 3], sc));
           const int f0 = nt * 128 + cq * 32;
           uint4* dq = reinterpret_cast<uint4*>(p.hq_pad + (size_t)prow * I + f0);
           dq[0] = make_uint4(w8[0], w8[1], w8[2], w8[3]);
@@ -388,7 +484,7 @@ gemm_fp8_kernel(const Fp8GemmParams p, const __grid_constant__ CUtensorMap tm_a,
             reinterpret_cast<uint32_t*>(p.hsf_atoms + ((size_t)mt * (I >> 7) + nt) * 512)[(row_in_tile & 31) * 4 + (row_in_tile >> 5)] =
                 code * 0x01010101u;
           if (p.h_export) {
-            const int drow = p.offsets[e] + (mt - p.tile_prefix[e]) * k8BM + row_in_tile;
+            const int drow = p.offsets[e] + (mt - p.tile_prefix[e]) * (kFew ? k8FewRows : k8BM) + row_in_tile;
             uint4* d = reinterpret_cast<uint4*>(p.h_export + (size_t)drow * I + f0);
 #pragma unroll
             for (int i = 0; i < 4; ++i)
@@ -413,21 +509,26 @@ gemm_fp8_kernel(const Fp8GemmParams p, const __grid_constant__ CUtensorMap tm_a,
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 1) tmem_dealloc<1>(tmem, 512);
+  if (warp == C::kMmaWarp) tmem_dealloc<1>(tmem, 512);
 }
 
 }  // namespace
 
-quads_status launch_gemm_fp8(int epi, const Fp8GemmParams& p, const CUtensorMap& tm_a, const CUtensorMap& tm_b, int n_sms,
-                             cudaStream_t stream) {
-  if (epi == kEpiSwiGLU) {
-    QUADS_CUDA_OK(set_max_dynamic_smem<gemm_fp8_kernel<kEpiSwiGLU>>(k8SmemBytes));
-    QUADS_CUDA_OK(launch_kernel(gemm_fp8_kernel<kEpiSwiGLU>, dim3(n_sms), dim3(k8Threads), (size_t)k8SmemBytes, stream, p, tm_a, tm_b));
-  } else {
-    QUADS_CUDA_OK(set_max_dynamic_smem<gemm_fp8_kernel<kEpiCombine>>(k8SmemBytes));
-    QUADS_CUDA_OK(launch_kernel(gemm_fp8_kernel<kEpiCombine>, dim3(n_sms), dim3(k8Threads), (size_t)k8SmemBytes, stream, p, tm_a, tm_b));
-  }
+template <int EPI, bool kFew>
+static quads_status launch_gemm_fp8_as(const Fp8GemmParams& p, const CUtensorMap& tm_a, const CUtensorMap& tm_b, int n_sms, cudaStream_t stream) {
+  constexpr int smem = F8Cfg<kFew>::kSmemBytes;
+  QUADS_CUDA_OK((set_max_dynamic_smem<gemm_fp8_kernel<EPI, kFew>>(smem)));
+  QUADS_CUDA_OK(launch_kernel(gemm_fp8_kernel<EPI, kFew>, dim3(n_sms), dim3(F8Cfg<kFew>::kThreads), (size_t)smem, stream, p, tm_a, tm_b));
   return QUADS_OK;
+}
+
+quads_status launch_gemm_fp8(int epi, bool few_rows, const Fp8GemmParams& p, const CUtensorMap& tm_a, const CUtensorMap& tm_b, int n_sms,
+                             cudaStream_t stream) {
+  if (epi == kEpiSwiGLU)
+    return few_rows ? launch_gemm_fp8_as<kEpiSwiGLU, true>(p, tm_a, tm_b, n_sms, stream)
+                    : launch_gemm_fp8_as<kEpiSwiGLU, false>(p, tm_a, tm_b, n_sms, stream);
+  return few_rows ? launch_gemm_fp8_as<kEpiCombine, true>(p, tm_a, tm_b, n_sms, stream)
+                  : launch_gemm_fp8_as<kEpiCombine, false>(p, tm_a, tm_b, n_sms, stream);
 }
 
 }  // namespace quads

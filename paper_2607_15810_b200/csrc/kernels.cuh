@@ -108,6 +108,7 @@ constexpr int kSmallMaxUnits = 16;    // units of 128 channels a CTA of the fron
 struct SmallRouteArgs {
   const float* logits;
   int T, E, topk, renormalize, e_lo, e_hi;
+  int slot_rows;                      // valid rows of a 128-row tile at most
   float* wts;
   int32_t *offsets, *tile_prefix, *tile_expert, *tile_rows, *header, *perm, *pos_pad, *row_token;
   unsigned long long* zero_u64;       // n_zero words cleared for the kernels that follow
@@ -129,6 +130,7 @@ struct SmallFrontArgs {
   float* gs_store;                    // exports, each may be NULL
   uint8_t *mask_out, *xq_exp, *xsf_exp, *rq_exp, *rsf_exp;
 };
+bool route_small_fits(int T);
 bool front_small_fits(int T, int H, bool token_order);
 quads_status launch_route_small(const SmallRouteArgs& a, cudaStream_t st);
 quads_status launch_front_small(const SmallFrontArgs& a, cudaStream_t st);
@@ -216,6 +218,9 @@ struct Fp8GemmParams {
   const uint8_t* a_sf;   // activation scale atoms, [m_tiles, K/128, 512]
   const uint8_t* b_sf;   // weight scale atoms, [E, rows/128, K/128, 512]
   size_t b_sf_expert_stride;
+  const int32_t* row_token;    // few-rows first projection: token of a padded row, scale bytes in token order [T, K/128]
+  const uint8_t* xe_tok;
+  int tables_late;             // few rows: the preceding kernel wrote the routing tables
   uint16_t* y_pad;       // kEpiCombine: bf16 [padded rows, n_out]
   uint8_t* hq_pad;       // kEpiSwiGLU: E4M3 codes of h, [padded rows, n_out]
   uint8_t* hsf_atoms;    // kEpiSwiGLU: scale atoms of h, [m_tiles, n_out/128, 512]
@@ -226,12 +231,13 @@ struct Fp8GemmParams {
   const int32_t* offsets;
   int32_t* status;
 };
+quads_status launch_fp8_quantize_act(const uint16_t* x, int64_t rows, int K, uint8_t* codes, uint8_t* exps, int sm_count, cudaStream_t st);
 quads_status launch_fp8_front(const uint16_t* x, int64_t rows, int K, uint8_t* codes, uint8_t* exps, const RouteArgs& r, int sm_count,
                               cudaStream_t st);
 __global__ void fp8_quantize_weight_kernel(const uint16_t* w, int N, int K, uint8_t* codes, uint8_t* exps, uint8_t* atoms);
 __global__ void fp8_dispatch_kernel(int H, const int32_t* header, const int32_t* tile_rows, const int32_t* row_token,
                                     const uint8_t* xq, const uint8_t* xe, uint8_t* xq_pad, uint8_t* xsf_atoms);
-quads_status launch_gemm_fp8(int epi, const Fp8GemmParams& p, const CUtensorMap& tm_a, const CUtensorMap& tm_b, int n_sms,
+quads_status launch_gemm_fp8(int epi, bool few_rows, const Fp8GemmParams& p, const CUtensorMap& tm_a, const CUtensorMap& tm_b, int n_sms,
                              cudaStream_t stream);
 
 quads_status launch_gemm(int epi, int cta_group, const GemmParams& p, const GemmMaps& m, int n_sms,

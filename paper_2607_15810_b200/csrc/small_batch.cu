@@ -122,7 +122,7 @@ route_small_kernel(const SmallRouteArgs p) {
         cnt += c;
         if (w < rank * TW) base += c;
       }
-    tiles = (cnt + 127) / 128;
+    tiles = (cnt + p.slot_rows - 1) / p.slot_rows;
     inc_c = cnt; inc_t = tiles;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -144,7 +144,7 @@ route_small_kernel(const SmallRouteArgs p) {
         if (p.offsets_out) p.offsets_out[e] = off;
         for (int m = 0; m < tiles; ++m) {
           p.tile_expert[tp + m] = e;
-          p.tile_rows[tp + m] = min(128, cnt - m * 128);
+          p.tile_rows[tp + m] = min(p.slot_rows, cnt - m * p.slot_rows);
         }
         if (e == E - 1) {
           p.offsets[E] = off + cnt;
@@ -178,7 +178,7 @@ route_small_kernel(const SmallRouteArgs p) {
 #pragma unroll
     for (int b = 0; b < TW; ++b)
       if (b < a) r += __popc(words[rank * TW + b][e]);
-    const int row = s_off[e] + r, pos = s_tile[e] * 128 + r;
+    const int slot = r / p.slot_rows, row = s_off[e] + r, pos = (s_tile[e] + slot) * 128 + (r - slot * p.slot_rows);
     p.perm[row] = flat;
     if (p.perm_out) p.perm_out[row] = flat;
     p.pos_pad[flat] = pos;
@@ -457,9 +457,11 @@ quads_status launch_route_nj(const SmallRouteArgs& a, cudaStream_t st) {
 
 }  // namespace
 
+bool route_small_fits(int T) { return T <= 2 * kRouteTokens * front_cluster_limit(); }
+
 bool front_small_fits(int T, int H, bool token_order) {
   const int n = front_ctas(H), upc = (H / 128 + n - 1) / n;
-  return T <= 2 * kRouteTokens * front_cluster_limit() && upc <= kSmallMaxUnits && front_small_smem(T, H, n, token_order) <= (size_t)kFrontMaxSmem;
+  return route_small_fits(T) && upc <= kSmallMaxUnits && front_small_smem(T, H, n, token_order) <= (size_t)kFrontMaxSmem;
 }
 
 quads_status launch_route_small(const SmallRouteArgs& a, cudaStream_t st) {

@@ -85,6 +85,11 @@ def _layer(B, sh, full=True):
 FP8_SHAPES = [synth.MOE_SHAPES["tiny"], synth.MOE_SHAPES["small"],
               synth.MoEShape("one_token", 31, 1, 128, 256, 1, 128, 0.05, 1, 3.0, 10.0),
               synth.MoEShape("k_tail", 34, 70, 384, 4, 2, 128, 0.05, 2, 3.0, 10.0),
+              # few rows per expert (tiles of at most 32 rows): an expert with several such tiles and K tails; the same with
+              # more tokens than the small-batch routing takes
+              synth.MoEShape("few_rows", 36, 200, 640, 16, 2, 384, 0.05, 2, 3.0, 10.0, 1, 0.45),
+              synth.MoEShape("few_rows_many_tokens", 37, 700, 256, 64, 2, 128, 0.05, 2, 3.0, 10.0, 1, 0.2),
+              synth.MoEShape("few_rows_edge", 38, 128, 128, 8, 2, 256, 0.05, 1, 3.0, 10.0),
               synth.MoEShape("many_tiles", 35, 2100, 256, 4, 2, 384, 0.05, 1, 3.0, 10.0)]
 
 
