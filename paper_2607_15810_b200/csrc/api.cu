@@ -99,7 +99,7 @@ quads_status make_sf_map(CUtensorMap* map, const void* base, uint64_t atoms) {
   return r == CUDA_SUCCESS ? QUADS_OK : QUADS_ERR_CUDA;
 }
 
-// 2D map over a bf16 matrix [rows, K] (K contiguous): box 64 elements (128 bytes) x 128 rows,
+// 2D map over a bf16 matrix [rows, K] (K contiguous): box 64 elements (128 bytes) x kBf16BoxRows rows,
 // 128-byte swizzle, zero fill outside.
 quads_status make_bf16_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t K) {
   EncodeTiledFn fn = encode_fn();
@@ -107,7 +107,7 @@ quads_status make_bf16_map(CUtensorMap* map, const void* base, uint64_t rows, ui
   if (rows == 0) rows = 1;
   cuuint64_t dims[2] = {K, rows};
   cuuint64_t strides[1] = {K * 2};
-  cuuint32_t box[2] = {64, 128};
+  cuuint32_t box[2] = {64, (cuuint32_t)kBf16BoxRows};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -219,6 +219,16 @@ quads_status launch_select_mask(uint8_t* codes, int n_rows_fixed, uint32_t flip,
   QUADS_CUDA_OK(set_max_dynamic_smem<select_mask_kernel>(16384 * 12 + 16384 / 2));
   QUADS_CUDA_OK(launch_kernel(select_mask_kernel, dim3(sm_count), dim3(kSelectThreads), (size_t)C * 12 + C / 2, st, codes, n_rows_fixed,
                               flip, header, tile_rows, keys, C, n_sel, mask_out));
+  return QUADS_OK;
+}
+
+quads_status launch_dequantize(const uint8_t* q, const uint8_t* sf, const float* gs, int64_t n_tensors, int64_t nblk, int64_t K, int tiled,
+                               int64_t sf_stride, uint16_t* out, int32_t* zero, int sm_count, cudaStream_t st) {
+  // four blocks of 16 elements per thread, and no more CTAs than a few rounds of the chip
+  const int64_t per_tensor = std::min<int64_t>((nblk + 1023) / 1024, std::max<int64_t>(1, (int64_t)sm_count * 16 / n_tensors));
+  QUADS_CUDA_OK(launch_kernel(dequantize_kernel, dim3((unsigned)per_tensor, (unsigned)n_tensors), dim3(256), (size_t)0, st, q, sf, gs, nblk,
+                              (uint32_t)(K / 16), (int)((K + 63) / 64), tiled, sf_stride, out, zero));
+  QUADS_CUDA_OK(cudaGetLastError());
   return QUADS_OK;
 }
 
@@ -395,13 +405,8 @@ quads_status quads_dequantize_nvfp4(const uint8_t* q, const uint8_t* sf, const f
   if (s != QUADS_OK) return s;
   const int tiled = sf_layout == QUADS_SF_TILED;
   const int64_t sf_stride = tiled ? (int64_t)quads_sf_tiled_bytes(rows, K) : nblk;
-  const int64_t want = (nblk * n_tensors + 255) / 256;
-  const int grid = (int)std::min<int64_t>(want, (int64_t)di.sm_count * 16);
-  QUADS_CUDA_OK(launch_kernel(dequantize_kernel, dim3(grid), dim3(256), (size_t)0, static_cast<cudaStream_t>(cuda_stream),
-                              q, sf, gs, (int)n_tensors, nblk, (uint32_t)(K / 16), (int)((K + 63) / 64), tiled, sf_stride,
-                              static_cast<uint16_t*>(out)));
-  QUADS_CUDA_OK(cudaGetLastError());
-  return QUADS_OK;
+  return launch_dequantize(q, sf, gs, n_tensors, nblk, K, tiled, sf_stride, static_cast<uint16_t*>(out), nullptr, di.sm_count,
+                           static_cast<cudaStream_t>(cuda_stream));
 }
 
 quads_status quads_fake_quant_activations(const void* x, int64_t rows, int64_t K, int64_t ld, const float* gs_in,
@@ -667,7 +672,8 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   g_trace.n = 0;
   trace_mark("start", st);
   // header (status word included) and the amax word start at zero
-  if (!small) QUADS_CUDA_OK(cudaMemsetAsync(ws, 0, L.ids, st));
+  const bool decodes = a->operand_mode == QUADS_W4A16;      // its first kernel clears the status word, all that it needs
+  if (!small && !decodes) QUADS_CUDA_OK(cudaMemsetAsync(ws, 0, L.ids, st));
   trace_mark("memset", st);
 
   if (dense && a->operand_mode != QUADS_W4A4) {
@@ -676,10 +682,9 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
     uint16_t* dec = reinterpret_cast<uint16_t*>(P(L.dec));
     const void *A_op = a->x, *B_op = a->w13_bf16;
     if (a->operand_mode == QUADS_W4A16) {
-      const int64_t nblk = (int64_t)a->N * (H / 16);
-      const int grid = (int)std::min<int64_t>((nblk + 255) / 256, (int64_t)di.sm_count * 16);
-      QUADS_CUDA_OK(launch_kernel(dequantize_kernel, dim3(grid), dim3(256), (size_t)0, st, a->w13_q, a->w13_sf, a->w13_gs, 1,
-                                  nblk, (uint32_t)(H / 16), (int)(H / 64), 1, (int64_t)quads_sf_tiled_bytes(a->N, H), dec));
+      s = launch_dequantize(a->w13_q, a->w13_sf, a->w13_gs, 1, (int64_t)a->N * (H / 16), H, 1, (int64_t)quads_sf_tiled_bytes(a->N, H), dec,
+                            header + kHdrStatus, di.sm_count, st);
+      if (s != QUADS_OK) return s;
       B_op = dec;
     } else if (a->operand_mode == QUADS_W16A4) {
       // Q_A(x) then decode, in one pass of the quantizer (its scratch: the 256 bytes at the amax slot)

@@ -34,8 +34,8 @@ __global__ void fake_quant_ring_kernel(const uint16_t* x, int64_t nblk, int64_t 
                                        uint32_t* pair, int per, int lead, int split, uint8_t* q, uint8_t* sf, uint16_t* fq,
                                        float* gs_out, int sf_tiled, int64_t sf_tensor_stride, uint32_t k16,
                                        int kt_count);
-__global__ void dequantize_kernel(const uint8_t* q, const uint8_t* sf, const float* gs, int n_tensors, int64_t nblk,
-                                  uint32_t k16, int kt_count, int sf_tiled, int64_t sf_tensor_stride, uint16_t* out);
+__global__ void dequantize_kernel(const uint8_t* q, const uint8_t* sf, const float* gs, int64_t nblk, uint32_t k16,
+                                  int kt_count, int sf_tiled, int64_t sf_tensor_stride, uint16_t* out, int32_t* zero);
 __global__ void channel_stats_kernel(const uint16_t* x, int T, int H, const float* gs_in, const uint32_t* amax_bits,
                                      int rows_per_cta, float* partials);
 constexpr int kScoreSlices = 16;
@@ -200,8 +200,9 @@ struct GemmMaps {
 bool gemm_swapped_ok(int64_t assignments, int n_experts, int m_tiles_max);
 quads_status launch_gemm_swapped(int epi, const GemmParams& p, const GemmMaps& m, int n_sms, cudaStream_t stream);
 
-// ---- gemm_bf16.cu: out[T, N] = A[T, K] B[N, K]^T, bf16 operands (tensor maps with boxes of 64 x 128
-// elements, 128-byte swizzle), float32 accumulation, bf16 output; K % 64 == 0, N % 128 == 0
+// ---- gemm_bf16.cu: out[T, N] = A[T, K] B[N, K]^T, bf16 operands (tensor maps with boxes of 64 elements x kBf16BoxRows
+// rows, 128-byte swizzle), float32 accumulation, bf16 output; K % 64 == 0, N % 128 == 0
+constexpr int kBf16BoxRows = 64;
 quads_status launch_gemm_bf16(const CUtensorMap& tm_a, const CUtensorMap& tm_b, int T, int N, int K, uint16_t* out,
                               int32_t* status, int n_sms, cudaStream_t stream);
 
