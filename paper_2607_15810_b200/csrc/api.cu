@@ -852,21 +852,17 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   // ---- site 2: selection and masking of the residual of h
   const int nsel2 = a->rac_nsel_2;
   uint8_t* mask2 = P(L.mask2);
-  if (nsel2 > 0) {
-    // the scores are complete when the first projection ends (integer totals)
-    const bool want_mask = a->sel2 || a->hq || a->hsf || a->r2q || a->r2sf;
-    if ((s = launch_select_mask(P(L.r2q_pad), 0, 0u, header, tile_rows, g.keys2, I, nsel2, want_mask ? mask2 : nullptr, di.sm_count, st)) != QUADS_OK)
-      return s;
-    if (a->sel2) QUADS_CUDA_OK(launch_kernel(sel_list_kernel, dim3(1), dim3(1024), (size_t)0, st, mask2, I, a->sel2));
-  } else if (a->r2q) {
-    QUADS_CUDA_OK(cudaMemsetAsync(mask2, 0, I, st));
-  }
-  if (a->hq || a->hsf || a->r2q || a->r2sf) {
-    const int64_t n = (int64_t)A * (I / 16);
-    QUADS_CUDA_OK(launch_kernel(export_site2_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), (size_t)(0), st, A, header + kHdrAssignments, I, perm, pos_pad, P(L.hq_pad), P(L.hsf), P(L.r2q_pad), P(L.r2sf), mask2, a->hq, a->hsf, a->r2q, a->r2sf));
-  }
-
-  trace_mark("select2+mask", st);
+  const bool want_mask = a->sel2 || a->hq || a->hsf || a->r2q || a->r2sf;
+  // The scores are complete when the first projection ends (integer totals).  The operand-swapped second projection
+  // selects and masks for itself where the channels fit its shared memory; else a kernel does in between.  (Row-major
+  // tiles masked in shared memory by a warp of the second projection: 16 KB per stage and a three-stage ring put that
+  // on the critical path, 186 us at 8192 tokens against 107 and 23 for the kernel in between.)
+  const bool selects = nsel2 > 0 && swapped && I <= kSwappedSelectMax;
+  if (nsel2 > 0 && !selects &&
+      (s = launch_select_mask(P(L.r2q_pad), 0, 0u, header, tile_rows, g.keys2, I, nsel2, want_mask ? mask2 : nullptr, di.sm_count, st)) != QUADS_OK)
+    return s;
+  if (nsel2 == 0 && a->r2q) QUADS_CUDA_OK(cudaMemsetAsync(mask2, 0, I, st));
+  trace_mark("select2", st);
   // ---- second projection + weighted combine
   uint16_t* y_pad = reinterpret_cast<uint16_t*>(P(L.y_pad));
   GemmMaps m2;
@@ -891,6 +887,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   g2.n_tiles_n = swapped ? H / 128 : (H + 255) / 256;
   g2.half1_row_offset = 128;
   g2.y_pad = y_pad;
+  if (selects) { g2.sel_keys = g.keys2; g2.n_sel = nsel2; g2.mask_out = want_mask ? mask2 : nullptr; }
   if (timing) QUADS_CUDA_OK(cudaEventRecord(g_timers.ev[2], st));
   s = swapped ? launch_gemm_swapped(kEpiCombine, g2, m2, di.sm_count, st)
               : launch_gemm(kEpiCombine, cta_group, g2, m2, di.sm_count, st);
@@ -898,6 +895,12 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   if (timing) {
     QUADS_CUDA_OK(cudaEventRecord(g_timers.ev[3], st));
     g_timers.valid = true;
+  }
+  // verification exports of site 2
+  if (nsel2 > 0 && a->sel2) QUADS_CUDA_OK(launch_kernel(sel_list_kernel, dim3(1), dim3(1024), (size_t)0, st, mask2, I, a->sel2));
+  if (a->hq || a->hsf || a->r2q || a->r2sf) {
+    const int64_t n = (int64_t)A * (I / 16);
+    QUADS_CUDA_OK(launch_kernel(export_site2_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), (size_t)(0), st, A, header + kHdrAssignments, I, perm, pos_pad, P(L.hq_pad), P(L.hsf), P(L.r2q_pad), P(L.r2sf), mask2, a->hq, a->hsf, a->r2q, a->r2sf));
   }
   trace_mark("gemm2", st);
   const int64_t n8 = (int64_t)T * (H / 8);

@@ -44,6 +44,7 @@ __global__ void score_reduce_kernel(const float* partials, const int* n_part_ptr
                                     unsigned long long* score_keys);
 __global__ void sel_list_kernel(const uint8_t* mask, int C, int32_t* sel_export);
 __global__ void export_residual_kernel(int T, int H, const uint8_t* mask, uint32_t flip, const uint8_t* rq, uint8_t* rq_exp);
+constexpr int kSwappedSelectMax = 2048;   // channels the operand-swapped second projection can select among
 constexpr int kSelectThreads = 512;   // one CTA per SM: the CTAs of an SM would only repeat each other's search
 __global__ void select_mask_kernel(uint8_t* codes, int n_rows_fixed, uint32_t flip, const int32_t* header, const int32_t* tile_rows,
                                    const unsigned long long* score_keys, int C, int n_sel, uint8_t* mask_out /* or NULL */);
@@ -170,6 +171,11 @@ struct GemmParams {
   const uint8_t* rsf_tok;
   uint16_t* out_bf16;    // kEpiStore: [dense_rows, n_out]
   uint16_t* y_pad;       // kEpiCombine: bf16 [padded dispatch rows, n_out], one row per assignment
+  // kEpiCombine with a residual, operand-swapped: the kernel selects the n_sel of K channels with the largest totals
+  // and masks the residual rows it loads (sel_keys == NULL: they are masked already)
+  const unsigned long long* sel_keys;
+  int n_sel;
+  uint8_t* mask_out;     // export, may be NULL
   // epilogue: SwiGLU + requantize (site 2)
   const float* h_gs;     // per-tensor scale of h
   int resid2;            // 1: also emit the residual of h and its column statistics
