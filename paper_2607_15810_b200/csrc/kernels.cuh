@@ -45,7 +45,7 @@ __global__ void score_reduce_kernel(const float* partials, const int* n_part_ptr
 __global__ void sel_list_kernel(const uint8_t* mask, int C, int32_t* sel_export);
 __global__ void export_residual_kernel(int T, int H, const uint8_t* mask, uint32_t flip, const uint8_t* rq, uint8_t* rq_exp);
 constexpr int kSwappedSelectMax = 2048;   // channels the operand-swapped second projection can select among
-constexpr int kSelectThreads = 512;   // one CTA per SM: the CTAs of an SM would only repeat each other's search
+constexpr int kSelectThreads = 1024;   // one CTA per SM: the CTAs of an SM would only repeat each other's search
 __global__ void select_mask_kernel(uint8_t* codes, int n_rows_fixed, uint32_t flip, const int32_t* header, const int32_t* tile_rows,
                                    const unsigned long long* score_keys, int C, int n_sel, uint8_t* mask_out /* or NULL */);
 __global__ void combine_kernel(const uint16_t* y_pad, const int32_t* pos_pad, const float* wts, int T, int H,

@@ -821,9 +821,9 @@ export_residual_kernel(int T, int H, const uint8_t* __restrict__ mask, uint32_t 
 // A thread keeps its 16-byte column chunk and walks down the rows, eight of them in flight; the first
 // eight are fetched before the search, which hides their latency.  CTA 0 also exports the mask when asked
 // to.  Rows beyond a tile's valid ones are left alone: with few rows per expert they are most of the matrix.
-// Against a ranking kernel (C / 16 CTAs, one rank per key) and a mask kernel behind it: decode layer of
-// 256 tokens 126.3 -> 120.4 us, of one token 55.8 -> 52.5 us, prefill of 8192 unchanged (522.7 us).  With
-// eight CTAs of 256 threads per SM, each repeating the search, the same layers took 133.6 and 65.7 us.
+// Latency-bound: one CTA of 1024 threads per SM (8192 tokens, 25 MB of codes: 18 us in a loop; with 512 threads 26, a
+// ranking kernel and a mask kernel behind it took 19; eight CTAs of 256 threads per SM, each repeating the
+// search, cost a decode layer 7 us more than those two did).
 // With n_rows_fixed > 0 the matrix has that many rows, all valid (site 13 in token order, dense projections); `flip` is XORed
 // into every word of the result (the residual operand is stored negated).
 // dynamic shared memory: C keys of 8 bytes, C words of scratch, C / 8 mask words.
