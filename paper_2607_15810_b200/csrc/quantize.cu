@@ -155,11 +155,10 @@ __device__ __forceinline__ void emit_block(const QuantSink& o, const QuantCtx& q
   if (o.fq) {
     float d[16];
     dequant_block(bq, d);
-    uint4* dst = reinterpret_cast<uint4*>(o.fq + b * 16);
-    __stcs(dst, make_uint4(f32x2_to_bf16x2(d[0], d[1]), f32x2_to_bf16x2(d[2], d[3]),
-                           f32x2_to_bf16x2(d[4], d[5]), f32x2_to_bf16x2(d[6], d[7])));
-    __stcs(dst + 1, make_uint4(f32x2_to_bf16x2(d[8], d[9]), f32x2_to_bf16x2(d[10], d[11]),
-                               f32x2_to_bf16x2(d[12], d[13]), f32x2_to_bf16x2(d[14], d[15])));
+    uint32_t w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = f32x2_to_bf16x2(d[2 * i], d[2 * i + 1]);
+    stg256_stream(o.fq + b * 16, w);
   }
 }
 
