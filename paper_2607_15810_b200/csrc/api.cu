@@ -213,6 +213,12 @@ int gemm_cta_group_for(int64_t rows, int experts) {
   return rows >= (int64_t)1024 * (experts > 0 ? experts : 1) ? 2 : 1;
 }
 
+// Zeroes the first `bytes` (a multiple of 16) of a workspace.
+cudaError_t clear_words(uint8_t* p, size_t bytes, cudaStream_t st) {
+  const int n = (int)(bytes / 16);
+  return launch_kernel(clear_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), (size_t)0, st, reinterpret_cast<uint4*>(p), n);
+}
+
 // Selection and masking of a code matrix in one launch (see select_mask_kernel).
 quads_status launch_select_mask(uint8_t* codes, int n_rows_fixed, uint32_t flip, const int32_t* header, const int32_t* tile_rows,
                                 const unsigned long long* keys, int C, int n_sel, uint8_t* mask_out, int sm_count, cudaStream_t st) {
@@ -673,8 +679,8 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   trace_mark("start", st);
   // header (status word included) and the amax word start at zero
   const bool decodes = a->operand_mode == QUADS_W4A16;      // its first kernel clears the status word, all that it needs
-  if (!small && !decodes) QUADS_CUDA_OK(cudaMemsetAsync(ws, 0, L.ids, st));
-  trace_mark("memset", st);
+  if (!small && !decodes) QUADS_CUDA_OK(clear_words(ws, L.ids, st));
+  trace_mark("clear", st);
 
   if (dense && a->operand_mode != QUADS_W4A4) {
     // ---- one-sided modes: decode the NVFP4 side to bf16 with the library's own kernels, then one
@@ -1023,7 +1029,7 @@ quads_status quads_moe_fp8_w8a8(const quads_moe_fp8_args* a, void* cuda_stream) 
     if ((s = launch_route_small(r, st)) != QUADS_OK) return s;
     if ((s = launch_fp8_quantize_act(x, T, H, xq_tok, xe_tok, di.sm_count, st)) != QUADS_OK) return s;
   } else {
-    QUADS_CUDA_OK(cudaMemsetAsync(ws, 0, L.ids, st));          // header, status word, route counts
+    QUADS_CUDA_OK(clear_words(ws, L.ids, st));          // header, status word, route counts
     RouteArgs r{};
     r.logits = a->router_logits;
     r.T = T; r.E = E; r.topk = topk; r.renormalize = a->renormalize; r.e_lo = 0; r.e_hi = E;

@@ -42,6 +42,7 @@ constexpr int kScoreSlices = 16;
 __global__ void score_reduce_kernel(const float* partials, const int* n_part_ptr, int n_part_mul,
                                     int n_part_fixed, int C, double* slice_sums, unsigned int* counters,
                                     unsigned long long* score_keys);
+__global__ void clear_kernel(uint4* p, int n);
 __global__ void sel_list_kernel(const uint8_t* mask, int C, int32_t* sel_export);
 __global__ void export_residual_kernel(int T, int H, const uint8_t* mask, uint32_t flip, const uint8_t* rq, uint8_t* rq_exp);
 constexpr int kSwappedSelectMax = 2048;   // channels the operand-swapped second projection can select among
