@@ -213,6 +213,15 @@ int gemm_cta_group_for(int64_t rows, int experts) {
   return rows >= (int64_t)1024 * (experts > 0 ? experts : 1) ? 2 : 1;
 }
 
+// Blocks of at most 256 threads: a token's 16-byte columns along x, tokens along y where a row has fewer than 256.
+quads_status launch_combine(const uint16_t* y_pad, const int32_t* pos_pad, const float* wts, int T, int H, int topk, uint16_t* out,
+                            float* out_f32, cudaStream_t st) {
+  const int per_row = H / 8, bx = std::min(per_row, 256), by = 256 / bx;
+  QUADS_CUDA_OK(launch_kernel(combine_kernel, dim3((unsigned)((T + by - 1) / by), (unsigned)((per_row + bx - 1) / bx)),
+                              dim3((unsigned)bx, (unsigned)by), (size_t)0, st, y_pad, pos_pad, wts, T, H, topk, out, out_f32));
+  return QUADS_OK;
+}
+
 // Zeroes the first `bytes` (a multiple of 16) of a workspace.
 cudaError_t clear_words(uint8_t* p, size_t bytes, cudaStream_t st) {
   const int n = (int)(bytes / 16);
@@ -909,8 +918,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
     QUADS_CUDA_OK(launch_kernel(export_site2_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), (size_t)(0), st, A, header + kHdrAssignments, I, perm, pos_pad, P(L.hq_pad), P(L.hsf), P(L.r2q_pad), P(L.r2sf), mask2, a->hq, a->hsf, a->r2q, a->r2sf));
   }
   trace_mark("gemm2", st);
-  const int64_t n8 = (int64_t)T * (H / 8);
-  QUADS_CUDA_OK(launch_kernel(combine_kernel, dim3((unsigned)((n8 + 255) / 256)), dim3(256), (size_t)(0), st, y_pad, pos_pad, wts, T, H, topk, static_cast<uint16_t*>(a->out), a->out_f32));
+  if ((s = launch_combine(y_pad, pos_pad, wts, T, H, topk, static_cast<uint16_t*>(a->out), a->out_f32, st)) != QUADS_OK) return s;
   trace_mark("combine", st);
   QUADS_CUDA_OK(cudaGetLastError());
   return QUADS_OK;
@@ -1077,9 +1085,7 @@ quads_status quads_moe_fp8_w8a8(const quads_moe_fp8_args* a, void* cuda_stream) 
     QUADS_CUDA_OK(cudaEventRecord(g_timers.ev[3], st));
     g_timers.valid = true;
   }
-  const int64_t n8 = (int64_t)T * (H / 8);
-  QUADS_CUDA_OK(launch_kernel(combine_kernel, dim3((unsigned)((n8 + 255) / 256)), dim3(256), (size_t)0, st, g2.y_pad, pos_pad, wts,
-                              T, H, topk, static_cast<uint16_t*>(a->out), (float*)nullptr));
+  if ((s = launch_combine(g2.y_pad, pos_pad, wts, T, H, topk, static_cast<uint16_t*>(a->out), nullptr, st)) != QUADS_OK) return s;
   QUADS_CUDA_OK(cudaGetLastError());
   return QUADS_OK;
 }
