@@ -36,9 +36,14 @@
 //                      memory: the ring of weights fills meanwhile, where a selection kernel in between kept this
 //                      one from starting (layer of 256 tokens 95.8 -> 91.6 us, of one token 32.9 -> 29.4).
 //
-// Roles: warp 0 loads weights and their scales into a ring of stages, warp 10 the activation side, warp 1
-// issues the MMAs, warps 2..9 are the epilogue (thread = feature, 16 token columns each), warp 11 masks.  Two accumulator
-// buffers.  Only the activation side and the epilogue wait for the preceding kernel: the weights and the
+// Roles: warp 0 loads weights and their scales into a ring of stages, warp 10 the activation side, warps 1 and 12
+// issue the MMAs, warps 2..9 are the epilogue (thread = feature, 16 token columns each), warp 11 masks.  Two accumulator
+// buffers.  The MMAs are so small (N = 16 or 32) that issuing them was the bound: about 30 to 60 cycles per MMA or
+// scale copy and 300 around them, 930 cycles per stage of the second projection with one issuer, where DRAM
+// needs 710.  Two issuers share every stage and have an accumulator each: the gate and the up rows, or half the
+// K steps, which the epilogue adds (61 tokens 77.4 -> 74.8 us, 256 tokens 91.0 -> 89.0, one token 29.2 -> 28.6).
+// (Letting them take alternate tiles is no option: with more stages per tile than in the ring, a phase parity no
+// longer tells the fills of a slot apart.)  Only the activation side and the epilogue wait for the preceding kernel: the weights and the
 // routing tables are older, so the ring fills while that kernel still runs.  Every wait is
 // bounded (status word, as in gemm.cu).
 #include "kernels.cuh"
@@ -58,8 +63,10 @@ constexpr int kTileW = 128 * kStageKBytes;          // 128 weight rows of one st
 constexpr int kTileX = kChunk * kStageKBytes;       // one chunk of activation rows
 constexpr int kSfStage = kKSteps * 512;             // one 128-row scale atom per K step
 constexpr int kEpiWarps = 8;
-constexpr int kThreads = 64 + 32 * kEpiWarps + 64;
+constexpr int kThreads = 64 + 32 * kEpiWarps + 96;
 constexpr int kMaskWarp = 3 + kEpiWarps;            // second projection: masks the residual rows of a stage
+constexpr int kMmaWarps = 2;
+constexpr int kMma2Warp = 4 + kEpiWarps;           // the second MMA issuer
 constexpr int kActWarp = 2 + kEpiWarps;             // loads the activation / residual rows and their scales
 constexpr int kMaxChunkList = 2048;                 // (slot, chunk) entries, 2 bytes each
 constexpr int kMaxSlots = kMaxChunkList / 4;
@@ -162,10 +169,10 @@ gemm_swapped_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_x
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(bar_full + 8 * s, 2);               // both loading warps
-      mbar_init(bar_empty + 8 * s, 1);
+      mbar_init(bar_empty + 8 * s, kMmaWarps);
       mbar_init(bar_masked + 8 * s, 1);
     }
-    for (int b = 0; b < 2; ++b) { mbar_init(bar_tfull + 8 * b, 1); mbar_init(bar_tempty + 8 * b, kEpiWarps); }
+    for (int b = 0; b < 2; ++b) { mbar_init(bar_tfull + 8 * b, kMmaWarps); mbar_init(bar_tempty + 8 * b, kEpiWarps); }
     bars->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     prefetch_tmap(&tm_x);
@@ -355,8 +362,13 @@ gemm_swapped_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_x
         }
       }
     }
-  } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer
+  } else if (warp == 1 || warp == kMma2Warp) {
+    // ------------------------------------------------------------ MMA issuers, each with an accumulator and scale columns of
+    // its own: of the gate or the up rows, or (second projection) of K steps j0, j0 + 1 of every stage
+    const int half = warp == 1 ? 0 : 1;
+    constexpr int kSteps = kDual ? kKSteps : kKSteps / kMmaWarps;
+    const int j0 = kDual ? 0 : half * kSteps;
+    const uint32_t w_off = kDual ? half * kTileW : 0, sfw_off = C::kOffSfW + (kDual ? half * kSfStage : 0);
     const bool issuer = elect_one();
     uint32_t stage = 0, phase = 0, kcount = 0;
     int it = 0;
@@ -374,7 +386,7 @@ gemm_swapped_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_x
       // E2M1 x E2M1, UE4M3 block scales, both operands K-major, M = 128, N = n_mma
       const uint32_t idesc = (1u << 7) | (1u << 10) | ((uint32_t)(n_mma >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
       const int buf = it & 1;
-      const uint32_t acc = tmem + (uint32_t)(buf * 128);
+      const uint32_t acc = tmem + (uint32_t)(buf * 128 + half * 64);
       ok = mbar_wait(bar_tempty + 8 * buf, (uint32_t)((it >> 1) & 1) ^ 1u, abort_flag, p.status);
       if (!ok) break;
       tc_fence_after();
@@ -385,40 +397,34 @@ gemm_swapped_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_x
         tc_fence_after();
         const int atoms = min(kKSteps, kt_count - ks * kKSteps);
         const uint32_t sb = smem_base + stage * C::kStageBytes;
-        const uint32_t sfcol = tmem + kTmemSfBase + (kcount & 1u) * kTmemSfPerBuf;
-        const uint32_t w0_lo = ((sb & 0x3FFFFu) >> 4) | (1u << 16);
-        const uint32_t w1_lo = (((sb + kTileW) & 0x3FFFFu) >> 4) | (1u << 16);
+        const uint32_t sfcol = tmem + kTmemSfBase + (2 * half + (kcount & 1u)) * kTmemSfPerBuf;
+        const uint32_t w_lo = (((sb + w_off) & 0x3FFFFu) >> 4) | (1u << 16);
         const uint32_t x_lo = (((sb + C::kOffX - n_lead * kStageKBytes) & 0x3FFFFu) >> 4) | (1u << 16);
         const uint32_t r_lo = (((sb + C::kOffR - n_lead * kStageKBytes) & 0x3FFFFu) >> 4) | (1u << 16);
-        const uint32_t sfw_lo = ((sb + C::kOffSfW) & 0x3FFFFu) >> 4;
+        const uint32_t sfw_lo = ((sb + sfw_off) & 0x3FFFFu) >> 4;
         const uint32_t sfx_lo = ((sb + C::kOffSfX) & 0x3FFFFu) >> 4;
         const uint32_t sfr_lo = ((sb + C::kOffSfR) & 0x3FFFFu) >> 4;
         if (issuer) {
-          // scale columns of K step j: weights 0 at 4j, weights 1 at 16+4j, X at 32+4j, R at 48+4j
+          // scale columns of K step j: weights at 4j, X at 16+4j, R at 32+4j
           auto copy_sf = [&](int j) {
             tc_cp_sf<1>(sfcol + 4 * j, ((uint64_t)kSfHi << 32) | (sfw_lo + 32 * j));
-            if (kDual) tc_cp_sf<1>(sfcol + 16 + 4 * j, ((uint64_t)kSfHi << 32) | (sfw_lo + (kSfStage >> 4) + 32 * j));
-            tc_cp_sf<1>(sfcol + 32 + 4 * j, ((uint64_t)kSfHi << 32) | (sfx_lo + 32 * j));
-            if (resid) tc_cp_sf<1>(sfcol + 48 + 4 * j, ((uint64_t)kSfHi << 32) | (sfr_lo + 32 * j));
+            tc_cp_sf<1>(sfcol + 16 + 4 * j, ((uint64_t)kSfHi << 32) | (sfx_lo + 32 * j));
+            if (resid) tc_cp_sf<1>(sfcol + 32 + 4 * j, ((uint64_t)kSfHi << 32) | (sfr_lo + 32 * j));
           };
-          if (atoms > 0) copy_sf(0);
+          if (j0 < atoms) copy_sf(j0);
 #pragma unroll
-          for (int j = 0; j < kKSteps; ++j) {
-            if (j + 1 < atoms) copy_sf(j + 1);
+          for (int jj = 0; jj < kSteps; ++jj) {
+            const int j = j0 + jj;
+            if (jj + 1 < kSteps && j + 1 < atoms) copy_sf(j + 1);
             if (j < atoms) {
-              const uint32_t accum = (ks > 0 || j > 0) ? 1u : 0u;
+              const uint32_t accum = (ks > 0 || jj > 0) ? 1u : 0u;
               const uint64_t xdesc = ((uint64_t)kSw128Hi << 32) | (x_lo + 2 * j);
               const uint64_t rdesc = ((uint64_t)kSw128Hi << 32) | (r_lo + 2 * j);
-              const uint64_t w0desc = ((uint64_t)kSw128Hi << 32) | (w0_lo + 2 * j);
+              const uint64_t wdesc = ((uint64_t)kSw128Hi << 32) | (w_lo + 2 * j);
               // token scales: the even column at or before the chunk's own column of the slot's atom
-              const uint32_t sfx = sfcol + 32 + 4 * j + (uint32_t)(c & 2), sfr = sfcol + 48 + 4 * j + (uint32_t)(c & 2);
-              tc_mma_nvf4<1>(acc, w0desc, xdesc, idesc, sfcol + 4 * j, sfx, accum);
-              if (resid) tc_mma_nvf4<1>(acc, w0desc, rdesc, idesc, sfcol + 4 * j, sfr, 1u);
-              if (kDual) {
-                const uint64_t w1desc = ((uint64_t)kSw128Hi << 32) | (w1_lo + 2 * j);
-                tc_mma_nvf4<1>(acc + 64, w1desc, xdesc, idesc, sfcol + 16 + 4 * j, sfx, accum);
-                if (resid) tc_mma_nvf4<1>(acc + 64, w1desc, rdesc, idesc, sfcol + 16 + 4 * j, sfr, 1u);
-              }
+              const uint32_t sfx = sfcol + 16 + 4 * j + (uint32_t)(c & 2), sfr = sfcol + 32 + 4 * j + (uint32_t)(c & 2);
+              tc_mma_nvf4<1>(acc, wdesc, xdesc, idesc, sfcol + 4 * j, sfx, accum);
+              if (resid) tc_mma_nvf4<1>(acc, wdesc, rdesc, idesc, sfcol + 4 * j, sfr, 1u);
             }
           }
           tc_commit<1>(bar_empty + 8 * stage);
@@ -464,13 +470,17 @@ gemm_swapped_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_x
       tc_fence_after();
       float g[16], u[16];
       tmem_ld16(lane_addr + buf * 128 + col0 + th * 16, g);
-      if (kDual) tmem_ld16(lane_addr + buf * 128 + 64 + col0 + th * 16, u);
+      if (kDual || kt_count > kKSteps / kMmaWarps) tmem_ld16(lane_addr + buf * 128 + 64 + col0 + th * 16, u);
       tmem_ld_wait();
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_tempty + 8 * buf);
 
       if (!kDual) {
+        if (kt_count > kKSteps / kMmaWarps) {                // the other issuer's part
+#pragma unroll
+          for (int i = 0; i < 16; ++i) g[i] += u[i];
+        }
         // y rows for the combine kernel: thread = output feature, one 2-byte store per token
         const int n_out = p.n_out;
         const int f = ft * 128 + f_in_tile;
