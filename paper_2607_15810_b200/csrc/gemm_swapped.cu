@@ -36,7 +36,8 @@
 //                      memory: the ring of weights fills meanwhile, where a selection kernel in between kept this
 //                      one from starting (layer of 256 tokens 95.8 -> 91.6 us, of one token 32.9 -> 29.4).
 //
-// Roles: warp 0 loads weights and their scales into a ring of stages, warp 10 the activation side, warps 1 and 12
+// Roles: warp 0 loads weights and their scales into a ring of stages, warp 10 the activation side (first projection: warp 11
+// its residual), warps 1 and 12
 // issue the MMAs, warps 2..9 are the epilogue (thread = feature, 16 token columns each), warp 11 masks.  Two accumulator
 // buffers.  The MMAs are so small (N = 16 or 32) that issuing them was the bound: about 30 to 60 cycles per MMA or
 // scale copy and 300 around them, 930 cycles per stage of the second projection with one issuer, where DRAM
@@ -64,7 +65,7 @@ constexpr int kTileX = kChunk * kStageKBytes;       // one chunk of activation r
 constexpr int kSfStage = kKSteps * 512;             // one 128-row scale atom per K step
 constexpr int kEpiWarps = 8;
 constexpr int kThreads = 64 + 32 * kEpiWarps + 96;
-constexpr int kMaskWarp = 3 + kEpiWarps;            // second projection: masks the residual rows of a stage
+constexpr int kMaskWarp = 3 + kEpiWarps;            // second projection: masks the residual rows of a stage; first: loads them
 constexpr int kMmaWarps = 2;
 constexpr int kMma2Warp = 4 + kEpiWarps;           // the second MMA issuer
 constexpr int kActWarp = 2 + kEpiWarps;             // loads the activation / residual rows and their scales
@@ -168,7 +169,7 @@ gemm_swapped_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_x
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
-      mbar_init(bar_full + 8 * s, 2);               // both loading warps
+      mbar_init(bar_full + 8 * s, kDual && p.has_resid ? 3 : 2);               // the loading warps
       mbar_init(bar_empty + 8 * s, kMmaWarps);
       mbar_init(bar_masked + 8 * s, 1);
     }
@@ -269,8 +270,9 @@ gemm_swapped_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_x
       ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, p.status);
       if (++stage == kStages) { stage = 0; phase ^= 1u; }
     }
-  } else if (warp == kActWarp) {
-    // ------------------------------------------------------------ activation loader
+  } else if (warp == kActWarp || (kDual && resid && warp == kMaskWarp)) {
+    // ------------------------------------------------------------ activation loader (first projection: the second warp loads
+    // the residual)
     uint32_t stage = 0, phase = 0;
     bool ok = true;
     for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x) {
@@ -278,40 +280,34 @@ gemm_swapped_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_x
       const int mt = chunk_list[ch] >> 2, c = chunk_list[ch] & 3;
       const int n_rows = min(kChunk, (int)tab_rows[mt] - c * kChunk);
       if (kDual) {
-        // lane = row of the chunk (rows beyond the valid ones repeat the last); lanes 0..7 gather four rows of
-        // codes each, lanes 8..15 four rows of the residual
+        // lane = row of the chunk (rows beyond the valid ones repeat the last); lanes 0..7 gather four rows of codes each
+        // (every gather costs its warp about 33 ns, so with X and R in one warp 32 rows took 0.5 of a stage's 0.74 us: 256
+        // tokens 89.0 us, 87.2 with a warp each)
+        const bool rsd = warp != kActWarp;
         const int tok = p.row_token[mt * 128 + c * kChunk + min(lane, n_rows - 1)];
         const int g4 = (lane & 7) * 4;
         const int y0 = __shfl_sync(0xFFFFFFFFu, tok, g4), y1 = __shfl_sync(0xFFFFFFFFu, tok, g4 + 1);
         const int y2 = __shfl_sync(0xFFFFFFFFu, tok, g4 + 2), y3 = __shfl_sync(0xFFFFFFFFu, tok, g4 + 3);
-        const bool gathers = g4 < n_rows && (lane < 8 || (resid && lane < 16));
-        const CUtensorMap* map = lane < 8 ? &tm_x : &tm_r;
-        const uint32_t dst = (lane < 8 ? C::kOffX : C::kOffR) + (uint32_t)g4 * kStageKBytes;
-        const uint32_t bytes = (uint32_t)((n_rows + 3) / 4) * (4 * kStageKBytes) * (resid ? 2u : 1u);
-        const size_t so = (size_t)tok * (p.K >> 4);
-        uint4 vx = load_row_scales(p.xsf_tok + so, min(kKSteps, kt_count)), vr = make_uint4(0, 0, 0, 0);
-        if (resid) vr = load_row_scales(p.rsf_tok + so, min(kKSteps, kt_count));
+        const bool gathers = g4 < n_rows && lane < 8;
+        const CUtensorMap* map = rsd ? &tm_r : &tm_x;
+        const uint32_t dst = (rsd ? C::kOffR : C::kOffX) + (uint32_t)g4 * kStageKBytes, dst_sf = (rsd ? C::kOffSfR : C::kOffSfX) + lane * 16;
+        const uint32_t bytes = (uint32_t)((n_rows + 3) / 4) * (4 * kStageKBytes);
+        const uint8_t* sf = (rsd ? p.rsf_tok : p.xsf_tok) + (size_t)tok * (p.K >> 4);
+        uint4 v = load_row_scales(sf, min(kKSteps, kt_count));
         for (int ks = 0; ks < k_stages; ++ks) {
           ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, p.status);
           if (!ok) break;
           const int atoms = min(kKSteps, kt_count - ks * kKSteps);
           const uint32_t sb = smem_base + stage * C::kStageBytes, full = bar_full + 8 * stage;
           if (gathers) tma_gather4(sb + dst, map, ks * kStageKBytes, y0, y1, y2, y3, full);
-          const uint32_t ax = sb + C::kOffSfX + lane * 16, ar = sb + C::kOffSfR + lane * 16;
-          st_shared_u32(ax, vx.x); st_shared_u32(ax + 512, vx.y);
-          if (atoms > 2) { st_shared_u32(ax + 1024, vx.z); st_shared_u32(ax + 1536, vx.w); }
-          if (resid) {
-            st_shared_u32(ar, vr.x); st_shared_u32(ar + 512, vr.y);
-            if (atoms > 2) { st_shared_u32(ar + 1024, vr.z); st_shared_u32(ar + 1536, vr.w); }
-          }
+          const uint32_t a = sb + dst_sf;
+          st_shared_u32(a, v.x); st_shared_u32(a + 512, v.y);
+          if (atoms > 2) { st_shared_u32(a + 1024, v.z); st_shared_u32(a + 1536, v.w); }
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // the copies to tensor memory read these words
           __syncwarp();
           if (lane == 0) mbar_expect_tx(full, bytes);
-          if (ks + 1 < k_stages) {                     // the next stage's scales, a stage ahead of their use
-            const int na = min(kKSteps, kt_count - (ks + 1) * kKSteps);
-            vx = load_row_scales(p.xsf_tok + so + (ks + 1) * 16, na);
-            if (resid) vr = load_row_scales(p.rsf_tok + so + (ks + 1) * 16, na);
-          }
+          if (ks + 1 < k_stages)                       // the next stage's scales, a stage ahead of their use
+            v = load_row_scales(sf + (ks + 1) * 16, min(kKSteps, kt_count - (ks + 1) * kKSteps));
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
       } else {
