@@ -290,6 +290,7 @@ typedef struct {
 } quads_moe_args;
 
 quads_status quads_moe_w4a4_rac(const quads_moe_args* args /* host */, void* cuda_stream);
+/* never smaller for a larger T: a workspace of the largest batch serves the smaller ones */
 size_t quads_moe_workspace_bytes(int32_t T, int32_t H, int32_t I, int32_t E, int32_t topk,
                                  int32_t N);
 /* Reads (with a device-to-host copy and a stream synchronise) the status word
@@ -359,6 +360,7 @@ typedef struct {
   size_t workspace_bytes;        /* >= quads_moe_fp8_workspace_bytes(T, H, I, E, topk), 256-byte aligned */
 } quads_moe_fp8_args;
 quads_status quads_moe_fp8_w8a8(const quads_moe_fp8_args* args /* host */, void* cuda_stream);
+/* never smaller for a larger T: a workspace of the largest batch serves the smaller ones */
 size_t quads_moe_fp8_workspace_bytes(int32_t T, int32_t H, int32_t I, int32_t E, int32_t topk);
 
 /*

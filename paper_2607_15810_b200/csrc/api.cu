@@ -939,7 +939,8 @@ bool fp8_few_rows(int T, int E, int topk) { return (int64_t)T * topk <= (int64_t
 Fp8Layout fp8_layout(int T, int H, int I, int E, int topk) {
   Fp8Layout L{};
   const int64_t A = (int64_t)T * topk;
-  L.m_tiles_max = (int)(A / (fp8_few_rows(T, E, topk) ? 32 : 128)) + E;
+  const bool few = fp8_few_rows(T, E, topk);
+  L.m_tiles_max = (int)(A / (few ? 32 : 128)) + E;
   const size_t pad_rows = (size_t)L.m_tiles_max * 128;
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
@@ -956,8 +957,10 @@ Fp8Layout fp8_layout(int T, int H, int I, int E, int topk) {
   L.row_token = take(pad_rows * 4);
   L.xq_tok = take((size_t)T * H);
   L.xe_tok = take((size_t)T * (H / 128));
-  L.xq_pad = take(pad_rows * (size_t)H);
-  L.xsf = take((size_t)L.m_tiles_max * (H / 128) * 512);
+  if (!few) {                                             // (few rows: the first projection gathers out of token order)
+    L.xq_pad = take(pad_rows * (size_t)H);
+    L.xsf = take((size_t)L.m_tiles_max * (H / 128) * 512);
+  }
   L.hq_pad = take(pad_rows * (size_t)I);
   L.hsf = take((size_t)L.m_tiles_max * (I / 128) * 512);
   L.y_pad = take(pad_rows * (size_t)H * 2);
@@ -986,7 +989,10 @@ quads_status quads_fp8_quantize_weights(const void* w, int64_t n_tensors, int64_
 
 size_t quads_moe_fp8_workspace_bytes(int32_t T, int32_t H, int32_t I, int32_t E, int32_t topk) {
   if (T < 0 || H <= 0 || I <= 0 || E < 1 || topk < 1) return 0;
-  return fp8_layout(T, H, I, E, topk).total;
+  // Few rows per expert take up to four times the tiles per assignment, so the largest batch of that form can need more
+  // than a larger one of the other: what is returned for T is enough for every smaller batch as well.
+  const int t_few = (int)std::min<int64_t>(T, (int64_t)E * 32 / topk);
+  return std::max(fp8_layout(T, H, I, E, topk).total, fp8_layout(t_few, H, I, E, topk).total);
 }
 
 

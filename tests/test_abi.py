@@ -60,3 +60,15 @@ def test_argument_errors_come_back_before_any_launch(lib):
     g.restype = C.c_int32
     g.argtypes = [C.c_void_p, C.c_void_p]
     assert g(None, None) == -1
+
+
+@pytest.mark.parametrize("E,topk,H,I", [(128, 8, 2048, 768), (8, 2, 256, 128), (5, 5, 384, 256), (256, 16, 128, 128), (3, 2, 128, 640)])
+def test_workspace_of_a_larger_batch_serves_smaller_ones(lib, E, topk, H, I):
+    """The forms a batch size selects (few rows per expert, CTA pairs) must not make a workspace shrink as T grows."""
+    fp8, moe = lib.quads_moe_fp8_workspace_bytes, lib.quads_moe_workspace_bytes
+    fp8.restype = moe.restype = C.c_size_t
+    fp8.argtypes, moe.argtypes = [C.c_int32] * 5, [C.c_int32] * 6
+    edge = 32 * E // topk
+    for sizes in ([fp8(T, H, I, E, topk) for T in range(0, 5 * edge)], [moe(T, H, I, E, topk, 0) for T in range(0, 5 * edge)],
+                  [moe(T, H, 0, 1, 1, I) for T in range(0, 1500)]):
+        assert all(a <= b for a, b in zip(sizes, sizes[1:]))

@@ -191,3 +191,19 @@ def test_fp8_prefill_layer_at_full_size_sampled(B):
             n_out += 128
     print("fp8 prefill: rows %d, h err/tol %.3f, out values %d err/tol %.3f" % (len(rows), worst_h, n_out, worst_o))
     assert worst_h <= 1.0 and worst_o <= 1.0 and n_out >= 64 * 128
+
+
+@pytest.mark.parametrize("big", [129, 300, 520])
+def test_workspace_of_a_larger_batch_serves_smaller_ones(B, big):
+    """8 experts, top 2: batches up to 128 tokens run the few-rows form, whose tiles take more room per token."""
+    sh = synth.MoEShape("ws", 39, 129, 256, 8, 2, 128, 0.05, 2, 3.0, 10.0)
+    x, _ = synth.activations(sh)
+    x, lg = x.cuda(), synth.router_logits(sh).cuda()
+    g13 = B.fp8_quantize_weights(synth.expert_weights(sh, "w13").cuda())
+    g2 = B.fp8_quantize_weights(synth.expert_weights(sh, "w2").cuda())
+    ws = torch.full((B.moe_fp8_workspace_bytes(big, sh.H, sh.I, sh.E, sh.topk),), 0xFF, dtype=torch.uint8, device="cuda")
+    for T in (129, 128, 127, 33, 1):
+        got = B.moe_fp8_w8a8(x[:T].contiguous(), lg[:T].contiguous(), g13, g2, sh.topk, workspace=ws)
+        assert B.moe_async_status(ws) == 0
+        want = B.moe_fp8_w8a8(x[:T].contiguous(), lg[:T].contiguous(), g13, g2, sh.topk)
+        assert torch.equal(got["out"], want["out"])
