@@ -119,7 +119,7 @@ inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_
 
 // ------------------------------------------------------------------ workspace
 struct MoeLayout {
-  size_t header, amax, keys13, keys2, ids, wts, route_counts, offsets, tile_prefix, tile_expert, tile_rows;
+  size_t header, amax, col_arrivals, keys2, keys13, partials13, ids, wts, route_counts, offsets, tile_prefix, tile_expert, tile_rows;
   size_t perm, pos_pad, row_token;
   size_t mask13, xq_tok, xsf_tok, rq_tok, rsf_tok, xq_pad, xsf, rq_pad, rsf;
   size_t hq_pad, hsf, r2q_pad, r2sf, mask2, y_pad, dec;
@@ -138,10 +138,12 @@ MoeLayout moe_layout(int T, int H, int I, int E, int topk, int N) {
   auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
   L.header = take(kHdrWords * 4);
   L.amax = take((size_t)kAmaxPartsMax * 4);    // the amax word; also the quantizer's scratch in the one-sided modes
-  L.keys13 = take((size_t)H * 8);                  // integer column scores of site 13, zeroed with the header
+  L.col_arrivals = take((size_t)kQuantColsMax * 4);   // zeroed with the header
   L.keys2 = take((size_t)I * 8);                   // zeroed with the header: the first projection's epilogue adds to it
   L.route_counts = take(dense ? 0 : (size_t)kRouteCtasMax * Ee * 4);   // zeroed with the header
   L.ids = take((size_t)A * 4);
+  L.keys13 = take((size_t)H * 8);                  // column scores of site 13, and the partial ones of row ranges
+  L.partials13 = take(quant_partial_floats(T, H) * 4);
   L.wts = take((size_t)A * 4);
   L.offsets = take((size_t)(Ee + 1) * 4);
   L.tile_prefix = take((size_t)(Ee + 1) * 4);
@@ -229,10 +231,11 @@ cudaError_t clear_words(uint8_t* p, size_t bytes, cudaStream_t st) {
 }
 
 // Selection and masking of a code matrix in one launch (see select_mask_kernel).
+template <bool kDoubleKeys>
 quads_status launch_select_mask(uint8_t* codes, int n_rows_fixed, uint32_t flip, const int32_t* header, const int32_t* tile_rows,
                                 const unsigned long long* keys, int C, int n_sel, uint8_t* mask_out, int sm_count, cudaStream_t st) {
-  QUADS_CUDA_OK(set_max_dynamic_smem<select_mask_kernel>(16384 * 12 + 16384 / 2));
-  QUADS_CUDA_OK(launch_kernel(select_mask_kernel, dim3(sm_count), dim3(kSelectThreads), (size_t)C * 12 + C / 2, st, codes, n_rows_fixed,
+  QUADS_CUDA_OK(set_max_dynamic_smem<select_mask_kernel<kDoubleKeys>>(16384 * 12 + 16384 / 2));
+  QUADS_CUDA_OK(launch_kernel(select_mask_kernel<kDoubleKeys>, dim3(sm_count), dim3(kSelectThreads), (size_t)C * 12 + C / 2, st, codes, n_rows_fixed,
                               flip, header, tile_rows, keys, C, n_sel, mask_out));
   return QUADS_OK;
 }
@@ -761,7 +764,8 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
     q.xq = P(dense ? L.xq_pad : L.xq_tok); q.xsf = P(dense ? L.xsf : L.xsf_tok);
     q.rq = P(dense ? L.rq_pad : L.rq_tok); q.rsf = P(dense ? L.rsf : L.rsf_tok);
     q.xq_exp = a->xq; q.xsf_exp = a->xsf; q.rsf_exp = a->rsf;
-    q.totals = keys13;
+    q.partials = reinterpret_cast<float*>(P(L.partials13)); q.keys = keys13;
+    q.col_arrivals = reinterpret_cast<unsigned int*>(P(L.col_arrivals));
     if (dense) {
       s = launch_quant_rows(q, di.sm_count, st);
     } else {
@@ -787,7 +791,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
       d.xq_pad = P(L.xq_pad); d.xsf_tiled = P(L.xsf); d.rq_pad = P(L.rq_pad); d.rsf_tiled = P(L.rsf);
       if ((s = launch_dispatch(d, L.m_tiles_max, di.sm_count, st)) != QUADS_OK) return s;
     } else if (nsel13 > 0) {
-      s = launch_select_mask(q.rq, T, 0x88888888u, header, tile_rows, keys13, H, nsel13, (a->sel13 || a->rq) ? mask13 : nullptr,
+      s = launch_select_mask<true>(q.rq, T, 0x88888888u, header, tile_rows, keys13, H, nsel13, (a->sel13 || a->rq) ? mask13 : nullptr,
                              di.sm_count, st);
       if (s != QUADS_OK) return s;
     }
@@ -874,7 +878,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   // on the critical path, 186 us at 8192 tokens against 107 and 23 for the kernel in between.)
   const bool selects = nsel2 > 0 && swapped && I <= kSwappedSelectMax;
   if (nsel2 > 0 && !selects &&
-      (s = launch_select_mask(P(L.r2q_pad), 0, 0u, header, tile_rows, g.keys2, I, nsel2, want_mask ? mask2 : nullptr, di.sm_count, st)) != QUADS_OK)
+      (s = launch_select_mask<false>(P(L.r2q_pad), 0, 0u, header, tile_rows, g.keys2, I, nsel2, want_mask ? mask2 : nullptr, di.sm_count, st)) != QUADS_OK)
     return s;
   if (nsel2 == 0 && a->r2q) QUADS_CUDA_OK(cudaMemsetAsync(mask2, 0, I, st));
   trace_mark("select2", st);

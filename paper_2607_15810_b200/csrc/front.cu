@@ -16,24 +16,52 @@ namespace quads {
 // quantization with the same per-tensor scale (the mask of Eq. residual-recon is
 // applied later: quantizing the residual does not depend on the selection).
 //
-// A CTA owns bw blocks of 16 channels (8, 16 or 32, whatever divides the row) for a range of rows;
+// A CTA owns bw blocks of 16 channels (8, 16 or 32, see plan_quant) for a range of rows;
 // thread = (block, row lane).  The grid is what is resident at once, so that the amax of x can be the
 // first phase of the same launch: the CTAs meet at a counter (bounded wait) and read their rows again, out of L2.
-// A CTA adds its row lanes' column sums up in shared memory and adds one 64-bit integer per channel to the
-// channel's total, which is complete when the kernel ends: with CTAs that own whole rows, four times as
-// many reductions arrive together (20 us at 8192 x 2048), and partial rows need a kernel to add them up.
+// A CTA adds its row lanes' column sums up in shared memory and leaves one float32 per channel; the last CTA of a
+// column group to finish adds the row ranges up in float64, in their order, so that the scores keep their
+// relative precision whatever the range of x and its scale, and do not depend on who finishes when.  Fixed-point
+// totals, one reduction per CTA and channel, cost 1 to 2 us less (dense 8192 x 4096 -> 4096 157.4 us, 158.6 so; 1200 x
+// 512 -> 128 18.5, 20.5; a MoE layer of 1500 tokens the same), but need a bound on the residual, which a given
+// scale that x exceeds does not have, and lose channels that are small beside an outlier.
 // Issue-bound: about 400 issue cycles per warp and block, 128 of them in the two conversions to E2M1.
 // Dense projection 8192 x 4096 -> 4096: amax, quantization, score reduction, ranking and copy took 16 + 27 + 12 +
-// 12 + 28 us as kernels of their own; this one takes 39.8 and the in-place mask behind it 10 (whole call
-// 205 -> 165 us).
+// 12 + 28 us as kernels of their own; this one takes about 40 and the in-place mask behind it 10 (whole call
+// 205 -> 159 us).
 // Scales are stored linear [T, H/16], or tiled when the rows are a dense projection's operand as they are.
 // ---------------------------------------------------------------------------
 struct QuantShared {
   float gs;
+  int last;
   uint32_t wmax[8];
   float inv_lut[128];
   __align__(16) float red[256 * 16];
 };
+
+// Adds up the partial scores of a column group (n_ch = 128, 256 or 512 channels, `part` its first one's, rows of H), one
+// row per row range.  Thread = (four channels, every n-th row); latency-bound, eight loads in flight.
+__device__ __forceinline__ void sum_partial_scores(const float* part, int n_rg, int H, int n_ch, unsigned long long* keys, double* red) {
+  const int quads = n_ch >> 2, q = threadIdx.x % quads, sl = threadIdx.x / quads, n_sl = 256 / quads;
+  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+  for (int r = sl; r < n_rg; r += 8 * n_sl) {
+    float4 v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      v[u] = r + u * n_sl < n_rg ? __ldcg(reinterpret_cast<const float4*>(part + (size_t)(r + u * n_sl) * H) + q)
+                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) { a0 += (double)v[u].x; a1 += (double)v[u].y; a2 += (double)v[u].z; a3 += (double)v[u].w; }
+  }
+  double* d = red + sl * n_ch + 4 * q;
+  d[0] = a0; d[1] = a1; d[2] = a2; d[3] = a3;
+  __syncthreads();
+  for (int c = threadIdx.x; c < n_ch; c += 256) {
+    double t = 0.0;
+    for (int l = 0; l < n_sl; ++l) t += red[l * n_ch + c];
+    keys[c] = (unsigned long long)__double_as_longlong(t);   // order-preserving: t >= 0
+  }
+}
 
 // CTA `cta` of `n_cta`.
 __device__ __forceinline__ void quant_role(const QuantRowsArgs& p, int cta, int n_cta, QuantShared* s) {
@@ -114,18 +142,26 @@ __device__ __forceinline__ void quant_role(const QuantRowsArgs& p, int cta, int 
     }
   }
   if (!p.with_residual) return;
-  {
-    float4* d = reinterpret_cast<float4*>(s->red + threadIdx.x * 16);
+  // column sums: the CTA's row lanes, then (by the last CTA) the row ranges
+  const int n_ch = p.bw * 16, n_rg = n_cta / p.n_col;        // channels of this CTA, row ranges
+  float4* d = reinterpret_cast<float4*>(s->red + threadIdx.x * 16);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) d[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
-    __syncthreads();
-    const int n_ch = p.bw * 16;                              // channels of this CTA, at most 512
-    for (int c = threadIdx.x; c < n_ch; c += 256) {
-      float t = 0.f;
-      for (int l = 0; l < lanes; ++l) t += s->red[l * n_ch + c];
-      add_score(p.totals + col * n_ch + c, t, gs, p.score_bits, p.cap_bits);
-    }
+  for (int i = 0; i < 4; ++i) d[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
+  __syncthreads();
+  for (int c = threadIdx.x; c < n_ch; c += 256) {
+    double t = 0.0;
+#pragma unroll 8
+    for (int l = 0; l < lanes; ++l) t += (double)s->red[l * n_ch + c];
+    p.partials[(size_t)rg * H + col * n_ch + c] = (float)t;
   }
+  __syncthreads();
+  if (threadIdx.x == 0) {                                    // (releases what the barrier ordered before it)
+    uint32_t before;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(before) : "l"(p.col_arrivals + col) : "memory");
+    s->last = before == (uint32_t)n_rg - 1u;
+  }
+  __syncthreads();
+  if (s->last) sum_partial_scores(p.partials + col * n_ch, n_rg, H, n_ch, p.keys + col * n_ch, reinterpret_cast<double*>(s->red));
 }
 
 // Asks L2 for the rows of quant_role's CTA.
@@ -293,21 +329,23 @@ cudaError_t resident_per_sm(K kernel, int threads, std::atomic<int>* cache, int*
   return cudaSuccess;
 }
 
-// Row ranges of the quantization role on at most `ctas` CTAs; returns the CTAs used.
+// Column groups and row ranges of the quantization role on at most `ctas` CTAs; returns the CTAs used.  Of the widths
+// that divide a row the one with the least time: rounds of 256 blocks per CTA (some 2 us each with four CTAs per
+// SM), and batches of partial scores that a group's last CTA adds up (some 0.4 us each).
 int plan_quant(QuantRowsArgs* q, int ctas) {
-  q->bw = (q->H / 16) % 32 == 0 ? 32 : ((q->H / 16) % 16 == 0 ? 16 : 8);
-  q->n_col = q->H / 16 / q->bw;
-  const int lanes = 256 / q->bw;                    // each range at least a row per row lane
-  const int n_rg = std::max(1, std::min(ctas / q->n_col, (q->T + lanes - 1) / lanes));
-  q->rows_per_cta = ((q->T + n_rg - 1) / n_rg + lanes - 1) / lanes * lanes;
-  const int n_used = (q->T + q->rows_per_cta - 1) / q->rows_per_cta;
-  // a CTA's column sum covers rows_per_cta rows (< rows * 2^18 in units of the squared scale); the sums of
-  // all row ranges must fit 62 bits together
-  int cap_bits = 18, ranges_log2 = 0;
-  while ((1 << (cap_bits - 18)) < q->rows_per_cta) ++cap_bits;
-  while ((1 << ranges_log2) < n_used) ++ranges_log2;
-  q->cap_bits = cap_bits;
-  q->score_bits = std::max(0, std::min(26, 62 - cap_bits - ranges_log2));
+  const int blocks = q->H / 16;
+  ctas = std::min(ctas, kQuantCtasMax);
+  int best = 0, n_used = 1;
+  for (int bw = 8; bw <= 32 && blocks % bw == 0; bw *= 2) {
+    const int n_col = blocks / bw, lanes = 256 / bw;  // each range at least a row per row lane
+    const int n_rg = std::max(1, std::min(ctas / n_col, (q->T + lanes - 1) / lanes));
+    const int rounds = ((q->T + n_rg - 1) / n_rg + lanes - 1) / lanes, rows = rounds * lanes, used = (q->T + rows - 1) / rows;
+    const int cost = 5 * rounds + (used * bw + 511) / 512;
+    if (bw > 8 && cost >= best) continue;
+    best = cost;
+    q->bw = bw; q->n_col = n_col; q->rows_per_cta = rows;
+    n_used = used;
+  }
   return n_used * q->n_col;
 }
 

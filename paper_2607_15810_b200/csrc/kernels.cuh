@@ -2,6 +2,8 @@
 #pragma once
 #include <cuda.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace quads {
@@ -47,6 +49,7 @@ __global__ void sel_list_kernel(const uint8_t* mask, int C, int32_t* sel_export)
 __global__ void export_residual_kernel(int T, int H, const uint8_t* mask, uint32_t flip, const uint8_t* rq, uint8_t* rq_exp);
 constexpr int kSwappedSelectMax = 2048;   // channels the operand-swapped second projection can select among
 constexpr int kSelectThreads = 1024;   // one CTA per SM: the CTAs of an SM would only repeat each other's search
+template <bool kDoubleKeys>            // site 13: float64 scores; site 2: integer totals
 __global__ void select_mask_kernel(uint8_t* codes, int n_rows_fixed, uint32_t flip, const int32_t* header, const int32_t* tile_rows,
                                    const unsigned long long* score_keys, int C, int n_sel, uint8_t* mask_out /* or NULL */);
 __global__ void combine_kernel(const uint16_t* y_pad, const int32_t* pos_pad, const float* wts, int T, int H,
@@ -71,9 +74,14 @@ struct QuantRowsArgs {
   float* gs_store;                    // exports, each may be NULL
   uint8_t *xq, *xsf, *rq, *rsf;
   uint8_t *xq_exp, *xsf_exp, *rsf_exp;
-  unsigned long long* totals;         // [H] integer channel scores, zero on entry
-  int bw, n_col, rows_per_cta, score_bits, cap_bits;   // filled in at launch
+  float* partials;                    // [quant_partial_floats(T, H)] scratch of the channel scores
+  unsigned int* col_arrivals;         // [kQuantColsMax] zero on entry
+  unsigned long long* keys;           // [H] out: channel scores, bit patterns of non-negative float64 values
+  int bw, n_col, rows_per_cta;        // filled in at launch
 };
+constexpr int kQuantCtasMax = 1024;   // CTAs of the quantization role, each with at most 512 channels of a row range ...
+constexpr int kQuantColsMax = 128;    // ... in so many column groups (H <= 16384), of at least eight rows but the last
+inline size_t quant_partial_floats(int T, int H) { return std::min<size_t>((size_t)kQuantCtasMax * 512, ((size_t)T + 7) / 8 * H); }
 // Top-k routing and dispatch order (routing.cuh).
 constexpr int kRouteCtasMax = 256;
 struct RouteArgs {
@@ -95,7 +103,7 @@ quads_status launch_quant_rows(const QuantRowsArgs& q, int sm_count, cudaStream_
 constexpr int kDispatchThreads = 512, kDispatchPerSm = 3;
 struct DispatchArgs {
   int H, n_sel;                       // n_sel == 0: no residual
-  const unsigned long long* keys;     // [H] channel scores
+  const unsigned long long* keys;     // [H] channel scores (QuantRowsArgs::keys)
   uint8_t* mask;                      // [H] out: 1 for the selected channels
   const int32_t *header, *tile_rows, *row_token;
   const uint8_t *xq, *xsf, *rq, *rsf; // token order, linear scales

@@ -824,7 +824,7 @@ export_residual_kernel(int T, int H, const uint8_t* __restrict__ mask, uint32_t 
 }
 
 // Site-2 selection and masking in one launch: every CTA finds the selection's threshold for itself (C
-// integer totals, 8 C bytes out of L2), turns it into nibble masks in shared memory and clears, in place,
+// scores, 8 C bytes out of L2), turns it into nibble masks in shared memory and clears, in place,
 // the codes of unselected channels in its share of the valid rows of the padded [rows, C/2] code matrix.
 // A thread keeps its 16-byte column chunk and walks down the rows, eight of them in flight; the first
 // eight are fetched before the search, which hides their latency.  CTA 0 also exports the mask when asked
@@ -832,9 +832,11 @@ export_residual_kernel(int T, int H, const uint8_t* __restrict__ mask, uint32_t 
 // Latency-bound: one CTA of 1024 threads per SM (8192 tokens, 25 MB of codes: 18 us in a loop; with 512 threads 26, a
 // ranking kernel and a mask kernel behind it took 19; eight CTAs of 256 threads per SM, each repeating the
 // search, cost a decode layer 7 us more than those two did).
-// With n_rows_fixed > 0 the matrix has that many rows, all valid (site 13 in token order, dense projections); `flip` is XORed
+// The scores are integer totals (site 2) or float64 bit patterns (site 13).  With n_rows_fixed > 0 the matrix has that many
+// rows, all valid (site 13 in token order, dense projections); `flip` is XORed
 // into every word of the result (the residual operand is stored negated).
 // dynamic shared memory: C keys of 8 bytes, C words of scratch, C / 8 mask words.
+template <bool kDoubleKeys>
 __global__ void __launch_bounds__(kSelectThreads)
 select_mask_kernel(uint8_t* __restrict__ codes, int n_rows_fixed, uint32_t flip, const int32_t* __restrict__ header,
                    const int32_t* __restrict__ tile_rows,
@@ -868,7 +870,7 @@ select_mask_kernel(uint8_t* __restrict__ codes, int n_rows_fixed, uint32_t flip,
   const int c_first = threadIdx.x % cols;
   fetch(c_first, first);
   __syncthreads();
-  const Selection sel = select_largest<false>(sc, images, C, n_sel, &scratch);
+  const Selection sel = select_largest<kDoubleKeys>(sc, images, C, n_sel, &scratch);
   for (int w = threadIdx.x; w < (C >> 3); w += kSelectThreads) {
     uint32_t m = 0;
 #pragma unroll
@@ -893,6 +895,11 @@ select_mask_kernel(uint8_t* __restrict__ codes, int n_rows_fixed, uint32_t flip,
     }
   }
 }
+
+template __global__ void select_mask_kernel<false>(uint8_t*, int, uint32_t, const int32_t*, const int32_t*, const unsigned long long*, int,
+                                                   int, uint8_t*);
+template __global__ void select_mask_kernel<true>(uint8_t*, int, uint32_t, const int32_t*, const int32_t*, const unsigned long long*, int,
+                                                  int, uint8_t*);
 
 // Weighted top-k combine: out[t, :] = sum over the token's slots, in slot order,
 // of weight * y[row of (t, slot), :], accumulated in float32, rounded to bf16.

@@ -7,6 +7,7 @@ import torch
 import moe_check as MC
 from oracle import moe as M
 from oracle import nvfp4 as Q
+from oracle import rac as R
 from paper_2607_15810_b200 import synth
 
 pytestmark = pytest.mark.gpu
@@ -67,3 +68,57 @@ def test_site2_mask_applied_inside_the_second_projection(B, T, I, E, nsel2):
     MC.check_moe(res, x, lg, w13o, w2o, 1, 64, nsel2, a2)
     plain = B.moe_w4a4_rac(*args)
     assert torch.equal(plain["out"], res["out"])
+
+
+def _separated_channels(T, H, lo, hi, seed):
+    """Channel c has one magnitude in every row, rising with c from lo to hi, and random signs: the scores of two
+    channels differ by far more than any order of float32 additions can change."""
+    g = torch.Generator().manual_seed(seed)
+    mag = lo + (hi - lo) * torch.arange(H, dtype=torch.float32) / H
+    return (mag * (torch.randint(0, 2, (T, H), generator=g) * 2 - 1)).to(torch.bfloat16)
+
+
+# a given scale that every channel exceeds by 1.5 to 3 times (all clip), and one outlier beside which the others vanish
+SCORE_RANGES = {"clipped": (4096.0, 8192.0, 1.0), "beside_an_outlier": (1e-5, 2e-5, None)}
+
+
+@pytest.mark.parametrize("kind", sorted(SCORE_RANGES))
+@pytest.mark.parametrize("T,K,nsel", [
+    (513, 512, 33), (600, 256, 100), (1111, 640, 300), (40, 512, 33),
+    (772, 3072, 900), (513, 4608, 700)])       # column groups of 256 and 512 channels
+def test_site13_scores_keep_their_order_dense(B, kind, T, K, nsel):
+    lo, hi, gs = SCORE_RANGES[kind]
+    x = _separated_channels(T, K, lo, hi, T)
+    if gs is None:
+        x[:, 0] = 1e4
+    _, w = synth.dense_inputs(T, T=8, K=K, N=128)
+    wq = B.fake_quant_weights(w.unsqueeze(0).cuda(), want_fq=False, sf_layout=B.SF_TILED)
+    res = B.dense_w4a4_rac(x.cuda(), wq, nsel, a_gs=None if gs is None else torch.tensor([gs], device="cuda"), export=True)
+    torch.cuda.synchronize()
+    assert B.moe_async_status(res["workspace"]) == 0
+    wo = MC.oracle_weights(w[None])
+    o = M.dense_w4a4_rac(MC.f32(x), wo["codes"][0], wo["sf"][0], wo["gs"][0], nsel, a_gs=None if gs is None else np.float32(gs))
+    MC.check_site1(res, dict(site13=o["site"]), nsel, {})
+
+
+@pytest.mark.parametrize("kind", sorted(SCORE_RANGES))
+@pytest.mark.parametrize("T,H,E,topk,nsel", [
+    (600, 256, 8, 2, 60),        # dispatched copies
+    (520, 640, 256, 8, 200),     # operand-swapped projections: masked in token order
+    (1771, 1024, 8, 2, 300),     # column groups of 256 channels, 111 row ranges
+    (994, 3584, 8, 1, 900)])     # of 512 channels
+def test_site13_scores_keep_their_order_moe(B, kind, T, H, E, topk, nsel):
+    lo, hi, gs = SCORE_RANGES[kind]
+    sh = synth.MoEShape("scores", 61 + T, T, H, E, topk, 128, 0.05, 2, 3.0, 10.0)
+    x = _separated_channels(T, H, lo, hi, T)
+    if gs is None:
+        x[:, 0] = 1e4
+    lg = synth.router_logits(sh)
+    gw13 = B.fake_quant_weights(synth.expert_weights(sh, "w13").cuda(), want_fq=False, sf_layout=B.SF_TILED)
+    gw2 = B.fake_quant_weights(synth.expert_weights(sh, "w2").cuda(), want_fq=False, sf_layout=B.SF_TILED)
+    res = B.moe_w4a4_rac(x.cuda(), lg.cuda(), gw13, gw2, topk, nsel, 64, torch.ones(1, device="cuda"),
+                         a13_gs=None if gs is None else torch.tensor([gs], device="cuda"), export=True)
+    torch.cuda.synchronize()
+    assert B.moe_async_status(res["workspace"]) == 0
+    site = R.rac(MC.f32(x), nsel, None if gs is None else np.float32(gs))
+    MC.check_site1(res, dict(site13=site), nsel, {})
