@@ -938,13 +938,15 @@ struct Fp8Layout {
   size_t perm, pos_pad, row_token, xq_tok, xe_tok, xq_pad, xsf, hq_pad, hsf, y_pad, total;
   int m_tiles_max;
 };
-// Few rows per expert (decode-sized batches): at most 32 rows per 128-row tile, see fp8.cu.
+// Few rows per expert (decode-sized batches): at most 32 on average, and at most kFp8FewRows per 128-row tile, see fp8.cu.
+// At the limit (512 tokens, 128 experts, top 8; even load / half of / all assignments on eight experts) it takes 137 / 152 / 70 us
+// where the other form takes 168 / 177 / 75; one token above it the other form takes 161 / 168 / 68 with its present front.
 bool fp8_few_rows(int T, int E, int topk) { return (int64_t)T * topk <= (int64_t)E * 32; }
 Fp8Layout fp8_layout(int T, int H, int I, int E, int topk) {
   Fp8Layout L{};
   const int64_t A = (int64_t)T * topk;
   const bool few = fp8_few_rows(T, E, topk);
-  L.m_tiles_max = (int)(A / (few ? 32 : 128)) + E;
+  L.m_tiles_max = (int)(A / (few ? kFp8FewRows : 128)) + E;
   const size_t pad_rows = (size_t)L.m_tiles_max * 128;
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
@@ -993,7 +995,7 @@ quads_status quads_fp8_quantize_weights(const void* w, int64_t n_tensors, int64_
 
 size_t quads_moe_fp8_workspace_bytes(int32_t T, int32_t H, int32_t I, int32_t E, int32_t topk) {
   if (T < 0 || H <= 0 || I <= 0 || E < 1 || topk < 1) return 0;
-  // Few rows per expert take up to four times the tiles per assignment, so the largest batch of that form can need more
+  // Few rows per expert take up to twice the tiles per assignment, so the largest batch of that form can need more
   // than a larger one of the other: what is returned for T is enough for every smaller batch as well.
   const int t_few = (int)std::min<int64_t>(T, (int64_t)E * 32 / topk);
   return std::max(fp8_layout(T, H, I, E, topk).total, fp8_layout(t_few, H, I, E, topk).total);
@@ -1040,7 +1042,7 @@ quads_status quads_moe_fp8_w8a8(const quads_moe_fp8_args* a, void* cuda_stream) 
   if (small) {
     SmallRouteArgs r{};
     r.logits = a->router_logits;
-    r.T = T; r.E = E; r.topk = topk; r.renormalize = a->renormalize; r.e_lo = 0; r.e_hi = E; r.slot_rows = 32;
+    r.T = T; r.E = E; r.topk = topk; r.renormalize = a->renormalize; r.e_lo = 0; r.e_hi = E; r.slot_rows = kFp8FewRows;
     r.wts = wts; r.offsets = offsets; r.tile_prefix = tile_prefix; r.tile_expert = tile_expert; r.tile_rows = tile_rows;
     r.header = header; r.perm = perm; r.pos_pad = pos_pad; r.row_token = row_token;
     r.ids_out = a->topk_ids; r.perm_out = a->perm;
@@ -1051,7 +1053,7 @@ quads_status quads_moe_fp8_w8a8(const quads_moe_fp8_args* a, void* cuda_stream) 
     RouteArgs r{};
     r.logits = a->router_logits;
     r.T = T; r.E = E; r.topk = topk; r.renormalize = a->renormalize; r.e_lo = 0; r.e_hi = E;
-    r.slot_rows = few ? 32 : 128; r.tile_group = 1;
+    r.slot_rows = few ? kFp8FewRows : 128; r.tile_group = 1;
     r.ids = ids; r.wts = wts; r.counts = reinterpret_cast<int32_t*>(P(L.route_counts));
     r.arrivals = reinterpret_cast<unsigned int*>(header + kHdrRouteArrivals); r.status = header + kHdrStatus;
     r.offsets = offsets; r.tile_prefix = tile_prefix; r.tile_expert = tile_expert; r.tile_rows = tile_rows; r.header = header;

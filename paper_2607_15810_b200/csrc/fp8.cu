@@ -216,27 +216,29 @@ namespace {
 
 constexpr int k8BM = 128, k8BN = 256;
 constexpr int k8TileA = k8BM * 128, k8TileB = k8BN * 128;
-constexpr int k8ActWarp = 3;                             // loads the activation side of the few-rows form
-constexpr int k8FewRows = 32;                            // rows of a tile in that form
+constexpr int k8ActWarp = 6;                             // loads the activation side of the few-rows form
+constexpr int k8FewRows = kFp8FewRows;                   // rows of a tile in that form
 constexpr int k8MaxStages = 5;
 
-// kFew: few rows per expert (decode-sized batches; the routing then puts at most 32 rows into a 128-row tile).  All
-// that matters there is the stream of weights: the activation operand takes 4 KB of a stage instead of 16 (the
-// MMA still reads 128 rows; what it finds behind the 32 gives accumulator rows nobody reads), which makes room for
+// kFew: few rows per expert (decode-sized batches; the routing then puts at most 64 rows into a 128-row tile).  All
+// that matters there is the stream of weights: the activation operand takes 8 KB of a stage instead of 16 (the
+// MMA still reads 128 rows; what it finds behind the 64 gives accumulator rows nobody reads), which makes room for
 // a fifth stage; the first projection gathers its rows and scales out of the token-order arrays instead of
 // reading copies of them; and the weights and routing tables are older than the preceding kernel, so the ring
-// fills while that one still runs.  Layer of 256 tokens (645 MB of weights and scale atoms): 164.9 -> 130.0 us; the
-// two GEMMs stream at 5.9 and 6.1 TB/s (4.7 and 5.5 with 128-row tiles, four stages and copied rows).
+// fills while that one still runs.  Layer of 256 tokens (645 MB of weights and scale atoms): 161 us with 128-row tiles,
+// four stages and copied rows, 124 so.  Tiles of 32 rows make an expert with many rows stream its weights, out of
+// L2, and run its MMAs up to four times as often: 256 tokens 123 us, but 512 tokens 156 (137 with 64 rows; 168 with 128),
+// and 88 (70; 75) when all of them choose the same eight experts.
 template <bool kFew>
 struct F8Cfg {
   static constexpr int kOffB = kFew ? k8FewRows * 128 : k8TileA;
   static constexpr int kOffSfA = kOffB + k8TileB;
   static constexpr int kOffSfB = kOffSfA + 512;
-  static constexpr int kStageBytes = (kOffSfB + 1024 + 1023) / 1024 * 1024;      // 51200 / 38912
+  static constexpr int kStageBytes = (kOffSfB + 1024 + 1023) / 1024 * 1024;      // 51200 / 43008
   static constexpr int kStages = kFew ? 5 : 4;
-  static constexpr int kThreads = kFew ? 416 : 576;
-  static constexpr int kLoadWarp = kFew ? 1 : 0, kMmaWarp = kFew ? 2 : 1;
-  static constexpr int kEpiWarps = kFew ? 4 : 16;        // the warps whose tensor-memory lanes hold rows (few: 0, 4, 8, 12)
+  static constexpr int kThreads = kFew ? 448 : 576;
+  static constexpr int kLoadWarp = kFew ? 2 : 0, kMmaWarp = kFew ? 3 : 1;
+  static constexpr int kEpiWarps = kFew ? 8 : 16;        // the warps whose tensor-memory lanes hold rows (few: 0, 1, 4, 5, 8, ...)
   static constexpr int kBarOffset = kStages * kStageBytes;
   static constexpr int kSmemBytes = kBarOffset + 256 + 2 * 128 * 4 * 4 + 1024;
   static_assert(kSmemBytes <= 232448 && kStages <= k8MaxStages, "shared memory");
@@ -347,25 +349,35 @@ gemm_fp8_kernel(const Fp8GemmParams p, const __grid_constant__ CUtensorMap tm_a,
       const int mt = tile / p.n_tiles_n;
       const int n_rows = p.tile_rows[mt];
       if (EPI == kEpiSwiGLU) {
-        // lane = row of the tile (rows beyond the valid ones repeat the last); lanes 0..7 gather four rows each
-        const int tok = p.row_token[mt * 128 + min(lane, n_rows - 1)];
-        const int g4 = (lane & 7) * 4;
-        const int y0 = __shfl_sync(0xFFFFFFFFu, tok, g4), y1 = __shfl_sync(0xFFFFFFFFu, tok, g4 + 1);
-        const int y2 = __shfl_sync(0xFFFFFFFFu, tok, g4 + 2), y3 = __shfl_sync(0xFFFFFFFFu, tok, g4 + 3);
-        const bool gathers = lane < 8 && g4 < n_rows;
+        // lane = rows lane and lane + 32 of the tile (rows beyond the valid ones repeat the last); lanes 0..15 gather four
+        // rows each
+        const int tok0 = p.row_token[mt * 128 + min(lane, n_rows - 1)], tok1 = p.row_token[mt * 128 + min(lane + 32, n_rows - 1)];
+        const int g4 = (lane & 15) * 4;
+        int y[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int lo = __shfl_sync(0xFFFFFFFFu, tok0, (g4 + i) & 31), hi = __shfl_sync(0xFFFFFFFFu, tok1, (g4 + i) & 31);
+          y[i] = g4 < 32 ? lo : hi;
+        }
+        const bool gathers = lane < 16 && g4 < n_rows;
         const uint32_t bytes = (uint32_t)((n_rows + 3) / 4) * 512u;
-        const uint8_t* xe = p.xe_tok + (size_t)tok * k_stages;
-        uint32_t code = __ldg(xe);
+        const uint8_t *xe0 = p.xe_tok + (size_t)tok0 * k_stages, *xe1 = p.xe_tok + (size_t)tok1 * k_stages;
+        const bool second = n_rows > 32;
+        uint32_t code0 = __ldg(xe0), code1 = second ? __ldg(xe1) : 0u;
         for (int ks = 0; ks < k_stages; ++ks) {
           ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, p.status);
           if (!ok) break;
           const uint32_t sb = smem_base + stage * k8StageBytes, full = bar_full + 8 * stage;
-          if (gathers) tma_gather4_rows(sb + (uint32_t)g4 * 128u, &tm_a, ks * 128, y0, y1, y2, y3, full);
-          asm volatile("st.shared.u32 [%0], %1;" ::"r"(sb + k8OffSfA + lane * 16), "r"(code * 0x01010101u) : "memory");
+          if (gathers) tma_gather4_rows(sb + (uint32_t)g4 * 128u, &tm_a, ks * 128, y[0], y[1], y[2], y[3], full);
+          asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(sb + k8OffSfA + lane * 16), "r"(code0 * 0x01010101u), "r"(code1 * 0x01010101u)
+                       : "memory");
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // the copy to tensor memory reads these words
           __syncwarp();
           if (lane == 0) mbar_expect_tx(full, bytes);
-          if (ks + 1 < k_stages) code = __ldg(xe + ks + 1);                 // a stage ahead of its use
+          if (ks + 1 < k_stages) {                               // a stage ahead of their use
+            code0 = __ldg(xe0 + ks + 1);
+            if (second) code1 = __ldg(xe1 + ks + 1);
+          }
           if (++stage == k8Stages) { stage = 0; phase ^= 1u; }
         }
       } else {
@@ -376,8 +388,10 @@ gemm_fp8_kernel(const Fp8GemmParams p, const __grid_constant__ CUtensorMap tm_a,
           if (!ok) break;
           if (issuer) {
             const uint32_t sb = smem_base + stage * k8StageBytes, full = bar_full + 8 * stage;
-            mbar_expect_tx(full, (uint32_t)(k8FewRows * 128 + 512));
+            const bool second = n_rows > 32;                   // (boxes of 32 rows)
+            mbar_expect_tx(full, (second ? 8192u : 4096u) + 512u);
             tma_load_2d(sb, &tm_a, ks * 128, mt * k8BM, full);
+            if (second) tma_load_2d(sb + 4096u, &tm_a, ks * 128, mt * k8BM + 32, full);
             bulk_load(sb + k8OffSfA, asf + (size_t)ks * 512u, 512u, full);
           }
           __syncwarp();
@@ -424,12 +438,12 @@ gemm_fp8_kernel(const Fp8GemmParams p, const __grid_constant__ CUtensorMap tm_a,
       if (ok && issuer) tc_commit<1>(bar_tfull);
       __syncwarp();
     }
-  } else if (!kFew || (warp & 3) == 0) {
+  } else if (!kFew || (warp & 3) < 2) {
     // ------------------------------------------------------------ epilogue
     const int q = warp & 3, cq = kFew ? warp >> 2 : (warp - 2) >> 2;
     const int row_in_tile = q * 32 + lane;
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
-    int it = 0;
+    int it = 0, turn = 0;                                  // tiles so far, and those with rows of this quadrant
     bool ok = true;
     for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++it) {
       const int mt = tile / p.n_tiles_n, nt = tile - mt * p.n_tiles_n;
@@ -438,6 +452,10 @@ gemm_fp8_kernel(const Fp8GemmParams p, const __grid_constant__ CUtensorMap tm_a,
       const bool valid = row_in_tile < n_valid;
       const int prow = mt * k8BM + row_in_tile;
       if (ok) ok = mbar_wait(bar_tfull, (uint32_t)(it & 1), abort_flag, p.status);
+      if (kFew && q * 32 >= n_valid) {                     // (all four warps of this quadrant)
+        if (ok && lane == 0) mbar_arrive(bar_tempty);
+        continue;
+      }
       float acc[64];
       if (ok) {
         tc_fence_after();
@@ -454,7 +472,8 @@ gemm_fp8_kernel(const Fp8GemmParams p, const __grid_constant__ CUtensorMap tm_a,
         if (lane == 0) mbar_arrive(bar_tempty);
       }
       if (EPI == kEpiSwiGLU) {
-        // every epilogue thread takes part in the tile's barrier, whether or not its wait succeeded
+        // the four warps of a quadrant, which exchange their rows' maxima, all take part in the tile's barrier, whether or
+        // not a wait succeeded
         const int I = p.n_out;
         float hb[32];
         float a = 0.f;
@@ -464,9 +483,9 @@ gemm_fp8_kernel(const Fp8GemmParams p, const __grid_constant__ CUtensorMap tm_a,
           hb[i] = __bfloat162float(__float2bfloat16_rn(__fdividef(g, 1.0f + __expf(-g)) * u));
           a = fmaxf(a, fabsf(hb[i]));
         }
-        float* slot = row_amax + (it & 1) * 512;
+        float* slot = row_amax + (turn++ & 1) * 512;
         slot[row_in_tile * 4 + cq] = a;
-        asm volatile("bar.sync 1, %0;" ::"n"(32 * k8EpiWarps) : "memory");
+        asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory");
         const float4 m4 = *reinterpret_cast<const float4*>(slot + row_in_tile * 4);
         const uint32_t code = fp8_scale_code(fmaxf(fmaxf(m4.x, m4.y), fmaxf(m4.z, m4.w)));
         const float sc = fp8_inv_scale(code);

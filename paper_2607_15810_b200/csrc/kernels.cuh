@@ -222,6 +222,7 @@ quads_status launch_gemm_bf16(const CUtensorMap& tm_a, const CUtensorMap& tm_b, 
                               int32_t* status, int n_sms, cudaStream_t stream);
 
 // ---- fp8.cu: the FP8 W8A8 comparison path
+constexpr int kFp8FewRows = 64;   // rows of a 128-row tile at most in the few-rows form
 struct Fp8GemmParams {
   int K;                 // contraction length in elements (multiple of 128)
   int n_tiles_n;         // tiles along the output features

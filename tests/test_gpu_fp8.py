@@ -207,3 +207,13 @@ def test_workspace_of_a_larger_batch_serves_smaller_ones(B, big):
         assert B.moe_async_status(ws) == 0
         want = B.moe_fp8_w8a8(x[:T].contiguous(), lg[:T].contiguous(), g13, g2, sh.topk)
         assert torch.equal(got["out"], want["out"])
+
+
+@pytest.mark.parametrize("T", [32, 33, 64, 65, 129])
+def test_fp8_few_rows_on_one_expert(B, T, monkeypatch):
+    """Every token goes to expert 5 first (tiles of at most 64 rows, copied in halves of 32) and to another one second."""
+    sh = synth.MoEShape("one_expert", 40, T, 256, 64, 2, 384, 0.05, 2, 3.0, 10.0)
+    lg = synth.router_logits(sh)
+    lg[:, 5] = 50.0
+    monkeypatch.setattr(synth, "router_logits", lambda s: lg)
+    _layer(B, sh)
