@@ -164,17 +164,6 @@ __device__ __forceinline__ void quant_role(const QuantRowsArgs& p, int cta, int 
   if (s->last) sum_partial_scores(p.partials + col * n_ch, n_rg, H, n_ch, p.keys + col * n_ch, reinterpret_cast<double*>(s->red));
 }
 
-// Asks L2 for the rows of quant_role's CTA.
-__device__ __forceinline__ void quant_prefetch(const QuantRowsArgs& p, int cta) {
-  const int col = cta % p.n_col, rg = cta / p.n_col;
-  const int r0 = rg * p.rows_per_cta, n_rows = min(p.T, r0 + p.rows_per_cta) - r0, lines = p.bw >> 2;   // of 128 bytes per row
-  const uint8_t* base = reinterpret_cast<const uint8_t*>(p.x + (size_t)col * p.bw * 16);
-  for (int i = threadIdx.x; i < n_rows * lines; i += 256) {
-    const int r = i / lines;
-    asm volatile("prefetch.global.L2::evict_last [%0];" ::"l"(base + (size_t)(r0 + r) * p.H * 2 + (size_t)(i - r * lines) * 128));
-  }
-}
-
 __global__ void __launch_bounds__(256, kQuantRowsPerSm) quant_rows_kernel(const QuantRowsArgs p) {
   pdl_sync();
   __shared__ QuantShared s;
@@ -185,13 +174,14 @@ __global__ void __launch_bounds__(256, kQuantRowsPerSm) quant_rows_kernel(const 
 // per SM beside them, quantize: the roles need nothing of one another, each has its own counters to meet at.
 // As five kernels on two streams (route, scan, permute beside quantize, rank) the last of them ended 44 us after
 // the call's start at 8192 tokens, because the quantization held the SMs; here codes, scores and tables are
-// there after 30 us (1500 tokens: 14 instead of 30).
+// there after 30 us (1500 tokens: 14 instead of 30).  Asking L2 for x before the tokens are routed gains nothing up to 4096 x
+// 4096 and loses beyond, where the lines it is asked to keep are evicted unread or evict others (this kernel with a cold
+// cache, 8192 x 4096 53 us, 57 so; 16384 x 4096 92 and 108; with a given scale 39 and 47).
 template <int NJ>
 __global__ void __launch_bounds__(256, kQuantRowsPerSm)
 front_kernel(const QuantRowsArgs q, const RouteArgs r, int n_groups) {
   pdl_sync();
   __shared__ union { QuantShared q; RouteShared r; } s;
-  if ((int)blockIdx.x >= n_groups) quant_prefetch(q, (int)blockIdx.x - n_groups);   // x arrives while the tokens are routed
   route_part1<NJ>(r, (int)blockIdx.x, (int)gridDim.x, n_groups);
   if ((int)blockIdx.x < n_groups) route_part2<NJ>(r, (int)blockIdx.x, n_groups, gridDim.x, &s.r);
   else quant_role(q, (int)blockIdx.x - n_groups, (int)gridDim.x - n_groups, &s.q);
