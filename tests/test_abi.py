@@ -3,6 +3,8 @@ and rejects bad arguments on the host before touching a device."""
 import ctypes as C
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -72,3 +74,13 @@ def test_workspace_of_a_larger_batch_serves_smaller_ones(lib, E, topk, H, I):
     for sizes in ([fp8(T, H, I, E, topk) for T in range(0, 5 * edge)], [moe(T, H, I, E, topk, 0) for T in range(0, 5 * edge)],
                   [moe(T, H, 0, 1, 1, I) for T in range(0, 1500)]):
         assert all(a <= b for a, b in zip(sizes, sizes[1:]))
+
+
+def test_binding_loads_where_torch_has_no_cuda():
+    """A build of torch without CUDA lacks these two functions; the library's host side (sizes, layouts) works there."""
+    code = ("import torch\n"
+            "for n in ('_cuda_getCurrentRawStream', '_cuda_getDevice'):\n"
+            "    if hasattr(torch._C, n): delattr(torch._C, n)\n"
+            "from paper_2607_15810_b200 import binding as B\n"
+            "assert B.sf_tiled_bytes(128, 64) == 512\n")
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT)
