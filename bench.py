@@ -837,7 +837,7 @@ def run_ours(args):
                 "rac_both_over_fp8": dcmp["fp8_w8a8"] / dcmp["nvfp4_rac_both"],
                 "rac_w13_slowdown_vs_plain": 1.0 - dcmp["nvfp4_plain"] / dcmp["nvfp4_rac_w13"],
                 "weight_bytes": {"fp8": fbytes, "nvfp4": wbytes},
-                "note": "T=%d, cold weights; the FP8 path runs 128-row tiles (no operand-swapped kernel for it)" % dsh.T}
+                "note": "T=%d, cold weights; the FP8 path runs tiles of at most 64 rows (no operand-swapped kernel for it)" % dsh.T}
             del dfws
             # the same call replayed from a CUDA graph (what a decode loop does)
             graph = torch.cuda.CUDAGraph()

@@ -536,7 +536,7 @@ quads_status quads_rac_channel_scores(const void* x, int64_t T, int64_t H, const
                               rpc, partials));
   // the order-preserving 64-bit keys of non-negative scores are the scores' own bit patterns
   QUADS_CUDA_OK(launch_kernel(score_reduce_kernel, dim3((unsigned)((H + 31) / 32), kScoreSlices), dim3(256), (size_t)0, st,
-                              (const float*)partials, (const int*)nullptr, 1, ctas, (int)H, slices, counters,
+                              (const float*)partials, ctas, (int)H, slices, counters,
                               reinterpret_cast<unsigned long long*>(scores)));
   QUADS_CUDA_OK(cudaGetLastError());
   return QUADS_OK;

@@ -168,7 +168,7 @@ fp8_quantize_weight_kernel(const uint16_t* __restrict__ w, int N, int K, uint8_t
   }
 }
 
-// Dispatch, driven by the destination tile (as rac_dispatch_kernel): the tile's rows of E4M3 codes
+// Dispatch, driven by the destination tile (as dispatch_kernel): the tile's rows of E4M3 codes
 // (H bytes each) and, per 128-channel stage, one 512-byte scale atom with every row's scale byte
 // repeated over the stage's four K = 32 MMAs.
 __global__ void __launch_bounds__(256)
@@ -259,13 +259,6 @@ __device__ __forceinline__ void tc_mma_mxf8(uint32_t d_tmem, uint64_t adesc, uin
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %6, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::mxf8f6f4.block_scale.scale_vec::1X [%0], %1, %2, %3, [%4], [%5], p;\n\t}"
       ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(sfa_tmem), "r"(sfb_tmem), "r"(accumulate) : "memory");
-}
-
-// Four rows of the tensor map (box: one row) into 4 x 128 bytes, swizzled like a tile.
-__device__ __forceinline__ void tma_gather4_rows(uint32_t dst, const CUtensorMap* map, int x, int y0, int y1, int y2, int y3, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cta.global.tile::gather4.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
-      ::"r"(dst), "l"(map), "r"(x), "r"(y0), "r"(y1), "r"(y2), "r"(y3), "r"(bar) : "memory");
 }
 
 template <int EPI, bool kFew>
@@ -368,7 +361,7 @@ gemm_fp8_kernel(const Fp8GemmParams p, const __grid_constant__ CUtensorMap tm_a,
           ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, p.status);
           if (!ok) break;
           const uint32_t sb = smem_base + stage * k8StageBytes, full = bar_full + 8 * stage;
-          if (gathers) tma_gather4_rows(sb + (uint32_t)g4 * 128u, &tm_a, ks * 128, y[0], y[1], y[2], y[3], full);
+          if (gathers) tma_gather4(sb + (uint32_t)g4 * 128u, &tm_a, ks * 128, y[0], y[1], y[2], y[3], full);
           asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(sb + k8OffSfA + lane * 16), "r"(code0 * 0x01010101u), "r"(code1 * 0x01010101u)
                        : "memory");
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // the copy to tensor memory reads these words

@@ -12,7 +12,7 @@ constexpr int kMaxTopk = 16;
 constexpr int kMaxExperts = 256;
 
 // header words written by the scan (device side sizes of the dispatch)
-enum { kHdrMTiles = 0, kHdrPaddedRows = 1, kHdrAssignments = 2, kHdrStatus = 3, kHdrArrivals = 4, kHdrRouteArrivals = 5, kHdrWords = 8 };
+enum { kHdrMTiles = 0, kHdrAssignments = 2, kHdrStatus = 3, kHdrArrivals = 4, kHdrRouteArrivals = 5, kHdrWords = 8 };
 
 constexpr int kAmaxPartsMax = 2048;   // partial maxima left by the first pass of the single-tensor quantizer
 
@@ -41,8 +41,7 @@ __global__ void dequantize_kernel(const uint8_t* q, const uint8_t* sf, const flo
 __global__ void channel_stats_kernel(const uint16_t* x, int T, int H, const float* gs_in, const uint32_t* amax_bits,
                                      int rows_per_cta, float* partials);
 constexpr int kScoreSlices = 16;
-__global__ void score_reduce_kernel(const float* partials, const int* n_part_ptr, int n_part_mul,
-                                    int n_part_fixed, int C, double* slice_sums, unsigned int* counters,
+__global__ void score_reduce_kernel(const float* partials, int n_part, int C, double* slice_sums, unsigned int* counters,
                                     unsigned long long* score_keys);
 __global__ void clear_kernel(uint4* p, int n);
 __global__ void sel_list_kernel(const uint8_t* mask, int C, int32_t* sel_export);

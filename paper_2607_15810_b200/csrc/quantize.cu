@@ -1,5 +1,5 @@
-// Streaming kernels: tensor amax, NVFP4 quantize / fake-quant, RAC statistics,
-// channel selection, masked residual quantize + dispatch scatter, small fix-ups.
+// Streaming kernels: tensor amax, NVFP4 quantize / fake-quant / decode, channel statistics, selection and masking of a
+// residual in place, the weighted sum over a token's experts, verification exports, mismatch norms.
 // All HBM- or latency-bound; no tensor cores here.
 #include "kernels.cuh"
 #include "select.cuh"
@@ -739,11 +739,9 @@ channel_stats_kernel(const uint16_t* __restrict__ x, int T, int H, const float* 
 // grid = (ceil(C/32), kScoreSlices), 256 threads = 32 columns x 8 row lanes.
 // `counters` (one per column group) must be zero on entry.
 __global__ void __launch_bounds__(256)
-score_reduce_kernel(const float* __restrict__ partials, const int* __restrict__ n_part_ptr, int n_part_mul,
-                    int n_part_fixed, int C, double* __restrict__ slice_sums, unsigned int* __restrict__ counters,
-                    unsigned long long* __restrict__ score_keys) {
+score_reduce_kernel(const float* __restrict__ partials, int n_part, int C, double* __restrict__ slice_sums,
+                    unsigned int* __restrict__ counters, unsigned long long* __restrict__ score_keys) {
   pdl_sync();
-  const int n_part = n_part_ptr ? *n_part_ptr * n_part_mul : n_part_fixed;
   const int per = (n_part + kScoreSlices - 1) / kScoreSlices;
   const int p0 = blockIdx.y * per, p1 = min(n_part, p0 + per);
   const int col = blockIdx.x * 32 + (threadIdx.x & 31);

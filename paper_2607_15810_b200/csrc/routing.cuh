@@ -201,7 +201,6 @@ __device__ void route_part2(const RouteArgs& p, int cta, int n_groups, uint32_t 
           p.tile_prefix[E] = tp + tiles;
           if (p.offsets_out) p.offsets_out[E] = off + cnt;
           p.header[kHdrMTiles] = tp + tiles;
-          p.header[kHdrPaddedRows] = (tp + tiles) * 128;
           p.header[kHdrAssignments] = off + cnt;
         }
       }

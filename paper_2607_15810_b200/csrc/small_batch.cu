@@ -151,7 +151,6 @@ route_small_kernel(const SmallRouteArgs p) {
           p.tile_prefix[E] = tp + tiles;
           if (p.offsets_out) p.offsets_out[E] = off + cnt;
           p.header[kHdrMTiles] = tp + tiles;
-          p.header[kHdrPaddedRows] = (tp + tiles) * 128;
           p.header[kHdrAssignments] = off + cnt;
         }
       }

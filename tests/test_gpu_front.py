@@ -1,5 +1,5 @@
 """The cooperative front of larger batches (routing and quantization as two roles of one launch, then selection and
-dispatch copies) at its edges: one token per routing warp and the four-token form, more than 32 tokens per routing
+dispatch copies) at its edges: one token per routing warp and the two-token form, more than 32 tokens per routing
 CTA, more tokens than the small-batch kernels take by one, channel groups of 128 / 256 / 512, slabs of 512 channels
 that do not divide the row, the widest top-k, no residual, a given scale, operand-swapped GEMMs behind it."""
 import numpy as np

@@ -1,5 +1,5 @@
 """The single-cluster front of a call with few tokens (routing, quantization, selection, dispatch) at the edges of
-its tiling: 32 tokens per word of the assignment matrix, 256 tokens where a warp takes a second one, 512 where the
+its tiling: 16 tokens per word of the assignment matrix, 256 tokens where a warp takes a second one, 512 where the
 grid-wide kernels take over; channel units of 128 that do not divide over the cluster; the widest top-k.  Every
 result is compared with the oracle as for any other layer (`moe_check`)."""
 import numpy as np
@@ -22,6 +22,7 @@ def B():
 
 
 @pytest.mark.parametrize("T,H,E,topk,f13,static", [
+    (15, 256, 16, 4, 0.5, False), (16, 128, 8, 2, 0.25, True), (17, 384, 33, 3, 0.5, False),
     (1, 128, 256, 16, 0.5, False), (31, 640, 33, 3, 0.25, False), (32, 256, 5, 5, 1.0, True), (33, 2176, 8, 2, 0.5, False),
     (255, 384, 64, 16, 0.0, False), (256, 256, 129, 8, 0.5, True), (257, 1024, 16, 4, 0.5, False), (511, 256, 32, 2, 0.5, False),
     (512, 128, 8, 8, 0.25, False), (513, 128, 8, 8, 0.25, False)])
