@@ -685,7 +685,11 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   static const bool no_swap = getenv("QUADS_NO_SWAP") != nullptr;
   const bool swapped = !dense && !no_swap && cta_group == 1 && gemm_swapped_ok(A, E, L.m_tiles_max);
   // Few tokens: the front of the call is two kernels of one cluster each (one for a dense projection), which
-  // clear what has to start at zero themselves.
+  // clear what has to start at zero themselves.  The line is the routing kernel's 512 tokens (or what fits shared memory).
+  // Whole calls, us, so / with the grid-wide front: layer of 128 experts, H = 2048, 1 token 27.9 / 50.0, 64 tokens 79.0 / 91.9,
+  // 256 87.0 / 96.4, 512 104.1 / 113.0; H = 4096, 256 tokens 266 / 268, 512 339 / 332; eight experts, 512 tokens, H = 2048 48.5 /
+  // 52.4, H = 4096 85.6 / 85.5; dense, K = 512, 256 tokens 18.4 / 20.9, 512 22.4 / 21.0; K = 4096, 128 tokens 31.1 / 32.8, 256 35.4 /
+  // 32.9, 512 42.9 / 35.0: for wide rows the line lies higher than it should.
   const bool small = a->operand_mode == QUADS_W4A4 && cta_group == 1 && front_small_fits(T, H, swapped);
   g_trace.n = 0;
   trace_mark("start", st);

@@ -267,7 +267,8 @@ __device__ __forceinline__ void stg256(void* addr, const uint32_t* v) {
 // The same, telling L2 that nobody reads it soon.  Fake-quantized weights leave by it: two 16-byte streaming stores
 // per thread write every sector in two halves (16 tensors of 3072 x 4096: 212 us, 203 with this one; 8 of
 // 1536 x 2048: 35 and 33), and without the hint the written lines push the tensor that is still to be quantized out
-// of L2 (220 us).
+// of L2 (220 us).  (The decoded operand of the one-sided mode W16A4 leaves by it too, although the product behind it reads
+// it back: not measured without the hint.)
 __device__ __forceinline__ void stg256_stream(void* addr, const uint32_t* v) {
   asm volatile("st.global.L2::evict_first.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]),
                "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");

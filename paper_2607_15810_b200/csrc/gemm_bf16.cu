@@ -234,7 +234,10 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_con
 quads_status launch_gemm_bf16(const CUtensorMap& tm_a, const CUtensorMap& tm_b, int T, int N, int K, uint16_t* out,
                               int32_t* status, int n_sms, cudaStream_t stream) {
   const int pair_tiles = ((T + 255) / 256) * ((N + 255) / 256);
-  if (pair_tiles >= n_sms / 2) {                     // at least one wave of pairs
+  // From one wave of pairs on, however full the last one is (us, pairs / best single-CTA width: 2304 x 4096 -> 2304, 81 tiles, 44.6 /
+  // 45.3; 2560 x 4096 -> 2560, 100 tiles, 44.4 / 50.1; 8192 x 2048 -> 640 25.0 / 25.3; 8192 x 4096 -> 4096 201 / 213; the one
+  // form it loses at is a single column tile, half of it missing: 18945 x 2048 -> 128 23.4 / 17.8).
+  if (pair_tiles >= n_sms / 2) {
     QUADS_CUDA_OK(set_max_dynamic_smem<gemm_bf16_pair_kernel>(FCfg<2>::kSmemBytes));
     QUADS_CUDA_OK(launch_kernel(gemm_bf16_pair_kernel, dim3(n_sms / 2 * 2), dim3(kFThreads), (size_t)FCfg<2>::kSmemBytes, stream, tm_a,
                                 tm_b, T, N, K, out, status));
