@@ -278,7 +278,8 @@ __device__ __forceinline__ void stg256_stream(void* addr, const uint32_t* v) {
 // `n_out` elements starting at `dst`, rows >= rows_valid skipped.  The 32-byte chunks are first
 // transposed inside every group of 4 lanes (two butterfly exchanges), so that each store
 // instruction of the warp writes eight complete 128-byte lines instead of a 32-byte piece of 32
-// different lines.  All 32 lanes must call it.
+// different lines.  All 32 lanes must call it.  kHalves: `dst` is 16-byte, not 32-byte aligned.
+template <bool kHalves = false>
 __device__ __forceinline__ void store_y_rows(const float* acc, float scale, uint16_t* dst, int n_out, int rows_valid,
                                              int lane) {
   uint32_t w[32];
@@ -304,7 +305,14 @@ __device__ __forceinline__ void store_y_rows(const float* acc, float scale, uint
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int r = 4 * g + i;
-    if (r < rows_valid) stg256(dst + (size_t)r * n_out + 16 * j, w + 8 * i);
+    if (r >= rows_valid) continue;
+    uint16_t* d = dst + (size_t)r * n_out + 16 * j;
+    if (!kHalves) {
+      stg256(d, w + 8 * i);
+    } else {
+      reinterpret_cast<uint4*>(d)[0] = make_uint4(w[8 * i], w[8 * i + 1], w[8 * i + 2], w[8 * i + 3]);
+      reinterpret_cast<uint4*>(d)[1] = make_uint4(w[8 * i + 4], w[8 * i + 5], w[8 * i + 6], w[8 * i + 7]);
+    }
   }
 }
 

@@ -184,6 +184,7 @@ __device__ __forceinline__ void gemm_bf16_body(const CUtensorMap* tm_a, const CU
     const int q = warp & 3, ch = (warp - 2) >> 2;
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
     const uint32_t tempty_addr = CG == 1 ? bar_tempty : map_to_cta(bar_tempty, 0);
+    const bool wide = (reinterpret_cast<size_t>(out) & 31) == 0;     // the caller's output may be aligned to 16 bytes only
     int it = 0;
     bool ok = true;
     for (int tile = first_tile; tile < total && ok; tile += tile_step, ++it) {
@@ -200,7 +201,10 @@ __device__ __forceinline__ void gemm_bf16_body(const CUtensorMap* tm_a, const CU
         tmem_ld32(lane_addr + buf * 256 + c, v);
         tmem_ld32(lane_addr + buf * 256 + c + 32, v + 32);
         tmem_ld_wait();
-        if (n0 < N) store_y_rows(v, 1.0f, out + (size_t)row0 * N + n0, N, T - row0, lane);
+        if (n0 < N) {
+          if (wide) store_y_rows(v, 1.0f, out + (size_t)row0 * N + n0, N, T - row0, lane);
+          else store_y_rows<true>(v, 1.0f, out + (size_t)row0 * N + n0, N, T - row0, lane);
+        }
       }
       tc_fence_before();
       __syncwarp();
