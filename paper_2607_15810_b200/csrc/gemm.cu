@@ -453,15 +453,14 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p, const CUtensorMap
         if (n0 < p.n_out)
           store_y_rows(acc, scale, p.y_pad + (size_t)(mt * kBM + q * 32) * p.n_out + n0, p.n_out, rows_of(mt) - q * 32, lane);
       } else {
+        // Complete lines through the lane transpose (the caller's output may be aligned to 16 bytes only).  One row per lane,
+        // 16 bytes at a time, is 32 half sectors per instruction: 128 x 512 -> 256 16.4 us per call, 14.6 with the transpose;
+        // 8192 x 4096 -> 4096 162.4 us, 154.0.
         const int n0 = nt * 256 + cq * 64;
-        if (valid && n0 < p.n_out) {
-          uint4* dst = reinterpret_cast<uint4*>(p.out_bf16 + (size_t)prow * p.n_out + n0);
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            dst[i] = make_uint4(f32x2_to_bf16x2(acc[8 * i] * scale, acc[8 * i + 1] * scale),
-                                f32x2_to_bf16x2(acc[8 * i + 2] * scale, acc[8 * i + 3] * scale),
-                                f32x2_to_bf16x2(acc[8 * i + 4] * scale, acc[8 * i + 5] * scale),
-                                f32x2_to_bf16x2(acc[8 * i + 6] * scale, acc[8 * i + 7] * scale));
+        if (n0 < p.n_out) {
+          uint16_t* dst = p.out_bf16 + (size_t)(mt * kBM + q * 32) * p.n_out + n0;
+          if ((reinterpret_cast<size_t>(p.out_bf16) & 31) == 0) store_y_rows(acc, scale, dst, p.n_out, rows_of(mt) - q * 32, lane);
+          else store_y_rows<true>(acc, scale, dst, p.n_out, rows_of(mt) - q * 32, lane);
         }
       }
     }
