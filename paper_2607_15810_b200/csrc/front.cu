@@ -129,12 +129,8 @@ __device__ __forceinline__ void quant_role(const QuantRowsArgs& p, int cta, int 
     if (p.xq_exp) *reinterpret_cast<uint2*>(p.xq_exp + qo) = make_uint2(bq.lo, bq.hi);
     if (p.xsf_exp) p.xsf_exp[so] = (uint8_t)bq.sf8;
     if (p.with_residual) {
-      dequant_block(bq, o);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        o[i] = __fsub_rn(o[i], f[i]);
-        acc[i] = __fmaf_rn(o[i], o[i], acc[i]);
-      }
+      residual_block(bq, f, o);
+      add_squares(o, acc);
       const BlockQ br = quantize_block(o, qc);
       *reinterpret_cast<uint2*>(p.rq + qo) = make_uint2(br.lo, br.hi);
       p.rsf[so_op] = (uint8_t)br.sf8;

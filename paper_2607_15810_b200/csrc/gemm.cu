@@ -423,9 +423,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p, const CUtensorMap
           }
           if (p.resid2) {
             float r[16];
-            dequant_block(bq, r);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) r[i] = __fsub_rn(r[i], hb[i]);
+            residual_block(bq, hb, r);
             const BlockQ br = quantize_block(r, qc);
             rs |= br.sf8 << (8 * c);
             if (valid)

@@ -521,9 +521,7 @@ gemm_swapped_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_x
           }
           if (p.resid2) {
             float r[16];
-            dequant_block(bq, r);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) r[i] = __fsub_rn(r[i], hb[i]);
+            residual_block(bq, hb, r);
             const BlockQ br = quantize_block(r, qc);
             if (valid) {
               *reinterpret_cast<uint2*>(p.r2q_pad + (size_t)prow * (I >> 1) + (f0 >> 1)) =

@@ -716,12 +716,8 @@ channel_stats_kernel(const uint16_t* __restrict__ x, int T, int H, const float* 
       float f[16], o[16];
       unpack8(v0, f);
       unpack8(v1, f + 8);
-      dequant_block(quantize_block(f, qc), o);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        o[i] = __fsub_rn(o[i], f[i]);
-        acc[i] = __fmaf_rn(o[i], o[i], acc[i]);
-      }
+      residual_block(quantize_block(f, qc), f, o);
+      add_squares(o, acc);
     }
     float4* dst = reinterpret_cast<float4*>(partials + (size_t)blockIdx.x * H + kb * 16);
     dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);

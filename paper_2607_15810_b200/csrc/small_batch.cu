@@ -280,12 +280,8 @@ front_small_kernel(const SmallFrontArgs p) {
       if (p.xsf_exp) p.xsf_exp[so] = (uint8_t)bq.sf8;
       if (p.n_sel > 0) {
         float o[16];
-        dequant_block(bq, o);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          o[i] = __fsub_rn(o[i], f[i]);
-          acc[i] = __fmaf_rn(o[i], o[i], acc[i]);
-        }
+        residual_block(bq, f, o);
+        add_squares(o, acc);
         const BlockQ br = quantize_block<false>(o, qc);
         reinterpret_cast<uint2*>(st_r)[idx * 8 + blk] = make_uint2(br.lo, br.hi);
         if (p.token_order) p.rsf[so] = (uint8_t)br.sf8;
