@@ -688,9 +688,11 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   // clear what has to start at zero themselves.  The line is the routing kernel's 512 tokens (or what fits shared memory).
   // Whole calls, us, so / with the grid-wide front: layer of 128 experts, H = 2048, 1 token 27.9 / 50.0, 64 tokens 79.0 / 91.9,
   // 256 87.0 / 96.4, 512 104.1 / 113.0; H = 4096, 256 tokens 266 / 268, 512 339 / 332; eight experts, 512 tokens, H = 2048 48.5 /
-  // 52.4, H = 4096 85.6 / 85.5; dense, K = 512, 256 tokens 18.4 / 20.9, 512 22.4 / 21.0; K = 4096, 128 tokens 31.1 / 32.8, 256 35.4 /
-  // 32.9, 512 42.9 / 35.0: for wide rows the line lies higher than it should.
-  const bool small = a->operand_mode == QUADS_W4A4 && cta_group == 1 && front_small_fits(T, H, swapped);
+  // 52.4, H = 4096 85.6 / 85.5.  Dense: K = 512, 256 rows 15.3 / 18.5, 512 18.4 / 18.5; K = 2048, 256 rows 19.4 / 22.6, 512 23.0 /
+  // 23.1; K = 4096, where a CTA of the cluster has two units of channels, 128 rows 25.1 / 26.7, 192 26.6 / 26.7, 256 28.7 / 26.8, 512
+  // 37.5 / 30.8.
+  const bool small = a->operand_mode == QUADS_W4A4 && cta_group == 1 && front_small_fits(T, H, swapped) &&
+                     !(dense && H > 2048 && (int64_t)T * H > 192 * 4096);
   g_trace.n = 0;
   trace_mark("start", st);
   // header (status word included) and the amax word start at zero
@@ -816,8 +818,9 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
     if ((s = make_gather_map(&m1.a, P(L.xq_tok), T, H / 2)) != QUADS_OK) return s;
     if ((s = make_gather_map(&m1.r, P(L.rq_tok), T, H / 2)) != QUADS_OK) return s;
   } else {
-    if ((s = make_codes_map(&m1.a, P(L.xq_pad), pad_rows, H / 2, act_box)) != QUADS_OK) return s;
-    if ((s = make_codes_map(&m1.r, P(L.rq_pad), pad_rows, H / 2, act_box)) != QUADS_OK) return s;
+    const uint64_t rows = dense ? (uint64_t)T : pad_rows;      // (rows beyond the map's end are zeros that nobody fetches)
+    if ((s = make_codes_map(&m1.a, P(L.xq_pad), rows, H / 2, act_box)) != QUADS_OK) return s;
+    if ((s = make_codes_map(&m1.r, P(L.rq_pad), rows, H / 2, act_box)) != QUADS_OK) return s;
   }
   if ((s = make_codes_map(&m1.b, a->w13_q, (uint64_t)e_cnt * N1, H / 2)) != QUADS_OK) return s;
   if (cta_group == 2) {
@@ -847,6 +850,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
     g.n_tiles_n = (a->N + 255) / 256;
     g.half1_row_offset = 128;
     g.out_bf16 = static_cast<uint16_t*>(a->out);
+    if (cta_group == 1 && gemm_dense_ok(T, H, a->N, di.sm_count)) return launch_gemm_dense(g, m1, di.sm_count, st);
     return launch_gemm(kEpiStore, cta_group, g, m1, di.sm_count, st);
   }
   g.n_out = I;

@@ -51,9 +51,9 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-// The same for a grid that is one thread-block cluster of n_cta CTAs.
+// The same for a grid of n_cta CTAs in clusters of `cluster`, and for a grid that is one cluster.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_cluster(void (*kernel)(KArgs...), int n_cta, int threads, size_t smem, cudaStream_t st, Args&&... args) {
+inline cudaError_t launch_clusters(void (*kernel)(KArgs...), int n_cta, int cluster, int threads, size_t smem, cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_cta);
   cfg.blockDim = dim3(threads);
@@ -61,13 +61,17 @@ inline cudaError_t launch_cluster(void (*kernel)(KArgs...), int n_cta, int threa
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = n_cta; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[0].val.clusterDim.x = cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl_enabled() ? 2 : 1;
   note_launch();
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_cluster(void (*kernel)(KArgs...), int n_cta, int threads, size_t smem, cudaStream_t st, Args&&... args) {
+  return launch_clusters(kernel, n_cta, n_cta, threads, smem, st, static_cast<Args&&>(args)...);
 }
 
 // Raise a kernel's dynamic shared-memory limit once per device (the attribute is per device; a

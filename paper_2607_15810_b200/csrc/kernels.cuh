@@ -214,6 +214,11 @@ struct GemmMaps {
 bool gemm_swapped_ok(int64_t assignments, int n_experts, int m_tiles_max);
 quads_status launch_gemm_swapped(int epi, const GemmParams& p, const GemmMaps& m, int n_sms, cudaStream_t stream);
 
+// ---- gemm_dense.cu: dense projection with few output tiles, K split over clusters
+constexpr int kDenseMaxSplit = 8;
+bool gemm_dense_ok(int rows, int K, int N, int n_sms);
+quads_status launch_gemm_dense(const GemmParams& p, const GemmMaps& m, int n_sms, cudaStream_t stream);
+
 // ---- gemm_bf16.cu: out[T, N] = A[T, K] B[N, K]^T, bf16 operands (tensor maps with boxes of 64 elements x kBf16BoxRows
 // rows, 128-byte swizzle), float32 accumulation, bf16 output; K % 64 == 0, N % 128 == 0
 constexpr int kBf16BoxRows = 64;

@@ -1,0 +1,36 @@
+"""The dense projection with few output tiles, at the edges of its tile width and of its split of K."""
+import numpy as np
+import pytest
+import torch
+
+import moe_check as MC
+from oracle import moe as M
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("T,K,N,nsel", [
+    (1, 4096, 128, 2048),      # eight CTAs per tile
+    (64, 4096, 128, 0),        # four, no residual
+    (128, 4096, 256, 4096),    # four, every row of the tile
+    (130, 2048, 128, 1024),    # two row tiles, two rows in the second
+    (40, 640, 128, 320),       # three stages for two CTAs, the last one half full
+    (17, 128, 128, 16),        # one stage
+    (129, 128, 9600, 64),      # tiles of 256 columns, half of the last one missing
+    (200, 4096, 128, 2048)])   # behind the grid-wide front
+def test_dense_tiles_and_splits(T, K, N, nsel):
+    from paper_2607_15810_b200 import binding as B
+    g = torch.Generator().manual_seed(T + K + N)
+    x = torch.randn(T, K, generator=g)
+    x[:, 3] *= 20
+    x = x.to(torch.bfloat16)
+    w = (torch.randn(N, K, generator=g) * 0.05).to(torch.bfloat16)
+    wo = MC.oracle_weights(w[None])
+    o = M.dense_w4a4_rac(MC.f32(x), wo["codes"][0], wo["sf"][0], wo["gs"][0], nsel)
+    wq = B.fake_quant_weights(w.unsqueeze(0).cuda(), want_fq=False, sf_layout=B.SF_TILED)
+    res = B.dense_w4a4_rac(x.cuda(), wq, nsel, export=True)
+    torch.cuda.synchronize()
+    assert B.moe_async_status(res["workspace"]) == 0
+    MC.check_site1(res, dict(site13=o["site"]), nsel, {})
+    got = MC.f32(res["out"]).astype(np.float64)
+    assert float((np.abs(got - o["y64"]) / MC.gemm_tol(o["absdot"], o["y64"])).max()) <= 1.0
