@@ -1,7 +1,10 @@
-"""Thin ctypes binding over libquads.so: argument marshalling only.  Every step
+"""Thin binding over libquads.so: argument marshalling only.  Every step
 of the path runs inside the library's CUDA kernels; torch is used for device
 memory and the current stream.  Importing this module fails loudly when the
-library has not been built (run `python -m paper_2607_15810_b200.build`)."""
+library has not been built (run `python -m paper_2607_15810_b200.build`).
+
+The ordinary calls -- plain CUDA tensors, no verification exports -- go through _native.so, which does the
+same in a third of the host time; everything else through ctypes."""
 import ctypes as C
 import os
 
@@ -76,6 +79,13 @@ class QuadsError(RuntimeError):
         super().__init__(lib.quads_status_string(int(status)).decode())
 
 
+try:
+    from . import _native
+    _native.set_error(QuadsError)
+except ImportError:                # a torch without CUDA, or another one than it was built for
+    _native = None
+
+
 def check(status):
     if status != QUADS_OK:
         raise QuadsError(status)
@@ -108,6 +118,8 @@ def _ws(nbytes, device):
 
 def quantize_nvfp4(x, gs=None, sf_layout=SF_LINEAR, out=None, workspace=None):
     """x: bf16 CUDA tensor [rows, K] (row stride allowed).  Returns (q, sf, gs)."""
+    if _native is not None and (r := _native.quantize_nvfp4(x, gs, sf_layout, out, workspace)) is not None:
+        return r
     assert x.dtype == torch.bfloat16 and x.is_cuda and x.dim() == 2 and x.stride(1) == 1
     rows, K = x.shape
     dev = x.device
@@ -202,6 +214,9 @@ def moe_w4a4_rac(x, logits, w13, w2, topk, nsel13, nsel2, a2_gs, a13_gs=None, re
                  export=False, workspace=None, out=None, expert_range=None, out_f32=None):
     """MoE layer forward.  w13 / w2: dicts with q [E,rows,K/2], sf (tiled, [E,bytes]), gs [E] as
     produced by fake_quant_weights(..., sf_layout=SF_TILED).  Returns dict(out=bf16 [T,H], ...)."""
+    if _native is not None and not export and expert_range is None and out_f32 is None and \
+            (r := _native.moe_w4a4_rac(x, logits, w13, w2, topk, nsel13, nsel2, a2_gs, a13_gs, renormalize, workspace, out)) is not None:
+        return r
     T, H = x.shape
     E = logits.shape[1]
     I = w2["q"].shape[2] * 2
@@ -255,6 +270,8 @@ def moe_w4a4_rac(x, logits, w13, w2, topk, nsel13, nsel2, a2_gs, a13_gs=None, re
 
 def dense_w4a4_rac(x, w, nsel, a_gs=None, export=False, workspace=None):
     """Single projection out[T,N] = W X~.  w: dict(q [1,N,K/2] or [N,K/2], sf tiled, gs [1])."""
+    if _native is not None and not export and (r := _native.dense_w4a4_rac(x, w, nsel, a_gs, workspace)) is not None:
+        return r
     T, K = x.shape
     N = w["q"].shape[-2]
     dev = x.device
@@ -290,6 +307,8 @@ def dense_one_sided(x, mode, w=None, w_bf16=None, a_gs=None, export=False, works
     """The one-sided rollout modes of the dense projection: mode = W4A16 (w: packed NVFP4 weight
     dict, x stays bf16) or W16A4 (w_bf16: bf16 [N, K] weight, x quantized online and decoded).
     Returns dict(out=bf16 [T, N], ...)."""
+    if _native is not None and not export and (r := _native.dense_one_sided(x, mode, w, w_bf16, a_gs, workspace)) is not None:
+        return r
     T, K = x.shape
     N = w["q"].shape[-2] if mode == W4A16 else w_bf16.shape[0]
     assert mode in (W4A16, W16A4, W16A16)
@@ -431,6 +450,9 @@ def moe_fp8_workspace_bytes(T, H, I, E, topk):
 
 def moe_fp8_w8a8(x, logits, w13, w2, topk, renormalize=True, export=False, workspace=None, out=None):
     """FP8 W8A8 MoE layer (comparison path).  w13 / w2: dicts from fp8_quantize_weights."""
+    if _native is not None and not export and \
+            (r := _native.moe_fp8_w8a8(x, logits, w13, w2, topk, renormalize, workspace, out)) is not None:
+        return r
     T, H = x.shape
     E = logits.shape[1]
     I = w2["q"].shape[2]

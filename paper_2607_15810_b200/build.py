@@ -1,11 +1,15 @@
-"""Builds libquads.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libquads.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _native.so, the binding's ordinary calls
+as native functions on top of it."""
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libquads.so")
+NATIVE = os.path.join(HERE, "_native.so")
+NATIVE_SOURCE = os.path.join(CSRC, "native.cpp")
 SOURCES = ["api.cu", "quantize.cu", "front.cu", "small_batch.cu", "gemm.cu", "gemm_dense.cu", "gemm_swapped.cu", "gemm_bf16.cu", "fp8.cu", "probe.cu"]
 HEADERS = ["common.cuh", "kernels.cuh", "routing.cuh", "select.cuh", "tcgen05.cuh", os.path.join("..", "..", "include", "quads.h")]
 
@@ -15,17 +19,47 @@ def _nvcc():
     return cand if os.path.exists(cand) else "nvcc"
 
 
+def _older(target, deps):
+    return not os.path.exists(target) or any(os.path.getmtime(d) > os.path.getmtime(target) for d in deps)
+
+
 def needs_build():
-    if not os.path.exists(LIB):
-        return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS]
-    return any(os.path.getmtime(d) > t for d in deps)
+    return _older(LIB, [os.path.join(CSRC, s) for s in SOURCES + HEADERS])
+
+
+def _start_native():
+    """The compiler of _native.so, or None where the installed torch has no CUDA (the binding then does without)."""
+    import torch
+    from torch.utils import cpp_extension
+    lib_dir = os.path.join(os.path.dirname(torch.__file__), "lib")
+    if torch.version.cuda is None or not os.path.exists(os.path.join(lib_dir, "libc10_cuda.so")):
+        return None
+    cuda_include = os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include") if os.path.isabs(_nvcc()) else "/usr/local/cuda/include"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-c", NATIVE_SOURCE, "-o", os.path.join(CSRC, "native.o"),
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)]
+    for d in cpp_extension.include_paths() + [sysconfig.get_paths()["include"], cuda_include]:
+        cmd += ["-isystem", d]
+    link = ["g++", "-shared", "-o", NATIVE, os.path.join(CSRC, "native.o"), "-L" + HERE, "-l:libquads.so", "-Wl,-rpath,$ORIGIN",
+            "-L" + lib_dir, "-Wl,-rpath," + lib_dir, "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    return subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True), link
 
 
 def build(force=False, verbose=False):
-    if not force and not needs_build():
-        return LIB
+    native = None
+    if force or _older(NATIVE, [NATIVE_SOURCE, os.path.join(CSRC, HEADERS[-1])]):
+        native = _start_native()
+    if force or needs_build():
+        _build_lib(verbose)
+    if native is not None:
+        out, _ = native[0].communicate()
+        if native[0].returncode != 0:
+            sys.stderr.write(out)
+            raise RuntimeError("g++ failed on native.cpp")
+        subprocess.check_call(native[1])
+    return LIB
+
+
+def _build_lib(verbose):
     objs = []
     procs = []
     for src in SOURCES:
@@ -43,7 +77,6 @@ def build(force=False, verbose=False):
             raise RuntimeError("nvcc failed on %s" % src)
     cmd = [_nvcc(), "-shared", "-o", LIB] + objs + ["-lcudart_static", "-ldl", "-lrt", "-lpthread"]
     subprocess.check_call(cmd)
-    return LIB
 
 
 if __name__ == "__main__":
