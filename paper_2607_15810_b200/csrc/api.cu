@@ -721,7 +721,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
     CUtensorMap tm_a, tm_b;
     if ((s = make_bf16_map(&tm_a, A_op, (uint64_t)T, (uint64_t)H)) != QUADS_OK) return s;
     if ((s = make_bf16_map(&tm_b, B_op, (uint64_t)a->N, (uint64_t)H)) != QUADS_OK) return s;
-    s = launch_gemm_bf16(tm_a, tm_b, T, a->N, H, static_cast<uint16_t*>(a->out), header + kHdrStatus, di.sm_count, st);
+    s = launch_gemm_bf16(tm_a, tm_b, T, a->N, H, A_op == a->x, B_op == a->w13_bf16, static_cast<uint16_t*>(a->out), header + kHdrStatus, di.sm_count, st);
     if (s != QUADS_OK) return s;
     QUADS_CUDA_OK(cudaGetLastError());
     return QUADS_OK;

@@ -52,10 +52,6 @@ struct __align__(8) DBarriers {
   int abort_flag;
 };
 
-__device__ __forceinline__ void st_cluster_f4(uint32_t addr, float a, float b, float c, float d) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
-}
-
 template <int BN>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_dense_kernel(const GemmParams p, int split_log2, const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_r,
@@ -217,14 +213,8 @@ gemm_dense_kernel(const GemmParams p, int split_log2, const __grid_constant__ CU
   const int r_log2 = w_log2 - 3;                       // a thread takes eight columns of a row
   for (int i = threadIdx.x - 64; i < rows_valid << r_log2; i += 32 * kEpiWarps) {
     const int r = i >> r_log2, c = (i & ((1 << r_log2) - 1)) * 8;
-    float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
-#pragma unroll 4
-    for (int s = 0; s < split; ++s) {
-      const float4* v = reinterpret_cast<const float4*>(part + (s * 128 + r) * ld + c);
-      const float4 a = v[0], b = v[1];
-      lo.x += a.x; lo.y += a.y; lo.z += a.z; lo.w += a.w;
-      hi.x += b.x; hi.y += b.y; hi.z += b.z; hi.w += b.w;
-    }
+    float4 lo, hi;
+    sum_parts(part + r * ld + c, 128 * ld, split, lo, hi);
     *reinterpret_cast<uint4*>(p.out_bf16 + (size_t)(mt * 128 + r) * p.n_out + n0 + c) =
         make_uint4(f32x2_to_bf16x2(lo.x * scale, lo.y * scale), f32x2_to_bf16x2(lo.z * scale, lo.w * scale),
                    f32x2_to_bf16x2(hi.x * scale, hi.y * scale), f32x2_to_bf16x2(hi.z * scale, hi.w * scale));
@@ -238,7 +228,11 @@ quads_status launch_bn(GemmParams p, int split, const GemmMaps& m, cudaStream_t 
   QUADS_CUDA_OK(set_max_dynamic_smem<gemm_dense_kernel<BN>>(DCfg<BN>::kSmemBytes));
   int split_log2 = 0;
   while (1 << split_log2 < split) ++split_log2;
-  QUADS_CUDA_OK(launch_clusters(gemm_dense_kernel<BN>, tiles * split, split, kThreads, (size_t)DCfg<BN>::kSmemBytes, stream, p, split_log2, m.a, m.r, m.b));
+  constexpr size_t kSmem = DCfg<BN>::kSmemBytes;
+  if (split == 1)
+    QUADS_CUDA_OK(launch_kernel(gemm_dense_kernel<BN>, dim3(tiles), dim3(kThreads), kSmem, stream, p, split_log2, m.a, m.r, m.b));
+  else
+    QUADS_CUDA_OK(launch_clusters(gemm_dense_kernel<BN>, tiles * split, split, kThreads, kSmem, stream, p, split_log2, m.a, m.r, m.b));
   return QUADS_OK;
 }
 

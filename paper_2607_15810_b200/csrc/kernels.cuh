@@ -222,7 +222,8 @@ quads_status launch_gemm_dense(const GemmParams& p, const GemmMaps& m, int n_sms
 // ---- gemm_bf16.cu: out[T, N] = A[T, K] B[N, K]^T, bf16 operands (tensor maps with boxes of 64 elements x kBf16BoxRows
 // rows, 128-byte swizzle), float32 accumulation, bf16 output; K % 64 == 0, N % 128 == 0
 constexpr int kBf16BoxRows = 64;
-quads_status launch_gemm_bf16(const CUtensorMap& tm_a, const CUtensorMap& tm_b, int T, int N, int K, uint16_t* out,
+// a_early / b_early: the operand is older than the preceding kernel of the stream, which has itself waited for its predecessor.
+quads_status launch_gemm_bf16(const CUtensorMap& tm_a, const CUtensorMap& tm_b, int T, int N, int K, bool a_early, bool b_early, uint16_t* out,
                               int32_t* status, int n_sms, cudaStream_t stream);
 
 // ---- fp8.cu: the FP8 W8A8 comparison path

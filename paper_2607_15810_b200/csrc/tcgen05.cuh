@@ -105,13 +105,12 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols) {
 }
 // Arrive on `bar` once all tcgen05 operations issued so far by this thread are
 // complete.  CG == 2: the arrival is delivered to the barrier at the same
-// shared-memory offset in both CTAs of the pair.
+// shared-memory offset in both CTAs of the pair (`mask`: their ranks in the cluster).
 template <int CG>
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
+__device__ __forceinline__ void tc_commit(uint32_t bar, uint16_t mask = 3) {
   if (CG == 1) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
   } else {
-    const uint16_t mask = 3;
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
                  ::"r"(bar), "h"(mask) : "memory");
   }
@@ -162,6 +161,20 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t saddr, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
   return r;
+}
+__device__ __forceinline__ void st_cluster_f4(uint32_t addr, float a, float b, float c, float d) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+// Eight consecutive sums of `n` partial tiles `pitch` floats apart, added in order.
+__device__ __forceinline__ void sum_parts(const float* v, int pitch, int n, float4& lo, float4& hi) {
+  lo = make_float4(0.f, 0.f, 0.f, 0.f);
+  hi = lo;
+#pragma unroll 4
+  for (int s = 0; s < n; ++s, v += pitch) {
+    const float4 a = reinterpret_cast<const float4*>(v)[0], b = reinterpret_cast<const float4*>(v)[1];
+    lo.x += a.x; lo.y += a.y; lo.z += a.z; lo.w += a.w;
+    hi.x += b.x; hi.y += b.y; hi.z += b.z; hi.w += b.w;
+  }
 }
 // No memory ordering: for hand-overs whose payload is tensor memory (ordered by tcgen05 fences),
 // so that the arrive does not wait for this thread's earlier global stores.

@@ -34,3 +34,26 @@ def test_dense_tiles_and_splits(T, K, N, nsel):
     MC.check_site1(res, dict(site13=o["site"]), nsel, {})
     got = MC.f32(res["out"]).astype(np.float64)
     assert float((np.abs(got - o["y64"]) / MC.gemm_tol(o["absdot"], o["y64"])).max()) <= 1.0
+
+
+@pytest.mark.parametrize("T,K,N", [
+    (1, 4096, 128),        # eight CTAs per tile
+    (70, 4096, 1024),      # four
+    (256, 2048, 2048),     # two, every row of both row tiles
+    (129, 384, 640),       # one, one row in the second row tile
+    (9000, 128, 384),      # tiles of 256 columns, half of the last one missing
+    (9000, 2176, 384)])    # the same number of tiles with a longer K: pairs, fewer tiles than pairs of SMs
+def test_bf16_product_of_one_wave(T, K, N):
+    """Against a float64 product of the same bf16 values: float32 accumulation of K exact products is within
+    K * 2^-24 * sum|a b| of it (partial sums of a split included), the result is rounded to bf16 once."""
+    from paper_2607_15810_b200 import binding as B
+    g = torch.Generator(device="cuda").manual_seed(T + K + N)
+    x = torch.randn(T, K, device="cuda", generator=g).to(torch.bfloat16)
+    w = (torch.randn(N, K, device="cuda", generator=g) * 0.05).to(torch.bfloat16)
+    res = B.dense_one_sided(x, B.W16A16, w_bf16=w)
+    torch.cuda.synchronize()
+    assert B.moe_async_status(res["workspace"]) == 0
+    want = x.double() @ w.double().t()
+    mag = x.double().abs() @ w.double().abs().t()
+    err = (res["out"].double() - want).abs()
+    assert bool((err <= K * 2.0 ** -24 * mag + 2.0 ** -8 * want.abs() + 1e-30).all())
