@@ -19,8 +19,8 @@
 // Every CTA loads what it needs itself; no load is shared across the cluster.
 //
 // One persistent CTA per SM, 19 warps:
-//   warp 0     producer: TMA tile loads of packed FP4 (128-byte swizzle) into a 3-stage
-//              shared-memory ring;
+//   warp 0     producer: TMA tile loads of packed FP4 (128-byte swizzle) into a ring of three
+//              shared-memory stages (four without the residual operand);
 //   warp 18    second producer: the bulk copies of the stage's 512-byte scale atoms (in the
 //              CTA-pair variant warp 0 issues those too, as TMA boxes, and this warp idles);
 //   warp 1     tensor-memory allocation; one thread copies scale atoms to TMEM
@@ -43,26 +43,27 @@ constexpr int kBM = 128;
 constexpr int kBN = 256;
 constexpr int kKSteps = kGemmKSteps;              // K = 64 MMAs per pipeline stage
 constexpr int kStageKBytes = kGemmStageKBytes;    // bytes of packed FP4 per row per stage
-constexpr int kTileA = kBM * kStageKBytes;
-constexpr int kSfA = kKSteps * 512;               // one atom (128 rows x 4 blocks) per K step
-constexpr int kSfB = 2 * kSfA;                    // scales of all 256 weight rows
-constexpr int kOffR = kTileA;
-constexpr int kOffB = 2 * kTileA;
 constexpr int kThreads = 608;
 constexpr int kEpiWarps = 16;
 constexpr int kTmemCols = 512;
 constexpr int kMaxTableTiles = 2048;               // M-tiles whose expert / row count fit the shared-memory tables
 constexpr int kTmemSfBase = 256;                  // accumulator: columns 0..255
 constexpr int kTmemSfPerBuf = 16 * kKSteps;       // SFA 4/step | SFR 4/step | SFB 8/step, double buffered
-
-template <int CG>
+// RES: the stage has room for the residual operand; without it another stage fits (a layer of 4096 tokens without compensation, H =
+// 2048 197.8 -> 184.8 us, with it at W13 only 229.5 -> 225.9; 1500 tokens 113.9 -> 111.1 and 131.0 -> 127.5).
+template <int CG, bool RES>
 struct Cfg {
-  static constexpr int kTileB = kBN * kStageKBytes / CG;     // weight rows held by one CTA
-  static constexpr int kStages = (CG == 1 ? 12 : 16) / kKSteps;   // ~216 KB of ring either way
+  static constexpr int kTileA = kBM * kStageKBytes;
+  static constexpr int kTileB = kBN * kStageKBytes / CG;        // weight rows held by one CTA
+  static constexpr int kSfA = kKSteps * 512;                      // one atom (128 rows x 4 blocks) per K step
+  static constexpr int kSfB = 2 * kSfA;                      // scales of all 256 weight rows
+  static constexpr int kOffR = kTileA;
+  static constexpr int kOffB = (RES ? 2 : 1) * kTileA;
   static constexpr int kOffSfA = kOffB + kTileB;
   static constexpr int kOffSfR = kOffSfA + kSfA;
-  static constexpr int kOffSfB = kOffSfR + kSfA;
-  static constexpr int kStageBytes = kOffSfB + kSfB;         // 73728 / 57344
+  static constexpr int kOffSfB = kOffSfA + (RES ? 2 : 1) * kSfA;
+  static constexpr int kStageBytes = kOffSfB + kSfB;         // 73728 / 57344 with the residual, 55296 / 38912 without
+  static constexpr int kStages = (216 + 8 * (CG - 1)) * 1024 / kStageBytes;      // 3 / 4, without the residual 4 / 5
   static constexpr int kBarOffset = kStages * kStageBytes;   // barriers after the ring
   static constexpr int kMetaBytes = 512 + (CG == 1 ? (2 * kMaxTableTiles + 4 * kMaxExperts) : 0);   // reciprocal table + per-tile tables
   static constexpr int kSmemBytes = kBarOffset + 256 + kMetaBytes + 1024; // + barrier block + tables + alignment slack
@@ -120,12 +121,12 @@ __device__ __forceinline__ float warp_colsum16(const float* v, int lane) {
   return d;
 }
 
-template <int EPI, int CG>
+template <int EPI, int CG, bool RES>
 __device__ __forceinline__ void gemm_body(const GemmParams& p, const CUtensorMap* tm_a, const CUtensorMap* tm_r,
                                           const CUtensorMap* tm_b, const CUtensorMap* tm_sfa,
                                           const CUtensorMap* tm_sfr, const CUtensorMap* tm_sfb) {
-  using C = Cfg<CG>;
-  constexpr int kStages = C::kStages;
+  using C = Cfg<CG, RES>;
+  constexpr int kStages = C::kStages, kTileA = C::kTileA, kSfA = C::kSfA, kOffR = C::kOffR, kOffB = C::kOffB;
   extern __shared__ uint8_t smem_dyn[];
   const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   uint8_t* smem_gen = smem_dyn + (smem_base - smem_u32(smem_dyn));
@@ -191,7 +192,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p, const CUtensorMap
   const int total_tiles = m_groups * p.n_tiles_n;
   const int kt_count = p.K >> 6;                    // scale atoms (K = 64 each) along K
   const int k_stages = (kt_count + kKSteps - 1) / kKSteps;
-  const bool resid = p.has_resid != 0;
+  const bool resid = RES && p.has_resid != 0;
   const int first_tile = blockIdx.x / CG, tile_step = gridDim.x / CG;
 
   // Two loading warps share a stage's copies: warp 0 the operand tiles (and the byte count), warp 18
@@ -289,9 +290,8 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p, const CUtensorMap
       bool ok = true;
       constexpr uint32_t idesc = idesc_nvf4<CG>();
       // constant high words of the two descriptor kinds; the low word carries the address
-      // swizzled K-major operand tiles: 8-row groups 8 * row bytes apart; 128-byte rows use the
-      // 128-byte swizzle (type 2), 64-byte rows the 64-byte swizzle (type 4)
-      constexpr uint32_t kSw128Hi = (uint32_t)((8 * kStageKBytes) >> 4) | (1u << 14) | ((kStageKBytes == 128 ? 2u : 4u) << 29);
+      // swizzled K-major operand tiles: 8-row groups 8 * row bytes apart, 128-byte swizzle (type 2)
+      constexpr uint32_t kSw128Hi = (uint32_t)((8 * kStageKBytes) >> 4) | (1u << 14) | (2u << 29);
       constexpr uint32_t kSfHi = (uint32_t)(128 >> 4) | (1u << 14);
       for (int tile = first_tile; tile < total_tiles && ok; tile += tile_step, ++it) {
         for (int ks = 0; ks < k_stages; ++ks, ++kcount) {
@@ -470,48 +470,49 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p, const CUtensorMap
   if (warp == 1) tmem_dealloc<CG>(tmem, kTmemCols);
 }
 
-template <int EPI>
+template <int EPI, bool RES>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_r,
             const __grid_constant__ CUtensorMap tm_b) {
-  gemm_body<EPI, 1>(p, &tm_a, &tm_r, &tm_b, nullptr, nullptr, nullptr);
+  gemm_body<EPI, 1, RES>(p, &tm_a, &tm_r, &tm_b, nullptr, nullptr, nullptr);
 }
 
-template <int EPI>
+template <int EPI, bool RES>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 gemm_kernel_pair(const GemmParams p, const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_r,
                  const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ CUtensorMap tm_sfa,
                  const __grid_constant__ CUtensorMap tm_sfr, const __grid_constant__ CUtensorMap tm_sfb) {
-  gemm_body<EPI, 2>(p, &tm_a, &tm_r, &tm_b, &tm_sfa, &tm_sfr, &tm_sfb);
+  gemm_body<EPI, 2, RES>(p, &tm_a, &tm_r, &tm_b, &tm_sfa, &tm_sfr, &tm_sfb);
 }
 
 }  // namespace
 
-template <int EPI>
+template <int EPI, bool RES>
 quads_status launch_one(const GemmParams& p, const GemmMaps& m, int n_sms, cudaStream_t stream) {
-  QUADS_CUDA_OK(set_max_dynamic_smem<gemm_kernel<EPI>>(Cfg<1>::kSmemBytes));
-  QUADS_CUDA_OK(launch_kernel(gemm_kernel<EPI>, dim3(n_sms), dim3(kThreads), (size_t)Cfg<1>::kSmemBytes, stream, p, m.a,
-                              m.r, m.b));
+  constexpr auto kKernel = gemm_kernel<EPI, RES>;
+  constexpr size_t kSmem = Cfg<1, RES>::kSmemBytes;
+  QUADS_CUDA_OK(set_max_dynamic_smem<kKernel>((int)kSmem));
+  QUADS_CUDA_OK(launch_kernel(kKernel, dim3(n_sms), dim3(kThreads), kSmem, stream, p, m.a, m.r, m.b));
+  return QUADS_OK;
+}
+template <int EPI, bool RES>
+quads_status launch_pair(const GemmParams& p, const GemmMaps& m, int n_sms, cudaStream_t stream) {
+  constexpr auto kKernel = gemm_kernel_pair<EPI, RES>;
+  constexpr size_t kSmem = Cfg<2, RES>::kSmemBytes;
+  QUADS_CUDA_OK(set_max_dynamic_smem<kKernel>((int)kSmem));
+  QUADS_CUDA_OK(launch_kernel(kKernel, dim3((n_sms / 2) * 2), dim3(kThreads), kSmem, stream, p, m.a, m.r, m.b, m.sfa, m.sfr, m.sfb));
   return QUADS_OK;
 }
 template <int EPI>
-quads_status launch_pair(const GemmParams& p, const GemmMaps& m, int n_sms, cudaStream_t stream) {
-  QUADS_CUDA_OK(set_max_dynamic_smem<gemm_kernel_pair<EPI>>(Cfg<2>::kSmemBytes));
-  QUADS_CUDA_OK(launch_kernel(gemm_kernel_pair<EPI>, dim3((n_sms / 2) * 2), dim3(kThreads), (size_t)Cfg<2>::kSmemBytes,
-                              stream, p, m.a, m.r, m.b, m.sfa, m.sfr, m.sfb));
-  return QUADS_OK;
+quads_status launch_epi(int cta_group, const GemmParams& p, const GemmMaps& m, int n_sms, cudaStream_t stream) {
+  if (cta_group == 2) return p.has_resid ? launch_pair<EPI, true>(p, m, n_sms, stream) : launch_pair<EPI, false>(p, m, n_sms, stream);
+  return p.has_resid ? launch_one<EPI, true>(p, m, n_sms, stream) : launch_one<EPI, false>(p, m, n_sms, stream);
 }
 
-quads_status launch_gemm(int epi, int cta_group, const GemmParams& p, const GemmMaps& m, int n_sms,
-                         cudaStream_t stream) {
-  if (cta_group == 2) {
-    return epi == kEpiStore ? launch_pair<kEpiStore>(p, m, n_sms, stream)
-                            : (epi == kEpiSwiGLU ? launch_pair<kEpiSwiGLU>(p, m, n_sms, stream)
-                                                 : launch_pair<kEpiCombine>(p, m, n_sms, stream));
-  }
-  return epi == kEpiStore ? launch_one<kEpiStore>(p, m, n_sms, stream)
-                          : (epi == kEpiSwiGLU ? launch_one<kEpiSwiGLU>(p, m, n_sms, stream)
-                                               : launch_one<kEpiCombine>(p, m, n_sms, stream));
+quads_status launch_gemm(int epi, int cta_group, const GemmParams& p, const GemmMaps& m, int n_sms, cudaStream_t stream) {
+  return epi == kEpiStore ? launch_epi<kEpiStore>(cta_group, p, m, n_sms, stream)
+                          : (epi == kEpiSwiGLU ? launch_epi<kEpiSwiGLU>(cta_group, p, m, n_sms, stream)
+                                               : launch_epi<kEpiCombine>(cta_group, p, m, n_sms, stream));
 }
 
 }  // namespace quads

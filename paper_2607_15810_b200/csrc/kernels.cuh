@@ -145,10 +145,7 @@ quads_status launch_route_small(const SmallRouteArgs& a, cudaStream_t st);
 quads_status launch_front_small(const SmallFrontArgs& a, cudaStream_t st);
 
 // ---- gemm.cu
-#ifndef QUADS_GEMM_KSTEPS
-#define QUADS_GEMM_KSTEPS 4
-#endif
-constexpr int kGemmKSteps = QUADS_GEMM_KSTEPS;        // K = 64 MMAs per pipeline stage (2 or 4)
+constexpr int kGemmKSteps = 4;                        // K = 64 MMAs per pipeline stage
 constexpr int kGemmStageKBytes = 32 * kGemmKSteps;    // packed FP4 bytes per operand row per stage
 enum { kEpiStore = 0, kEpiSwiGLU = 1, kEpiCombine = 2 };
 
