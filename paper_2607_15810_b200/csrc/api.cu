@@ -224,6 +224,11 @@ quads_status launch_combine(const uint16_t* y_pad, const int32_t* pos_pad, const
   return QUADS_OK;
 }
 
+// CTAs (and partial maxima) of the first pass of a single-tensor quantization of `chunks` eight-element chunks.
+int amax_parts_for(int64_t chunks, int sm_count) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>((chunks + 2047) / 2048, std::min(sm_count * 8, kAmaxPartsMax - 1)));
+}
+
 // Zeroes the first `bytes` (a multiple of 16) of a workspace.
 cudaError_t clear_words(uint8_t* p, size_t bytes, cudaStream_t st) {
   const int n = (int)(bytes / 16);
@@ -321,8 +326,9 @@ static quads_status quantize_common(const void* x, int64_t n_tensors, int64_t ro
   int n_parts = 0;
   if (two_pass) {
     const int64_t chunks = rows * (K / 8);
-    n_parts = (int)std::max<int64_t>(1, std::min<int64_t>((chunks + 2047) / 2048, std::min(di.sm_count * 8, kAmaxPartsMax)));
-    QUADS_CUDA_OK(launch_kernel(amax_partial_kernel, dim3(n_parts), dim3(256), (size_t)0, st, xp, rows, K, ld, amax_bits));
+    n_parts = amax_parts_for(chunks, di.sm_count);
+    QUADS_CUDA_OK(launch_kernel(amax_partial_kernel, dim3(n_parts), dim3(256), (size_t)0, st, xp, rows, K, ld, amax_bits,
+                                static_cast<uint32_t*>(nullptr), 0, static_cast<uint32_t*>(nullptr), 0));
   }
   uint16_t* fqp = static_cast<uint16_t*>(fq);
   int nt = (int)n_tensors;
@@ -697,7 +703,20 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   trace_mark("start", st);
   // header (status word included) and the amax word start at zero
   const bool decodes = a->operand_mode == QUADS_W4A16;      // its first kernel clears the status word, all that it needs
-  if (!small && !decodes) QUADS_CUDA_OK(clear_words(ws, L.ids, st));
+  // A dense projection behind the small batches: its first kernel takes x's partial maxima, and clears as well, while the quantization's
+  // CTAs need not meet, i.e. no cooperative launch, which waits for the chip to be empty and lets nothing start behind it.  For a
+  // large x the CTAs' own maxima are ahead: they find the rows they read again nearer (loops, us, so / cooperative: 520 x 1024 ->
+  // 1024 18.8 / 20.5, 1000 x 2048 -> 1024 23.0 / 24.8, 2000 x 4096 -> 1024 39.2 / 39.1, 4000 x 2048 -> 1024 34.1 / 34.8, 4000 x 4096 ->
+  // 1024 50.6 / 49.5, 8192 x 4096 -> 1024 83.4 / 78.8).
+  const bool amax_first = dense && !small && a->operand_mode == QUADS_W4A4 && !a->a13_gs && (int64_t)T * H <= (int64_t)1 << 23;
+  int n_amax_parts = 0;
+  if (amax_first) {
+    n_amax_parts = amax_parts_for((int64_t)T * (H / 8), di.sm_count);
+    QUADS_CUDA_OK(launch_kernel(amax_partial_kernel, dim3(n_amax_parts), dim3(256), (size_t)0, st, x, (int64_t)T, (int64_t)H, (int64_t)H, amax_bits,
+                                reinterpret_cast<uint32_t*>(header), kHdrWords, reinterpret_cast<uint32_t*>(P(L.col_arrivals)), kQuantColsMax));
+  } else if (!small && !decodes) {
+    QUADS_CUDA_OK(clear_words(ws, L.ids, st));
+  }
   trace_mark("clear", st);
 
   if (dense && a->operand_mode != QUADS_W4A4) {
@@ -765,6 +784,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
     QuantRowsArgs q{};
     q.x = x; q.T = T; q.H = H; q.with_residual = nsel13 > 0; q.sf_tiled = dense;
     q.gs_in = a->a13_gs; q.amax_bits = amax_bits;
+    if (amax_first) { q.amax_parts = amax_bits; q.n_amax_parts = n_amax_parts; q.amax_bits = amax_bits + kAmaxPartsMax - 1; }
     q.arrivals = reinterpret_cast<unsigned int*>(header + kHdrArrivals);
     q.status = header + kHdrStatus; q.gs_store = a->a13_gs_out;
     q.xq = P(dense ? L.xq_pad : L.xq_tok); q.xsf = P(dense ? L.xsf : L.xsf_tok);
@@ -837,7 +857,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   g.header = header; g.tile_expert = tile_expert; g.tile_rows = tile_rows;
   g.a_sf = P(L.xsf); g.r_sf = P(L.rsf);
   g.b_sf = a->w13_sf; g.b_sf_expert_stride = quads_sf_tiled_bytes(N1, H);
-  g.b_gs = a->w13_gs; g.a_gs = a->a13_gs; g.a_amax_bits = amax_bits;
+  g.b_gs = a->w13_gs; g.a_gs = a->a13_gs; g.a_amax_bits = amax_first ? amax_bits + kAmaxPartsMax - 1 : amax_bits;
   g.tile_prefix = tile_prefix; g.offsets = offsets;
   g.row_token = row_token; g.xsf_tok = P(L.xsf_tok); g.rsf_tok = P(L.rsf_tok);
   g.status = header + kHdrStatus;

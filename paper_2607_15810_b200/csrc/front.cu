@@ -71,7 +71,20 @@ __device__ __forceinline__ void quant_role(const QuantRowsArgs& p, int cta, int 
   const int kb = col * p.bw + blk;
   const int r0 = rg * p.rows_per_cta + lane_r, r1 = min(p.T, (rg + 1) * p.rows_per_cta);
   const uint16_t* xk = p.x + kb * 16;
-  if (!p.gs_in) {
+  if (!p.gs_in && p.amax_parts) {
+    uint32_t m = 0;
+    for (int i = threadIdx.x; i < p.n_amax_parts; i += 256) m = max(m, __ldcg(p.amax_parts + i));
+    m = __reduce_max_sync(0xFFFFFFFFu, m);
+    if ((threadIdx.x & 31) == 0) s->wmax[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      uint32_t tm = 0;
+      for (int i = 0; i < 8; ++i) tm = max(tm, s->wmax[i]);
+      if (cta == 0) p.amax_bits[0] = tm;
+      s->gs = gs_from_amax_bits(tm);
+    }
+    __syncthreads();
+  } else if (!p.gs_in) {
     uint32_t m = 0;
     int r = r0;
     for (; r + 3 * lanes < r1; r += 4 * lanes) {
@@ -363,7 +376,7 @@ quads_status launch_quant_rows(const QuantRowsArgs& args, int sm_count, cudaStre
   int per_sm = 0;
   QUADS_CUDA_OK(resident_per_sm(quant_rows_kernel, 256, &cache, &per_sm));
   const int n = plan_quant(&q, per_sm * sm_count);
-  if (!q.gs_in) {                                    // its CTAs wait for one another
+  if (!q.gs_in && !q.amax_parts) {                   // its CTAs wait for one another
     void* kargs[] = {&q};
     QUADS_CUDA_OK(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(quant_rows_kernel), dim3(n), dim3(256), kargs, 0, st));
     note_launch();

@@ -24,7 +24,8 @@ __global__ void fused_quantize_kernel(const uint16_t* x, int64_t rows, int64_t K
                                       uint8_t* q, uint8_t* sf, uint16_t* fq, float* gs_out, int sf_tiled,
                                       int64_t sf_tensor_stride, int n_groups, long long wait_cycles,
                                       int extra_arrivals, const uint32_t* amax_parts, int n_amax_parts);
-__global__ void amax_partial_kernel(const uint16_t* x, int64_t rows, int64_t K, int64_t ld, uint32_t* partials);
+__global__ void amax_partial_kernel(const uint16_t* x, int64_t rows, int64_t K, int64_t ld, uint32_t* partials, uint32_t* zero0, int n0,
+                                    uint32_t* zero1, int n1);
 // Fake-quant of a batch of tensors through shared-memory rings of bulk copies (one CTA per SM,
 // four groups of 7 consumer warps + 1 producer warp, one ring of 14 KB stages per group).
 constexpr int kRingThreads = 1024;
@@ -66,9 +67,11 @@ constexpr int kQuantRowsPerSm = 4;    // resident CTAs of the front kernels
 struct QuantRowsArgs {
   const uint16_t* x;
   int T, H, with_residual, sf_tiled;
-  const float* gs_in;                 // per-tensor scale, or NULL: amax-derived (then the launch is cooperative)
-  uint32_t* amax_bits;
-  unsigned int* arrivals;             // it and amax_bits are zero on entry
+  const float* gs_in;                 // per-tensor scale, or NULL: amax-derived, ...
+  const uint32_t* amax_parts;         // ... from n_amax_parts partial maxima of the preceding kernel, or (NULL) by the CTAs themselves
+  int n_amax_parts;
+  uint32_t* amax_bits;                // out; zero on entry where the CTAs derive it
+  unsigned int* arrivals;             // zero on entry
   int32_t* status;
   float* gs_store;                    // exports, each may be NULL
   uint8_t *xq, *xsf, *rq, *rsf;

@@ -76,10 +76,16 @@ __global__ void __launch_bounds__(256) amax_kernel(const uint16_t* __restrict__ 
 // ---------------------------------------------------------------------------
 // First pass of the single-tensor quantizer: CTA b leaves the |x| maximum of its share in
 // partials[b] (every CTA stores, so the array needs no initialisation and there is no atomic);
-// the 32-byte loads ask L2 to keep the lines for the pass that follows.
+// the 32-byte loads ask L2 to keep the lines for the pass that follows.  In front of a dense projection it also
+// clears the words that the call starts at zero (n0 and n1 words, by CTA 0).
 __global__ void __launch_bounds__(256) amax_partial_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t K,
-                                                           int64_t ld, uint32_t* __restrict__ partials) {
+                                                           int64_t ld, uint32_t* __restrict__ partials, uint32_t* __restrict__ zero0,
+                                                           int n0, uint32_t* __restrict__ zero1, int n1) {
   pdl_sync();
+  if (blockIdx.x == 0) {
+    for (int i = threadIdx.x; i < n0; i += 256) zero0[i] = 0u;
+    for (int i = threadIdx.x; i < n1; i += 256) zero1[i] = 0u;
+  }
   const int64_t k16 = K >> 4, nblk = rows * k16;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   uint32_t m = 0;

@@ -57,3 +57,26 @@ def test_bf16_product_of_one_wave(T, K, N):
     mag = x.double().abs() @ w.double().abs().t()
     err = (res["out"].double() - want).abs()
     assert bool((err <= K * 2.0 ** -24 * mag + 2.0 ** -8 * want.abs() + 1e-30).all())
+
+
+@pytest.mark.parametrize("T,K", [(513, 512), (2049, 4096), (2047, 4096)])      # either side of the two forms of the amax
+def test_scale_of_x_and_scores_behind_either_amax(T, K):
+    """The per-tensor scale and the codes are those of the stand-alone quantizer, twice in a row on one workspace (words of the
+    first call must not survive)."""
+    from paper_2607_15810_b200 import binding as B
+    g = torch.Generator(device="cuda").manual_seed(T)
+    w = B.fake_quant_weights(torch.randn(1, 128, K, device="cuda", generator=g).to(torch.bfloat16), want_fq=False, sf_layout=B.SF_TILED)
+    ws = torch.empty(B.moe_workspace_bytes(T, K, 0, 1, 1, 128), dtype=torch.uint8, device="cuda").fill_(255)
+    for scale in (30.0, 0.1):
+        x = (torch.randn(T, K, device="cuda", generator=g) * scale).to(torch.bfloat16)
+        res = B.dense_w4a4_rac(x, w, K // 4, export=True, workspace=ws)
+        q, sf, gs = B.quantize_nvfp4(x)
+        torch.cuda.synchronize()
+        assert B.moe_async_status(ws) == 0
+        assert torch.equal(res["a13_gs"], gs) and torch.equal(res["xq"], q) and torch.equal(res["xsf"], sf)
+        scores = B.rac_channel_scores(x)
+        kept = torch.zeros(K, dtype=torch.bool, device="cuda")
+        kept[res["sel13"].long()] = True
+        assert int(kept.sum()) == K // 4
+        # float32 partial sums of T squares, added in float64: relative error below T * 2^-24 each
+        assert float(scores[kept].min()) >= float(scores[~kept].max()) * (1 - 2 * T * 2.0 ** -24)
