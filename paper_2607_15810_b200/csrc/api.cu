@@ -246,11 +246,11 @@ quads_status launch_select_mask(uint8_t* codes, int n_rows_fixed, uint32_t flip,
 }
 
 quads_status launch_dequantize(const uint8_t* q, const uint8_t* sf, const float* gs, int64_t n_tensors, int64_t nblk, int64_t K, int tiled,
-                               int64_t sf_stride, uint16_t* out, int32_t* zero, int sm_count, cudaStream_t st) {
+                               int64_t sf_stride, uint16_t* out, int sm_count, cudaStream_t st) {
   // four blocks of 16 elements per thread, and no more CTAs than a few rounds of the chip
   const int64_t per_tensor = std::min<int64_t>((nblk + 1023) / 1024, std::max<int64_t>(1, (int64_t)sm_count * 16 / n_tensors));
   QUADS_CUDA_OK(launch_kernel(dequantize_kernel, dim3((unsigned)per_tensor, (unsigned)n_tensors), dim3(256), (size_t)0, st, q, sf, gs, nblk,
-                              (uint32_t)(K / 16), (int)((K + 63) / 64), tiled, sf_stride, out, zero));
+                              (uint32_t)(K / 16), (int)((K + 63) / 64), tiled, sf_stride, out));
   QUADS_CUDA_OK(cudaGetLastError());
   return QUADS_OK;
 }
@@ -429,7 +429,7 @@ quads_status quads_dequantize_nvfp4(const uint8_t* q, const uint8_t* sf, const f
   if (s != QUADS_OK) return s;
   const int tiled = sf_layout == QUADS_SF_TILED;
   const int64_t sf_stride = tiled ? (int64_t)quads_sf_tiled_bytes(rows, K) : nblk;
-  return launch_dequantize(q, sf, gs, n_tensors, nblk, K, tiled, sf_stride, static_cast<uint16_t*>(out), nullptr, di.sm_count,
+  return launch_dequantize(q, sf, gs, n_tensors, nblk, K, tiled, sf_stride, static_cast<uint16_t*>(out), di.sm_count,
                            static_cast<cudaStream_t>(cuda_stream));
 }
 
@@ -701,32 +701,33 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
                      !(dense && H > 2048 && (int64_t)T * H > 192 * 4096);
   g_trace.n = 0;
   trace_mark("start", st);
-  // header (status word included) and the amax word start at zero
-  const bool decodes = a->operand_mode == QUADS_W4A16;      // its first kernel clears the status word, all that it needs
+  // header (status word included) and the amax word start at zero; the one-sided modes need the status word alone, which
+  // their last kernel clears
+  const bool one_sided = a->operand_mode != QUADS_W4A4;
   // A dense projection behind the small batches: its first kernel takes x's partial maxima, and clears as well, while the quantization's
   // CTAs need not meet, i.e. no cooperative launch, which waits for the chip to be empty and lets nothing start behind it.  For a
   // large x the CTAs' own maxima are ahead: they find the rows they read again nearer (loops, us, so / cooperative: 520 x 1024 ->
   // 1024 18.8 / 20.5, 1000 x 2048 -> 1024 23.0 / 24.8, 2000 x 4096 -> 1024 39.2 / 39.1, 4000 x 2048 -> 1024 34.1 / 34.8, 4000 x 4096 ->
   // 1024 50.6 / 49.5, 8192 x 4096 -> 1024 83.4 / 78.8).
-  const bool amax_first = dense && !small && a->operand_mode == QUADS_W4A4 && !a->a13_gs && (int64_t)T * H <= (int64_t)1 << 23;
+  const bool amax_first = dense && !small && !one_sided && !a->a13_gs && (int64_t)T * H <= (int64_t)1 << 23;
   int n_amax_parts = 0;
   if (amax_first) {
     n_amax_parts = amax_parts_for((int64_t)T * (H / 8), di.sm_count);
     QUADS_CUDA_OK(launch_kernel(amax_partial_kernel, dim3(n_amax_parts), dim3(256), (size_t)0, st, x, (int64_t)T, (int64_t)H, (int64_t)H, amax_bits,
                                 reinterpret_cast<uint32_t*>(header), kHdrWords, reinterpret_cast<uint32_t*>(P(L.col_arrivals)), kQuantColsMax));
-  } else if (!small && !decodes) {
+  } else if (!small && !one_sided) {
     QUADS_CUDA_OK(clear_words(ws, L.ids, st));
   }
   trace_mark("clear", st);
 
-  if (dense && a->operand_mode != QUADS_W4A4) {
+  if (one_sided) {
     // ---- one-sided modes: decode the NVFP4 side to bf16 with the library's own kernels, then one
     // bf16 tensor-core product
     uint16_t* dec = reinterpret_cast<uint16_t*>(P(L.dec));
     const void *A_op = a->x, *B_op = a->w13_bf16;
     if (a->operand_mode == QUADS_W4A16) {
       s = launch_dequantize(a->w13_q, a->w13_sf, a->w13_gs, 1, (int64_t)a->N * (H / 16), H, 1, (int64_t)quads_sf_tiled_bytes(a->N, H), dec,
-                            header + kHdrStatus, di.sm_count, st);
+                            di.sm_count, st);
       if (s != QUADS_OK) return s;
       B_op = dec;
     } else if (a->operand_mode == QUADS_W16A4) {
@@ -740,7 +741,8 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
     CUtensorMap tm_a, tm_b;
     if ((s = make_bf16_map(&tm_a, A_op, (uint64_t)T, (uint64_t)H)) != QUADS_OK) return s;
     if ((s = make_bf16_map(&tm_b, B_op, (uint64_t)a->N, (uint64_t)H)) != QUADS_OK) return s;
-    s = launch_gemm_bf16(tm_a, tm_b, T, a->N, H, A_op == a->x, B_op == a->w13_bf16, static_cast<uint16_t*>(a->out), header + kHdrStatus, di.sm_count, st);
+    s = launch_gemm_bf16(tm_a, tm_b, T, a->N, H, a->operand_mode == QUADS_W4A16, a->operand_mode == QUADS_W16A4,
+                         static_cast<uint16_t*>(a->out), header + kHdrStatus, di.sm_count, st);
     if (s != QUADS_OK) return s;
     QUADS_CUDA_OK(cudaGetLastError());
     return QUADS_OK;

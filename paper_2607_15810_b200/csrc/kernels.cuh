@@ -38,7 +38,7 @@ __global__ void fake_quant_ring_kernel(const uint16_t* x, int64_t nblk, int64_t 
                                        float* gs_out, int sf_tiled, int64_t sf_tensor_stride, uint32_t k16,
                                        int kt_count);
 __global__ void dequantize_kernel(const uint8_t* q, const uint8_t* sf, const float* gs, int64_t nblk, uint32_t k16,
-                                  int kt_count, int sf_tiled, int64_t sf_tensor_stride, uint16_t* out, int32_t* zero);
+                                  int kt_count, int sf_tiled, int64_t sf_tensor_stride, uint16_t* out);
 __global__ void channel_stats_kernel(const uint16_t* x, int T, int H, const float* gs_in, const uint32_t* amax_bits,
                                      int rows_per_cta, float* partials);
 constexpr int kScoreSlices = 16;

@@ -644,14 +644,13 @@ fake_quant_ring_kernel(const uint16_t* __restrict__ x, int64_t nblk, int64_t ten
 // blockIdx.y = tensor; a thread decodes 16-element blocks, 8 B of codes + 1 B of scale in, one 32-byte store out,
 // four blocks in flight.  In the one-sided dense projection the result is read back out of L2 by the product
 // behind it (no streaming hint on the stores).  4096 x 4096 in front of that product: 11.5 us with one block at
-// a time and a 64-bit division for its tensor, 7.5 now (43 MB: 6.6 us).  `zero` (or NULL) is a word the kernel clears.
+// a time and a 64-bit division for its tensor, 7.5 now (43 MB: 6.6 us).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
 dequantize_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ sf, const float* __restrict__ gs,
                   int64_t nblk, uint32_t k16, int kt_count, int sf_tiled, int64_t sf_tensor_stride,
-                  uint16_t* __restrict__ out, int32_t* __restrict__ zero) {
+                  uint16_t* __restrict__ out) {
   pdl_sync();
-  if (zero && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *zero = 0;
   QuantSink geo{nullptr, nullptr, nullptr, sf_tiled, k16, kt_count, 0, 0};
   quant_sink_divisor(geo);
   const size_t t = blockIdx.y;
