@@ -327,7 +327,7 @@ static quads_status quantize_common(const void* x, int64_t n_tensors, int64_t ro
   if (two_pass) {
     const int64_t chunks = rows * (K / 8);
     n_parts = amax_parts_for(chunks, di.sm_count);
-    QUADS_CUDA_OK(launch_kernel(amax_partial_kernel, dim3(n_parts), dim3(256), (size_t)0, st, xp, rows, K, ld, amax_bits,
+    QUADS_CUDA_OK(launch_kernel(amax_partial_kernel<false>, dim3(n_parts), dim3(256), (size_t)0, st, xp, rows, K, ld, amax_bits,
                                 static_cast<uint32_t*>(nullptr), 0, static_cast<uint32_t*>(nullptr), 0));
   }
   uint16_t* fqp = static_cast<uint16_t*>(fq);
@@ -713,7 +713,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   int n_amax_parts = 0;
   if (amax_first) {
     n_amax_parts = amax_parts_for((int64_t)T * (H / 8), di.sm_count);
-    QUADS_CUDA_OK(launch_kernel(amax_partial_kernel, dim3(n_amax_parts), dim3(256), (size_t)0, st, x, (int64_t)T, (int64_t)H, (int64_t)H, amax_bits,
+    QUADS_CUDA_OK(launch_kernel(amax_partial_kernel<true>, dim3(n_amax_parts), dim3(256), (size_t)0, st, x, (int64_t)T, (int64_t)H, (int64_t)H, amax_bits,
                                 reinterpret_cast<uint32_t*>(header), kHdrWords, reinterpret_cast<uint32_t*>(P(L.col_arrivals)), kQuantColsMax));
   } else if (!small && !one_sided) {
     QUADS_CUDA_OK(clear_words(ws, L.ids, st));

@@ -25,7 +25,8 @@ namespace quads {
 // totals, one reduction per CTA and channel, cost 1 to 2 us less (dense 8192 x 4096 -> 4096 157.4 us, 158.6 so; 1200 x
 // 512 -> 128 18.5, 20.5; a MoE layer of 1500 tokens the same), but need a bound on the residual, which a given
 // scale that x exceeds does not have, and lose channels that are small beside an outlier.
-// Issue-bound: about 400 issue cycles per warp and block, 128 of them in the two conversions to E2M1.
+// Bound by the arithmetic, about 240 cycles per warp and block with its loads, 64 of them in the two conversions to E2M1, and by
+// reading x a second time out of L2 (some 6.6 TB/s).
 // Dense projection 8192 x 4096 -> 4096: amax, quantization, score reduction, ranking and copy took 16 + 27 + 12 +
 // 12 + 28 us as kernels of their own; this one takes about 40 and the in-place mask behind it 10 (whole call
 // 205 -> 159 us).

@@ -24,6 +24,7 @@ __global__ void fused_quantize_kernel(const uint16_t* x, int64_t rows, int64_t K
                                       uint8_t* q, uint8_t* sf, uint16_t* fq, float* gs_out, int sf_tiled,
                                       int64_t sf_tensor_stride, int n_groups, long long wait_cycles,
                                       int extra_arrivals, const uint32_t* amax_parts, int n_amax_parts);
+template <bool kClear>
 __global__ void amax_partial_kernel(const uint16_t* x, int64_t rows, int64_t K, int64_t ld, uint32_t* partials, uint32_t* zero0, int n0,
                                     uint32_t* zero1, int n1);
 // Fake-quant of a batch of tensors through shared-memory rings of bulk copies (one CTA per SM,

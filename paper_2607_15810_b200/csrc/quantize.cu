@@ -76,13 +76,14 @@ __global__ void __launch_bounds__(256) amax_kernel(const uint16_t* __restrict__ 
 // ---------------------------------------------------------------------------
 // First pass of the single-tensor quantizer: CTA b leaves the |x| maximum of its share in
 // partials[b] (every CTA stores, so the array needs no initialisation and there is no atomic);
-// the 32-byte loads ask L2 to keep the lines for the pass that follows.  In front of a dense projection it also
+// the 32-byte loads ask L2 to keep the lines for the pass that follows.  kClear: in front of a dense projection it also
 // clears the words that the call starts at zero (n0 and n1 words, by CTA 0).
+template <bool kClear>
 __global__ void __launch_bounds__(256) amax_partial_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t K,
                                                            int64_t ld, uint32_t* __restrict__ partials, uint32_t* __restrict__ zero0,
                                                            int n0, uint32_t* __restrict__ zero1, int n1) {
   pdl_sync();
-  if (blockIdx.x == 0) {
+  if (kClear && blockIdx.x == 0) {
     for (int i = threadIdx.x; i < n0; i += 256) zero0[i] = 0u;
     for (int i = threadIdx.x; i < n1; i += 256) zero1[i] = 0u;
   }
@@ -119,6 +120,9 @@ __global__ void __launch_bounds__(256) amax_partial_kernel(const uint16_t* __res
     partials[blockIdx.x] = t << 16;
   }
 }
+
+template __global__ void amax_partial_kernel<false>(const uint16_t*, int64_t, int64_t, int64_t, uint32_t*, uint32_t*, int, uint32_t*, int);
+template __global__ void amax_partial_kernel<true>(const uint16_t*, int64_t, int64_t, int64_t, uint32_t*, uint32_t*, int, uint32_t*, int);
 
 // Where the quantizer's outputs of one tensor go (any pointer may be null).
 struct QuantSink {
