@@ -27,13 +27,23 @@ def needs_build():
     return _older(LIB, [os.path.join(CSRC, s) for s in SOURCES + HEADERS])
 
 
+def _without_native(why):
+    """The binding does without _native.so; an object of older sources must not be what it finds."""
+    if os.path.exists(NATIVE):
+        os.remove(NATIVE)
+    sys.stderr.write("_native.so is not built (%s): the ordinary calls go through ctypes, at more host time each\n" % why)
+
+
 def _start_native():
-    """The compiler of _native.so, or None where the installed torch has no CUDA (the binding then does without)."""
-    import torch
-    from torch.utils import cpp_extension
+    """The compiler of _native.so and the link behind it, or None where something that it needs is missing."""
+    try:
+        import torch
+        from torch.utils import cpp_extension
+    except ImportError as e:
+        return _without_native(e)
     lib_dir = os.path.join(os.path.dirname(torch.__file__), "lib")
     if torch.version.cuda is None or not os.path.exists(os.path.join(lib_dir, "libc10_cuda.so")):
-        return None
+        return _without_native("a torch without CUDA")
     cuda_include = os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include") if os.path.isabs(_nvcc()) else "/usr/local/cuda/include"
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-c", NATIVE_SOURCE, "-o", os.path.join(CSRC, "native.o"),
            "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)]
@@ -41,21 +51,32 @@ def _start_native():
         cmd += ["-isystem", d]
     link = ["g++", "-shared", "-o", NATIVE, os.path.join(CSRC, "native.o"), "-L" + HERE, "-l:libquads.so", "-Wl,-rpath,$ORIGIN",
             "-L" + lib_dir, "-Wl,-rpath," + lib_dir, "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
-    return subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True), link
+    try:
+        return subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True), link
+    except OSError as e:
+        return _without_native(e)
+
+
+def _finish_native(compiler, link):
+    out, _ = compiler.communicate()
+    if compiler.returncode == 0:
+        done = subprocess.run(link, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+        if done.returncode == 0:
+            return
+        out += done.stdout
+    sys.stderr.write(out)
+    _without_native("g++ failed")
 
 
 def build(force=False, verbose=False):
+    """libquads.so, and where this machine has what it takes _native.so."""
     native = None
     if force or _older(NATIVE, [NATIVE_SOURCE, os.path.join(CSRC, HEADERS[-1])]):
         native = _start_native()
     if force or needs_build():
         _build_lib(verbose)
     if native is not None:
-        out, _ = native[0].communicate()
-        if native[0].returncode != 0:
-            sys.stderr.write(out)
-            raise RuntimeError("g++ failed on native.cpp")
-        subprocess.check_call(native[1])
+        _finish_native(*native)
     return LIB
 
 
