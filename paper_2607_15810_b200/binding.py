@@ -7,8 +7,11 @@ The ordinary calls -- plain CUDA tensors, no verification exports -- go through 
 same in a third of the host time; everything else through ctypes."""
 import ctypes as C
 import os
+import warnings
 
 import torch
+
+from . import build as _build
 
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libquads.so")
 if not os.path.exists(_LIB_PATH):
@@ -79,11 +82,22 @@ class QuadsError(RuntimeError):
         super().__init__(lib.quads_status_string(int(status)).decode())
 
 
-try:
-    from . import _native
+def _load_native():
+    """_native.so if it was built for this torch and this Python, or None."""
+    if not os.path.exists(_build.NATIVE):
+        return None
+    try:
+        if not _build.native_matches():
+            raise ImportError("built for another torch or Python")
+        from . import _native
+    except ImportError as e:
+        warnings.warn("_native.so is left out (%s): the ordinary calls go through ctypes, at more host time each" % e)
+        return None
     _native.set_error(QuadsError)
-except ImportError:                # a torch without CUDA, or another one than it was built for
-    _native = None
+    return _native
+
+
+_native = _load_native()
 
 
 def check(status):

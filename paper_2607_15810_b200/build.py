@@ -23,6 +23,26 @@ def _older(target, deps):
     return not os.path.exists(target) or any(os.path.getmtime(d) > os.path.getmtime(target) for d in deps)
 
 
+def native_tag():
+    """What _native.so has to have been compiled for: it reads torch's C++ objects through inline code, so another torch or Python may
+    load it (its symbols resolve) and then read wrong memory.  None without torch."""
+    try:
+        import torch
+    except ImportError:
+        return None
+    return "torch %s, CUDA %s, cxx11 ABI %d, %s" % (torch.__version__, torch.version.cuda, int(torch._C._GLIBCXX_USE_CXX11_ABI),
+                                                    sysconfig.get_config_var("SOABI"))
+
+
+def native_matches():
+    """Whether the built _native.so carries this process's tag, without loading it."""
+    tag = native_tag()
+    if tag is None or not os.path.exists(NATIVE):
+        return False
+    with open(NATIVE, "rb") as f:
+        return ("built for " + tag + "\0").encode() in f.read()
+
+
 def needs_build():
     return _older(LIB, [os.path.join(CSRC, s) for s in SOURCES + HEADERS])
 
@@ -46,7 +66,7 @@ def _start_native():
         return _without_native("a torch without CUDA")
     cuda_include = os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include") if os.path.isabs(_nvcc()) else "/usr/local/cuda/include"
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-c", NATIVE_SOURCE, "-o", os.path.join(CSRC, "native.o"),
-           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)]
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), '-DQUADS_NATIVE_TAG="%s"' % native_tag()]
     for d in cpp_extension.include_paths() + [sysconfig.get_paths()["include"], cuda_include]:
         cmd += ["-isystem", d]
     link = ["g++", "-shared", "-o", NATIVE, os.path.join(CSRC, "native.o"), "-L" + HERE, "-l:libquads.so", "-Wl,-rpath,$ORIGIN",
@@ -71,7 +91,7 @@ def _finish_native(compiler, link):
 def build(force=False, verbose=False):
     """libquads.so, and where this machine has what it takes _native.so."""
     native = None
-    if force or _older(NATIVE, [NATIVE_SOURCE, os.path.join(CSRC, HEADERS[-1])]):
+    if force or not native_matches() or _older(NATIVE, [NATIVE_SOURCE, os.path.join(CSRC, HEADERS[-1])]):
         native = _start_native()
     if force or needs_build():
         _build_lib(verbose)

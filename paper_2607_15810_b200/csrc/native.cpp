@@ -18,6 +18,9 @@
 
 namespace {
 
+// The torch and Python whose inline code this object holds; the binding looks for it in the file before it loads it.
+__attribute__((used)) const char g_tag[] = "built for " QUADS_NATIVE_TAG;
+
 PyObject* g_error = nullptr;                               // the binding's exception class
 PyObject *s_q, *s_sf, *s_gs, *s_atoms, *s_out, *s_workspace;
 

@@ -42,3 +42,25 @@ def test_library_is_built_where_the_native_calls_do_not_compile(built, monkeypat
     monkeypatch.setattr(Bd, "NATIVE_SOURCE", str(broken))
     monkeypatch.setattr(Bd, "CSRC", str(tmp_path))
     _built_without_native(built, capsys)
+
+
+def test_native_calls_of_another_torch_are_rebuilt(monkeypatch, tmp_path):
+    """Newer than its sources is not enough."""
+    monkeypatch.setattr(Bd, "NATIVE", str(tmp_path / "_native.so"))
+    monkeypatch.setattr(Bd, "needs_build", lambda: False)
+    started = []
+    monkeypatch.setattr(Bd, "_start_native", lambda: started.append(Bd.native_tag()))
+    for tag, times in ((Bd.native_tag(), 0), ("torch 1.0, CUDA 9.0, cxx11 ABI 0, cpython-36m", 1), (Bd.native_tag() + "0", 2)):
+        (tmp_path / "_native.so").write_bytes(b"\x7fELF built for " + tag.encode() + b"\0")
+        Bd.build()
+        assert len(started) == times, tag
+
+
+def test_native_calls_of_another_torch_are_not_loaded(monkeypatch):
+    from paper_2607_15810_b200 import binding as B
+    if not os.path.exists(Bd.NATIVE):
+        pytest.skip("_native.so is not built here")
+    assert Bd.native_matches() and B._native is not None
+    monkeypatch.setattr(Bd, "native_tag", lambda: "torch 1.0, CUDA 9.0, cxx11 ABI 0, cpython-36m")
+    with pytest.warns(UserWarning, match="_native.so is left out"):
+        assert B._load_native() is None
