@@ -246,11 +246,11 @@ quads_status launch_select_mask(uint8_t* codes, int n_rows_fixed, uint32_t flip,
 }
 
 quads_status launch_dequantize(const uint8_t* q, const uint8_t* sf, const float* gs, int64_t n_tensors, int64_t nblk, int64_t K, int tiled,
-                               int64_t sf_stride, uint16_t* out, int sm_count, cudaStream_t st) {
+                               int64_t sf_stride, uint16_t* out, int32_t* zero, int sm_count, cudaStream_t st) {
   // four blocks of 16 elements per thread, and no more CTAs than a few rounds of the chip
   const int64_t per_tensor = std::min<int64_t>((nblk + 1023) / 1024, std::max<int64_t>(1, (int64_t)sm_count * 16 / n_tensors));
   QUADS_CUDA_OK(launch_kernel(dequantize_kernel, dim3((unsigned)per_tensor, (unsigned)n_tensors), dim3(256), (size_t)0, st, q, sf, gs, nblk,
-                              (uint32_t)(K / 16), (int)((K + 63) / 64), tiled, sf_stride, out));
+                              (uint32_t)(K / 16), (int)((K + 63) / 64), tiled, sf_stride, out, zero));
   QUADS_CUDA_OK(cudaGetLastError());
   return QUADS_OK;
 }
@@ -300,7 +300,7 @@ void quads_debug_set_quantize_wait(int64_t clock_cycles, int32_t extra_arrivals)
 static quads_status quantize_common(const void* x, int64_t n_tensors, int64_t rows, int64_t K, int64_t ld,
                                     int64_t tensor_stride, const float* gs_in, void* fq, uint8_t* q, uint8_t* sf,
                                     float* gs_out, int sf_layout, void* workspace, size_t workspace_bytes,
-                                    cudaStream_t st) {
+                                    cudaStream_t st, int32_t* zero = nullptr /* a word that the first kernel clears */) {
   g_launch_count = 0;
   if (rows < 0 || n_tensors < 0 || K <= 0 || (K % 16) != 0 || ld < K || (ld % 16) != 0) return QUADS_ERR_SHAPE;
   if (sf_layout != QUADS_SF_LINEAR && sf_layout != QUADS_SF_TILED) return QUADS_ERR_SHAPE;
@@ -323,12 +323,14 @@ static quads_status quantize_common(const void* x, int64_t n_tensors, int64_t ro
   // quantizes out of L2.  The kernel boundary is the only synchronisation.
   const bool two_pass = !gs_in && n_tensors == 1 && rows > 0 && !getenv("QUADS_QUANT_COOPERATIVE");
   if (!gs_in && !two_pass) QUADS_CUDA_OK(cudaMemsetAsync(amax_bits, 0, (size_t)n_tensors * 8, st));
+  if (!gs_in && !two_pass && zero) QUADS_CUDA_OK(cudaMemsetAsync(zero, 0, 4, st));
+  if (gs_in) counters = reinterpret_cast<uint32_t*>(zero);      // (no arrivals to count: the kernel clears the word)
   int n_parts = 0;
   if (two_pass) {
     const int64_t chunks = rows * (K / 8);
     n_parts = amax_parts_for(chunks, di.sm_count);
     QUADS_CUDA_OK(launch_kernel(amax_partial_kernel<false>, dim3(n_parts), dim3(256), (size_t)0, st, xp, rows, K, ld, amax_bits,
-                                static_cast<uint32_t*>(nullptr), 0, static_cast<uint32_t*>(nullptr), 0));
+                                reinterpret_cast<uint32_t*>(zero), 0, static_cast<uint32_t*>(nullptr), 0));
   }
   uint16_t* fqp = static_cast<uint16_t*>(fq);
   int nt = (int)n_tensors;
@@ -429,7 +431,7 @@ quads_status quads_dequantize_nvfp4(const uint8_t* q, const uint8_t* sf, const f
   if (s != QUADS_OK) return s;
   const int tiled = sf_layout == QUADS_SF_TILED;
   const int64_t sf_stride = tiled ? (int64_t)quads_sf_tiled_bytes(rows, K) : nblk;
-  return launch_dequantize(q, sf, gs, n_tensors, nblk, K, tiled, sf_stride, static_cast<uint16_t*>(out), di.sm_count,
+  return launch_dequantize(q, sf, gs, n_tensors, nblk, K, tiled, sf_stride, static_cast<uint16_t*>(out), nullptr, di.sm_count,
                            static_cast<cudaStream_t>(cuda_stream));
 }
 
@@ -702,7 +704,7 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   g_trace.n = 0;
   trace_mark("start", st);
   // header (status word included) and the amax word start at zero; the one-sided modes need the status word alone, which
-  // their last kernel clears
+  // their first kernel clears
   const bool one_sided = a->operand_mode != QUADS_W4A4;
   // A dense projection behind the small batches: its first kernel takes x's partial maxima, and clears as well, while the quantization's
   // CTAs need not meet, i.e. no cooperative launch, which waits for the chip to be empty and lets nothing start behind it.  For a
@@ -727,13 +729,14 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
     const void *A_op = a->x, *B_op = a->w13_bf16;
     if (a->operand_mode == QUADS_W4A16) {
       s = launch_dequantize(a->w13_q, a->w13_sf, a->w13_gs, 1, (int64_t)a->N * (H / 16), H, 1, (int64_t)quads_sf_tiled_bytes(a->N, H), dec,
-                            di.sm_count, st);
+                            header + kHdrStatus, di.sm_count, st);
       if (s != QUADS_OK) return s;
       B_op = dec;
     } else if (a->operand_mode == QUADS_W16A4) {
       // Q_A(x) then decode, in one pass of the quantizer (its scratch: the 256 bytes at the amax slot)
       const int launches = g_launch_count;
-      s = quantize_common(a->x, 1, T, H, H, 0, a->a13_gs, dec, a->xq, a->xsf, a->a13_gs_out, QUADS_SF_LINEAR, P(L.amax), (size_t)kAmaxPartsMax * 4, st);
+      s = quantize_common(a->x, 1, T, H, H, 0, a->a13_gs, dec, a->xq, a->xsf, a->a13_gs_out, QUADS_SF_LINEAR, P(L.amax), (size_t)kAmaxPartsMax * 4, st,
+                          header + kHdrStatus);
       g_launch_count += launches;
       if (s != QUADS_OK) return s;
       A_op = dec;

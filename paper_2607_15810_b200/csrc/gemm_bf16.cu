@@ -17,9 +17,10 @@
 // tcgen05.commit; warps 2..9 drain one of TWO float32 accumulators (all 512 columns of tensor memory)
 // while the MMAs of the next tile fill the other.  2048 x 4096 -> 4096: 45.8 us (1.50 PFLOP/s, 0.89 of the measured burst
 // rate; 128 tiles on 74 pairs leave the second wave a quarter empty).
-// Every wait is bounded; a wait that gives up records QUADS_ERR_TIMEOUT and all roles leave.  The kernels clear the status word
-// themselves: a kernel in front that did nothing else cost a call 1 to 1.4 us (replayed from a graph, W16A16 64 x 512 -> 512 5.4
-// us, 4.0 so; 64 x 4096 -> 4096 9.7, 8.9; 2048 x 2048 -> 2048 14.9, 13.9).
+// Every wait is bounded; a wait that gives up records QUADS_ERR_TIMEOUT and all roles leave.  The status word is cleared by the
+// first kernel of a call: the decode or the quantizer in front, or with nothing in front (`first`) the product itself, all
+// of whose waits then begin behind the preceding kernel's end.  A kernel that did nothing else cost a call 1 to 1.4 us (replayed
+// from a graph, W16A16 64 x 512 -> 512 5.4 us, 4.0 so; 64 x 4096 -> 4096 9.7, 8.9; 2048 x 2048 -> 2048 14.9, 13.9).
 #include <algorithm>
 
 #include "kernels.cuh"
@@ -66,7 +67,7 @@ __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t adesc, uin
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kFThreads, 1)
 gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, int T, int N, int K,
-                      uint16_t* __restrict__ out, int32_t* __restrict__ status) {
+                      int first, uint16_t* __restrict__ out, int32_t* __restrict__ status) {
   extern __shared__ uint8_t smem_dyn[];
   const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   uint8_t* smem_gen = smem_dyn + (smem_base - smem_u32(smem_dyn));
@@ -92,7 +93,7 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_con
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
   pdl_sync();                                        // the decoded operand comes from the preceding kernel
-  if (blockIdx.x == 0 && threadIdx.x == 0) *status = 0;      // (a wait gives up seconds later at the earliest)
+  if (first && blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
 
   const int m_tiles = (T + 255) / 256, n_tiles = (N + kFTileN - 1) / kFTileN;
   const int total = m_tiles * n_tiles;
@@ -270,10 +271,14 @@ gemm_bf16_wave_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_con
   const int k_stages = K / kFStageK;
   const int ks0 = (part * k_stages) >> split_log2, ks1 = ((part + 1) * k_stages) >> split_log2;      // never empty: split <= k_stages
   const int row0 = mt * 128;
+  // The MMA warp goes ahead behind a kernel of this call, which waited for its own predecessor before this one could start; behind
+  // somebody else's, which may run for longer than a wait is allowed to take, nobody does.
+  const bool first = !(a_early | b_early);
+  const bool early = (warp == 1 && !first) || (warp == 0 && a_early) || (warp == kWLoadB && b_early);
   // launch_dependents lets the following kernel start; it waits for this one's end itself
-  const bool early = warp == 1 || (warp == 0 && a_early) || (warp == kWLoadB && b_early);
-  if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); else pdl_sync();
-  if (blockIdx.x == 0 && threadIdx.x == 64) *status = 0;     // an epilogue thread's; a wait gives up seconds later at the earliest
+  if (warp == 1 || early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (!early) pdl_sync();
+  if (first && blockIdx.x == 0 && threadIdx.x == 64) *status = 0;
 
   if (warp == 0 || warp == kWLoadB) {
     // ------------------------------------------------------------ loaders
@@ -410,7 +415,7 @@ quads_status launch_gemm_bf16(const CUtensorMap& tm_a, const CUtensorMap& tm_b, 
     return launch_wave<256>(tm_a, tm_b, T, N, K, 0, a_early, b_early, out, status, stream);
   QUADS_CUDA_OK(set_max_dynamic_smem<gemm_bf16_pair_kernel>(kFSmemBytes));
   QUADS_CUDA_OK(launch_kernel(gemm_bf16_pair_kernel, dim3(n_sms / 2 * 2), dim3(kFThreads), (size_t)kFSmemBytes, stream, tm_a,
-                              tm_b, T, N, K, out, status));
+                              tm_b, T, N, K, a_early || b_early ? 0 : 1, out, status));
   return QUADS_OK;
 }
 

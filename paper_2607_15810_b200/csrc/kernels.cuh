@@ -39,7 +39,7 @@ __global__ void fake_quant_ring_kernel(const uint16_t* x, int64_t nblk, int64_t 
                                        float* gs_out, int sf_tiled, int64_t sf_tensor_stride, uint32_t k16,
                                        int kt_count);
 __global__ void dequantize_kernel(const uint8_t* q, const uint8_t* sf, const float* gs, int64_t nblk, uint32_t k16,
-                                  int kt_count, int sf_tiled, int64_t sf_tensor_stride, uint16_t* out);
+                                  int kt_count, int sf_tiled, int64_t sf_tensor_stride, uint16_t* out, int32_t* zero);
 __global__ void channel_stats_kernel(const uint16_t* x, int T, int H, const float* gs_in, const uint32_t* amax_bits,
                                      int rows_per_cta, float* partials);
 constexpr int kScoreSlices = 16;
@@ -223,7 +223,8 @@ quads_status launch_gemm_dense(const GemmParams& p, const GemmMaps& m, int n_sms
 // ---- gemm_bf16.cu: out[T, N] = A[T, K] B[N, K]^T, bf16 operands (tensor maps with boxes of 64 elements x kBf16BoxRows
 // rows, 128-byte swizzle), float32 accumulation, bf16 output; K % 64 == 0, N % 128 == 0
 constexpr int kBf16BoxRows = 64;
-// a_early / b_early: the operand is older than the preceding kernel of the stream, which has itself waited for its predecessor.
+// a_early / b_early: the operand is older than the preceding kernel of the stream, which has itself waited for its predecessor
+// and has cleared the status word.  Neither: the product is the call's first kernel and clears the word.
 quads_status launch_gemm_bf16(const CUtensorMap& tm_a, const CUtensorMap& tm_b, int T, int N, int K, bool a_early, bool b_early, uint16_t* out,
                               int32_t* status, int n_sms, cudaStream_t stream);
 

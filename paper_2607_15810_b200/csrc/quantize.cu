@@ -76,8 +76,8 @@ __global__ void __launch_bounds__(256) amax_kernel(const uint16_t* __restrict__ 
 // ---------------------------------------------------------------------------
 // First pass of the single-tensor quantizer: CTA b leaves the |x| maximum of its share in
 // partials[b] (every CTA stores, so the array needs no initialisation and there is no atomic);
-// the 32-byte loads ask L2 to keep the lines for the pass that follows.  kClear: in front of a dense projection it also
-// clears the words that the call starts at zero (n0 and n1 words, by CTA 0).
+// the 32-byte loads ask L2 to keep the lines for the pass that follows.  `zero0` (or NULL) is a word
+// that it clears; kClear: in front of a dense projection it clears all the words that the call starts at zero (n0 and n1 of them, by CTA 0).
 template <bool kClear>
 __global__ void __launch_bounds__(256) amax_partial_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t K,
                                                            int64_t ld, uint32_t* __restrict__ partials, uint32_t* __restrict__ zero0,
@@ -118,6 +118,7 @@ __global__ void __launch_bounds__(256) amax_partial_kernel(const uint16_t* __res
     uint32_t t = 0;
     for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t = max(t, wmax[i]);
     partials[blockIdx.x] = t << 16;
+    if (!kClear && zero0 && blockIdx.x == 0) *zero0 = 0u;
   }
 }
 
@@ -172,6 +173,8 @@ __device__ __forceinline__ void emit_block(const QuantSink& o, const QuantCtx& q
   }
 }
 
+// With given scales there are no arrivals to count: `counters` (or NULL) is then a word that the kernel clears.  (As one more parameter it
+// cost every call 0.37 us of host time.)
 __global__ void __launch_bounds__(256, 4)
 fused_quantize_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t K, int64_t ld, int64_t tensor_stride,
                       int n_tensors, const float* __restrict__ gs_in, uint32_t* __restrict__ amax_bits,
@@ -180,6 +183,7 @@ fused_quantize_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t K, i
                       int n_groups, long long wait_cycles, int extra_arrivals, const uint32_t* __restrict__ amax_parts,
                       int n_amax_parts) {
   pdl_sync();
+  if (gs_in && counters && blockIdx.x == 0 && threadIdx.x == 0) *counters = 0u;
   const int group = blockIdx.x % n_groups;
   const int rank = blockIdx.x / n_groups;
   const int gsize = ((int)gridDim.x - group + n_groups - 1) / n_groups;
@@ -648,13 +652,14 @@ fake_quant_ring_kernel(const uint16_t* __restrict__ x, int64_t nblk, int64_t ten
 // blockIdx.y = tensor; a thread decodes 16-element blocks, 8 B of codes + 1 B of scale in, one 32-byte store out,
 // four blocks in flight.  In the one-sided dense projection the result is read back out of L2 by the product
 // behind it (no streaming hint on the stores).  4096 x 4096 in front of that product: 11.5 us with one block at
-// a time and a 64-bit division for its tensor, 7.5 now (43 MB: 6.6 us).
+// a time and a 64-bit division for its tensor, 7.5 now (43 MB: 6.6 us).  `zero` (or NULL) is a word the kernel clears.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
 dequantize_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ sf, const float* __restrict__ gs,
                   int64_t nblk, uint32_t k16, int kt_count, int sf_tiled, int64_t sf_tensor_stride,
-                  uint16_t* __restrict__ out) {
+                  uint16_t* __restrict__ out, int32_t* __restrict__ zero) {
   pdl_sync();
+  if (zero && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *zero = 0;
   QuantSink geo{nullptr, nullptr, nullptr, sf_tiled, k16, kt_count, 0, 0};
   quant_sink_divisor(geo);
   const size_t t = blockIdx.y;
