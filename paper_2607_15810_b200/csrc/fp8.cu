@@ -522,6 +522,7 @@ gemm_fp8_kernel(const Fp8GemmParams p, const __grid_constant__ CUtensorMap tm_a,
   __syncthreads();
   tc_fence_after();
   if (warp == C::kMmaWarp) tmem_dealloc<1>(tmem, 512);
+  if (warp == 0) settle_if_abandoned(abort_flag);
 }
 
 }  // namespace

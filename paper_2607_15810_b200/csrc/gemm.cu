@@ -465,9 +465,11 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p, const CUtensorMap
   }
   tc_fence_before();
   __syncthreads();
+  if (CG == 2 && warp == 0) settle_if_abandoned(abort_flag);
   if (CG == 2) cluster_sync_all();          // the peer may still be signalling this CTA's barriers
   tc_fence_after();
   if (warp == 1) tmem_dealloc<CG>(tmem, kTmemCols);
+  if (CG == 1 && warp == 0) settle_if_abandoned(abort_flag);
 }
 
 template <int EPI, bool RES>

@@ -203,6 +203,7 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_con
   }
   tc_fence_before();
   __syncthreads();
+  if (warp == 0) settle_if_abandoned(abort_flag);
   cluster_sync_all();                   // the peer may still be signalling this CTA's barriers
   tc_fence_after();
   if (warp == 1) tmem_dealloc<2>(tmem, 512);
@@ -361,6 +362,7 @@ gemm_bf16_wave_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_con
   if (split > 1) cluster_sync_all(); else __syncthreads();
   tc_fence_after();
   if (warp == 1) tmem_dealloc<1>(tmem, BN);
+  if (warp == 0) settle_if_abandoned(abort_flag);
   const int n0 = nt * BN + part * w;
   if (!epi || split == 1 || n0 >= N) return;           // (w <= 128: a CTA's columns are all there or all missing)
   const float* sums = reinterpret_cast<const float*>(smem_gen);

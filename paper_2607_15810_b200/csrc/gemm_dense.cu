@@ -207,6 +207,7 @@ gemm_dense_kernel(const GemmParams p, int split_log2, const __grid_constant__ CU
   if (split > 1) cluster_sync_all(); else __syncthreads();
   tc_fence_after();
   if (warp == 1) tmem_dealloc<1>(tmem, kTmemCols);
+  if (warp == 0) settle_if_abandoned(abort_flag);
   const int n0 = nt * BN + rank * w;
   if (!epi || split == 1 || n0 >= p.n_out) return;     // (w <= 128: a CTA's columns are all there or all missing)
   const float* part = reinterpret_cast<const float*>(smem_gen);

@@ -552,6 +552,7 @@ gemm_swapped_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tm_x
   __syncthreads();
   tc_fence_after();
   if (warp == 1) tmem_dealloc<1>(tmem, kTmemCols);
+  if (warp == 0) settle_if_abandoned(abort_flag);
 }
 
 }  // namespace
