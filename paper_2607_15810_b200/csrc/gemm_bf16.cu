@@ -272,12 +272,18 @@ gemm_bf16_wave_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_con
   const int k_stages = K / kFStageK;
   const int ks0 = (part * k_stages) >> split_log2, ks1 = ((part + 1) * k_stages) >> split_log2;      // never empty: split <= k_stages
   const int row0 = mt * 128;
-  // The MMA warp goes ahead behind a kernel of this call, which waited for its own predecessor before this one could start; behind
-  // somebody else's, which may run for longer than a wait is allowed to take, nobody does.
+  // Behind a kernel of this call, which waited for its own predecessor before this one could start, the loader of the older operand goes
+  // ahead, and with the weights (W16A4) the MMA warp too; behind somebody else's kernel (`first`: W16A16), which may run for
+  // longer than a wait is allowed to take, nobody does.
   const bool first = !(a_early | b_early);
-  const bool early = (warp == 1 && !first) || (warp == 0 && a_early) || (warp == kWLoadB && b_early);
-  // launch_dependents lets the following kernel start; it waits for this one's end itself
-  if (warp == 1 || early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const bool early = (warp == 0 && a_early) || ((warp == 1 || warp == kWLoadB) && b_early);
+  // When the following kernel may start (it waits for this one's end itself).  Let go at once, the decode of a next W4A16 call gathers on
+  // the SMs that this product leaves free, several CTAs to an SM, and the clusters of a next W16A16 product find too few free
+  // SMs side by side (replayed from a graph, us, at once / behind the wait: W4A16 78 x 1024 -> 3968 10.0 / 9.3, 1045 x 640 -> 1408 8.2 / 7.7,
+  // 132 x 1152 -> 3968 11.5 / 10.8, 173 x 768 -> 640 7.2 / 7.3; W16A16 235 x 2944 -> 640, 40 CTAs, 9.3 / 8.6, 366 x 2560 -> 512, 48 CTAs,
+  // 8.9 / 8.4, 68 x 3968 -> 512, 32 CTAs, 7.0 / 7.2, 70 x 1408 -> 512, 16 CTAs, 5.7 / 5.9, 64 x 512 -> 512, no split, 3.85 / 4.0).
+  const bool at_once = b_early || (first && (split == 1 || gridDim.x <= 32));
+  if (warp == 1 && at_once) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (!early) pdl_sync();
   if (first && blockIdx.x == 0 && threadIdx.x == 64) *status = 0;
 
