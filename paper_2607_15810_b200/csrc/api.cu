@@ -206,13 +206,15 @@ inline void trace_mark(const char* name, cudaStream_t st) {
 // here; QUADS_GEMM_CTA_GROUP=1|2 forces a variant.  (When the experts' tile counts happen to be
 // even -- the skewed prefill benchmark: 410 rows = 4 tiles for most experts -- pairs already win at
 // 512 rows per expert: 477 vs 488 us per layer.)
-int gemm_cta_group_for(int64_t rows, int experts) {
+// `one_wave`: a dense projection, which is padded by at most one tile either way, whose tiles all have an SM of their own
+// (gemm_dense_ahead_of_pairs).
+int gemm_cta_group_for(int64_t rows, int experts, bool one_wave) {
   static const int forced = [] {
     const char* e = getenv("QUADS_GEMM_CTA_GROUP");
     return (e && (e[0] == '1' || e[0] == '2')) ? e[0] - '0' : 0;
   }();
   if (forced) return forced;
-  return rows >= (int64_t)1024 * (experts > 0 ? experts : 1) ? 2 : 1;
+  return !one_wave && rows >= (int64_t)1024 * (experts > 0 ? experts : 1) ? 2 : 1;
 }
 
 // Blocks of at most 256 threads: a token's 16-byte columns along x, tokens along y where a row has fewer than 256.
@@ -687,7 +689,8 @@ quads_status quads_moe_w4a4_rac(const quads_moe_args* a, void* cuda_stream) {
   const uint16_t* x = static_cast<const uint16_t*>(a->x);
   const int A = T * topk;
   const size_t pad_rows = (size_t)L.m_tiles_max * 128;
-  const int cta_group = gemm_cta_group_for(dense ? (int64_t)T : (int64_t)A, dense ? 1 : E);
+  const int cta_group = gemm_cta_group_for(dense ? (int64_t)T : (int64_t)A, dense ? 1 : E,
+                                           dense && gemm_dense_ahead_of_pairs(T, H, a->N, a->rac_nsel_13 > 0, di.sm_count));
 
   // few rows per expert (decode-sized batches): operands swapped, weights on the M side
   static const bool no_swap = getenv("QUADS_NO_SWAP") != nullptr;

@@ -264,6 +264,16 @@ DensePlan plan_dense(int rows, int K, int N, int n_sms) {
 
 bool gemm_dense_ok(int rows, int K, int N, int n_sms) { return plan_dense(rows, K, N, n_sms).split > 0; }
 
+// From 1024 rows on, where the persistent CTA pairs are the other form: ahead of them in one wave, but for a long K without residual
+// in tiles of 256 columns, which the pairs' deeper ring suits better (replayed from a graph, us, pairs / so: 1024 x 512 -> 1024 10.3 / 7.9,
+// with residual 18.5 / 15.9; 1500 x 2048 -> 512 13.7 / 11.7, 25.6 / 22.1; 4000 x 2048 -> 1024 17.0 / 17.1, 31.4 / 29.8; 2000 x 4096 -> 1024
+// 19.5 / 17.6, 36.3 / 31.3; 8192 x 4096 -> 256 36.9 / 35.0, 62.3 / 58.0; 2000 x 4096 -> 2048 19.9 / 21.1, 37.6 / 36.0; beyond one wave 3000 x
+// 2048 -> 2048 19.1 / 20.2).
+bool gemm_dense_ahead_of_pairs(int rows, int K, int N, bool resid, int n_sms) {
+  const DensePlan d = plan_dense(rows, K, N, n_sms);
+  return d.split > 0 && (d.bn == 128 || resid || K <= 2048);
+}
+
 quads_status launch_gemm_dense(const GemmParams& p, const GemmMaps& m, int n_sms, cudaStream_t stream) {
   const DensePlan d = plan_dense(p.dense_rows, p.K, p.n_out, n_sms);
   return d.bn == 128 ? launch_bn<128>(p, d.split, m, stream) : launch_bn<256>(p, d.split, m, stream);

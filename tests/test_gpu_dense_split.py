@@ -17,7 +17,9 @@ pytestmark = pytest.mark.gpu
     (40, 640, 128, 320),       # three stages for two CTAs, the last one half full
     (17, 128, 128, 16),        # one stage
     (129, 128, 9600, 64),      # tiles of 256 columns, half of the last one missing
-    (200, 4096, 128, 2048)])   # behind the grid-wide front
+    (200, 4096, 128, 2048),    # behind the grid-wide front
+    (1025, 2048, 384, 0),      # more rows than the CTA pairs' line, tiles in one wave
+    (2049, 2176, 1152, 1088)]) # the same in tiles of 256 columns
 def test_dense_tiles_and_splits(T, K, N, nsel):
     from paper_2607_15810_b200 import binding as B
     g = torch.Generator().manual_seed(T + K + N)

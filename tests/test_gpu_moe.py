@@ -77,12 +77,14 @@ def test_dense_exact_integer_case(B):
     assert np.array_equal(got, MC.f32(torch.from_numpy(want).to(torch.bfloat16)).astype(np.float64))
 
 
-def test_dense_at_the_size_where_cta_pairs_are_chosen(B):
+@pytest.mark.parametrize("N", [640, 2176])
+def test_dense_at_the_size_where_cta_pairs_are_chosen(B, N):
     """From 1024 rows per weight matrix the call takes the CTA-pair kernel (256 x 256 tiles,
-    cta_group::2) on its own; compared element by element with the oracle, ragged last pair."""
-    x, w = synth.dense_inputs(seed=9, T=2300, K=1024, N=640)
+    cta_group::2) on its own, unless its tiles fit the chip at once (N = 640); compared element by element with the oracle, ragged last
+    pair."""
+    x, w = synth.dense_inputs(seed=9, T=2300, K=1024, N=N)
     ratio = _dense_case(B, x, w, 512)
-    print("cta-pair dense 2300x1024x640: worst err / tol = %.3f" % ratio)
+    print("dense 2300x1024x%d: worst err / tol = %.3f" % (N, ratio))
 
 
 def _sweep_operands():
