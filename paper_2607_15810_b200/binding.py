@@ -4,7 +4,7 @@ memory and the current stream.  Importing this module fails loudly when the
 library has not been built (run `python -m paper_2607_15810_b200.build`).
 
 The ordinary calls -- plain CUDA tensors, no verification exports -- go through _native.so, which does the
-same in a third of the host time; everything else through ctypes."""
+same in half to three quarters of the time a call takes the host; everything else through ctypes."""
 import ctypes as C
 import os
 import warnings

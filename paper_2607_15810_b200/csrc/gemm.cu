@@ -49,8 +49,10 @@ constexpr int kTmemCols = 512;
 constexpr int kMaxTableTiles = 2048;               // M-tiles whose expert / row count fit the shared-memory tables
 constexpr int kTmemSfBase = 256;                  // accumulator: columns 0..255
 constexpr int kTmemSfPerBuf = 16 * kKSteps;       // SFA 4/step | SFR 4/step | SFB 8/step, double buffered
-// RES: the stage has room for the residual operand; without it another stage fits (a layer of 4096 tokens without compensation, H =
-// 2048 197.8 -> 184.8 us, with it at W13 only 229.5 -> 225.9; 1500 tokens 113.9 -> 111.1 and 131.0 -> 127.5).
+// RES: the stage has room for the residual operand; without it another stage fits (layers in a loop, us per call, H = 2048: 4096
+// tokens without compensation 212.7 -> 201.9, with it at W13 only 258.8 -> 256.1; 1500 tokens 113.8 -> 111.9 and 133.2 -> 132.6; 8192, W13
+// only, 450.3 -> 444.0; H = 4096: 1000 tokens without 303.4 -> 296.2, 3000, W13 only, 643.4 -> 631.6; dense 2000 x 2048 -> 4096 without 23.2 ->
+// 22.5).
 template <int CG, bool RES>
 struct Cfg {
   static constexpr int kTileA = kBM * kStageKBytes;

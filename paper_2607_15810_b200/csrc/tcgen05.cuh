@@ -117,12 +117,13 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols) {
 }
 // Arrive on `bar` once all tcgen05 operations issued so far by this thread are
 // complete.  CG == 2: the arrival is delivered to the barrier at the same
-// shared-memory offset in both CTAs of the pair (`mask`: their ranks in the cluster).
+// shared-memory offset in both CTAs of the pair.
 template <int CG>
-__device__ __forceinline__ void tc_commit(uint32_t bar, uint16_t mask = 3) {
+__device__ __forceinline__ void tc_commit(uint32_t bar) {
   if (CG == 1) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
   } else {
+    const uint16_t mask = 3;
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
                  ::"r"(bar), "h"(mask) : "memory");
   }
