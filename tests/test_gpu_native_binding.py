@@ -1,4 +1,6 @@
-"""The binding's native calls against its ctypes path: the same results, objects and errors."""
+"""The binding's native calls against its ctypes path: the same results, objects and errors, each through the path it is meant for."""
+from collections import OrderedDict
+
 import pytest
 import torch
 
@@ -9,23 +11,46 @@ class Sub(torch.Tensor):
     pass
 
 
+class Recorder:
+    """The native module, with what became of each call: "done", the status of its error, or None where it was left to ctypes."""
+
+    def __init__(self, module):
+        self.module, self.seen = module, []
+
+    def __getattr__(self, name):
+        def call(*args):
+            from paper_2607_15810_b200 import binding as B
+            try:
+                r = getattr(self.module, name)(*args)
+            except B.QuadsError as e:
+                self.seen.append(e.status)
+                raise
+            self.seen.append(None if r is None else "done")
+            return r
+        return call
+
+
 def _both(monkeypatch, B, call):
-    """The call's result (or status of its error) through either path."""
+    """The call's result (or status of its error) through either path, and what the native function made of it."""
     got = []
     assert B._native is not None
-    for native in (B._native, None):
+    rec = Recorder(B._native)
+    for native in (rec, None):
         monkeypatch.setattr(B, "_native", native)
         try:
             r = call()
             got.append(r)
         except B.QuadsError as e:
             got.append(e.status)
-    return got
+    assert len(rec.seen) == 1
+    return got + rec.seen
 
 
 def _same(a, b):
     if isinstance(a, dict):
         assert a.keys() == b.keys()
+        wa, wb = a["workspace"], b["workspace"]
+        assert wa.dtype == wb.dtype and wa.shape == wb.shape and wa.device == wb.device
         return _same(a["out"], b["out"])
     if isinstance(a, tuple):
         assert len(a) == len(b)
@@ -48,27 +73,40 @@ def test_same_results_objects_and_errors(monkeypatch):
     w = B.fake_quant_weights(wb.unsqueeze(0), want_fq=False, sf_layout=B.SF_TILED)
     a2, gs = torch.tensor([0.01], device="cuda"), torch.tensor([0.002], device="cuda")
     wide = bf(T, 2 * H)[:, :H]                                              # a row stride
-    calls = [
+    tiled = (torch.empty(T, H // 2, dtype=torch.uint8, device="cuda"), torch.zeros(B.sf_tiled_bytes(T, H), dtype=torch.uint8, device="cuda"),
+             torch.empty(1, device="cuda"))
+    native = [
         lambda: B.moe_w4a4_rac(x, lg, w13, w2, 2, H // 2, I // 2, a2),
         lambda: B.moe_w4a4_rac(x, lg, w13, w2, 2, 0, 0, a2, a13_gs=gs, renormalize=False),
         lambda: B.moe_fp8_w8a8(x, lg, p13, p2, 2),
         lambda: B.dense_w4a4_rac(x, w, 64), lambda: B.dense_w4a4_rac(x, w, 0, a_gs=gs),
         lambda: B.dense_one_sided(x, B.W4A16, w=w), lambda: B.dense_one_sided(x, B.W16A4, w_bf16=wb, a_gs=gs),
         lambda: B.dense_one_sided(x, B.W16A16, w_bf16=wb), lambda: B.dense_w4a4_rac(torch.nn.Parameter(x), w, 64),
-        lambda: B.dense_w4a4_rac(x.as_subclass(Sub), w, 64),
         lambda: B.quantize_nvfp4(x), lambda: B.quantize_nvfp4(x, gs=gs), lambda: B.quantize_nvfp4(wide),
-        lambda: B.quantize_nvfp4(x[:1, :48]),
-        # refused
+        lambda: B.quantize_nvfp4(x[:1, :48]), lambda: B.quantize_nvfp4(x, sf_layout=B.SF_TILED, out=tiled)]
+    refused = [
         lambda: B.dense_w4a4_rac(x, w, H + 1), lambda: B.moe_w4a4_rac(x, lg, w13, w2, 9, 0, 0, a2),
         lambda: B.moe_w4a4_rac(x, lg, w13, w2, 2, 0, 0, None), lambda: B.quantize_nvfp4(x[:, :40]),
         lambda: B.dense_w4a4_rac(x, w, 64, workspace=torch.empty(512, dtype=torch.uint8, device="cuda"))]
-    for i, call in enumerate(calls):
-        a, b = _both(monkeypatch, B, call)
-        monkeypatch.undo()
-        assert _same(a, b), i
-    for bad in (lambda: B.quantize_nvfp4(x.float()), lambda: B.quantize_nvfp4(x.t())):
+    left_to_ctypes = [
+        lambda: B.dense_w4a4_rac(x.as_subclass(Sub), w, 64), lambda: B.dense_w4a4_rac(x, OrderedDict(w), 64), lambda: B.dense_w4a4_rac(x, w, True),
+        lambda: B.moe_w4a4_rac(x, lg.as_subclass(Sub), w13, w2, 2, 0, 0, a2), lambda: B.moe_fp8_w8a8(x.as_subclass(Sub), lg, p13, p2, 2),
+        lambda: B.dense_one_sided(x.as_subclass(Sub), B.W16A16, w_bf16=wb),
+        lambda: B.quantize_nvfp4(x.as_subclass(Sub)), lambda: B.quantize_nvfp4(x, sf_layout=B.SF_TILED, out=list(tiled))]
+    for group, calls in (("done", native), ("refused", refused), (None, left_to_ctypes)):
+        for i, call in enumerate(calls):
+            a, b, seen = _both(monkeypatch, B, call)
+            monkeypatch.undo()
+            assert _same(a, b), (group, i)
+            assert seen == (a if group == "refused" else group), (group, i)
+            assert (group == "refused") == isinstance(a, int), (group, i)
+    for bad in (lambda: B.quantize_nvfp4(x.float()), lambda: B.quantize_nvfp4(x.t()), lambda: B.quantize_nvfp4(x.cpu())):
+        rec = Recorder(B._native)
+        monkeypatch.setattr(B, "_native", rec)
         with pytest.raises(AssertionError):
             bad()
+        monkeypatch.undo()
+        assert rec.seen == [None]
     # the caller's buffers come back as they are
     ws = torch.empty(B.moe_workspace_bytes(T, H, I, E, 2), dtype=torch.uint8, device="cuda")
     out = torch.empty(T, H, dtype=torch.bfloat16, device="cuda")
