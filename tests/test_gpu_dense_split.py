@@ -1,4 +1,5 @@
-"""The dense projection with few output tiles, at the edges of its tile width and of its split of K."""
+"""The dense projection with few output tiles, at the edges of its tile width and of its split of K; the rings of the larger
+tiles; operands that the preceding kernel has only just written."""
 import numpy as np
 import pytest
 import torch
@@ -19,7 +20,10 @@ pytestmark = pytest.mark.gpu
     (129, 128, 9600, 64),      # tiles of 256 columns, half of the last one missing
     (200, 4096, 128, 2048),    # behind the grid-wide front
     (1025, 2048, 384, 0),      # more rows than the CTA pairs' line, tiles in one wave
-    (2049, 2176, 1152, 1088)]) # the same in tiles of 256 columns
+    (2049, 2176, 1152, 1088),  # the same in tiles of 256 columns
+    (1030, 2048, 4352, 0),     # CTA pairs without a residual: eight K steps through five stages, six rows in the last row tile
+    (1030, 1664, 4352, 0),     # the same with a half-full last K step
+    (1030, 1664, 4352, 832)])  # with a residual, four stages
 def test_dense_tiles_and_splits(T, K, N, nsel):
     from paper_2607_15810_b200 import binding as B
     g = torch.Generator().manual_seed(T + K + N)
@@ -40,8 +44,10 @@ def test_dense_tiles_and_splits(T, K, N, nsel):
 
 @pytest.mark.parametrize("T,K,N", [
     (1, 4096, 128),        # eight CTAs per tile
-    (70, 4096, 1024),      # four
+    (70, 4096, 1024),      # eight, a tile of 70 rows
+    (70, 1408, 512),       # four
     (256, 2048, 2048),     # two, every row of both row tiles
+    (661, 2176, 640),      # two, where four would fit, too
     (129, 384, 640),       # one, one row in the second row tile
     (9000, 128, 384),      # tiles of 256 columns, half of the last one missing
     (9000, 2176, 384)])    # the same number of tiles with a longer K: pairs, fewer tiles than pairs of SMs
@@ -82,3 +88,49 @@ def test_scale_of_x_and_scores_behind_either_amax(T, K):
         assert int(kept.sum()) == K // 4
         # float32 partial sums of T squares, added in float64: relative error below T * 2^-24 each
         assert float(scores[kept].min()) >= float(scores[~kept].max()) * (1 - 2 * T * 2.0 ** -24)
+
+
+def _fill(gen, t, std):
+    t.copy_((torch.randn(t.shape, device="cuda", generator=gen) * std).to(torch.bfloat16))
+
+
+def test_operands_written_right_before_the_call():
+    """What a loader fetches ahead of the preceding kernel's end is complete all the same: weights packed or decoded, and an x computed,
+    by the library's kernels immediately before the call, in buffers that hold other values every time.  A chain without a
+    synchronisation against the same chain with one behind every call."""
+    from paper_2607_15810_b200 import binding as B
+    T, K, N = 64, 4096, 4096
+
+    def chain(sync):
+        g = torch.Generator(device="cuda").manual_seed(11)
+        x, wb = (torch.empty(n, K, dtype=torch.bfloat16, device="cuda") for n in (T, N))
+        packed = (None, torch.empty(1, N, K // 2, dtype=torch.uint8, device="cuda"),
+                  torch.zeros(1, B.sf_tiled_bytes(N, K), dtype=torch.uint8, device="cuda"), torch.empty(1, device="cuda"))
+        dec = torch.empty(1, N, K, dtype=torch.bfloat16, device="cuda")
+        ws = torch.empty(B.moe_workspace_bytes(T, K, 0, 1, 1, N), dtype=torch.uint8, device="cuda")
+        wait = torch.cuda.synchronize if sync else (lambda: None)
+        got = []
+        for _ in range(12):
+            _fill(g, x, 1.0)
+            _fill(g, wb, 0.02)
+            wait()
+            w = B.fake_quant_weights(wb.view(1, N, K), want_fq=False, sf_layout=B.SF_TILED, out=packed)
+            wait()
+            y = B.dense_w4a4_rac(x, w, K // 2, workspace=ws)["out"]                    # weights older than the front by one kernel
+            wait()
+            z = B.dense_one_sided(y, B.W4A16, w=w, workspace=ws)["out"]                # x: the result just above
+            wait()
+            B.dequantize_nvfp4(w["q"], w["sf"], w["gs"], N, K, sf_layout=B.SF_TILED, out=dec)
+            wait()
+            u = B.dense_one_sided(z, B.W16A4, w_bf16=dec[0], workspace=ws)["out"]      # weights decoded just above
+            wait()
+            v = B.dense_one_sided(u, B.W16A16, w_bf16=dec[0], workspace=ws)["out"]
+            wait()
+            t = B.dense_w4a4_rac(v, w, 0, workspace=ws)["out"]
+            wait()
+            got += [y, z, u, v, t]
+        torch.cuda.synchronize()
+        return got
+
+    for i, (a, b) in enumerate(zip(chain(False), chain(True))):
+        assert torch.equal(a, b), (i // 5, i % 5)
