@@ -11,7 +11,7 @@ LIB = os.path.join(HERE, "libquads.so")
 NATIVE = os.path.join(HERE, "_native.so")
 NATIVE_SOURCE = os.path.join(CSRC, "native.cpp")
 SOURCES = ["api.cu", "quantize.cu", "front.cu", "small_batch.cu", "gemm.cu", "gemm_dense.cu", "gemm_swapped.cu", "gemm_bf16.cu", "fp8.cu", "probe.cu"]
-HEADERS = ["common.cuh", "kernels.cuh", "routing.cuh", "select.cuh", "tcgen05.cuh", os.path.join("..", "..", "include", "quads.h")]
+HEADERS = ["common.cuh", "kernels.cuh", "routing.cuh", "select.cuh", "split_k.cuh", "tcgen05.cuh", os.path.join("..", "..", "include", "quads.h")]
 
 
 def _nvcc():

@@ -21,9 +21,8 @@
 // first kernel of a call: the decode or the quantizer in front, or with nothing in front (`first`) the product itself, all
 // of whose waits then begin behind the preceding kernel's end.  A kernel that did nothing else cost a call 1 to 1.4 us (replayed
 // from a graph, W16A16 64 x 512 -> 512 5.4 us, 4.0 so; 64 x 4096 -> 4096 9.7, 8.9; 2048 x 2048 -> 2048 14.9, 13.9).
-#include <algorithm>
-
 #include "kernels.cuh"
+#include "split_k.cuh"
 #include "tcgen05.cuh"
 
 namespace quads {
@@ -220,14 +219,13 @@ constexpr int kWThreads = 352;
 constexpr int kWLoadB = 10;
 
 constexpr int kWTile = 128 * 128;                              // 128 rows of either operand
-constexpr int kWMaxSplit = 8;
 template <int BN>
 struct WCfg {
   static constexpr int kStages = BN == 128 ? 7 : 4;
   static constexpr int kStageBytes = (1 + BN / 128) * kWTile;
   static constexpr int kBarOffset = kStages * kStageBytes;
   static constexpr int kSmemBytes = kBarOffset + 256 + 1024;
-  static_assert(128 * 4 * (BN + 4 * kWMaxSplit) <= kBarOffset, "the exchange fits the ring");
+  static_assert(128 * 4 * (BN + 4 * kSplitMax) <= kBarOffset, "the exchange fits the ring");
   static_assert(kSmemBytes <= 232448, "shared memory");
 };
 
@@ -398,20 +396,11 @@ quads_status launch_wave(const CUtensorMap& tm_a, const CUtensorMap& tm_b, int T
 
 // The split of K (log2) of a problem of one wave, or -1.  Fitted in us (replayed from a graph, 4096 -> 512, S = 1 / 2 / 4 / 8: 64 rows
 // 15.6 / 11.1 / 8.6 / 8.0, 128 rows 15.8 / 12.3 / 10.5 / 11.0; 2048 -> 2048, 256 rows 10.1 / 9.7 / 10.7).  Clusters of four and eight do
-// not fill every SM (see plan_dense); from 17 clusters of four on two calls' do not fit side by side, which costs 1 to 2 us (S = 1 /
+// not fill every SM (see plan_split); from 17 clusters of four on two calls' do not fit side by side, which costs 1 to 2 us (S = 1 /
 // 2 / 4: 30 tiles, W16A16 661 x 2176 -> 640 9.2 / 8.5 / 9.6, W4A16 11.7 / 10.8 / 13.6; 31 tiles, 93 x 2944 -> 3968 11.9 / 9.7 / 10.3; 32,
 // 64 x 4096 -> 4096 15.2 / 11.1 / 10.8; 17, W4A16 84 x 1408 -> 2176 9.8 / 9.4 / 10.5; against 12, 366 x 2560 -> 512 10.2 / 8.8 / 8.4).
 int plan_wave(int T, int N, int K, int n_sms) {
-  const int k_stages = K / kFStageK, tiles = (int)std::min<int64_t>((int64_t)((T + 127) / 128) * (N / 128), n_sms + 1);
-  int best = -1;
-  double cost = 1e30;
-  for (int lg = 0; 1 << lg <= kWMaxSplit && 1 << lg <= k_stages; ++lg) {
-    if (tiles << lg > (lg < 2 ? n_sms : lg == 2 ? 128 : 64)) continue;
-    const double c = ((k_stages + (1 << lg) - 1) >> lg) * 0.185 + (lg ? std::min(T, 128) / 128.0 * 1.25 * (1 + lg) + 0.05 * lg : 0.0) +
-                     (lg == 2 && tiles > 16 ? 1.3 : 0.0);
-    if (c < cost) { cost = c; best = lg; }
-  }
-  return best;
+  return plan_split((int64_t)((T + 127) / 128) * (N / 128), T, K / kFStageK, 0.185, 1.25, 1.3, n_sms);
 }
 
 }  // namespace

@@ -11,9 +11,8 @@
 // One tile per CTA.  Warp 0 loads weights and their scales, which are older than the preceding kernel, without waiting
 // for it; warp 10 loads the activation side behind it; warp 1 issues the MMAs; warps 2..9 are the epilogue.
 // Every wait is bounded (status word, as in gemm.cu).
-#include <algorithm>
-
 #include "kernels.cuh"
+#include "split_k.cuh"
 #include "tcgen05.cuh"
 
 namespace quads {
@@ -41,7 +40,7 @@ struct DCfg {
   static constexpr int kStages = BN == 128 ? 4 : 3;
   static constexpr int kBarOffset = kStages * kStageBytes;
   static constexpr int kSmemBytes = kBarOffset + 256 + 1024;
-  static_assert(128 * 4 * (BN + 4 * kDenseMaxSplit) <= kBarOffset, "the exchange fits the ring");
+  static_assert(128 * 4 * (BN + 4 * kSplitMax) <= kBarOffset, "the exchange fits the ring");
 };
 
 struct __align__(8) DBarriers {
@@ -223,46 +222,35 @@ gemm_dense_kernel(const GemmParams p, int split_log2, const __grid_constant__ CU
 }
 
 template <int BN>
-quads_status launch_bn(GemmParams p, int split, const GemmMaps& m, cudaStream_t stream) {
+quads_status launch_bn(GemmParams p, int split_log2, const GemmMaps& m, cudaStream_t stream) {
   p.n_tiles_n = (p.n_out + BN - 1) / BN;
   const int tiles = (p.dense_rows + 127) / 128 * p.n_tiles_n;
   QUADS_CUDA_OK(set_max_dynamic_smem<gemm_dense_kernel<BN>>(DCfg<BN>::kSmemBytes));
-  int split_log2 = 0;
-  while (1 << split_log2 < split) ++split_log2;
   constexpr size_t kSmem = DCfg<BN>::kSmemBytes;
-  if (split == 1)
+  if (split_log2 == 0)
     QUADS_CUDA_OK(launch_kernel(gemm_dense_kernel<BN>, dim3(tiles), dim3(kThreads), kSmem, stream, p, split_log2, m.a, m.r, m.b));
   else
-    QUADS_CUDA_OK(launch_clusters(gemm_dense_kernel<BN>, tiles * split, split, kThreads, kSmem, stream, p, split_log2, m.a, m.r, m.b));
+    QUADS_CUDA_OK(launch_clusters(gemm_dense_kernel<BN>, tiles << split_log2, 1 << split_log2, kThreads, kSmem, stream, p, split_log2, m.a, m.r, m.b));
   return QUADS_OK;
 }
 
-// Tile width and split of K of a dense projection; split = 0 where the persistent kernels take it (more tiles than SMs).
+// Tile width and split of K (log2) of a dense projection; split_log2 = -1 where the persistent kernels take it (more tiles than SMs).
 // Tiles of 128 columns if they fit one wave, else of 256 (700 x 4096 -> 4096 32.5 us per call with the persistent kernel, 31.2 so; where
-// both fit, 128 are ahead: 512 x 2048 -> 2048 24.4 / 22.4).  A stage of K takes a CTA 0.39 us; the exchange costs about
-// 1 + log2(S) us with 128 rows in a tile, and in proportion with fewer (4096 -> 1024, S = 1 / 2 / 4 / 8: one row 20.9 / 17.9 / 16.4 /
-// 15.6, 64 rows 22.0 / 20.0 / 18.9 / 19.1, 128 rows 24.4 / 23.4 / 22.9 / 23.8; 2048 -> 2048, 128 rows 16.6 / 17.2 / 17.8).  The
-// clusters have to be resident together: eight CTAs find room for 16 clusters at best (one row, 2048 -> 2048: 12.7 with 64 CTAs
-// in clusters of four, 15.9 with 128 in clusters of eight).
-struct DensePlan { int bn, split; };
+// both fit, 128 are ahead: 512 x 2048 -> 2048 24.4 / 22.4).  A stage of K takes a CTA 0.39 us, the exchange about 1 + log2(S) us with 128
+// rows (4096 -> 1024, S = 1 / 2 / 4 / 8: one row 20.9 / 17.9 / 16.4 / 15.6, 64 rows 22.0 / 20.0 / 18.9 / 19.1, 128 rows 24.4 / 23.4 / 22.9 /
+// 23.8; 2048 -> 2048, 128 rows 16.6 / 17.2 / 17.8; one row, 2048 -> 2048: 12.7 with 64 CTAs in clusters of four, 15.9 with 128 in clusters
+// of eight).
+struct DensePlan { int bn, split_log2; };
 DensePlan plan_dense(int rows, int K, int N, int n_sms) {
   const int k_stages = (K + 64 * kSteps - 1) / (64 * kSteps), m_tiles = (rows + 127) / 128;
-  const int64_t tiles = (int64_t)m_tiles * (N / 128);
-  if (tiles > n_sms) return DensePlan{256, m_tiles * (int64_t)((N + 255) / 256) <= n_sms ? 1 : 0};
-  DensePlan best{128, 1};
-  double cost = 1e30;
-  for (int lg = 0; 1 << lg <= kDenseMaxSplit && 1 << lg <= k_stages; ++lg) {
-    const int s = 1 << lg;
-    if (tiles * s > (s == 1 ? n_sms : s == 2 ? n_sms / 2 * 2 : s == 4 ? 128 : 64)) continue;
-    const double c = (k_stages + s - 1) / s * 0.39 + (s > 1 ? std::min(rows, 128) / 128.0 * (1 + lg) + 0.05 * lg : 0.0);
-    if (c < cost) { cost = c; best.split = s; }
-  }
-  return best;
+  const int lg = plan_split((int64_t)m_tiles * (N / 128), rows, k_stages, 0.39, 1.0, 0.0, n_sms);
+  if (lg >= 0) return DensePlan{128, lg};
+  return DensePlan{256, m_tiles * (int64_t)((N + 255) / 256) <= n_sms ? 0 : -1};
 }
 
 }  // namespace
 
-bool gemm_dense_ok(int rows, int K, int N, int n_sms) { return plan_dense(rows, K, N, n_sms).split > 0; }
+bool gemm_dense_ok(int rows, int K, int N, int n_sms) { return plan_dense(rows, K, N, n_sms).split_log2 >= 0; }
 
 // From 1024 rows on, where the persistent CTA pairs are the other form: ahead of them in one wave, but for a long K without residual
 // in tiles of 256 columns, which the pairs' deeper ring suits better (replayed from a graph, us, pairs / so: 1024 x 512 -> 1024 10.3 / 7.9,
@@ -271,12 +259,12 @@ bool gemm_dense_ok(int rows, int K, int N, int n_sms) { return plan_dense(rows, 
 // 2048 -> 2048 19.1 / 20.2).
 bool gemm_dense_ahead_of_pairs(int rows, int K, int N, bool resid, int n_sms) {
   const DensePlan d = plan_dense(rows, K, N, n_sms);
-  return d.split > 0 && (d.bn == 128 || resid || K <= 2048);
+  return d.split_log2 >= 0 && (d.bn == 128 || resid || K <= 2048);
 }
 
 quads_status launch_gemm_dense(const GemmParams& p, const GemmMaps& m, int n_sms, cudaStream_t stream) {
   const DensePlan d = plan_dense(p.dense_rows, p.K, p.n_out, n_sms);
-  return d.bn == 128 ? launch_bn<128>(p, d.split, m, stream) : launch_bn<256>(p, d.split, m, stream);
+  return d.bn == 128 ? launch_bn<128>(p, d.split_log2, m, stream) : launch_bn<256>(p, d.split_log2, m, stream);
 }
 
 }  // namespace quads

@@ -216,7 +216,6 @@ bool gemm_swapped_ok(int64_t assignments, int n_experts, int m_tiles_max);
 quads_status launch_gemm_swapped(int epi, const GemmParams& p, const GemmMaps& m, int n_sms, cudaStream_t stream);
 
 // ---- gemm_dense.cu: dense projection with few output tiles, K split over clusters
-constexpr int kDenseMaxSplit = 8;
 bool gemm_dense_ok(int rows, int K, int N, int n_sms);
 bool gemm_dense_ahead_of_pairs(int rows, int K, int N, bool resid, int n_sms);
 quads_status launch_gemm_dense(const GemmParams& p, const GemmMaps& m, int n_sms, cudaStream_t stream);
