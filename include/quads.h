@@ -219,8 +219,9 @@ quads_status quads_fake_quant_weights_noalloc(const void* w, int64_t n_tensors, 
  * The call allocates nothing, never synchronises the host and enqueues all of
  * its work on `cuda_stream`, so it can be captured into a CUDA graph (make one
  * ordinary call first: kernel attributes are set on first use).  Beyond a few
- * hundred tokens its first kernel is a cooperative launch whose thread blocks
- * meet at counters.  Device-side waits are bounded; one that gives up writes
+ * hundred tokens its first kernel (in dense mode: the quantization, from 8 M
+ * elements of x on) is a cooperative launch whose thread blocks meet at
+ * counters.  Device-side waits are bounded; one that gives up writes
  * QUADS_ERR_TIMEOUT to a status word in the workspace, read with
  * quads_moe_async_status().  Every call resets that word on its stream before
  * its first kernel or in it: poll after each call whose status matters.  The
